@@ -3,8 +3,9 @@
 // One thread per output site and right-hand side.  Each of the 8 hops loads the
 // neighbour spinor, projects it to a 2-spin half spinor with (1 -/+ gamma_mu) in the
 // chiral basis, multiplies by U_mu(x) or U_mu(x-mu)^dag, and reconstructs the lower
-// spin pair from the upper one.  Spinor loads are 16-byte vector loads of the
-// [site][spin][colour] layout; links are read through the read-only path.
+// spin pair from the upper one.  Spinor loads are 32-byte vector loads of the
+// [site][spin][colour] layout (16-byte where the fields are only so aligned); links are read
+// through the read-only path.
 #include <cstring>
 #include <type_traits>
 
@@ -27,28 +28,9 @@ dslash_kernel(typename S::elem* __restrict__ out, const typename S::elem* __rest
               size_t in_stride, size_t out_stride) {
   dep_entry();
   typedef typename S::real R;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nsites) return;
-  size_t rhs = blockIdx.y;
-  int site;
-  if (parity < 0) {
-    site = i;
-  } else {
-    int s0 = 2 * i;
-    int x0 = s0 % g.L[0];
-    int rest = s0 / g.L[0];
-    int y = rest % g.L[1];
-    int z = (rest / g.L[1]) % g.L[2];
-    int t = rest / (g.L[1] * g.L[2]);
-    site = s0 + (((x0 + y + z + t) & 1) != parity ? 1 : 0);
-  }
-  int c[4];
-  c[0] = site % g.L[0];
-  int rest = site / g.L[0];
-  c[1] = rest % g.L[1];
-  rest /= g.L[1];
-  c[2] = rest % g.L[2];
-  c[3] = rest / g.L[2];
+  const size_t rhs = blockIdx.y;
+  int i, site, c[4];
+  if (!stencil_work(g, parity, nsites, threadIdx.x, TPB, i, site, c)) return;
   cplx<R> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
@@ -90,18 +72,15 @@ dslash_split_kernel(typename S::elem* __restrict__ out, const typename S::elem* 
   typedef typename S::real R;
   __shared__ cplx<R> sacc[12][64];
   const int half = threadIdx.x >> 6, ls = threadIdx.x & 63;
-  const int i = blockIdx.x * 64 + ls;
-  const bool active = i < nsites;
+  int i = 0, site = 0, c[4] = {0, 0, 0, 0};
+  const bool active = stencil_work(g, parity, nsites, ls, 64, i, site, c);
   const size_t rhs = blockIdx.y;
   const bool half_in = parity >= 0;
   const size_t in_off = rhs * in_stride;
   cplx<R> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
-  int site = 0;
-  int c[4] = {0, 0, 0, 0};
   if (active) {
-    site = stencil_site(g, parity, i, c);
     if (half == 0) {
       hop_fwd<0, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
       hop_fwd<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
@@ -141,81 +120,109 @@ dslash_split_kernel(typename S::elem* __restrict__ out, const typename S::elem* 
   }
 }
 
-// Launch shapes: threads per CTA and the minimum resident CTAs per SM requested from
-// the register allocator (register cap = 64K / (TPB * MINB)).  The autotuner below
-// picks one per (dtype, parity, dagger, volume, nrhs).
-struct Shape {
-  int tpb, minb;
-};
-constexpr Shape kShapes[] = {{128, 1}, {128, 6}, {128, 8}, {256, 4}, {64, 16}, {128, 0},
-                             {128, 0}, {128, 0}};
-// entry 5 is the two-threads-per-site kernel (dslash_split_kernel); entries 6 and 7 take
-// 2 and 4 right-hand sides per thread (dslash_mrhs_kernel), candidates only when nrhs > 1
-constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
-constexpr int kNumSingle = 6;
+// Launch variants of an aligned call, searched by the autotuner per (dtype, layout, parity,
+// dagger, volume, nrhs): 0 and 1 one site per thread, 128 threads, registers uncapped and capped
+// at 128; 2 two threads per site (dslash_split_kernel); 3 one site per thread at 80 registers; 4
+// and 5 take 2 and 4 right-hand sides per thread (dslash_mrhs_kernel), candidates only when nrhs
+// > 1.  Complex double stops at 2: its later forms spill kilobytes per thread.
+constexpr int kNumVariants = 6, kNumSingle = 4, kNumF64 = 3;
 
-template <typename S, int DAG, int TPB, int MINB, int LL>
+template <typename S, int DAG, int MINB, int LL>
 void launch_shape(void* out, const void* in, const void* links, const KGeom& k, int parity,
                   int nsites, int nrhs, cudaStream_t st, size_t in_stride, size_t out_stride) {
   typedef typename S::elem E;
-  dim3 grid((nsites + TPB - 1) / TPB, nrhs);
-  launch_dep(dslash_kernel<S, DAG, TPB, MINB, LL>, grid, TPB, 0, st, (E*)out, (const E*)in, (const E*)links, k, parity, nsites, in_stride, out_stride);
+  dim3 grid(stencil_ctas(k.tile, nsites, 128), nrhs);
+  launch_dep(dslash_kernel<S, DAG, 128, MINB, LL>, grid, 128, 0, st, (E*)out, (const E*)in,
+             (const E*)links, k, parity, nsites, in_stride, out_stride);
 }
 
 template <typename S, int DAG, int LL>
 void launch_variant(int v, void* out, const void* in, const void* links, const KGeom& k,
                     int parity, int nsites, int nrhs, cudaStream_t st, size_t is, size_t os) {
-  switch (v) {
-    case 1: launch_shape<S, DAG, 128, 6, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os); break;
-    case 2: launch_shape<S, DAG, 128, 8, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os); break;
-    case 3: launch_shape<S, DAG, 256, 4, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os); break;
-    case 4: launch_shape<S, DAG, 64, 16, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os); break;
-    case 5: {
-      typedef typename S::elem E;
-      dim3 grid((nsites + 63) / 64, nrhs);
-      launch_dep(dslash_split_kernel<S, DAG, LL>, grid, 128, 0, st, (E*)out, (const E*)in,
-                 (const E*)links, k, parity, nsites, is, os);
-      break;
-    }
-    case 6: launch_dslash_mrhs<S>(2, DAG, LL, out, in, links, k, parity, nsites, nrhs, st, is, os); break;
-    case 7: launch_dslash_mrhs<S>(4, DAG, LL, out, in, links, k, parity, nsites, nrhs, st, is, os); break;
-    default: launch_shape<S, DAG, 128, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os); break;
+  if (v == 2) {
+    typedef typename S::elem E;
+    KGeom k64 = k;
+    k64.tile = pick_tile(k.L, parity, 64);
+    dim3 grid(stencil_ctas(k64.tile, nsites, 64), nrhs);
+    launch_dep(dslash_split_kernel<S, DAG, LL>, grid, 128, 0, st, (E*)out, (const E*)in,
+               (const E*)links, k64, parity, nsites, is, os);
+    return;
   }
+  if constexpr (!std::is_same<S, StC128>::value) {
+    if (v == 3) return launch_shape<S, DAG, 6, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os);
+    if (v >= 4)
+      return launch_dslash_mrhs<S>(v == 4 ? 2 : 4, DAG, LL, out, in, links, k, parity, nsites, nrhs, st, is, os);
+  }
+  if (v == 1) launch_shape<S, DAG, 4, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os);
+  else launch_shape<S, DAG, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os);
 }
 
-template <typename S>
+template <typename S, int LL>
+void launch_dag(int v, int dagger, void* out, const void* in, const void* links, const KGeom& k,
+                int parity, int nsites, int nrhs, cudaStream_t st, size_t is, size_t os) {
+  if (dagger) launch_variant<S, 1, LL>(v, out, in, links, k, parity, nsites, nrhs, st, is, os);
+  else launch_variant<S, 0, LL>(v, out, in, links, k, parity, nsites, nrhs, st, is, os);
+}
+
+// S: the storage type; SN: its form for fields that are only 16-byte aligned (or, where the ABI
+// links are not 16-byte aligned, for links read element by element): one launch shape.
+template <typename S, typename SN>
 int launch_typed(void* out, const void* in, const void* links, const Geom& g, int parity,
                  int dagger, int nrhs, cudaStream_t st, size_t in_stride, size_t out_stride,
                  int dtype, int layout, const void* subf) {
+  constexpr bool f64 = std::is_same<S, StC128>::value;
+  constexpr bool site32 = !std::is_same<S, SN>::value;   // 32-byte site accesses
+  if (layout == 2 && f64)
+    return fail(MG_EINVAL, "dslash: two-row links are not used with complex double fields");
   KGeom k = to_kgeom(g);
   k.sub = parity >= 0 ? subf : nullptr;
+  k.tile = pick_tile(g.L, parity, 128);
   int nsites = parity < 0 ? g.V : g.V / 2;
-  auto run = [&](int v) {
-    if (layout == 0) {
-      if (dagger) launch_variant<S, 1, 0>(v, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else launch_variant<S, 0, 0>(v, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-    } else if (layout == 1) {
-      if (dagger) launch_variant<S, 1, 1>(v, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else launch_variant<S, 0, 1>(v, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-    } else if constexpr (!std::is_same<S, StC128>::value) {
-      // two stored rows (FP32 and half storage only: the FP64 stencil is bound by its FMA
-      // rate, where rebuilding the third row would cost more than the bytes it saves)
-      if (dagger) launch_variant<S, 1, 2>(v, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else launch_variant<S, 0, 2>(v, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-    }
-  };
-  if (layout == 2 && std::is_same<S, StC128>::value)
-    return fail(MG_EINVAL, "dslash: two-row links are not used with complex double fields");
-  int v = tuned_variant(dtype + 16 * layout, parity, dagger, g.V, nrhs, st,
-                        nrhs > 1 ? kNumShapes : kNumSingle, run);
-  if (v < 0) return fail(MG_ECUDA, "dslash autotune failed");
+  const size_t es = sizeof(typename S::elem);
+  uintptr_t al = (uintptr_t)out | (uintptr_t)in | (uintptr_t)k.sub;
+  if (nrhs > 1) al |= (in_stride * es) | (out_stride * es);
+  bool wide = !site32 || (al & 31) == 0;
+  // the windowed link loads (load_link, LL = 3) start at a 16-byte boundary
+  if (layout == 0 && !f64) wide = wide && ((uintptr_t)links & 15) == 0;
   // algorithmic bytes: in + out spinors per rhs and each link once (parity: all 4V links),
   // 18 reals per link whatever the stored form
   double real_bytes = (double)sizeof(typename S::real) * (sizeof(typename S::elem) == 4 ? 0.5 : 1.0);
   double per_site = parity < 0 ? 48.0 * nrhs + 72.0 : 48.0 * nrhs + 144.0;
-  ProfScope ps(dtype == MG_C128 ? "dslash_c128" : dtype == MG_C64 ? "dslash_c64"
-               : dtype == MG_F16 ? "dslash_f16" : "dslash_bf16",
-               per_site * real_bytes * nsites, 1320.0 * nsites * nrhs, st);
+  const char* name = dtype == MG_C128 ? "dslash_c128" : dtype == MG_C64 ? "dslash_c64"
+                     : dtype == MG_F16 ? "dslash_f16" : "dslash_bf16";
+  const double pbytes = per_site * real_bytes * nsites, pflops = 1320.0 * nsites * nrhs;
+  if (!wide) {
+    ProfScope ps(name, pbytes, pflops, st);
+    const bool d = dagger != 0;
+    auto one = [&](auto ll) {
+      constexpr int LL = decltype(ll)::value;
+      if (d) launch_shape<SN, 1, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+      else launch_shape<SN, 0, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+    };
+    if (layout == 0) one(std::integral_constant<int, 0>{});
+    if constexpr (site32) {
+      if (layout == 1) one(std::integral_constant<int, 1>{});
+      if constexpr (!f64) if (layout == 2) one(std::integral_constant<int, 2>{});
+    }
+    WMG_LAUNCHED();
+    return MG_OK;
+  }
+  auto run = [&](int v) {
+    if constexpr (f64) {
+      if (layout == 0) launch_dag<S, 0>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+      else launch_dag<S, 1>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+    } else {
+      // two stored rows (FP32 and half storage only: the FP64 stencil is bound by its FMA
+      // rate, where rebuilding the third row would cost more than the bytes it saves)
+      if (layout == 0) launch_dag<S, 3>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+      else if (layout == 1) launch_dag<S, 1>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+      else launch_dag<S, 2>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+    }
+  };
+  int v = tuned_variant(dtype + 16 * layout, parity, dagger, g.V, nrhs, st,
+                        f64 ? kNumF64 : nrhs > 1 ? kNumVariants : kNumSingle, run);
+  if (v < 0) return fail(MG_ECUDA, "dslash autotune failed");
+  ProfScope ps(name, pbytes, pflops, st);
   run(v);
   WMG_LAUNCHED();
   return MG_OK;
@@ -377,6 +384,77 @@ int su3_deviation_df(double* dev_out, const zdf* links, size_t nlinks, cudaStrea
   return MG_OK;
 }
 
+namespace stencil {
+
+// The tile of at most `most` sites with the least L2 -> L1 traffic per site: its own spinors, the
+// 2 / t_mu neighbours outside it in every direction it does not span, and the links' part-used
+// 32-byte sectors, times the idle lanes of its last warp.  Consecutive sites are the tile's rival:
+// `most` of them span x, and y as far as they reach.
+TileMap pick_tile(const int L[4], int parity, int most) {
+  struct Key {
+    int L[4], half, most;
+  };
+  struct Entry {
+    Key k;
+    TileMap m;
+  };
+  // the last few answers of this thread (a solver asks for the same two lattices again and again)
+  static thread_local Entry cache[4];
+  static thread_local int used = 0, next = 0;
+  const Key key = {{L[0], L[1], L[2], L[3]}, parity >= 0 ? 1 : 0, most};
+  for (int i = 0; i < used; ++i)
+    if (std::memcmp(&cache[i].k, &key, sizeof(Key)) == 0) return cache[i].m;
+  const int E[4] = {key.half ? L[0] / 2 : L[0], L[1], L[2], L[3]};
+  auto halo = [](int t, int e) { return t == e ? 0.0 : 2.0 / t; };
+  TileMap m;
+  // consecutive sites: rows of x, then of y, inside one CTA
+  const int lx = E[0] < most ? E[0] : most;
+  const int ly = E[0] < most ? (most / E[0] < E[1] ? most / E[0] : E[1]) : 1;
+  double best = 96.0 * (1.0 + halo(lx, E[0]) + halo(ly, E[1]) + halo(1, E[2]) + halo(1, E[3])) +
+                384.0 + 192.0 / lx;
+  const int xmin = E[0] < 8 ? E[0] : 8;
+  for (int a = xmin; a <= E[0] && a <= most; ++a) {
+    if (E[0] % a) continue;
+    for (int b = 1; b <= E[1] && a * b <= most; ++b) {
+      if (E[1] % b) continue;
+      for (int c = 1; c <= E[2] && a * b * c <= most; ++c) {
+        if (E[2] % c) continue;
+        for (int d = 1; d <= E[3] && a * b * c * d <= most; ++d) {
+          if (E[3] % d) continue;
+          const int n = a * b * c * d;
+          const double links = (a % 4 ? (8.0 * a + 24.0) / (8.0 * a) : 1.0) + 0.5 / a;
+          const double cost = (96.0 * (1.0 + halo(a, E[0]) + halo(b, E[1]) + halo(c, E[2]) +
+                                       halo(d, E[3])) + 384.0 * links) *
+                              ((n + 31) / 32 * 32) / n;
+          if (cost < best - 1e-9) {
+            best = cost;
+            m.on = 1;
+            m.t[0] = a; m.t[1] = b; m.t[2] = c; m.t[3] = d;
+          }
+        }
+      }
+    }
+  }
+  if (m.on) {
+    m.sites = m.t[0] * m.t[1] * m.t[2] * m.t[3];
+    const long long tiles = (long long)E[0] * E[1] * E[2] * E[3] / m.sites;
+    for (int a = 0; a < 3; ++a) {
+      m.n[a] = E[a] / m.t[a];
+      // u / t = (u tm) >> 16 for u t < 2^16 (u, t <= 128); b / n = high word of b nm for
+      // b n < 2^32
+      m.tm[a] = (65536u + m.t[a] - 1) / m.t[a];
+      m.nm[a] = m.n[a] == 1 ? 0u : 0xffffffffu / (unsigned)m.n[a] + 1u;
+      if (tiles * m.n[a] >= (1LL << 32)) m.on = 0;
+    }
+  }
+  cache[next] = {key, m};
+  next = (next + 1) % 4;
+  if (used < 4) ++used;
+  return m;
+}
+
+}  // namespace stencil
+
 int dslash_launch(int dtype, void* out, const void* in, const void* links, const Geom& g,
                   int parity, int dagger, int nrhs, cudaStream_t st, size_t in_stride,
                   size_t out_stride, int link_layout, const void* sub) {
@@ -385,16 +463,16 @@ int dslash_launch(int dtype, void* out, const void* in, const void* links, const
   if (out_stride == 0) out_stride = half;
   switch (dtype) {
     case MG_C128:
-      return launch_typed<StC128>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
+      return launch_typed<StC128, StC128N>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
                                   link_layout, sub);
     case MG_C64:
-      return launch_typed<StC64>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
+      return launch_typed<StC64, StC64N>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
                                   link_layout, sub);
     case MG_F16:
-      return launch_typed<StF16>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
+      return launch_typed<StF16, StF16>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
                                   link_layout, sub);
     case MG_BF16:
-      return launch_typed<StBF16>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
+      return launch_typed<StBF16, StBF16>(out, in, links, g, parity, dagger, nrhs, st, in_stride, out_stride, dtype,
                                   link_layout, sub);
   }
   return fail(MG_EINVAL, "dslash: unknown dtype");

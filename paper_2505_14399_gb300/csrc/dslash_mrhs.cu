@@ -35,10 +35,8 @@ __device__ __forceinline__ void hop_fwd_m(const KGeom& g, int site, const int c[
       cplx<R> p[12], h[6], gg[6];
       SiteIO<S>::load(in + (r < nr ? r : nr - 1) * in_stride, idx, p);
       project<MU, SF, R>(p, h);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) h[i] = cf * h[i];
       mul_link<R>(u, h, gg);
-      accumulate<MU, SF, R>(acc[r], gg);
+      accumulate<MU, SF, R>(acc[r], gg, cf);
     }
   }
 }
@@ -64,10 +62,8 @@ __device__ __forceinline__ void hop_bwd_m(const KGeom& g, int site, const int c[
       cplx<R> p[12], h[6], gg[6];
       SiteIO<S>::load(in + (r < nr ? r : nr - 1) * in_stride, idx, p);
       project<MU, SB, R>(p, h);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) h[i] = cf * h[i];
       mul_link_dag<R>(u, h, gg);
-      accumulate<MU, SB, R>(acc[r], gg);
+      accumulate<MU, SB, R>(acc[r], gg, cf);
     }
   }
 }
@@ -81,12 +77,10 @@ dslash_mrhs_kernel(typename S::elem* __restrict__ out, const typename S::elem* _
                    int nrhs, size_t in_stride, size_t out_stride) {
   dep_entry();
   typedef typename S::real R;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nsites) return;
+  int i, site, c[4];
+  if (!stencil_work(g, parity, nsites, threadIdx.x, 128, i, site, c)) return;
   const int r0 = blockIdx.y * NR;
   const int nr = min(NR, nrhs - r0);
-  int c[4];
-  const int site = stencil_site(g, parity, i, c);
   const bool half_in = parity >= 0;
   const typename S::elem* inr = in + (size_t)r0 * in_stride;
   cplx<R> acc[NR][12];
@@ -131,7 +125,7 @@ template <typename S, int DAG, int NR, int LL, int MINB>
 void launch_nr(void* out, const void* in, const void* links, const KGeom& k, int parity,
                int nsites, int nrhs, cudaStream_t st, size_t is, size_t os) {
   typedef typename S::elem E;
-  dim3 grid((nsites + 127) / 128, (nrhs + NR - 1) / NR);
+  dim3 grid(stencil_ctas(k.tile, nsites, 128), (nrhs + NR - 1) / NR);
   launch_dep(dslash_mrhs_kernel<S, DAG, NR, LL, MINB>, grid, 128, 0, st, (E*)out, (const E*)in,
              (const E*)links, k, parity, nsites, nrhs, is, os);
 }
@@ -153,20 +147,16 @@ template <typename S>
 void launch_dslash_mrhs(int nr, int dagger, int layout, void* out, const void* in,
                         const void* links, const KGeom& k, int parity, int nsites, int nrhs,
                         cudaStream_t st, size_t is, size_t os) {
-  if (layout == 0) {
-    if (dagger) launch_dl<S, 1, 0>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
-    else launch_dl<S, 0, 0>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
-  } else if (layout == 1) {
-    if (dagger) launch_dl<S, 1, 1>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
-    else launch_dl<S, 0, 1>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
-  } else if constexpr (!std::is_same<S, StC128>::value) {
-    if (dagger) launch_dl<S, 1, 2>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
-    else launch_dl<S, 0, 2>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
-  }
+  auto go = [&](auto ll) {
+    constexpr int LL = decltype(ll)::value;
+    if (dagger) launch_dl<S, 1, LL>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
+    else launch_dl<S, 0, LL>(nr, out, in, links, k, parity, nsites, nrhs, st, is, os);
+  };
+  if (layout == 1) go(std::integral_constant<int, 1>{});
+  else if (layout == 2) go(std::integral_constant<int, 2>{});
+  else go(std::integral_constant<int, 3>{});
 }
 
-template void launch_dslash_mrhs<StC128>(int, int, int, void*, const void*, const void*,
-                                         const KGeom&, int, int, int, cudaStream_t, size_t, size_t);
 template void launch_dslash_mrhs<StC64>(int, int, int, void*, const void*, const void*,
                                         const KGeom&, int, int, int, cudaStream_t, size_t, size_t);
 template void launch_dslash_mrhs<StF16>(int, int, int, void*, const void*, const void*,

@@ -508,13 +508,11 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   for (int q = 0; q < NVM; ++q) { ar[q] = 0.f; ai[q] = 0.f; }
   float ss = 0.f;
   // one site per thread (the launcher sizes the grid to cover every site): with no loop the
-  // projection accumulators are not live across the stencil's hops, which need the registers
-  const int site = blockIdx.x * BT + threadIdx.x;
-  if (site < nsites) {
-    int c[4];
-    // site: the output index (lexicographic, or the checkerboard index with par); ls: the
-    // lattice site the hops start from
-    const int ls = stencil_site(g, par ? 0 : -1, site, c);
+  // projection accumulators are not live across the stencil's hops, which need the registers.
+  // site: the output index (lexicographic, or the checkerboard index with par); ls: the lattice
+  // site the hops start from
+  int site, ls, c[4];
+  if (stencil_work(g, par ? 0 : -1, nsites, threadIdx.x, BT, site, ls, c)) {
     zf acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = {0.f, 0.f};
@@ -578,45 +576,37 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   }
 }
 
-// launch shapes of the fused kernel: threads per CTA and resident CTAs per SM asked of the
-// register allocator (register cap 64K / (BT MINB), allocated in steps of 8): 256 x 2 and
-// 128 x 4 (128 registers), 128 x 5 (96), 128 x 6 (80; spills 12-64 bytes per thread).
-constexpr int kProjShapes = 4;
-
-template <int NVM, bool FIRST, int LL, int BT, int MINB>
-void launch_proj_shape(int nv, int V, int nblk, int nrhs, cudaStream_t st, zf* w, zf* V_,
-                       size_t fs, size_t n, const float2* L32, const stencil::KGeom& kg, zd* small,
-                       SmallLayout L, double* dnorm, ReduceWork& rw, const zf* b0,
-                       const double* beta0, const zf* sin, int par, cudaError_t* err) {
-  const int ns = par ? V / 2 : V;
-  const int nb = (ns + BT - 1) / BT;   // one site per thread; launch_proj checked nb <= nblk
-  *err = launch_dep(dslash_proj_kernel<NVM, FIRST, LL, BT, MINB>, dim3(nb, nrhs), BT, 0, st, w,
-                    V_, fs, nv, n, L32, kg, small, L, dnorm, rw.partial, rw.counter, rw.maxvec,
-                    b0, beta0, sin, par);
-}
+// launch shapes of the fused kernel: 128 threads and 4, 5 or 6 resident CTAs per SM asked of the
+// register allocator (128, 96 or 80 registers).
+constexpr int kProjShapes = 3;
 
 template <int NVM, bool FIRST, int LL>
-void launch_proj_v(int v, int nv, int nrhs, cudaStream_t st, zf* w, zf* V_, size_t fs, size_t n,
+void launch_proj_v(int v, int nv, int nrhs, cudaStream_t st, zf* w, zf* V, size_t fs, size_t n,
                    const float2* L32, const stencil::KGeom& kg, zd* small, SmallLayout L,
                    double* dnorm, ReduceWork& rw, const zf* b0, const double* beta0,
                    const zf* sin, int par, cudaError_t* err) {
-  switch (v) {
-    case 1: launch_proj_shape<NVM, FIRST, LL, 128, 4>(nv, kg.V, rw.cap, nrhs, st, w, V_, fs, n, L32, kg, small, L, dnorm, rw, b0, beta0, sin, par, err); break;
-    case 2: launch_proj_shape<NVM, FIRST, LL, 128, 5>(nv, kg.V, rw.cap, nrhs, st, w, V_, fs, n, L32, kg, small, L, dnorm, rw, b0, beta0, sin, par, err); break;
-    case 3: launch_proj_shape<NVM, FIRST, LL, 128, 6>(nv, kg.V, rw.cap, nrhs, st, w, V_, fs, n, L32, kg, small, L, dnorm, rw, b0, beta0, sin, par, err); break;
-    default: launch_proj_shape<NVM, FIRST, LL, 256, 2>(nv, kg.V, rw.cap, nrhs, st, w, V_, fs, n, L32, kg, small, L, dnorm, rw, b0, beta0, sin, par, err); break;
-  }
+  // one site per thread; launch_proj checked that the partial slots hold every CTA
+  const dim3 grid(stencil::stencil_ctas(kg.tile, par ? kg.V / 2 : kg.V, 128), nrhs);
+  auto go = [&](auto kernel) {
+    *err = launch_dep(kernel, grid, 128, 0, st, w, V, fs, nv, n, L32, kg, small, L, dnorm,
+                      rw.partial, rw.counter, rw.maxvec, b0, beta0, sin, par);
+  };
+  if (v == 1) go(dslash_proj_kernel<NVM, FIRST, LL, 128, 5>);
+  else if (v == 2) go(dslash_proj_kernel<NVM, FIRST, LL, 128, 6>);
+  else go(dslash_proj_kernel<NVM, FIRST, LL, 128, 4>);
 }
 
 template <int LL>
 int launch_proj(int nv, bool first, int nrhs, cudaStream_t st, zf* w, zf* V, size_t fs,
-                size_t n, const float2* L32, const stencil::KGeom& kg, zd* small, SmallLayout L,
+                size_t n, const float2* L32, stencil::KGeom kg, zd* small, SmallLayout L,
                 double* dnorm, ReduceWork& rw, const zf* b0, const double* beta0, const zf* sin,
                 int par) {
   const int nvm = first ? 0 : nv <= 4 ? 4 : nv <= 8 ? 8 : 16;
-  // every shape takes one site per thread, so its grid (at least 128 threads per CTA) must
-  // fit the partial slots of the reduction workspace
+  // one site per thread: the grid must fit the partial slots of the reduction workspace, which
+  // hold a CTA per 128 consecutive sites; tiles of fewer sites are used where they fit as well
   const int ns = par ? kg.V / 2 : kg.V;
+  kg.tile = stencil::pick_tile(kg.L, par ? 0 : -1, 128);
+  if (stencil::stencil_ctas(kg.tile, ns, 128) > rw.cap) kg.tile.on = 0;
   if ((ns + 127) / 128 > rw.cap)
     return fail(MG_EINVAL, "dslash_proj: reduction workspace holds too few CTA partials");
   cudaError_t err = cudaSuccess;

@@ -11,10 +11,74 @@
 namespace wmg {
 namespace stencil {
 
-// 16-byte vector loads/stores of one site's 12 complex numbers.
+// 32-byte global accesses (sm_100 and later).  volatile: they stay behind the dependent-launch
+// wait of dep_entry() in program order.
+__device__ __forceinline__ void ld32(const void* p, float v[8]) {
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                 "=f"(v[6]), "=f"(v[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void st32(void* p, const float v[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]),
+               "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void ld32(const void* p, double v[4]) {
+  asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+               : "l"(p));
+}
+__device__ __forceinline__ void st32(void* p, const double v[4]) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]),
+               "d"(v[2]), "d"(v[3])
+               : "memory");
+}
+
+// Loads/stores of one site's 12 complex numbers (complex float: 96 bytes, complex double: 192).
+// Consecutive threads take consecutive sites, so a 16-byte load of a warp touches 32 half-used
+// sectors in 24 lines, and the stencil is bound by the L1's passes over them (80 % busy, DRAM
+// 41 %, ncu at 24^3x48).  32-byte accesses use every sector they touch: 201 -> 161 us per FP32
+// stencil at 32^3x64 (two-row links), 256 -> 208 us with ABI links.  They need 32-byte aligned
+// fields; StC64N / StC128N are the 16-byte forms for fields that are only 16-byte aligned.
 template <typename S> struct SiteIO;
 
-template <> struct SiteIO<StC128> {
+template <typename S> struct SiteIO32 {
+  typedef typename S::real R;
+  static constexpr int N = 32 / sizeof(R);        // reals per access
+  static __device__ __forceinline__ void load(const typename S::elem* p, size_t site,
+                                              cplx<R> v[12]) {
+    const char* q = reinterpret_cast<const char*>(p + site * 12);
+#pragma unroll
+    for (int i = 0; i < 24 / N; ++i) {
+      R t[N];
+      ld32(q + 32 * i, t);
+#pragma unroll
+      for (int j = 0; j < N / 2; ++j) v[i * (N / 2) + j] = {t[2 * j], t[2 * j + 1]};
+    }
+  }
+  static __device__ __forceinline__ void store(typename S::elem* p, size_t site,
+                                               const cplx<R> v[12]) {
+    char* q = reinterpret_cast<char*>(p + site * 12);
+#pragma unroll
+    for (int i = 0; i < 24 / N; ++i) {
+      R t[N];
+#pragma unroll
+      for (int j = 0; j < N / 2; ++j) {
+        t[2 * j] = v[i * (N / 2) + j].re;
+        t[2 * j + 1] = v[i * (N / 2) + j].im;
+      }
+      st32(q + 32 * i, t);
+    }
+  }
+};
+template <> struct SiteIO<StC128> : SiteIO32<StC128> {};
+template <> struct SiteIO<StC64> : SiteIO32<StC64> {};
+
+// 16-byte forms
+struct StC128N : StC128 {};
+struct StC64N : StC64 {};
+template <> struct SiteIO<StC128N> {
   static __device__ __forceinline__ void load(const double2* p, size_t site, zd v[12]) {
     const double2* q = p + site * 12;
 #pragma unroll
@@ -26,7 +90,7 @@ template <> struct SiteIO<StC128> {
     for (int i = 0; i < 12; ++i) q[i] = make_double2(v[i].re, v[i].im);
   }
 };
-template <> struct SiteIO<StC64> {
+template <> struct SiteIO<StC64N> {
   static __device__ __forceinline__ void load(const float2* p, size_t site, zf v[12]) {
     const float4* q = reinterpret_cast<const float4*>(p + site * 12);
 #pragma unroll
@@ -74,28 +138,67 @@ template <> struct SiteIO<StBF16> : SiteIOHalf<__nv_bfloat162, StBF16> {};
 // consecutive sites touches one contiguous 32 x element_size span (the solver's copy);
 // LL = 2: the same with the first two rows only, [mu][6 entry][site]: for U in SU(3) the rows
 // are orthonormal and det U = 1, so the third row is the complex conjugate of the cross
-// product of the first two (12 of the 18 reals cross HBM).
+// product of the first two (12 of the 18 reals cross HBM);
+// LL = 3: ABI layout of 4- or 8-byte elements with a 16-byte aligned base: the aligned 16-byte
+// pieces that cover the link (5 of a 72-byte link that starts at 0 or 8 mod 16, 3 of a 36-byte
+// link that starts at 0, 4, 8 or 12 mod 16) instead of nine element loads, then a select by the
+// offset (208 -> 205 us at 32^3x64 in FP32, 18.4 -> 16.5 us at 16^3x32).  The window never
+// leaves the array: 4 V is a multiple of 4, so the first link starts and the last one ends on a
+// 16-byte boundary.
 template <typename S, int LL>
 __device__ __forceinline__ void load_link(const typename S::elem* L, int V, int mu, int site,
                                           cplx<typename S::real> u[9]) {
-  if (LL == 0) {
+  if constexpr (LL == 0) {
     size_t idx = ((size_t)mu * V + site) * 9;
 #pragma unroll
     for (int i = 0; i < 9; ++i) u[i] = S::ld(L, idx + i);
-  } else if (LL == 1) {
+  } else if constexpr (LL == 1) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) u[i] = S::ld(L, ((size_t)mu * 9 + i) * V + site);
-  } else {
+  } else if constexpr (LL == 2) {
 #pragma unroll
     for (int i = 0; i < 6; ++i) u[i] = S::ld(L, ((size_t)mu * 6 + i) * V + site);
     u[6] = conj(u[1] * u[5] - u[2] * u[4]);
     u[7] = conj(u[2] * u[3] - u[0] * u[5]);
     u[8] = conj(u[0] * u[4] - u[1] * u[3]);
+  } else if constexpr (sizeof(typename S::elem) == 8) {
+    const size_t e0 = ((size_t)mu * V + site) * 9;   // first element of the link
+    const bool odd = (e0 & 1) != 0;
+    const float4* q = reinterpret_cast<const float4*>(L) + (e0 >> 1);
+    float w[20];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      float4 t = __ldg(q + i);
+      w[4 * i] = t.x; w[4 * i + 1] = t.y; w[4 * i + 2] = t.z; w[4 * i + 3] = t.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      u[i] = {odd ? w[2 * i + 2] : w[2 * i], odd ? w[2 * i + 3] : w[2 * i + 1]};
+  } else {
+    const size_t e0 = ((size_t)mu * V + site) * 9;
+    const int off = (int)(e0 & 3);
+    const uint4* q = reinterpret_cast<const uint4*>(L) + (e0 >> 2);
+    unsigned w[12], x[11];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      uint4 t = __ldg(q + i);
+      w[4 * i] = t.x; w[4 * i + 1] = t.y; w[4 * i + 2] = t.z; w[4 * i + 3] = t.w;
+    }
+    // shift by off = 2 b1 + b0 elements
+#pragma unroll
+    for (int i = 0; i < 11; ++i) x[i] = (off & 1) ? w[i + 1] : w[i];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      typename S::elem h;
+      const unsigned v = (off & 2) ? x[i + 2] : x[i];
+      memcpy(&h, &v, 4);
+      u[i] = S::ld(&h, 0);
+    }
   }
 }
 
-// Project psi with (1 + s gamma_mu) to the upper spin pair h (2 spins x 3 colours),
-// scaled by c.  mu = 0,1,2: h = psi_up - s i sigma_mu psi_dn; mu = 3: h = psi_up + s psi_dn.
+// Project psi with (1 + s gamma_mu) to the upper spin pair h (2 spins x 3 colours).
+// mu = 0,1,2: h = psi_up - s i sigma_mu psi_dn; mu = 3: h = psi_up + s psi_dn.
 template <int MU, int SGN, typename R>
 __device__ __forceinline__ void project(const cplx<R> p[12], cplx<R> h[6]) {
 #pragma unroll
@@ -116,22 +219,29 @@ __device__ __forceinline__ void project(const cplx<R> p[12], cplx<R> h[6]) {
   }
 }
 
-// acc += (1 + s gamma_mu) reconstructed from the transported half spinor g:
-// upper = g; lower = s i sigma_mu g (mu < 3) or s g (mu = 3).
+// acc += c (1 + s gamma_mu) reconstructed from the transported half spinor g:
+// upper = g; lower = s i sigma_mu g (mu < 3) or s g (mu = 3).  The hop's coefficient c (weight
+// and boundary phase) rides on the multiply-adds: scaling the half spinor first would be 12
+// multiplications more per hop (a tenth of the FP64 stencil's instructions).
 template <int MU, int SGN, typename R>
-__device__ __forceinline__ void accumulate(cplx<R> acc[12], const cplx<R> g[6]) {
+__device__ __forceinline__ void accumulate(cplx<R> acc[12], const cplx<R> g[6], R c) {
+  const R cs = SGN > 0 ? c : -c;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    cplx<R> g0 = g[c], g1 = g[3 + c];
-    acc[0 * 3 + c] += g0;
-    acc[1 * 3 + c] += g1;
+  for (int i = 0; i < 3; ++i) {
+    cplx<R> g0 = g[i], g1 = g[3 + i];
     cplx<R> a, b;  // i sigma g or g
     if (MU == 0) { a = ti(g1); b = ti(g0); }
     else if (MU == 1) { a = g1; b = -g0; }
     else if (MU == 2) { a = ti(g0); b = tmi(g1); }
     else { a = g0; b = g1; }
-    if (SGN > 0) { acc[2 * 3 + c] += a; acc[3 * 3 + c] += b; }
-    else { acc[2 * 3 + c] -= a; acc[3 * 3 + c] -= b; }
+    acc[i].re = fma(c, g0.re, acc[i].re);
+    acc[i].im = fma(c, g0.im, acc[i].im);
+    acc[3 + i].re = fma(c, g1.re, acc[3 + i].re);
+    acc[3 + i].im = fma(c, g1.im, acc[3 + i].im);
+    acc[6 + i].re = fma(cs, a.re, acc[6 + i].re);
+    acc[6 + i].im = fma(cs, a.im, acc[6 + i].im);
+    acc[9 + i].re = fma(cs, b.re, acc[9 + i].re);
+    acc[9 + i].im = fma(cs, b.im, acc[9 + i].im);
   }
 }
 
@@ -161,6 +271,19 @@ __device__ __forceinline__ void mul_link_dag(const cplx<R> u[9], const cplx<R> h
     }
 }
 
+// Sites of a CTA.  Off: consecutive sites.  On: a tile of t0 x t1 x t2 x t3 sites (t0 in half
+// sites for a single-parity stencil), so that neighbours in y, z and t come from the CTA's own
+// L1 lines more often: the L2 -> L1 traffic of a 128-site tile of a 16^3x32 lattice is 4 spinors
+// per site instead of 5-6 (18.6 -> 18.0 us cold, 14.5 -> 12.5 us warm per FP32 stencil there,
+// 164 -> 162 us at 32^3x64).  Chosen on the host by pick_tile.
+struct TileMap {
+  int on = 0;
+  int sites = 0;          // t0 t1 t2 t3
+  int t[4];               // tile extents
+  int n[3];               // tiles along the first three axes
+  unsigned tm[3], nm[3];  // reciprocals of t[0..2] (16 bit) and n[0..2] (32 bit, 0 for 1)
+};
+
 struct KGeom {
   int L[4];
   int stride[4];
@@ -172,6 +295,7 @@ struct KGeom {
   // single-parity form only: when set, out_p = sub_p - (-kappa H_{p,1-p} in) (the even-odd
   // Schur complement and its source / reconstruction steps), sub with out's layout and stride
   const void* sub = nullptr;
+  TileMap tile;
 };
 
 // res <- sub[rhs][i] - res for the single-parity form with a subtrahend field
@@ -197,11 +321,9 @@ __device__ __forceinline__ void hop_fwd(const KGeom& g, int site, const int c[4]
   cplx<R> p[12], h[6], gg[6], u[9];
   SiteIO<S>::load(in + in_off, half_in ? (size_t)(nb >> 1) : (size_t)nb, p);
   project<MU, SF, R>(p, h);
-#pragma unroll
-  for (int i = 0; i < 6; ++i) h[i] = cf * h[i];
   load_link<S, LL>(links, g.V, MU, site, u);
   mul_link<R>(u, h, gg);
-  accumulate<MU, SF, R>(acc, gg);
+  accumulate<MU, SF, R>(acc, gg, cf);
 }
 
 // backward hop of direction MU: (1 + SB gamma) U_mu(x - mu)^dag psi(x - mu)
@@ -218,11 +340,9 @@ __device__ __forceinline__ void hop_bwd(const KGeom& g, int site, const int c[4]
   cplx<R> p[12], h[6], gg[6], u[9];
   SiteIO<S>::load(in + in_off, half_in ? (size_t)(nb >> 1) : (size_t)nb, p);
   project<MU, SB, R>(p, h);
-#pragma unroll
-  for (int i = 0; i < 6; ++i) h[i] = cf * h[i];
   load_link<S, LL>(links, g.V, MU, nb, u);
   mul_link_dag<R>(u, h, gg);
-  accumulate<MU, SB, R>(acc, gg);
+  accumulate<MU, SB, R>(acc, gg, cf);
 }
 
 template <int MU, int DAG, typename S, int LL>
@@ -258,6 +378,40 @@ __device__ __forceinline__ int stencil_site(const KGeom& g, int parity, int i, i
   return site;
 }
 
+// Work item of thread `u` (of `per` sites per CTA) in CTA blockIdx.x: output index i (the site,
+// or the checkerboard index of a single-parity stencil), lattice site and coordinates; false when
+// there is none.
+__device__ __forceinline__ bool stencil_work(const KGeom& g, int parity, int nsites, int u, int per,
+                                             int& i, int& site, int c[4]) {
+  const TileMap& m = g.tile;
+  if (!m.on) {
+    i = blockIdx.x * per + u;
+    if (i >= nsites) return false;
+    site = stencil_site(g, parity, i, c);
+    return true;
+  }
+  if (u >= m.sites) return false;
+  unsigned r = (unsigned)u, b = blockIdx.x;
+  int x[4];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const unsigned q = (r * m.tm[a]) >> 16;
+    const unsigned bq = m.nm[a] ? __umulhi(b, m.nm[a]) : b;
+    x[a] = (int)(b - bq * m.n[a]) * m.t[a] + (int)(r - q * m.t[a]);
+    r = q;
+    b = bq;
+  }
+  x[3] = (int)b * m.t[3] + (int)r;
+  const int row = x[1] + g.L[1] * (x[2] + g.L[2] * x[3]);
+  c[0] = parity < 0 ? x[0] : 2 * x[0] + ((x[1] + x[2] + x[3] + parity) & 1);
+  c[1] = x[1];
+  c[2] = x[2];
+  c[3] = x[3];
+  site = c[0] + g.L[0] * row;
+  i = parity < 0 ? site : site >> 1;
+  return true;
+}
+
 template <typename S>
 __device__ __forceinline__ void apply_sub(const KGeom& g, size_t rhs_off, int i,
                                           cplx<typename S::real> res[12]) {
@@ -285,8 +439,16 @@ inline KGeom to_kgeom(const Geom& g) {
   return k;
 }
 
-// Stencil with 2 or 4 right-hand sides per thread (nr), defined in dslash_mrhs.cu for the four
-// storage types; layout 0: ABI links, 1: lane-contiguous links.
+// Tile of at most `most` sites for the stencil of the given parity (< 0: full lattice); off when
+// no tile beats consecutive sites (csrc/dslash.cu).
+TileMap pick_tile(const int L[4], int parity, int most);
+// CTAs of a launch over nsites sites with `per` site slots per CTA
+inline int stencil_ctas(const TileMap& m, int nsites, int per) {
+  return m.on ? nsites / m.sites : (nsites + per - 1) / per;
+}
+
+// Stencil with 2 or 4 right-hand sides per thread (nr), defined in dslash_mrhs.cu for the
+// FP32-arithmetic storage types; layouts as load_link's LL.
 template <typename S>
 void launch_dslash_mrhs(int nr, int dagger, int layout, void* out, const void* in,
                         const void* links, const KGeom& k, int parity, int nsites, int nrhs,

@@ -77,3 +77,18 @@ def test_digit_products_accumulate_exactly_in_fp32():
     for d in range(7):
         w = F(2.0) ** F(-12 - 8 * d)
         assert float(w) == 2.0 ** (-12 - 8 * d) and np.isfinite(w) and w > np.finfo(F).tiny
+
+
+def test_tile_reciprocals_of_the_stencil_are_exact():
+    """u / t = (u ceil(2^16 / t)) >> 16 for thread indices u < 128 and tile extents t <= 128, and
+    b / n = high word of b (floor((2^32 - 1) / n) + 1) while b n < 2^32 (the CTA's tile index)."""
+    u = np.arange(128, dtype=np.int64)
+    for t in range(1, 129):
+        m = (65536 + t - 1) // t
+        assert np.array_equal((u * m) >> 16, u // t)
+    rng = np.random.default_rng(0)
+    for n in list(range(2, 200)) + [1000, 4096, 65535]:
+        m = 0xFFFFFFFF // n + 1
+        b = np.unique(np.concatenate([np.arange(min(4 * n, 4096)),
+                                      rng.integers(0, (2 ** 32 - 1) // n, 2000)])).astype(np.uint64)
+        assert np.array_equal((b * np.uint64(m)) >> np.uint64(32), b // np.uint64(n))
