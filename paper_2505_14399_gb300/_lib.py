@@ -5,6 +5,7 @@ The shared library is built in-tree by ``paper_2505_14399_gb300._build`` (or
 CPU fallback for any entry point.
 """
 import ctypes as C
+import functools
 import os
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -133,9 +134,21 @@ def check(status, where):
     return status
 
 
-def ivec(v):
+@functools.lru_cache(maxsize=256)
+def _ivec(v):
     return (C.c_int * 4)(*[int(x) for x in v])
 
 
-def dvec(v):
+@functools.lru_cache(maxsize=256)
+def _dvec(v):
     return (C.c_double * 4)(*[float(x) for x in v])
+
+
+def ivec(v):
+    """Four C ints; arrays of equal values are shared (the library only reads them)."""
+    return _ivec(tuple(v))
+
+
+def dvec(v):
+    """Four C doubles; arrays of equal values are shared (the library only reads them)."""
+    return _dvec(tuple(v))

@@ -18,17 +18,21 @@ _DT = {torch.complex128: L.MG_C128, torch.complex64: L.MG_C64,
 
 
 def _stream(t=None):
-    if t is not None and not t.is_cuda:
+    """torch's current stream as an integer handle (None: the legacy default stream)."""
+    if t is None:
+        if not torch.cuda.is_available():
+            return None
+        return torch.cuda.current_stream().cuda_stream
+    if not t.is_cuda:
         return None
-    if not torch.cuda.is_available():
-        return None
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle, without the Stream object of torch.cuda.current_stream()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def params(dims, block, kappa, k, r, n_s, sweeps=5, seed=3000, hop_weight=(1, 1, 1, 1),

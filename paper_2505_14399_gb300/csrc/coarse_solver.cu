@@ -579,7 +579,7 @@ __global__ void barrier_timeout_kernel(BarrierState* bs, long long limit) {
 
 int barrier_timeout_selftest(cudaStream_t st) {
   BarrierState* bs = nullptr;
-  WMG_CUDA(cudaMallocAsync(&bs, sizeof(BarrierState), st));
+  WMG_CUDA(scratch_alloc(&bs, sizeof(BarrierState), st));
   WMG_CUDA(cudaMemsetAsync(bs, 0, sizeof(BarrierState), st));
   long long limit = 1ll << 16;
   barrier_timeout_kernel<<<2, 32, 0, st>>>(bs, limit);
@@ -587,7 +587,7 @@ int barrier_timeout_selftest(cudaStream_t st) {
   BarrierState h;
   WMG_CUDA(cudaMemcpyAsync(&h, bs, sizeof(h), cudaMemcpyDeviceToHost, st));
   WMG_CUDA(cudaStreamSynchronize(st));
-  WMG_CUDA(cudaFreeAsync(bs, st));
+  scratch_free(bs, st);
   WMG_CUDA(cudaStreamSynchronize(st));
   if (h.err) return fail(MG_ETIMEOUT, "barrier self-test: bounded wait gave up as designed");
   return fail(MG_ECUDA, "barrier self-test: the wait did not time out");

@@ -27,6 +27,13 @@ int dev_alloc_bytes(void** p, size_t bytes);
 void dev_free(void* p);
 int host_alloc_bytes(void** p, size_t bytes);
 void host_free(void* p);
+// Stream-ordered scratch of one call, from the library's own pool; see runtime.cu.
+cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st);
+void scratch_free(void* p, cudaStream_t st);
+template <typename T>
+inline cudaError_t scratch_alloc(T** p, size_t bytes, cudaStream_t st) {
+  return scratch_alloc_bytes(reinterpret_cast<void**>(p), bytes, st);
+}
 template <typename T>
 inline int dev_alloc(T** p, size_t bytes) { return dev_alloc_bytes(reinterpret_cast<void**>(p), bytes); }
 template <typename T>

@@ -356,7 +356,7 @@ __global__ void su3_deviation_df_kernel(unsigned long long* out, const zdf* __re
 
 int su3_deviation(double* dev_out, const zd* links, size_t nlinks, cudaStream_t st) {
   unsigned long long* d = nullptr;
-  WMG_CUDA(cudaMallocAsync(&d, sizeof(*d), st));
+  WMG_CUDA(scratch_alloc(&d, sizeof(*d), st));
   WMG_CUDA(cudaMemsetAsync(d, 0, sizeof(*d), st));
   size_t g = (nlinks + 255) / 256, cap = (size_t)num_sms() * 8;
   su3_deviation_kernel<<<(unsigned)(g < cap ? (g < 1 ? 1 : g) : cap), 256, 0, st>>>(d, links, nlinks);
@@ -364,14 +364,14 @@ int su3_deviation(double* dev_out, const zd* links, size_t nlinks, cudaStream_t 
   unsigned long long bits = 0;
   WMG_CUDA(cudaMemcpyAsync(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost, st));
   WMG_CUDA(cudaStreamSynchronize(st));
-  cudaFreeAsync(d, st);
+  scratch_free(d, st);
   std::memcpy(dev_out, &bits, sizeof(double));
   return MG_OK;
 }
 
 int su3_deviation_df(double* dev_out, const zdf* links, size_t nlinks, cudaStream_t st) {
   unsigned long long* d = nullptr;
-  WMG_CUDA(cudaMallocAsync(&d, sizeof(*d), st));
+  WMG_CUDA(scratch_alloc(&d, sizeof(*d), st));
   WMG_CUDA(cudaMemsetAsync(d, 0, sizeof(*d), st));
   size_t g = (nlinks + 255) / 256, cap = (size_t)num_sms() * 8;
   su3_deviation_df_kernel<<<(unsigned)(g < cap ? (g < 1 ? 1 : g) : cap), 256, 0, st>>>(d, links, nlinks);
@@ -379,7 +379,7 @@ int su3_deviation_df(double* dev_out, const zdf* links, size_t nlinks, cudaStrea
   unsigned long long bits = 0;
   WMG_CUDA(cudaMemcpyAsync(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost, st));
   WMG_CUDA(cudaStreamSynchronize(st));
-  cudaFreeAsync(d, st);
+  scratch_free(d, st);
   std::memcpy(dev_out, &bits, sizeof(double));
   return MG_OK;
 }

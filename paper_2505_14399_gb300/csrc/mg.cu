@@ -1008,11 +1008,11 @@ extern "C" int coarse_build(mg_handle* h, void* stream) {
     h->lv.clear();
   }
   zd* Xpart = nullptr;
-  WMG_CUDA(cudaMallocAsync(&Xpart, (size_t)4 * h->B.d * ne * sizeof(zd), st));
+  WMG_CUDA(scratch_alloc(&Xpart, (size_t)4 * h->B.d * ne * sizeof(zd), st));
   bool df = galerkin_df(h->p);
   int s = galerkin_build(h->Op64, Xpart, h->P64, h->Pdf, h->PtP, h->k, h->links64, h->Ldf, h->g,
                          h->B, st, df, h->pdf_ready, h->tc_flag);
-  cudaFreeAsync(Xpart, st);
+  scratch_free(Xpart, st);
   WMG_TRY(s);
   if (h->clov64) WMG_TRY(clover_galerkin_add(h->Op64, h->P64, h->clov64, h->k, h->B, st));
   WMG_TRY((convert<float, double>(h->Op32, h->Op64, nullptr, 0, (size_t)h->B.d * 9 * ne, 1, st)));
@@ -1100,7 +1100,7 @@ static int solve_entry(mg_handle* h, void* x, const void* b, int nrhs, double to
   const zd* bb = (const zd*)sb.dev;
   zd* gb = nullptr;
   if (adjoint) {
-    WMG_CUDA(cudaMallocAsync(&gb, fb, st));
+    WMG_CUDA(scratch_alloc(&gb, fb, st));
     WMG_TRY(apply_gamma5<double>(gb, bb, (size_t)h->g.V * nrhs, st));
     bb = gb;
   }
@@ -1110,7 +1110,7 @@ static int solve_entry(mg_handle* h, void* x, const void* b, int nrhs, double to
       int s2 = apply_gamma5<double>((zd*)sx.dev, (const zd*)sx.dev, (size_t)h->g.V * nrhs, st);
       if (s2 != MG_OK) s = s2;
     }
-    cudaFreeAsync(gb, st);
+    scratch_free(gb, st);
   }
   if (s != MG_OK && s != MG_ENOCONV) return s;
   std::string msg = s == MG_ENOCONV ? std::string(mg_last_error()) : std::string();
@@ -1151,22 +1151,22 @@ extern "C" int mg_test_vectors(void* out, const void* links, const mg_params* p,
   WMG_TRY(stage_out_alloc(so, out, fr * sizeof(zd), st));
   if (p->setup_dtype == MG_C128) {
     zd* tmp;
-    WMG_CUDA(cudaMallocAsync(&tmp, fr * sizeof(zd), st));
+    WMG_CUDA(scratch_alloc(&tmp, fr * sizeof(zd), st));
     Gmres<double> gm;
     int s = smooth_stream<double>(h, (zd*)so.dev, tmp, gm, stream_index, st);
     cudaStreamSynchronize(st);
-    cudaFreeAsync(tmp, st);
+    scratch_free(tmp, st);
     WMG_TRY(s);
   } else {
     zf *tmp, *psi;
-    WMG_CUDA(cudaMallocAsync(&tmp, fr * sizeof(zf), st));
-    WMG_CUDA(cudaMallocAsync(&psi, fr * sizeof(zf), st));
+    WMG_CUDA(scratch_alloc(&tmp, fr * sizeof(zf), st));
+    WMG_CUDA(scratch_alloc(&psi, fr * sizeof(zf), st));
     Gmres<float> gm;
     int s = smooth_stream<float>(h, psi, tmp, gm, stream_index, st);
     if (s == MG_OK) s = convert<double, float>((zd*)so.dev, psi, nullptr, 0, fr, 1, st);
     cudaStreamSynchronize(st);
-    cudaFreeAsync(tmp, st);
-    cudaFreeAsync(psi, st);
+    scratch_free(tmp, st);
+    scratch_free(psi, st);
     WMG_TRY(s);
   }
   WMG_TRY(stage_out_finish(so, out, fr * sizeof(zd), st));

@@ -43,7 +43,7 @@ int probe(double* tflops, int iters, cudaStream_t st) {
   if (occ < 1) occ = 1;
   int blocks = occ * num_sms();
   T* out = nullptr;
-  WMG_CUDA(cudaMallocAsync(&out, sizeof(T) * (size_t)blocks * PROBE_THREADS, st));
+  WMG_CUDA(scratch_alloc(&out, sizeof(T) * (size_t)blocks * PROBE_THREADS, st));
   cudaEvent_t e0, e1;
   WMG_CUDA(cudaEventCreate(&e0));
   WMG_CUDA(cudaEventCreate(&e1));
@@ -64,7 +64,7 @@ int probe(double* tflops, int iters, cudaStream_t st) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  cudaFreeAsync(out, st);
+  scratch_free(out, st);
   if (status != MG_OK) return status;
   WMG_CUDA(cudaStreamSynchronize(st));
   double fmas = (double)blocks * PROBE_THREADS * iters * PROBE_UNROLL * PROBE_CHAINS;

@@ -197,7 +197,7 @@ extern "C" int wilson_schur(void* out, const void* in, const void* links, const 
   if (((uintptr_t)sin.dev | (uintptr_t)sout.dev) & 15)
     return fail(MG_EINVAL, "wilson_schur: spinor fields must be 16-byte aligned");
   void* tmp = nullptr;
-  WMG_CUDA(cudaMallocAsync(&tmp, fbytes, st));
+  WMG_CUDA(scratch_alloc(&tmp, fbytes, st));
   int s = MG_OK;
   switch (dtype) {
     case MG_C128: s = schur_apply<zd>((zd*)sout.dev, (const zd*)sin.dev, (zd*)tmp, sl.dev, 0, g, dagger, nrhs, st); break;
@@ -205,7 +205,7 @@ extern "C" int wilson_schur(void* out, const void* in, const void* links, const 
     case MG_F16: s = schur_apply<zh>((zh*)sout.dev, (const zh*)sin.dev, (zh*)tmp, sl.dev, 0, g, dagger, nrhs, st); break;
     default: s = schur_apply<zbf>((zbf*)sout.dev, (const zbf*)sin.dev, (zbf*)tmp, sl.dev, 0, g, dagger, nrhs, st); break;
   }
-  cudaFreeAsync(tmp, st);
+  scratch_free(tmp, st);
   WMG_TRY(s);
   WMG_TRY(stage_out_finish(sout, out, fbytes, st));
   return MG_OK;
