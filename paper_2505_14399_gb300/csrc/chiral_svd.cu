@@ -24,25 +24,26 @@ namespace wmg {
 
 namespace {
 
+// One thread per (site, chirality) of one vector: six components from one contiguous span into
+// one (the aggregate's index arithmetic once per six, in 32 bits).
 template <typename R, typename TO>
-__global__ void gather_kernel(TO* tiles, int cmax, int col0, const cplx<R>* __restrict__ f,
-                              int nvec, Blocking B) {
-  size_t total = (size_t)nvec * B.L[0] * B.L[1] * B.L[2] * B.L[3] * 12;
-  size_t V12 = total / nvec;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    int v = (int)(e / V12);
-    size_t rem = e % V12;
-    int s = (int)(rem / 12), comp = (int)(rem % 12);
-    int spin = comp / 3, col = comp % 3;
-    int j, l;
-    B.block_of(s, &j, &l);
-    int alpha = spin >> 1;
-    int row = (l * 2 + (spin & 1)) * 3 + col;
-    size_t t = (size_t)j * 2 + alpha;
-    cplx<R> x = f[e];
-    if constexpr (std::is_same<TO, zdf>::value) tiles[(t * cmax + col0 + v) * B.M + row] = zdf_from(x);
-    else tiles[(t * cmax + col0 + v) * B.M + row] = {(double)x.re, (double)x.im};
+__global__ void __launch_bounds__(256)
+gather_kernel(TO* tiles, int cmax, int col0, const cplx<R>* __restrict__ f, Blocking B) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  const int V = B.nd * B.d;
+  if (e >= 2 * V) return;
+  const int v = blockIdx.y, s = e >> 1, alpha = e & 1;
+  const cplx<R>* src = f + ((size_t)v * V + s) * 12 + 6 * alpha;
+  cplx<R> x[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) x[i] = src[i];
+  int j, l;
+  B.block_of(s, &j, &l);
+  TO* dst = tiles + ((size_t)(2 * j + alpha) * cmax + col0 + v) * B.M + 6 * l;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    if constexpr (std::is_same<TO, zdf>::value) dst[i] = zdf_from(x[i]);
+    else dst[i] = {(double)x[i].re, (double)x[i].im};
   }
 }
 
@@ -54,29 +55,25 @@ constexpr int JT = 128;
 constexpr int GR = 32;    // rows staged per chunk
 constexpr int MAXC = 64;  // max columns per tile
 
-// G = A^dag A, upper triangle computed, mirrored.  DF: df64 arithmetic (FP32 units,
-// error-free transformations) instead of FP64.  MAXP: column pairs per thread
+// G = A^dag A in FP64, upper triangle computed, mirrored.  MAXP: column pairs per thread
 // (>= pairs / blockDim), which sets the accumulator registers.
 // The first kd columns may be known to be orthogonal with squared norms lamp[t][0..kd-1]
 // (the previous stream's Phi = A V_k, whose Gram matrix is V_k^dag G V_k = Lambda_k): their
 // block is then written as that diagonal and only the pairs (i, j), i <= j, j >= kd are summed.
-template <bool DF, int MAXP>
-__global__ void __launch_bounds__(GT) gram_kernel(zd* G, const void* __restrict__ tiles, int cmax,
+template <int MAXP>
+__global__ void __launch_bounds__(GT) gram_kernel(zd* G, const zd* __restrict__ tiles, int cmax,
                                                   int c, int M, int kd, const double* lamp,
                                                   int cprev) {
-  typedef typename std::conditional<DF, zdf, zd>::type T;
-  typedef typename std::conditional<DF, zdfacc, zd>::type TA;
-  extern __shared__ zd smraw_g[];
-  T* sA = reinterpret_cast<T*>(smraw_g);  // [GR][c]
+  extern __shared__ zd sA[];  // [GR][c]
   int t = blockIdx.x;
-  const T* A = reinterpret_cast<const T*>(tiles) + (size_t)t * cmax * M;
+  const zd* A = tiles + (size_t)t * cmax * M;
   const int nth = blockDim.x;
   const int npairs = c * (c + 1) / 2 - kd * (kd + 1) / 2;
-  TA acc[MAXP];
+  zd acc[MAXP];
   int pi[MAXP], pj[MAXP];
 #pragma unroll
   for (int q = 0; q < MAXP; ++q) {
-    acc[q] = TA{};
+    acc[q] = zd{};
     int p = threadIdx.x + q * nth;
     // p -> (i, j) with i <= j and j >= kd, column by column (column j holds j + 1 pairs)
     int j = kd, rem = p;
@@ -94,19 +91,15 @@ __global__ void __launch_bounds__(GT) gram_kernel(zd* G, const void* __restrict_
     __syncthreads();
     for (int e = threadIdx.x; e < nr * c; e += nth) {
       int col = e / nr, rr = e % nr;
-      if constexpr (DF) sA[rr * c + col] = zdf_ld(A + (size_t)col * M + r0 + rr);
-      else sA[rr * c + col] = A[(size_t)col * M + r0 + rr];
+      sA[rr * c + col] = A[(size_t)col * M + r0 + rr];
     }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < MAXP; ++q) {
       int p = threadIdx.x + q * nth;
       if (p < npairs) {
-        TA a = acc[q];
-        for (int rr = 0; rr < nr; ++rr) {
-          if constexpr (DF) zdf_fmac(a, sA[rr * c + pi[q]], sA[rr * c + pj[q]]);
-          else cfmac(a, sA[rr * c + pi[q]], sA[rr * c + pj[q]]);
-        }
+        zd a = acc[q];
+        for (int rr = 0; rr < nr; ++rr) cfmac(a, sA[rr * c + pi[q]], sA[rr * c + pj[q]]);
         acc[q] = a;
       }
     }
@@ -115,11 +108,149 @@ __global__ void __launch_bounds__(GT) gram_kernel(zd* G, const void* __restrict_
   for (int q = 0; q < MAXP; ++q) {
     int p = threadIdx.x + q * nth;
     if (p < npairs) {
-      zd v;
-      if constexpr (DF) v = zdf_result(acc[q]);
-      else v = acc[q];
+      zd v = acc[q];
       Gt[pi[q] * c + pj[q]] = v;
       if (pi[q] != pj[q]) Gt[pj[q] * c + pi[q]] = conj(v);
+    }
+  }
+}
+
+// G = A^dag A on double-float tiles, on the FP32 units, with biased accumulators (df64.cuh).
+// A thread sums a 2 x 2 block of column pairs over every eighth row, the block's two right
+// columns in the two halves of packed instructions: its four operands come from shared memory
+// once per four products (24 packed instructions per two products), the eight row groups of a
+// block are neighbouring lanes, so a quarter warp reads eight rows at an odd stride (no bank
+// conflicts) and the groups meet in shuffles.  Rows arrive in chunks of GR through registers
+// (loads of the next chunk in flight during this one's products) and two shared buffers, one
+// barrier per chunk.  A group's sums over a chunk (four rows) start at a bias from the norms n of
+// the columns over those rows (Cauchy and Schwarz: every partial sum is within n_i n_j) and then
+// join a (hi, lo) total.  Against one long double-float sum (df_fma, 12 instructions per product)
+// it is half the instructions and more exact: P^dag P of orthonormal 1536-row tiles (the Galerkin
+// diagonal) is off by 1.4e-14 instead of 5.6e-13, of 192-row tiles by 2.4e-14 instead of 7.4e-14.
+// 16^3x32, four streams (c = 8, 16, 20, 20): 1.88 -> 1.14 ms.
+// kd, lamp: as for gram_kernel.  cn[t][i] (leading dimension cld, may be null): the columns'
+// squared norms.  nt: 2 x 2 blocks in all, ntc of them per CTA (blockIdx.y picks the slice).
+constexpr int GDF_G = 8;        // row groups
+constexpr int GDF_T = 40;       // blocks per CTA at most (320 threads)
+// PRE: staged column pairs of a row per thread and chunk at most (2, or 4 above 40 columns)
+template <int PRE>
+__global__ void __launch_bounds__(GDF_T * GDF_G, 2)
+gram_df_kernel(zd* G, float* cn, int cld, const zdf* __restrict__ tiles, int cmax, int c, int M,
+               int kd, const double* lamp, int cprev, int nt, int ntc) {
+  extern __shared__ __align__(16) unsigned char smraw_gd[];
+  const int np = (c + 1) / 2, ld = np | 1;      // column pairs, odd row stride
+  // [2][re, im][GR][ld]: (hi, hi, lo, lo) of a column pair
+  float4* sA = reinterpret_cast<float4*>(smraw_gd);
+  float2* snrm = reinterpret_cast<float2*>(sA + 4 * GR * ld);   // [2][GDF_G][np]
+  const int t = blockIdx.x, nth = blockDim.x;
+  const zdf* A = tiles + (size_t)t * cmax * M;
+  const int g = threadIdx.x & (GDF_G - 1);
+  int blk = blockIdx.y * ntc + (threadIdx.x / GDF_G);
+  const bool work = (int)(threadIdx.x / GDF_G) < ntc && blk < nt;
+  if (!work) blk = nt - 1;
+  // block index -> (I, J), I <= J, J >= kd / 2, column pair by column pair
+  int J = kd / 2, I = blk;
+  while (I >= J + 1) { I -= J + 1; ++J; }
+  const zdf zero = {{0.f, 0.f}, {0.f, 0.f}};
+  zdf pre[PRE][2];
+  const int npre = GR * np;
+  auto load = [&](int r0) {
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) {
+      const int e = threadIdx.x + u * nth;   // whole warps: 32 rows of one column pair
+      const int col = 2 * (e / GR), r = r0 + (e & (GR - 1));
+      pre[u][0] = pre[u][1] = zero;
+      if (e < npre && r < M) {
+        pre[u][0] = zdf_ld(A + (size_t)col * M + r);
+        if (col + 1 < c) pre[u][1] = zdf_ld(A + (size_t)(col + 1) * M + r);
+      }
+    }
+  };
+  f32x2 th[2][2] = {}, tl[2][2] = {};
+  load(0);
+  int buf = 0;
+  for (int r0 = 0; r0 < M; r0 += GR, buf ^= 1) {
+    float4* sre = sA + buf * 2 * GR * ld;
+    float4* sim = sre + GR * ld;
+    float2* sn = snrm + buf * GDF_G * np;
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) {
+      const int e = threadIdx.x + u * nth;
+      if (e < npre) {
+        const int at = (e & (GR - 1)) * ld + e / GR;
+        const zdf &v = pre[u][0], &w = pre[u][1];
+        sre[at] = make_float4(v.re.hi, w.re.hi, v.re.lo, w.re.lo);
+        sim[at] = make_float4(v.im.hi, w.im.hi, v.im.lo, w.im.lo);
+        // squared norms over the rows of each group: lanes g, g + 8, g + 16, g + 24
+        float n0 = fmaf(v.re.hi, v.re.hi, v.im.hi * v.im.hi);
+        float n1 = fmaf(w.re.hi, w.re.hi, w.im.hi * w.im.hi);
+#pragma unroll
+        for (int o = GDF_G; o < 32; o <<= 1) {
+          n0 += __shfl_xor_sync(0xffffffffu, n0, o);
+          n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+        }
+        if ((threadIdx.x & 31) < GDF_G)
+          sn[(threadIdx.x & 31) * np + e / GR] = make_float2(sqrtf(n0), sqrtf(n1));
+      }
+    }
+    __syncthreads();
+    if (r0 + GR < M) load(r0 + GR);
+    const float2 ni = sn[g * np + I], nj = sn[g * np + J];
+    zbacc2 acc[2];
+    f32x2 C[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      acc[q] = zbacc2{};
+      const float n = 1.001f * (q ? ni.y : ni.x);
+      C[q] = f2_pack(bacc_bias(n * nj.x), bacc_bias(n * nj.y));
+      acc[q].re.s = acc[q].im.s = C[q];
+    }
+#pragma unroll
+    for (int u = 0; u < GR / GDF_G; ++u) {
+      const int row = (g + u * GDF_G) * ld;
+      const float4 ar = sre[row + I], ai = sim[row + I];
+      const zdf2 b = {df2_ld(sre + row + J), df2_ld(sim + row + J)};
+      zbacc2_fmac(acc[0], zdf_dup({{ar.x, ar.z}, {ai.x, ai.z}}), b);
+      zbacc2_fmac(acc[1], zdf_dup({{ar.y, ar.w}, {ai.y, ai.w}}), b);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        const bacc2& a = z ? acc[q].im : acc[q].re;
+        const df2 v = df2_two_sum(th[q][z], f2_sub(a.s, C[q]));
+        th[q][z] = v.hi;
+        tl[q][z] = f2_add(tl[q][z], f2_add(v.lo, f2_add(a.e, a.x)));
+      }
+  }
+  zd* Gt = G + (size_t)t * c * c;
+  if (blockIdx.y == 0)
+    for (int e = threadIdx.x; e < kd * kd; e += nth) {
+      const int i = e / kd, j = e % kd;
+      const double l = lamp[(size_t)t * cprev + i];
+      Gt[i * c + j] = i == j ? zd{l, 0.0} : zd{0.0, 0.0};
+      if (i == j && cn) cn[(size_t)t * cld + i] = (float)l;
+    }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    df v[2];
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      const f32x2 h = th[q >> 1][z], l = tl[q >> 1][z];
+      df x = (q & 1) ? df_two_sum(f2_hi(h), f2_hi(l)) : df_two_sum(f2_lo(h), f2_lo(l));
+#pragma unroll
+      for (int o = 1; o < GDF_G; o <<= 1) {
+        const df y = {__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
+        x = (g & o) ? df_add(y, x) : df_add(x, y);   // one order in every lane
+      }
+      v[z] = x;
+    }
+    const int i = 2 * I + (q >> 1), j = 2 * J + (q & 1);
+    if (work && g == 0 && i <= j && j < c && j >= kd) {
+      const zd w = {df_val(v[0]), i == j ? 0.0 : df_val(v[1])};
+      Gt[i * c + j] = w;
+      if (i != j) Gt[j * c + i] = conj(w);
+      else if (cn) cn[(size_t)t * cld + i] = df_to_float(v[0]);
     }
   }
 }
@@ -180,9 +311,29 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(double* lam, zd* Vec, const 
   int t = blockIdx.x;
   const zd* Gt = G + (size_t)t * c * c;
   const float rtol2 = (float)(rtol * rtol);
+  // double-float: scaled by a power of two (exact) to a largest diagonal entry in [1/2, 1), since
+  // the angles square FP32 copies of the entries
+  __shared__ double gscale[2];   // 2^-e, 2^e
+  if constexpr (DF) {
+    if (threadIdx.x < 32) {
+      double m = 0;
+      for (int i = threadIdx.x; i < c; i += 32) m = fmax(m, fabs(Gt[i * c + i].re));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (threadIdx.x == 0) {
+        int e = 0;
+        if (m > 0 && isfinite(m)) frexp(m, &e);
+        gscale[0] = ldexp(1.0, -e);
+        gscale[1] = ldexp(1.0, e);
+      }
+    }
+    __syncthreads();
+  }
   for (int e = threadIdx.x; e < ce * ce; e += blockDim.x) {
     int i = e / ce, j = e % ce;
-    A[e] = (i < c && j < c) ? J::from(Gt[i * c + j]) : J::zero();
+    zd v = (i < c && j < c) ? Gt[i * c + j] : zd{0, 0};
+    if constexpr (DF) v = gscale[0] * v;
+    A[e] = J::from(v);
     Vv[e] = (i == j) ? J::one() : J::zero();
   }
   // the round-robin schedule of all ce - 1 rounds of a sweep, once: pairs (top[p], bot[p])
@@ -360,7 +511,7 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(double* lam, zd* Vec, const 
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < c; i += blockDim.x) lam[(size_t)t * c + i] = dg[order[i]];
+  for (int i = threadIdx.x; i < c; i += blockDim.x) lam[(size_t)t * c + i] = DF ? gscale[1] * dg[order[i]] : dg[order[i]];
   zd* Vt = Vec + (size_t)t * c * c;
   for (int e = threadIdx.x; e < c * c; e += blockDim.x) {
     int row = e / c, i = e % c;
@@ -370,15 +521,12 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(double* lam, zd* Vec, const 
 
 constexpr int UK = 64;  // max output columns per update
 
-template <bool DF>
-__global__ void __launch_bounds__(GT) update_kernel(void* out, int cmax_out,
-                                                    const void* __restrict__ tiles, int cmax, int c,
+// out = A V (FP64), optionally with columns scaled by 1 / sqrt(lam)
+__global__ void __launch_bounds__(GT) update_kernel(zd* out, int cmax_out,
+                                                    const zd* __restrict__ tiles, int cmax, int c,
                                                     const zd* __restrict__ Vec, const double* lam,
                                                     int kout, int scale_inv, int M) {
-  typedef typename std::conditional<DF, zdf, zd>::type T;
-  typedef typename std::conditional<DF, zdfacc, zd>::type TA;
-  extern __shared__ zd smraw_u[];
-  T* sV = reinterpret_cast<T*>(smraw_u);  // [c][kout]
+  extern __shared__ zd sV[];  // [c][kout]
   int t = blockIdx.x;
   const zd* Vt = Vec + (size_t)t * c * c;
   for (int e = threadIdx.x; e < c * kout; e += blockDim.x) {
@@ -389,35 +537,150 @@ __global__ void __launch_bounds__(GT) update_kernel(void* out, int cmax_out,
       double f = l > 0 ? 1.0 / sqrt(l) : 0.0;
       v = f * v;
     }
-    if constexpr (DF) sV[e] = zdf_from(v);
-    else sV[e] = v;
+    sV[e] = v;
   }
   __syncthreads();
-  const T* A = reinterpret_cast<const T*>(tiles) + (size_t)t * cmax * M;
-  T* O = reinterpret_cast<T*>(out) + (size_t)t * cmax_out * M;
+  const zd* A = tiles + (size_t)t * cmax * M;
+  zd* O = out + (size_t)t * cmax_out * M;
   for (int r = threadIdx.x; r < M; r += blockDim.x) {
     for (int i0 = 0; i0 < kout; i0 += 16) {
-      TA acc[16];
+      zd acc[16];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) acc[q] = TA{};
+      for (int q = 0; q < 16; ++q) acc[q] = zd{};
       for (int col = 0; col < c; ++col) {
-        if constexpr (DF) {
-          zdf a = zdf_ld(A + (size_t)col * M + r);
+        zd a0 = A[(size_t)col * M + r];
 #pragma unroll
-          for (int q = 0; q < 16; ++q)
-            if (i0 + q < kout) zdf_fma(acc[q], a, sV[col * kout + i0 + q]);
-        } else {
-          zd a0 = A[(size_t)col * M + r];
+        for (int q = 0; q < 16; ++q)
+          if (i0 + q < kout) cfma(acc[q], a0, sV[col * kout + i0 + q]);
+      }
 #pragma unroll
-          for (int q = 0; q < 16; ++q)
-            if (i0 + q < kout) cfma(acc[q], a0, sV[col * kout + i0 + q]);
+      for (int q = 0; q < 16; ++q)
+        if (i0 + q < kout) O[(size_t)(i0 + q) * M + r] = acc[q];
+    }
+  }
+}
+
+// The same on double-float tiles, on the FP32 units with biased accumulators (df64.cuh): a thread
+// takes one row and OB output columns at a time, two outputs per packed instruction, and adds the
+// columns of A in groups of UDG.  A group's bias comes from Cauchy and Schwarz with the columns
+// scaled by their norms n_c (cn, squared, from the Gram kernel): every partial sum of the group's
+// A_rc V_ci lies within R F_i, R^2 = sum_c |A_rc|^2 / n_c^2 and F_i^2 = sum_c n_c^2 |V_ci|^2,
+// which follows small singular values; the group then joins a (hi, lo) total.  Groups of four
+// lose less than one sum over all columns by the square of their number (its bias is larger, and
+// it collects more roundings): relative error of a column 4.8e-13 -> 6e-14 at c = 20 (float32
+// emulation); the streaming SVD's P is then as exact as with the 12-instruction df_fma or more.
+// 16^3x32, four streams (c x kout = 8 x 8, 16 x 12, 20 x 12 twice): 2.52 -> 1.22 ms.
+// Each CTA takes `rows` rows of a tile (blockIdx.y picks them).  kp: kout padded to a multiple of
+// OB (even).
+constexpr int UDT = 128, UDG = 4;
+template <int OB>
+__global__ void __launch_bounds__(UDT, 4)
+update_df_kernel(zdf* out, int cmax_out, const zdf* __restrict__ tiles, int cmax, int c,
+                 const zd* __restrict__ Vec, const double* lam, const float* __restrict__ cn,
+                 int cld, int kout, int kp, int scale_inv, int M, int rows) {
+  extern __shared__ __align__(16) unsigned char smraw_ud[];
+  const int ng = (c + UDG - 1) / UDG, cpad = ng * UDG;
+  // [cpad][kp / 2][re, im]: (hi, hi, lo, lo) of an output pair
+  float4* sV = reinterpret_cast<float4*>(smraw_ud);
+  float* sF = reinterpret_cast<float*>(sV + (size_t)cpad * kp);  // [ng][kp] F_i of a group
+  float* sI = sF + ng * kp;                                      // [cpad] 1 / n_c
+  float* sN = sI + cpad;                                         // [cpad] n_c / max
+  __shared__ float nmax;
+  const int t = blockIdx.x;
+  const zd* Vt = Vec + (size_t)t * c * c;
+  if (threadIdx.x < 32) {
+    float m = 0.f;
+    for (int q = threadIdx.x; q < c; q += 32) m = fmaxf(m, sqrtf(cn[(size_t)t * cld + q]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int q = threadIdx.x; q < cpad; q += 32) {
+      const float n = q < c ? sqrtf(cn[(size_t)t * cld + q]) : 0.f;
+      sI[q] = n > 1e-20f ? 1.0f / n : 0.0f;   // below: n^2 has lost its digits
+      sN[q] = m > 0.f ? n / m : 0.f;
+    }
+    if (threadIdx.x == 0) nmax = m;
+  }
+  for (int e = threadIdx.x; e < cpad * kp; e += UDT) {
+    const int row = e / kp, i = e % kp;
+    zdf w = {{0.f, 0.f}, {0.f, 0.f}};
+    if (i < kout && row < c) {
+      zd v = Vt[row * c + i];
+      if (scale_inv) {
+        double l = lam[(size_t)t * c + i];
+        double f = l > 0 ? 1.0 / sqrt(l) : 0.0;
+        v = f * v;
+      }
+      w = zdf_from(v);
+    }
+    float* q = reinterpret_cast<float*>(sV + (size_t)row * kp + (i & ~1)) + (i & 1);
+    q[0] = w.re.hi; q[2] = w.re.lo; q[4] = w.im.hi; q[6] = w.im.lo;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < ng * kp; e += UDT) {
+    const int g = e / kp, i = e % kp;
+    float f = 0.f;
+    for (int q = g * UDG; q < (g + 1) * UDG; ++q) {
+      const float* v = reinterpret_cast<const float*>(sV + (size_t)q * kp + (i & ~1)) + (i & 1);
+      const float x = sN[q] * v[0], y = sN[q] * v[4];
+      f = fmaf(x, x, fmaf(y, y, f));
+    }
+    sF[e] = 1.001f * nmax * sqrtf(f);
+  }
+  __syncthreads();
+  const zdf* A = tiles + (size_t)t * cmax * M;
+  zdf* O = out + (size_t)t * cmax_out * M;
+  const int r1 = min(M, ((int)blockIdx.y + 1) * rows);
+  const zdf zero = {{0.f, 0.f}, {0.f, 0.f}};
+  for (int r = blockIdx.y * rows + threadIdx.x; r < r1; r += UDT) {
+    for (int i0 = 0; i0 < kout; i0 += OB) {
+      f32x2 th[OB / 2][2], tl[OB / 2][2];
+#pragma unroll
+      for (int q = 0; q < OB / 2; ++q) th[q][0] = th[q][1] = tl[q][0] = tl[q][1] = 0;
+      zdf a[UDG];
+#pragma unroll
+      for (int u = 0; u < UDG; ++u) a[u] = u < c ? zdf_ld(A + (size_t)u * M + r) : zero;
+      for (int g = 0; g < ng; ++g) {
+        float R = 0.f;
+        zdfdup ad[UDG];
+#pragma unroll
+        for (int u = 0; u < UDG; ++u) {
+          const float x = sI[g * UDG + u] * a[u].re.hi, y = sI[g * UDG + u] * a[u].im.hi;
+          R = fmaf(x, x, fmaf(y, y, R));
+          ad[u] = zdf_dup(a[u]);
+          const int col = (g + 1) * UDG + u;   // the next group's loads, under this one's products
+          a[u] = col < c ? zdf_ld(A + (size_t)col * M + r) : zero;
+        }
+        R = sqrtf(R);
+        const float4* v = sV + (size_t)g * UDG * kp + i0;
+#pragma unroll
+        for (int q = 0; q < OB / 2; ++q) {
+          const float2 F = *reinterpret_cast<const float2*>(sF + g * kp + i0 + 2 * q);
+          const f32x2 C = f2_pack(bacc_bias(R * F.x), bacc_bias(R * F.y));
+          zbacc2 acc = {};
+          acc.re.s = acc.im.s = C;
+#pragma unroll
+          for (int u = 0; u < UDG; ++u)
+            zbacc2_fma(acc, ad[u], {df2_ld(v + u * kp + 2 * q), df2_ld(v + u * kp + 2 * q + 1)});
+#pragma unroll
+          for (int z = 0; z < 2; ++z) {
+            const bacc2& b = z ? acc.im : acc.re;
+            const df2 w = df2_two_sum(th[q][z], f2_sub(b.s, C));
+            th[q][z] = w.hi;
+            tl[q][z] = f2_add(tl[q][z], f2_add(w.lo, f2_add(b.e, b.x)));
+          }
         }
       }
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
+      for (int q = 0; q < OB; ++q) {
         if (i0 + q < kout) {
-          if constexpr (DF) O[(size_t)(i0 + q) * M + r] = zdf_norm(acc[q]);
-          else O[(size_t)(i0 + q) * M + r] = acc[q];
+          df x[2];
+#pragma unroll
+          for (int z = 0; z < 2; ++z) {
+            const f32x2 h = th[q >> 1][z], l = tl[q >> 1][z];
+            x[z] = (q & 1) ? df_two_sum(f2_hi(h), f2_hi(l)) : df_two_sum(f2_lo(h), f2_lo(l));
+          }
+          reinterpret_cast<float4*>(O)[(size_t)(i0 + q) * M + r] =
+              make_float4(x[0].hi, x[0].lo, x[1].hi, x[1].lo);
         }
       }
     }
@@ -621,12 +884,9 @@ int make_blocking(Blocking& B, const int dims[4], const int block[4]) {
 template <typename R>
 int chiral_gather(void* tiles, int cmax, int col0, const cplx<R>* fields, int nvec,
                   const Blocking& B, cudaStream_t st, bool df64) {
-  size_t total = (size_t)nvec * B.nd * B.d * 12;
-  size_t g = (total + 255) / 256;
-  size_t cap = (size_t)num_sms() * 16;
-  unsigned grid = (unsigned)(g < cap ? g : cap);
-  if (df64) gather_kernel<R, zdf><<<grid, 256, 0, st>>>((zdf*)tiles, cmax, col0, fields, nvec, B);
-  else gather_kernel<R, zd><<<grid, 256, 0, st>>>((zd*)tiles, cmax, col0, fields, nvec, B);
+  const dim3 grid((2 * B.nd * B.d + 255) / 256, nvec);
+  if (df64) gather_kernel<R, zdf><<<grid, 256, 0, st>>>((zdf*)tiles, cmax, col0, fields, B);
+  else gather_kernel<R, zd><<<grid, 256, 0, st>>>((zd*)tiles, cmax, col0, fields, B);
   WMG_LAUNCHED();
   return MG_OK;
 }
@@ -634,31 +894,43 @@ template int chiral_gather<float>(void*, int, int, const zf*, int, const Blockin
 template int chiral_gather<double>(void*, int, int, const zd*, int, const Blocking&, cudaStream_t, bool);
 
 int tile_gram(zd* G, const void* tiles, int cmax, int c, const Blocking& B, cudaStream_t st,
-              bool df64, int kd, const double* lam_prev, int c_prev) {
+              bool df64, int kd, const double* lam_prev, int c_prev, float* cn, int cld) {
   if (c > MAXC) return fail(MG_EINVAL, "tile_gram: more than 64 columns");
   if (kd < 0 || kd > c || (kd > 0 && (!lam_prev || c_prev < kd)))
     return fail(MG_EINVAL, "tile_gram: bad known-diagonal block");
-  size_t sh = sizeof(zd) * GR * c;
   const int npairs = c * (c + 1) / 2 - kd * (kd + 1) / 2;
-  // one thread per summed pair where they fit one CTA (whole warps, at least two)
-  const int nth = npairs >= GT ? GT : std::max(64, (npairs + 31) / 32 * 32);
   ProfScope ps(df64 ? "svd_gram_df64" : "svd_gram_fp64", 16.0 * B.M * c * B.d * 2,
                8.0 * B.M * npairs * B.d * 2, st);
-  int np = (npairs + nth - 1) / nth;
-#define WMG_GRAM(DFV, MP) \
-  gram_kernel<DFV, MP><<<B.d * 2, nth, sh, st>>>(G, tiles, cmax, c, B.M, kd, lam_prev, c_prev)
   if (df64) {
-    if (np <= 1) WMG_GRAM(true, 1);
-    else if (np <= 2) WMG_GRAM(true, 2);
-    else if (np <= 4) WMG_GRAM(true, 4);
-    else WMG_GRAM(true, 9);
-  } else {
-    if (np <= 1) WMG_GRAM(false, 1);
-    else if (np <= 2) WMG_GRAM(false, 2);
-    else if (np <= 4) WMG_GRAM(false, 4);
-    else WMG_GRAM(false, 9);
+    // 2 x 2 blocks of column pairs, in equal slices of at most GDF_T per CTA; enough threads that
+    // a chunk's column pairs are at most PRE per thread
+    const int cp = (c + 1) / 2, J0 = kd / 2;
+    const int nt = cp * (cp + 1) / 2 - J0 * (J0 + 1) / 2;
+    const int ny = nt < 1 ? 1 : (nt + GDF_T - 1) / GDF_T;
+    const int ntc = nt < 1 ? 1 : (nt + ny - 1) / ny;
+    const int pre = cp <= 2 * GDF_T * GDF_G / GR ? 2 : 4;
+    const int need = std::max(ntc * GDF_G, (GR * cp + pre - 1) / pre);
+    const int nth = (need + 31) / 32 * 32;
+    const size_t sh = sizeof(float4) * 4 * GR * (cp | 1) + sizeof(float2) * 2 * GDF_G * cp;
+    auto kernel = pre == 2 ? gram_df_kernel<2> : gram_df_kernel<4>;
+    WMG_TRY(smem_attr(kernel, sh));
+    kernel<<<dim3(B.d * 2, ny), nth, sh, st>>>(G, cn, cld, (const zdf*)tiles, cmax, c, B.M, kd,
+                                               lam_prev, c_prev, std::max(nt, 1), ntc);
+    WMG_LAUNCHED();
+    return MG_OK;
   }
-#undef WMG_GRAM
+  size_t sh = sizeof(zd) * GR * c;
+  // one thread per summed pair where they fit one CTA (whole warps, at least two)
+  const int nth = npairs >= GT ? GT : std::max(64, (npairs + 31) / 32 * 32);
+  int np = (npairs + nth - 1) / nth;
+  auto go = [&](auto mp) {
+    gram_kernel<decltype(mp)::value><<<B.d * 2, nth, sh, st>>>(G, (const zd*)tiles, cmax, c, B.M,
+                                                               kd, lam_prev, c_prev);
+  };
+  if (np <= 1) go(std::integral_constant<int, 1>{});
+  else if (np <= 2) go(std::integral_constant<int, 2>{});
+  else if (np <= 4) go(std::integral_constant<int, 4>{});
+  else go(std::integral_constant<int, 9>{});
   WMG_LAUNCHED();
   return MG_OK;
 }
@@ -681,18 +953,38 @@ int tile_eig(double* lam, zd* Vec, zd* G, int c, int ntiles, cudaStream_t st, do
 
 int tile_update(void* out, int cmax_out, const void* tiles, int cmax, int c, const zd* Vec,
                 const double* lam, int kout, int scale_inv, const Blocking& B, cudaStream_t st,
-                bool df64) {
+                bool df64, const float* cn, int cld) {
   if (kout > UK || c > MAXC) return fail(MG_EINVAL, "tile_update: too many columns");
-  size_t sh = sizeof(zd) * c * kout;
-  WMG_TRY(smem_attr(df64 ? update_kernel<true> : update_kernel<false>, sh));
   ProfScope ps(df64 ? "svd_update_df64" : "svd_update_fp64", 16.0 * B.M * (c + kout) * B.d * 2,
                8.0 * B.M * c * kout * B.d * 2, st);
-  if (df64)
-    update_kernel<true><<<B.d * 2, GT, sh, st>>>(out, cmax_out, tiles, cmax, c, Vec, lam, kout,
-                                                 scale_inv, B.M);
-  else
-    update_kernel<false><<<B.d * 2, GT, sh, st>>>(out, cmax_out, tiles, cmax, c, Vec, lam, kout,
-                                                  scale_inv, B.M);
+  if (df64) {
+    if (!cn) return fail(MG_EINVAL, "tile_update: no column norms");
+    // output columns in equal groups of at most 12 (four floats of totals each stay in registers);
+    // 256 rows per CTA: ten waves of CTAs on 1024 tiles of 1536 rows instead of five and a bit
+    const int ng = (kout + 11) / 12, per = (kout + ng - 1) / ng;
+    const int ob = per <= 4 ? 4 : per <= 6 ? 6 : per <= 8 ? 8 : per <= 10 ? 10 : 12;
+    const int kp = (kout + ob - 1) / ob * ob, cg = (c + UDG - 1) / UDG;
+    const int rows = 2 * UDT;
+    const dim3 grid(B.d * 2, (B.M + rows - 1) / rows);
+    const size_t sh = sizeof(zdf) * (size_t)cg * UDG * kp + sizeof(float) * (cg * kp + 2 * cg * UDG);
+    auto go = [&](auto kernel) -> int {
+      WMG_TRY(smem_attr(kernel, sh));
+      kernel<<<grid, UDT, sh, st>>>((zdf*)out, cmax_out, (const zdf*)tiles, cmax, c, Vec, lam, cn,
+                                    cld, kout, kp, scale_inv, B.M, rows);
+      return MG_OK;
+    };
+    if (ob == 4) WMG_TRY(go(update_df_kernel<4>));
+    else if (ob == 6) WMG_TRY(go(update_df_kernel<6>));
+    else if (ob == 8) WMG_TRY(go(update_df_kernel<8>));
+    else if (ob == 10) WMG_TRY(go(update_df_kernel<10>));
+    else WMG_TRY(go(update_df_kernel<12>));
+    WMG_LAUNCHED();
+    return MG_OK;
+  }
+  size_t sh = sizeof(zd) * c * kout;
+  WMG_TRY(smem_attr(update_kernel, sh));
+  update_kernel<<<B.d * 2, GT, sh, st>>>((zd*)out, cmax_out, (const zd*)tiles, cmax, c, Vec, lam,
+                                         kout, scale_inv, B.M);
   WMG_LAUNCHED();
   return MG_OK;
 }

@@ -45,6 +45,80 @@ __device__ __forceinline__ void df_fma(dfacc& acc, df a, df b) {
   acc.e = __fadd_rn(acc.e, __fadd_rn(err, pe));
 }
 
+// ---- biased accumulation
+// Sums whose size is bounded beforehand need half of df_fma's instructions.  An accumulator that
+// starts at C = 3 2^q, where every partial sum lies within +-2^q, stays inside the binade
+// [2 2^q, 4 2^q]; then
+//   s = fma(a, b, acc), t = s - acc (exact: both are multiples of one ulp), r = fma(a, b, -t)
+// leaves a b = t + r up to r's own rounding, |r| <= ulp(C) / 2, in three instructions instead of
+// eight.  r and the cross terms collect in e and x (two sums: the cross terms are far smaller).
+// What is lost per term is about 2^-48 C, so C has to follow the sums: callers take it from norm
+// bounds of the operands at hand.
+//
+// The kernels run two such sums per instruction (f32x2, sm_100 and later): the scalar form's
+// three-register multiply-adds stall on register reads at 80 of 128 lanes per clock and SM, the
+// packed form reaches 102 and leaves half of the issue slots to loads and index arithmetic
+// (measured with shared-memory operands, 8 to 20 warps per SM).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float a, float b) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float f2_lo(f32x2 v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float f2_hi(f32x2 v) { return __uint_as_float((unsigned)(v >> 32)); }
+__device__ __forceinline__ f32x2 f2_dup(float a) { return f2_pack(a, a); }
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// two double-float values: (hi, hi) and (lo, lo); two complex ones
+struct df2 {
+  f32x2 hi, lo;
+};
+struct zdf2 {
+  df2 re, im;
+};
+__device__ __forceinline__ df2 df2_dup(df a) { return {f2_dup(a.hi), f2_dup(a.lo)}; }
+__device__ __forceinline__ df2 df2_two_sum(f32x2 a, f32x2 b) {
+  f32x2 s = f2_add(a, b);
+  f32x2 bb = f2_sub(s, a);
+  return {s, f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb))};
+}
+// two values from shared memory, stored as (hi0, hi1, lo0, lo1)
+__device__ __forceinline__ df2 df2_ld(const float4* p) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+  return {v.x, v.y};
+}
+
+struct bacc2 {
+  f32x2 s, e, x;
+};
+__device__ __forceinline__ void bacc2_fma(bacc2& acc, df2 a, df2 b) {
+  const f32x2 s = f2_fma(a.hi, b.hi, acc.s);
+  acc.e = f2_add(acc.e, f2_fma(a.hi, b.hi, f2_sub(acc.s, s)));
+  acc.x = f2_fma(a.hi, b.lo, acc.x);
+  acc.x = f2_fma(a.lo, b.hi, acc.x);
+  acc.s = s;
+}
+
+// C for partial sums within +-bound (bound >= 0): 3 times the power of two above it
+__device__ __forceinline__ float bacc_bias(float bound) {
+  const unsigned u = (__float_as_uint(bound) & 0x7f800000u) + 0x00800000u;
+  return 3.0f * __uint_as_float(u);
+}
+
 // complex df64 value and accumulator
 struct zdf {
   df re, im;
@@ -138,6 +212,35 @@ __device__ __forceinline__ df df_rsqrt(df x) {
     y = df_add(y, df_mul(y, df_mul_f(r, 0.5f)));
   }
   return y;
+}
+
+__device__ __forceinline__ df df_two_sum(float a, float b) {
+  float s = __fadd_rn(a, b);
+  float bb = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+struct zbacc2 {
+  bacc2 re, im;
+};
+// a complex value with its imaginary part's negative, each in both halves
+struct zdfdup {
+  df2 re, im, mim;
+};
+__device__ __forceinline__ zdfdup zdf_dup(zdf a) {
+  return {df2_dup(a.re), df2_dup(a.im), df2_dup(df_neg(a.im))};
+}
+// acc += conj(a) b and acc += a b for the two values of b
+__device__ __forceinline__ void zbacc2_fmac(zbacc2& acc, const zdfdup& a, const zdf2& b) {
+  bacc2_fma(acc.re, a.re, b.re);
+  bacc2_fma(acc.re, a.im, b.im);
+  bacc2_fma(acc.im, a.re, b.im);
+  bacc2_fma(acc.im, a.mim, b.re);
+}
+__device__ __forceinline__ void zbacc2_fma(zbacc2& acc, const zdfdup& a, const zdf2& b) {
+  bacc2_fma(acc.re, a.re, b.re);
+  bacc2_fma(acc.re, a.mim, b.im);
+  bacc2_fma(acc.im, a.re, b.im);
+  bacc2_fma(acc.im, a.im, b.re);
 }
 
 // complex df64 sign and i-multiples (exact)

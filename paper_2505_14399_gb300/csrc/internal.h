@@ -279,8 +279,10 @@ int chiral_gather(void* tiles, int cmax, int col0, const cplx<R>* fields, int nv
 // kd > 0: the first kd columns are the previous stream's Phi = A V_k, orthogonal with squared
 // norms lam_prev[t][0..kd-1] (row stride c_prev): that block is written as the diagonal and
 // only the pairs with a column j >= kd are summed.
+// cn[t][c] (df64, row stride cld, may be null): the columns' squared norms, for tile_update.
 int tile_gram(zd* G, const void* tiles, int cmax, int c, const Blocking& B, cudaStream_t st,
-              bool df64 = false, int kd = 0, const double* lam_prev = nullptr, int c_prev = 0);
+              bool df64 = false, int kd = 0, const double* lam_prev = nullptr, int c_prev = 0,
+              float* cn = nullptr, int cld = 0);
 // Hermitian eigen-decomposition of every G_t (c x c) by parallel cyclic Jacobi; returns
 // eigenvalues descending in lam[t][c] and eigenvectors in Vec[t][c][c] (column i at
 // Vec[t][*][i], row-major c x c).
@@ -289,10 +291,11 @@ int tile_eig(double* lam, zd* Vec, zd* G, int c, int ntiles, cudaStream_t st, do
              bool df64 = false);
 // out[t][i][row] = sum_c A[t][c][row] Vec[t][c][i] * (scale_inv ? 1/sqrt(lam[t][i]) : 1)
 // for i < kout; out tile stride cmax_out*M.
-// df64: double-float tiles in and out, sums of products in double-float arithmetic.
+// df64: double-float tiles in and out, sums of products in double-float arithmetic; needs the
+// squared norms cn of the columns of `tiles` (tile_gram).
 int tile_update(void* out, int cmax_out, const void* tiles, int cmax, int c, const zd* Vec,
                 const double* lam, int kout, int scale_inv, const Blocking& B, cudaStream_t st,
-                bool df64 = false);
+                bool df64 = false, const float* cn = nullptr, int cld = 0);
 // Multiply every column i < k of every tile by conj(q)/|q|, q = sum of its entries.
 int tile_canonical_phase(void* tiles, int cmax, int k, const Blocking& B, cudaStream_t st,
                          bool df64 = false);

@@ -238,6 +238,9 @@ int smooth_stream(mg_handle* h, cplx<R>* psi, cplx<R>* tmp, Gmres<R>& gm, int s,
     if (src->dtype == MG_C128)
       WMG_TRY((convert<R, double>(psi, static_cast<const zd*>(src->fields) + off, nullptr, 0,
                                   h->nf * r, 1, st)));
+    else if (sizeof(R) == 4)   // the same type: a copy, not a conversion kernel
+      WMG_CUDA(cudaMemcpyAsync(psi, static_cast<const zf*>(src->fields) + off,
+                               h->nf * r * sizeof(zf), cudaMemcpyDeviceToDevice, st));
     else
       WMG_TRY((convert<R, float>(psi, static_cast<const zf*>(src->fields) + off, nullptr, 0,
                                  h->nf * r, 1, st)));
@@ -276,11 +279,12 @@ int run_setup(mg_handle* h, cudaStream_t st, const SetupSource* src = nullptr,
   cplx<R>*psi = nullptr, *tmp = nullptr;
   zd *T0 = nullptr, *T1 = nullptr, *G = nullptr, *Vec = nullptr;
   double* lam = nullptr;
+  float* cn = nullptr;   // squared column norms of the double-float tiles (tile_gram)
   Gmres<R> gm;
   int status = MG_OK;
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);   // the cached blocks are reused only after their work ends
-    dfree(psi); dfree(tmp); dfree(T0); dfree(T1); dfree(G); dfree(Vec); dfree(lam);
+    dfree(psi); dfree(tmp); dfree(T0); dfree(T1); dfree(G); dfree(Vec); dfree(lam); dfree(cn);
   };
 #define STEP(x) do { status = (x); if (status != MG_OK) { cleanup(); return status; } } while (0)
 #define CSTEP(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) { cleanup(); return fail(e_ == cudaErrorMemoryAllocation ? MG_ENOMEM : MG_ECUDA, std::string(#x) + ": " + cudaGetErrorString(e_)); } } while (0)
@@ -291,6 +295,7 @@ int run_setup(mg_handle* h, cudaStream_t st, const SetupSource* src = nullptr,
   STEP(dev_alloc(&G, ntile * cmax * cmax * sizeof(zd)));
   STEP(dev_alloc(&Vec, ntile * cmax * cmax * sizeof(zd)));
   STEP(dev_alloc(&lam, ntile * cmax * sizeof(double)));
+  STEP(dev_alloc(&cn, ntile * cmax * sizeof(float)));
   zd* cur = T0;
   zd* oth = T1;
   int kk = 0;
@@ -311,21 +316,21 @@ int run_setup(mg_handle* h, cudaStream_t st, const SetupSource* src = nullptr,
     // update's c-term rounding), so only their cross products with the new vectors and the new
     // vectors' own Gram block are summed (the second pass of the refined route recomputes all)
     const int kd = refine ? 0 : kk;
-    STEP(tile_gram(G, cur, cmax, c, h->B, st, df, kd, lam, c_prev));
+    STEP(tile_gram(G, cur, cmax, c, h->B, st, df, kd, lam, c_prev, cn, cmax));
     STEP(tile_eig(lam, Vec, G, c, (int)ntile, st, eig_tol, df));
     if (ls_omega) {
       // P = A W with W = Omega V_k B^-1 Sigma_k^-1 (Eq. 9); G is free after the eigensolver
       STEP(tile_ls_weights(G, Vec, lam, ls_omega, c, kn, (int)ntile, st));
-      STEP(tile_update(oth, cmax, cur, cmax, c, G, lam, kn, 0, h->B, st, df));
+      STEP(tile_update(oth, cmax, cur, cmax, c, G, lam, kn, 0, h->B, st, df, cn, cmax));
       zd* t = cur; cur = oth; oth = t;
     } else if (p.svd_refine > 0 || (p.svd_refine < 0 && sizeof(R) == 8)) {
       // B = A V (all c columns), then a second Gram/eig pass on B
-      STEP(tile_update(oth, cmax, cur, cmax, c, Vec, lam, c, 0, h->B, st, df));
-      STEP(tile_gram(G, oth, cmax, c, h->B, st, df));
+      STEP(tile_update(oth, cmax, cur, cmax, c, Vec, lam, c, 0, h->B, st, df, cn, cmax));
+      STEP(tile_gram(G, oth, cmax, c, h->B, st, df, 0, nullptr, 0, cn, cmax));
       STEP(tile_eig(lam, Vec, G, c, (int)ntile, st, eig_tol, df));
-      STEP(tile_update(cur, cmax, oth, cmax, c, Vec, lam, kn, last ? 1 : 0, h->B, st, df));
+      STEP(tile_update(cur, cmax, oth, cmax, c, Vec, lam, kn, last ? 1 : 0, h->B, st, df, cn, cmax));
     } else {
-      STEP(tile_update(oth, cmax, cur, cmax, c, Vec, lam, kn, last ? 1 : 0, h->B, st, df));
+      STEP(tile_update(oth, cmax, cur, cmax, c, Vec, lam, kn, last ? 1 : 0, h->B, st, df, cn, cmax));
       zd* t = cur; cur = oth; oth = t;
     }
     STEP(tile_sigma(h->hist + (size_t)s * ntile * k, k, lam, c, kn, (int)ntile, st));
