@@ -83,6 +83,9 @@ __device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// a b as a multiply-add of zero: ptxas 13.0 contracts a packed multiplication into a packed
+// addition that follows (measured: dfacc2_fma with mul.rn.f32x2 loses all its low bits)
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) { return f2_fma(a, b, 0); }
 // two double-float values: (hi, hi) and (lo, lo); two complex ones
 struct df2 {
   f32x2 hi, lo;
@@ -100,6 +103,29 @@ __device__ __forceinline__ df2 df2_two_sum(f32x2 a, f32x2 b) {
 __device__ __forceinline__ df2 df2_ld(const float4* p) {
   const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
   return {v.x, v.y};
+}
+
+// df_fma on two values (f32x2 has no negation: mah = -a.hi)
+struct dfacc2 {
+  f32x2 s, e;
+};
+__device__ __forceinline__ void dfacc2_fma(dfacc2& acc, df2 a, f32x2 mah, df2 b, bool first) {
+  const f32x2 p = f2_mul(a.hi, b.hi);
+  f32x2 pe = f2_fma(a.hi, b.hi, f2_mul(mah, b.hi));
+  pe = f2_fma(a.hi, b.lo, pe);
+  pe = f2_fma(a.lo, b.hi, pe);
+  if (first) {
+    acc = {p, pe};
+    return;
+  }
+  const df2 s = df2_two_sum(acc.s, p);
+  acc.s = s.hi;
+  acc.e = f2_add(acc.e, f2_add(s.lo, pe));
+}
+// an accumulator as normalised values (|s| >= |e|)
+__device__ __forceinline__ df2 df2_norm(const dfacc2& a) {
+  const f32x2 h = f2_add(a.s, a.e);
+  return {h, f2_sub(a.e, f2_sub(h, a.s))};
 }
 
 struct bacc2 {

@@ -7,13 +7,14 @@
 // Every staged double-float entry v satisfies |v| < 2 (|P| <= 1 entrywise for orthonormal
 // columns; |U h| <= sqrt(3) for unitary U and |h| <= 1), so it is written exactly enough as
 // fixed-point digits in base 256,
-//     v = sum_{i < NS} s_i 2^{-6-8i},  s_i integers, |s_i| <= 129,  NS = 7
-// (error at most 2^-55 (1 + 2^-16)),
+//     v = sum_{i < NS} s_i 2^{-6-8i},  s_i integers, |s_i| <= 128,  NS = 7
+// (error at most 2^-55),
 // each digit exact in bfloat16.  A product of digit planes is an integer matrix product:
 // bf16 x bf16 tensor-core MMAs with FP32 accumulation are exact while the partial sums stay
-// below 2^24, which holds for one staging batch (<= 7 digit pairs x 96 stacked rows x 129^2).
-// Digit pairs i + j = d of the same weight 2^{-12-8d} share an FP32 accumulator; pairs with
-// i + j >= NS (weight below 2^-68) are dropped.  After every batch the exact FP32 sums are
+// below 2^24, which holds for three staging batches (7 digit pairs x 3 x 48 stacked rows x
+// 128^2 = 0.984 2^24).  Digit pairs i + j = d of the same weight 2^{-12-8d} share an FP32
+// accumulator; pairs with i + j >= NS (weight below 2^-68) are dropped.  After every third batch
+// (every one where a warp's tiles leave no registers for that) the exact FP32 sums are
 // scaled by their weights (exact) and added to double-float accumulators with error-free
 // two-sums, so the result carries double-float accuracy (~2^-48 relative), not bf16's.
 //
@@ -26,11 +27,14 @@
 // planes are stored k'-major (SA[k'][b'], SB[k'][a]) so that staging threads with consecutive
 // columns write consecutive addresses, and read with ldmatrix .trans; every row stride is an
 // odd number of 16-byte units, so the eight rows of an ldmatrix phase hit distinct banks.
-// A batch is NB = 4 sites (one warp group, three k' steps) or, for 2k <= 24, NB = 8 sites (two
-// warp groups split its six 16-row k' steps; the digit planes and the double-buffered raw
-// inputs of one CTA then take ~195 KB, one CTA per SM).  At 4 sites a CTA fits its shared
-// memory up to the paper's k = 24, and for 2k <= 24 two CTAs share an SM, so one CTA's staging
-// overlaps the other's products; the autotuner picks between the two where both fit.
+// A batch is NB = 4 sites: three k' steps of 16 stacked rows.  For 2k <= 24 two CTAs (three and
+// four for 2k <= 16 and 8) share an SM, so one CTA's staging overlaps the other's products.
+//
+// Staging (double-float colour transport, digit split) runs on two adjacent columns at once in
+// packed FP32 instructions.  It was the bound, with the per-batch fold: 3.11 ms at 16^3x32, k =
+// 12, tensor pipe a fifth busy; 2.57 ms now (21.7 -> 19.8 ms at 16^3x64, k = 24), where the FP32
+// pipe is busy 61 % of the time, the tensor pipe 27 %, and the warps wait for the barriers
+// between staging and products.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -46,29 +50,30 @@ namespace {
 
 constexpr int TC_MAXT4 = 6;            // 2k <= 48
 
-// Per column-tile count T4 (2k <= 8 T4) and sites per batch NB_ (8 or 4): stacked rows, warp
-// groups, warps.
-template <int T4, int NB_>
+constexpr int NB = 4;                  // fine sites staged per batch
+constexpr int KB = NB * 6;             // staged rows per batch
+constexpr int TCK = 2 * KB;            // stacked real rows per batch
+
+// Per column-tile count T4 (2k <= 8 T4): tiles, warps.
+template <int T4>
 struct TcCfg {
-  static constexpr int NB = NB_;                       // fine sites staged per batch
-  static constexpr int KB = NB * 6;                    // staged rows per batch
-  static constexpr int K = 2 * KB;                     // stacked real rows (96 or 48)
-  static constexpr int WG = (K / 16) % 2 == 0 ? 2 : 1; // warp groups (each takes k' steps)
   static constexpr int NTILES = T4 * T4;
-  // warps per group: at most 12 (two groups) or 16 (one group), tiles spread evenly
-  static constexpr int MAXW = WG == 2 ? 12 : 16;
+  static constexpr int MAXW = T4 == 6 ? 18 : 16;           // warps that take tiles, at most
   static constexpr int TPW = (NTILES + MAXW - 1) / MAXW;   // tiles per warp
   static constexpr int NW = (NTILES + TPW - 1) / TPW;
-  // resident CTAs per SM asked of the register allocator: two for 4-site batches of 2k <= 24
-  // (about 100 KB of shared memory each), whose staging and products then overlap
-  static constexpr int MINB = (NB == 4 && T4 <= 3) ? 2 : 1;
+  // warps of the CTA: one staging item (row, column pair) per thread
+  static constexpr int WARPS = NW > 3 * T4 ? NW : 3 * T4;
+  // resident CTAs per SM asked of the register allocator
+  static constexpr int MINB = T4 == 1 ? 4 : T4 == 2 ? 3 : T4 == 3 ? 2 : 1;
+  // batches between folds
+  static constexpr int FOLD = TPW == 1 ? 3 : 1;
 };
 
 // Row strides (bf16) of the k'-major digit planes: odd multiples of 8 (16 bytes).
 __host__ __device__ constexpr int tc_lda(int t4) { return 16 * t4 + 8; }
 __host__ __device__ constexpr int tc_ldb(int t4) { return 8 * t4 + ((t4 & 1) ? 0 : 8); }
-__host__ __device__ constexpr size_t tc_smem(int t4, int nb) {
-  return sizeof(__nv_bfloat16) * (size_t)TC_NS * 12 * nb * (tc_lda(t4) + tc_ldb(t4));
+__host__ __device__ constexpr size_t tc_smem(int t4) {
+  return sizeof(__nv_bfloat16) * (size_t)TC_NS * TCK * (tc_lda(t4) + tc_ldb(t4));
 }
 
 // Shared memory of one CTA beyond the digit planes: two raw input buffers (P(x + mu) and P(x)
@@ -78,35 +83,57 @@ __host__ __device__ constexpr size_t tc_smem(int t4, int nb) {
 // sits in slot (b odd ? k : 0) + b / 2, so that the staging threads, which take the column
 // pairs (2q, 2q + 1) for consecutive q, read consecutive 16-byte slots.
 __host__ __device__ constexpr int tc_nrp(int t4) { return 8 * t4 + 1; }
-__host__ __device__ constexpr size_t tc_raw_bytes(int t4, int nb) {
-  return sizeof(zdf) * 2 * ((size_t)2 * nb * 6 * tc_nrp(t4) + nb * 9);
+__host__ __device__ constexpr size_t tc_raw_bytes(int t4) {
+  return sizeof(zdf) * 2 * ((size_t)2 * NB * 6 * tc_nrp(t4) + NB * 9);
 }
 __host__ __device__ inline size_t tc_table_bytes(int nd) { return sizeof(int) * 8 * (size_t)nd + 16; }
-__host__ __device__ inline size_t tc_cta_bytes(int t4, int nb, int nd) {
-  return tc_smem(t4, nb) + tc_raw_bytes(t4, nb) + tc_table_bytes(nd);
+__host__ __device__ inline size_t tc_cta_bytes(int t4, int nd) {
+  return tc_smem(t4) + tc_raw_bytes(t4) + tc_table_bytes(nd);
 }
-template <int T4, int NB_>
-__global__ void __launch_bounds__(32 * TcCfg<T4, NB_>::WG * TcCfg<T4, NB_>::NW,
-                                  TcCfg<T4, NB_>::MINB)
+
+// i^rot x for the two halves of x, rot 0 .. 3 per half (sign changes and swaps: exact)
+__device__ __forceinline__ zdf2 rot_i(zdf2 x, int rot0, int rot1) {
+  auto one = [](float re, float im, int rot, float& ore, float& oim) {
+    const float a = (rot & 1) ? im : re, b = (rot & 1) ? re : im;
+    // rot 1: (-im, re), 2: (-re, -im), 3: (im, -re)
+    const unsigned sa = (rot == 1 || rot == 2) ? 0x80000000u : 0u;
+    const unsigned sb = (rot & 2) ? 0x80000000u : 0u;
+    ore = __uint_as_float(__float_as_uint(a) ^ sa);
+    oim = __uint_as_float(__float_as_uint(b) ^ sb);
+  };
+  float h[4], l[4];
+  one(f2_lo(x.re.hi), f2_lo(x.im.hi), rot0, h[0], h[1]);
+  one(f2_hi(x.re.hi), f2_hi(x.im.hi), rot1, h[2], h[3]);
+  one(f2_lo(x.re.lo), f2_lo(x.im.lo), rot0, l[0], l[1]);
+  one(f2_hi(x.re.lo), f2_hi(x.im.lo), rot1, l[2], l[3]);
+  return {{f2_pack(h[0], h[2]), f2_pack(l[0], l[2])}, {f2_pack(h[1], h[3]), f2_pack(l[1], l[3])}};
+}
+__device__ __forceinline__ zdf2 zdf2_pair(const zdf& a, const zdf& b) {
+  return {{f2_pack(a.re.hi, b.re.hi), f2_pack(a.re.lo, b.re.lo)},
+          {f2_pack(a.im.hi, b.im.hi), f2_pack(a.im.lo, b.im.lo)}};
+}
+
+template <int T4>
+__global__ void __launch_bounds__(32 * TcCfg<T4>::WARPS, TcCfg<T4>::MINB)
 galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
                    const zdf* __restrict__ Ldf, HopGeom g, Blocking B, int* range_flag) {
-  using C = TcCfg<T4, NB_>;
+  using C = TcCfg<T4>;
   constexpr int NR = 8 * T4;                  // columns a (>= 2k)
   constexpr int NTILES = C::NTILES;
   constexpr int NW = C::NW;
   constexpr int TPW = C::TPW;                 // tiles per warp
-  constexpr int NB = C::NB, KB = C::KB, K = C::K, WG = C::WG;
+  constexpr int K = TCK;
   constexpr int ND = TC_NS;                   // digit-pair weights d = i + j < NS
   constexpr int LDA = tc_lda(T4), LDB = tc_ldb(T4);
   extern __shared__ __align__(16) unsigned char tc_raw[];
   __nv_bfloat16* SA = reinterpret_cast<__nv_bfloat16*>(tc_raw);   // [NS][K][LDA]
   __nv_bfloat16* SB = SA + (size_t)TC_NS * K * LDA;                // [NS][K][LDB]
   constexpr int NRP = tc_nrp(T4);
-  zdf* sPy = reinterpret_cast<zdf*>(tc_raw + tc_smem(T4, NB));     // [2][NB][6][NRP]
+  zdf* sPy = reinterpret_cast<zdf*>(tc_raw + tc_smem(T4));     // [2][NB][6][NRP]
   zdf* sPx = sPy + (size_t)2 * NB * 6 * NRP;                       // [2][NB][6][NRP]
   zdf* sU = sPx + (size_t)2 * NB * 6 * NRP;                        // [2][NB][9]
   const int nd = B.nd;
-  int* tx = reinterpret_cast<int*>(tc_raw + tc_smem(T4, NB) + tc_raw_bytes(T4, NB));   // site x
+  int* tx = reinterpret_cast<int*>(tc_raw + tc_smem(T4) + tc_raw_bytes(T4));   // site x
   int* toy = tx + nd;      // P offset of (2 j(y)) k M, y = x + mu
   int* tox = toy + nd;     // P offset of (2 j(x)) k M
   int* tly = tox + nd;     // local site of y, x
@@ -121,8 +148,8 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
   const int M = B.M;
   const size_t V = (size_t)B.nd * B.d;
   const int lane = threadIdx.x & 31;
-  const int wid = (threadIdx.x >> 5) % NW, grp = (threadIdx.x >> 5) / NW;   // tile slot, k' half
-  const size_t plane16 = tc_smem(T4, NB) / 16;   // 16-byte chunks of SA + SB
+  const int wid = threadIdx.x >> 5;   // tile slot; warps beyond NW only stage
+  const size_t plane16 = tc_smem(T4) / 16;   // 16-byte chunks of SA + SB
   bool bad = false;
 
   // ---- per-site tables of this aggregate, and the two passes' site lists
@@ -204,11 +231,10 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
     // zero both digit planes: padding rows and columns stay zero for the whole pass
     for (size_t e = threadIdx.x; e < plane16; e += blockDim.x)
       reinterpret_cast<uint4*>(tc_raw)[e] = make_uint4(0u, 0u, 0u, 0u);
-    dfacc dacc[TPW][4];
+    dfacc2 dacc[TPW][2];
+    float acc[TPW][ND][4];
 #pragma unroll
-    for (int t = 0; t < TPW; ++t)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) dacc[t][e] = {0.0f, 0.0f};
+    for (int t = 0; t < TPW; ++t) dacc[t][0] = dacc[t][1] = {0, 0};
     const int nbat = (nsel[pass] + NB - 1) / NB;
     if (nbat > 0) prefetch(pass, 0, 0);
     for (int b = 0; b < nbat; ++b) {
@@ -245,81 +271,83 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
         const int q = sq;
         const int s = r / 3, cc = r - 3 * s;
         const zdf* U = pu + h * 9 + cc * 3;
-        const zdf u0 = U[0], u1 = U[1], u2 = U[2];
         const bool neg = tng[ls[h]] != 0;
-        float cr[2][TC_NS], ci[2][TC_NS], tr[2][TC_NS], ti[2][TC_NS];
+        // columns of chirality 1 take i sigma_mu psi_dn (mu < 3) or -psi_dn (mu = 3): one
+        // component of the pair times a power of i, which commutes with the colour transport
+        const zdf* Py = py + (size_t)h * 6 * NRP + q;
+        const zdf* Px = px + (size_t)h * 6 * NRP + q;
+        int pi[2], rot[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int bcol = 2 * q + u;
-          const int beta = bcol >= k;
-          // component q' of this column at this site: P*[q' * NRP] (slot u k + q)
-          const zdf* Py = py + (size_t)h * 6 * NRP + u * k + q;
-          const zdf* Px = px + (size_t)h * 6 * NRP + u * k + q;
-          zdf hv[3];
+          const bool up = 2 * q + u < k;
+          pi[u] = u * k + NRP * 3 * ((up || mu >= 2) ? s : 1 - s);   // column slot, spin row
+          rot[u] = up ? 0 : mu == 0 ? 1 : mu == 1 ? 2 * s : mu == 2 ? 1 + 2 * s : 2;
+        }
+        dfacc2 tre, tim;
 #pragma unroll
-          for (int c2 = 0; c2 < 3; ++c2) {
-            if (beta == 0) {
-              hv[c2] = Py[(s * 3 + c2) * NRP];
-            } else {
-              zdf p0 = Py[c2 * NRP], p1 = Py[(3 + c2) * NRP];
-              hv[c2] = mu < 3 ? isigma_df(mu, s, p0, p1) : zdf_neg(s == 0 ? p0 : p1);
-            }
-          }
-          zdfacc t{};
-          zdf_fma(t, u0, hv[0]);
-          zdf_fma(t, u1, hv[1]);
-          zdf_fma(t, u2, hv[2]);
-          zdf ch = zdf_norm(t);
-          if (neg) ch = zdf_neg(ch);
-          zdf pt;
-          if (beta == 0) {
-            pt = Px[(s * 3 + cc) * NRP];
-          } else {
-            zdf p0 = Px[cc * NRP], p1 = Px[(3 + cc) * NRP];
-            pt = mu < 3 ? isigma_df(mu, s, p0, p1) : zdf_neg(s == 0 ? p0 : p1);
-          }
-          bad |= !(tc_in_range(ch.re) && tc_in_range(ch.im) && tc_in_range(pt.re) &&
-                   tc_in_range(pt.im));
-          tc_digits(ch.re, cr[u]);
-          tc_digits(ch.im, ci[u]);
-          tc_digits(pt.re, tr[u]);
-          tc_digits(pt.im, ti[u]);
+        for (int c2 = 0; c2 < 3; ++c2) {
+          const zdf u = U[c2];
+          const zdf2 v = zdf2_pair(Py[pi[0] + c2 * NRP], Py[pi[1] + c2 * NRP]);
+          const df2 ur = df2_dup(u.re), ui = df2_dup(u.im), mi = df2_dup(df_neg(u.im));
+          const f32x2 mr = f2_dup(-u.re.hi);
+          dfacc2_fma(tre, ur, mr, v.re, c2 == 0);
+          dfacc2_fma(tre, mi, ui.hi, v.im, false);
+          dfacc2_fma(tim, ur, mr, v.im, c2 == 0);
+          dfacc2_fma(tim, ui, mi.hi, v.re, false);
         }
         const int kk = h * 6 + r;
+        f32x2 dr[TC_NS], di[TC_NS];
+        {
+          const int n2 = neg ? 2 : 0;
+          const zdf2 ch = rot_i({df2_norm(tre), df2_norm(tim)}, (rot[0] + n2) & 3, (rot[1] + n2) & 3);
+          bad |= !(tc_in_range(ch.re) && tc_in_range(ch.im));
+          tc_digits2(ch.re, dr);
+          tc_digits2(ch.im, di);
 #pragma unroll
-        for (int i = 0; i < TC_NS; ++i) {
-          __nv_bfloat16* a0 = SA + ((size_t)i * K + kk) * LDA;          // re rows k
-          __nv_bfloat16* a1 = SA + ((size_t)i * K + KB + kk) * LDA;     // im rows k
-          const unsigned pr = tc_pack(cr[0][i], cr[1][i]), pi = tc_pack(ci[0][i], ci[1][i]);
-          *reinterpret_cast<unsigned*>(a0 + 2 * q) = pr;
-          *reinterpret_cast<unsigned*>(a1 + 2 * q) = pi;
-          *reinterpret_cast<unsigned*>(a0 + n2k + 2 * q) = pi;
-          *reinterpret_cast<unsigned*>(a1 + n2k + 2 * q) = pr ^ 0x80008000u;   // -Ch_re
-          *reinterpret_cast<unsigned*>(SB + ((size_t)i * K + kk) * LDB + 2 * q) =
-              tc_pack(tr[0][i], tr[1][i]);
-          *reinterpret_cast<unsigned*>(SB + ((size_t)i * K + KB + kk) * LDB + 2 * q) =
-              tc_pack(ti[0][i], ti[1][i]);
+          for (int i = 0; i < TC_NS; ++i) {
+            __nv_bfloat16* a0 = SA + ((size_t)i * K + kk) * LDA;          // re rows k
+            __nv_bfloat16* a1 = SA + ((size_t)i * K + KB + kk) * LDA;     // im rows k
+            const unsigned pr = tc_pack(dr[i]), pim = tc_pack(di[i]);
+            *reinterpret_cast<unsigned*>(a0 + 2 * q) = pr;
+            *reinterpret_cast<unsigned*>(a1 + 2 * q) = pim;
+            *reinterpret_cast<unsigned*>(a0 + n2k + 2 * q) = pim;
+            *reinterpret_cast<unsigned*>(a1 + n2k + 2 * q) = pr ^ 0x80008000u;   // -Ch_re
+          }
+        }
+        {
+          const zdf2 pt = rot_i(zdf2_pair(Px[pi[0] + cc * NRP], Px[pi[1] + cc * NRP]), rot[0], rot[1]);
+          bad |= !(tc_in_range(pt.re) && tc_in_range(pt.im));
+          tc_digits2(pt.re, dr);
+          tc_digits2(pt.im, di);
+#pragma unroll
+          for (int i = 0; i < TC_NS; ++i) {
+            *reinterpret_cast<unsigned*>(SB + ((size_t)i * K + kk) * LDB + 2 * q) = tc_pack(dr[i]);
+            *reinterpret_cast<unsigned*>(SB + ((size_t)i * K + KB + kk) * LDB + 2 * q) =
+                tc_pack(di[i]);
+          }
         }
       }
       __syncthreads();
       // exact digit-plane products of this warp's output tiles, folded into double-float
+      const bool start = b % C::FOLD == 0, fold = b % C::FOLD == C::FOLD - 1 || b == nbat - 1;
 #pragma unroll
       for (int tt = 0; tt < TPW; ++tt) {
         const int tile = wid + tt * NW;
-        if (tile < NTILES) {
+        if (wid < NW && tile < NTILES) {
           const int mt = tile / T4, nt = tile % T4;
-          float acc[ND][4];
+          if (start) {
 #pragma unroll
-          for (int d = 0; d < ND; ++d)
+            for (int d = 0; d < ND; ++d)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[d][e] = 0.0f;
+              for (int e = 0; e < 4; ++e) acc[tt][d][e] = 0.0f;
+          }
           // ldmatrix .trans row addresses: A matrices (b' 0-7 | 8-15) x (k 0-7 | 8-15) in the
           // order of the A fragment, B matrices k 0-7 | 8-15 for columns a of this tile
           const int mq = lane >> 3, rr = lane & 7;
           const __nv_bfloat16* arow = SA + (size_t)(8 * (mq >> 1) + rr) * LDA + 16 * mt + 8 * (mq & 1);
           const __nv_bfloat16* brow = SB + (size_t)(8 * (mq & 1) + rr) * LDB + 8 * nt;
 #pragma unroll 1
-          for (int ks = grp * (K / 16 / WG); ks < (grp + 1) * (K / 16 / WG); ++ks) {
+          for (int ks = 0; ks < K / 16; ++ks) {
             unsigned bfr[TC_NS][2];
 #pragma unroll
             for (int i = 0; i < TC_NS; ++i)
@@ -330,44 +358,43 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
               ldm_x4t(af, arow + ((size_t)i * K + 16 * ks) * LDA);
 #pragma unroll
               for (int jd = 0; jd < TC_NS; ++jd)
-                if (i + jd < ND) mma_bf16(acc[i + jd], af, bfr[jd]);
+                if (i + jd < ND) mma_bf16(acc[tt][i + jd], af, bfr[jd]);
             }
           }
-          // weights 2^{-12-8d}: exact FP32 constants
-          float wgt = 1.0f / 4096.0f;
+          if (fold) {
+            // weights 2^{-12-8d}: exact FP32 constants
+            float wgt = 1.0f / 4096.0f;
 #pragma unroll
-          for (int d = 0; d < ND; ++d) {
+            for (int d = 0; d < ND; ++d) {
+              const f32x2 w2 = f2_dup(wgt);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc_add(dacc[tt][e], acc[d][e] * wgt);
-            wgt *= 1.0f / 256.0f;
+              for (int e = 0; e < 2; ++e)
+                acc_add(dacc[tt][e], f2_mul(f2_pack(acc[tt][d][2 * e], acc[tt][d][2 * e + 1]), w2));
+              wgt *= 1.0f / 256.0f;
+            }
           }
         }
       }
     }
-    // this pass's blocks: tiles -> shared memory (over the digit planes) -> Op / Xpart; the
-    // second warp group adds its half of the rows to the first group's
+    // this pass's blocks: tiles -> shared memory (over the digit planes) -> Op / Xpart
     __syncthreads();
     df* sOut = reinterpret_cast<df*>(tc_raw);   // [16 T4][NR]
-    for (int g2 = 0; g2 < WG; ++g2) {
-      if (grp == g2) {
 #pragma unroll
-        for (int tt = 0; tt < TPW; ++tt) {
-          const int tile = wid + tt * NW;
-          if (tile < NTILES) {
-            const int mt = tile / T4, nt = tile % T4;
-            const int row = 16 * mt + (lane >> 2), col = 8 * nt + 2 * (lane & 3);
-            const size_t o[4] = {(size_t)row * NR + col, (size_t)row * NR + col + 1,
-                                 (size_t)(row + 8) * NR + col, (size_t)(row + 8) * NR + col + 1};
+    for (int tt = 0; tt < TPW; ++tt) {
+      const int tile = wid + tt * NW;
+      if (wid < NW && tile < NTILES) {
+        const int mt = tile / T4, nt = tile % T4;
+        const int row = 16 * mt + (lane >> 2), col = 8 * nt + 2 * (lane & 3);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              df v = df_norm(dacc[tt][e]);
-              sOut[o[e]] = g2 == 0 ? v : df_add(sOut[o[e]], v);
-            }
-          }
+        for (int e = 0; e < 2; ++e) {
+          const df2 v = df2_norm(dacc[tt][e]);
+          df* o = sOut + (size_t)(row + 8 * e) * NR + col;
+          o[0] = {f2_lo(v.hi), f2_lo(v.lo)};
+          o[1] = {f2_hi(v.hi), f2_hi(v.lo)};
         }
       }
-      __syncthreads();
     }
+    __syncthreads();
     zd* out = pass == 1 ? Op + ((size_t)j * 9 + 1 + dir) * ne
                         : Xpart + ((size_t)mu * B.d + j) * ne;
     for (int e = threadIdx.x; e < ne; e += blockDim.x) {
@@ -380,18 +407,17 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
   if (bad) atomicExch(range_flag, 1);
 }
 
-template <int T4, int NB>
+template <int T4>
 int launch_tc(zd* Op, zd* Xpart, const zdf* Pdf, int k, const zdf* Ldf, const HopGeom& g,
               const Blocking& B, int* range_flag, cudaStream_t st) {
-  constexpr int NW = TcCfg<T4, NB>::NW * TcCfg<T4, NB>::WG;
-  size_t sh = tc_cta_bytes(T4, NB, B.nd);
-  WMG_TRY(smem_attr(galerkin_tc_kernel<T4, NB>, sh));
-  if (TcCfg<T4, NB>::MINB > 1)   // room for two CTAs: the largest shared-memory carveout
-    WMG_CUDA(cudaFuncSetAttribute(galerkin_tc_kernel<T4, NB>,
+  size_t sh = tc_cta_bytes(T4, B.nd);
+  WMG_TRY(smem_attr(galerkin_tc_kernel<T4>, sh));
+  if (TcCfg<T4>::MINB > 1)   // room for several CTAs: the largest shared-memory carveout
+    WMG_CUDA(cudaFuncSetAttribute(galerkin_tc_kernel<T4>,
                                   cudaFuncAttributePreferredSharedMemoryCarveout,
                                   (int)cudaSharedmemCarveoutMaxShared));
-  galerkin_tc_kernel<T4, NB><<<dim3(B.d, 4), 32 * NW, sh, st>>>(Op, Xpart, Pdf, k, Ldf, g, B,
-                                                                range_flag);
+  galerkin_tc_kernel<T4><<<dim3(B.d, 4), 32 * TcCfg<T4>::WARPS, sh, st>>>(Op, Xpart, Pdf, k, Ldf, g,
+                                                                          B, range_flag);
   WMG_LAUNCHED();
   return MG_OK;
 }
@@ -402,64 +428,31 @@ constexpr size_t kTcSmemMax = (size_t)227 * 1024 - 1024;
 
 bool galerkin_tc_supported(int k, const Blocking& B) {
   if (k < 1 || (k + 3) / 4 > TC_MAXT4) return false;
-  // shared memory of one CTA at 4 sites per batch, and tile offsets that fit an int
+  // shared memory of one CTA, and tile offsets that fit an int
   const int t4 = (k + 3) / 4;
-  return tc_cta_bytes(t4, 4, B.nd) <= kTcSmemMax &&
+  return tc_cta_bytes(t4, B.nd) <= kTcSmemMax &&
          (size_t)B.d * 2 * k * B.M < ((size_t)1 << 31);
 }
 
-double galerkin_tc_issued_flops(int k, const Blocking& B, int nb) {
+double galerkin_tc_issued_flops(int k, const Blocking& B) {
   // bf16 digit-plane products issued: 28 digit pairs of a (16 T4) x (8 T4) x (12 NB) real
   // product per batch and hop direction, about n_d / NB + 1 batches per CTA
   const int t4 = (k + 3) / 4;
-  return 2.0 * (16.0 * t4) * (8.0 * t4) * (12.0 * nb) * 28.0 * 4.0 * B.d *
-         ((double)B.nd / nb + 1.0);
+  return 2.0 * (16.0 * t4) * (8.0 * t4) * (12.0 * NB) * 28.0 * 4.0 * B.d *
+         ((double)B.nd / NB + 1.0);
 }
 
 int galerkin_hops_tc(zd* Op, zd* Xpart, const zdf* Pdf, int k, const zdf* Ldf, const HopGeom& g,
-                     const Blocking& B, int nb, int* range_flag, cudaStream_t st) {
-  if (nb == 8) {
-    switch ((k + 3) / 4) {
-      case 1: return launch_tc<1, 8>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-      case 2: return launch_tc<2, 8>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-      case 3: return launch_tc<3, 8>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-      default: return fail(MG_EINVAL, "galerkin (tensor pipe): 8-site batches need 2k <= 24");
-    }
-  }
-  if (nb != 4) return fail(MG_EINVAL, "galerkin (tensor pipe): batches of 4 or 8 sites");
+                     const Blocking& B, int* range_flag, cudaStream_t st) {
   switch ((k + 3) / 4) {
-    case 1: return launch_tc<1, 4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-    case 2: return launch_tc<2, 4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-    case 3: return launch_tc<3, 4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-    case 4: return launch_tc<4, 4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-    case 5: return launch_tc<5, 4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
-    case 6: return launch_tc<6, 4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
+    case 1: return launch_tc<1>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
+    case 2: return launch_tc<2>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
+    case 3: return launch_tc<3>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
+    case 4: return launch_tc<4>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
+    case 5: return launch_tc<5>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
+    case 6: return launch_tc<6>(Op, Xpart, Pdf, k, Ldf, g, B, range_flag, st);
     default: return fail(MG_EINVAL, "galerkin (tensor pipe): 2k > 48");
   }
-}
-
-int galerkin_tc_batch(int* nb, zd* Op, zd* Xpart, const zdf* Pdf, int k, const zdf* Ldf,
-                      const HopGeom& g, const Blocking& B, int* range_flag, cudaStream_t st) {
-  // 8-site batches (one CTA per SM: the staging and the products of a CTA alternate) or
-  // 4-site batches (two CTAs per SM whose phases overlap, twice the per-batch folds): the
-  // autotuner times both on the live arguments where both fit (2k <= 24); the kernel is
-  // idempotent (it rewrites its outputs from inputs it does not modify; the range flag, which
-  // the caller clears before its own launch, can only be raised)
-  const int t4 = (k + 3) / 4;
-  if (t4 > 3 || tc_cta_bytes(t4, 8, B.nd) > kTcSmemMax) {
-    *nb = 4;
-    return MG_OK;
-  }
-  int err = MG_OK;
-  auto run = [&](int v) {
-    int e = galerkin_hops_tc(Op, Xpart, Pdf, k, Ldf, g, B, v == 0 ? 8 : 4, range_flag, st);
-    if (e != MG_OK) err = e;
-  };
-  int v = tuned_variant(2000 + t4, -3, 0, B.d * B.nd, k, st, 2, run);
-  if (err != MG_OK) return err;
-  if (v < 0) return fail(MG_ECUDA, "galerkin (tensor pipe): autotune failed");
-  *nb = v == 0 ? 8 : 4;
-  return MG_OK;
 }
 
 }  // namespace wmg

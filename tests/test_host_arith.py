@@ -92,3 +92,53 @@ def test_tile_reciprocals_of_the_stencil_are_exact():
         b = np.unique(np.concatenate([np.arange(min(4 * n, 4096)),
                                       rng.integers(0, (2 ** 32 - 1) // n, 2000)])).astype(np.uint64)
         assert np.array_equal((b * np.uint64(m)) >> np.uint64(32), b // np.uint64(n))
+
+
+def test_digit_split_by_magic_sums():
+    """The kernel's digit split: v plus 1.5 2^k (and 128 units) in units of 2^-14, 2^-30, 2^-46 and
+    2^-54, the remainders renormalised by fast two-sums, digits from the bytes of the sums' words.
+    Every remainder is exact as rationals, every digit has |d| <= 128, and the value minus its
+    expansion sum_i d_i 2^(-6-8i) is at most 2^-55 (half of the last unit)."""
+    def word(x):
+        return int(np.array(x, dtype=F).view(np.uint32))
+
+    magic = [F(float.fromhex("0x1.8p9") + float.fromhex("0x1p-7")),
+             F(float.fromhex("0x1.8p-7") + float.fromhex("0x1p-23")),
+             F(float.fromhex("0x1.8p-23") + float.fromhex("0x1p-39")),
+             F(float.fromhex("0x1.8p-31") + float.fromhex("0x1p-40"))]
+    units = [Fraction(1, 2 ** e) for e in (14, 30, 46, 54)]
+    for m, u, off in zip(magic, units, (128, 128, 128, 2 ** 14)):
+        # exact constants: 1.5 2^23 units and the offset, in a word whose bit 23 is clear
+        assert Fraction(float(m)) == u * (3 * 2 ** 22 + off) and not word(m) >> 23 & 1
+    rng = np.random.default_rng(3)
+    xs = _values() + [s * (2 - 2.0 ** -23) for s in (1, -1)]
+    # remainders at their largest: halves of the first two units, on both sides
+    xs += [float(n) * 2.0 ** -14 + s * 2.0 ** -15 + t * 2.0 ** -31
+           for n in rng.integers(-20000, 20000, 200) for s in (1, -1) for t in (1, 0, -1)]
+    for x in xs:
+        hi = F(x)
+        lo = F(x - float(hi))
+        ds, h, l = [], hi, lo
+        for i, (m, u) in enumerate(zip(magic, units)):
+            before = Fraction(float(h)) + Fraction(float(l))
+            if i == 3:
+                h, l = F(h + l), F(0)     # the last remainder in one word
+            a = F(h + m)
+            n = Fraction(float(F(a - m)))
+            w = word(a)
+            if i < 3:
+                ds += [((w >> 8) & 0xFFFF) - 2 ** 14, (w & 0xFF) - 128]
+                assert 256 * ds[-2] + ds[-1] == n / u
+                r = F(h - F(a - m))
+                h = F(r + l)
+                l = F(l - F(h - r))
+                assert Fraction(float(h)) + Fraction(float(l)) == before - n, (x, i)
+            else:
+                ds.append((w & 0xFFFF) - 2 ** 14)
+                assert ds[-1] == n / u
+        assert all(abs(d) <= 128 for d in ds), (x, ds)
+        v = Fraction(float(hi)) + Fraction(float(lo))
+        expansion = sum(Fraction(d) * Fraction(1, 2 ** (6 + 8 * i)) for i, d in enumerate(ds))
+        assert abs(v - expansion) <= Fraction(1, 2 ** 55), x
+    # three batches of 48 stacked rows, 7 digit pairs each, stay exact in FP32
+    assert 3 * 7 * 48 * 128 ** 2 < 2 ** 24
