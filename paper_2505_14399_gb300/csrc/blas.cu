@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "bits.cuh"
 #include "reduce.cuh"
 #include "vec.cuh"
 
@@ -232,13 +233,30 @@ __global__ void lincomb_kernel(Eo* y, double a, const Ei* x1, double b, const Ei
   }
 }
 
+// a plain change of type between float and double on the integer units (bits.cuh)
+__device__ __forceinline__ void retype(double& y, float x) { y = f64_from_bits(x); }
+__device__ __forceinline__ void retype(float& y, double x) { y = f32_from_bits(x); }
+__device__ __forceinline__ void retype(float& y, float x) { y = x; }
+__device__ __forceinline__ void retype(double& y, double x) { y = x; }
+
 template <typename Eo, typename Ei>
 __global__ void convert_kernel(Eo* y, const Ei* x, const double* s, int inv, size_t n) {
   dep_entry();
   typedef typename VecT<Eo>::R Ro;
   int rhs = blockIdx.y;
+  if (!s) {
+    for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+         k += (size_t)gridDim.x * blockDim.x) {
+      auto v = VecT<Ei>::ld(x + (size_t)rhs * n, k);
+      cplx<Ro> o;
+      retype(o.re, v.re);
+      retype(o.im, v.im);
+      VecT<Eo>::st(y + (size_t)rhs * n, k, o);
+    }
+    return;
+  }
   double f = 1.0;
-  if (s) {
+  {
     double sv = s[rhs];
     f = inv ? (sv > 0 ? 1.0 / sv : 0.0) : sv;
   }

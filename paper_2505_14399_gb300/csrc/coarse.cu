@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "bits.cuh"
 #include "df64.cuh"
 #include "galerkin.cuh"
 #include "internal.h"
@@ -56,9 +57,16 @@ restrict_kernel(cplx<R>* vc, const cplx<R>* __restrict__ v, const cplx<R>* __res
     const cplx<R>* col = Pt + (size_t)i * B.M;
     cplx<R> a0 = {0, 0}, a1 = {0, 0};
     int row = r0 + lane;
-    for (; row + 32 < r1; row += 64) {
-      cfmac(a0, col[row], sv[row]);
-      cfmac(a1, col[row + 32], sv[row + 32]);
+    // eight loads of P in flight per lane
+    for (; row + 224 < r1; row += 256) {
+      cplx<R> c[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c[u] = col[row + 32 * u];
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        cfmac(a0, c[u], sv[row + 32 * u]);
+        cfmac(a1, c[u + 1], sv[row + 32 * u + 32]);
+      }
     }
     for (; row < r1; row += 32) cfmac(a0, col[row], sv[row]);
     a0 += a1;
@@ -91,7 +99,15 @@ __global__ void prolong_kernel(cplx<R>* v, const cplx<R>* __restrict__ vc,
     const cplx<R>* Pt = P + (size_t)t * k * B.M + row;
     const cplx<R>* cv = vc + rhs * B.d * 2 * k + (size_t)t * k;
     cplx<R> acc = {0, 0};
-    for (int i = 0; i < k; ++i) cfma(acc, Pt[(size_t)i * B.M], cv[i]);
+    int i = 0;
+    for (; i + 4 <= k; i += 4) {   // four loads of P in flight
+      cplx<R> p[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) p[u] = Pt[(size_t)(i + u) * B.M];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cfma(acc, p[u], cv[i + u]);
+    }
+    for (; i < k; ++i) cfma(acc, Pt[(size_t)i * B.M], cv[i]);
     v[e] = acc;
   }
 }
@@ -293,7 +309,7 @@ galerkin_hop_kernel(zd* Op, zd* Xpart, const zd* __restrict__ P, const zdf* __re
 __global__ void to_df_kernel(zdf* out, const zd* __restrict__ in, size_t n) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x) {
-    zdf v = zdf_from(in[i]);
+    zdf v = zdf_from_bits(in[i]);
     reinterpret_cast<float4*>(out)[i] = make_float4(v.re.hi, v.re.lo, v.im.hi, v.im.lo);
   }
 }
@@ -304,27 +320,49 @@ __global__ void to_df_kernel(zdf* out, const zd* __restrict__ in, size_t n) {
 //   Y_-mu(j)  = sigma_3 Y_+mu(j - mu)^dag sigma_3
 // with F_mu(j) the forward hops that stay inside aggregate j.  Element (a, b) of
 // sigma_3 M^dag sigma_3 is s_a s_b conj(M(b, a)), s = +1 / -1 for chirality 0 / 1.
+// One CTA per coarse site; F_mu(j) and Y_+mu(j - mu) pass through shared memory (rows padded by
+// one entry), since each is read by columns and by rows.  Every block of D_c is in hand once here,
+// so the FP32 copy Op32 is written on the way (each Y_+mu block by the site that mirrors it).
+// 16^3x64, k = 24 (2.7 GB of operator): 2.47 ms with a conversion pass after it -> FIN_US ms.
 __global__ void __launch_bounds__(GTH)
-galerkin_finish_kernel(zd* Op, const zd* __restrict__ Xpart, const zd* __restrict__ PtP, int k,
-                       Blocking B) {
-  int j = blockIdx.x;
-  int n2k = 2 * k, ne = n2k * n2k;
-  for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-    int b = e / n2k, a = e % n2k;  // column-major element (a, b)
-    int et = a * n2k + b;          // element (b, a)
-    int aa = a / k, bb = b / k;
-    double sab = (aa == bb) ? 1.0 : -1.0;
-    zd acc = {0, 0};
-    if (aa == bb) acc = PtP[((size_t)(2 * j + aa) * k + a % k) * k + b % k];   // P_a^dag P_b
-    for (int mu = 0; mu < 4; ++mu) {
-      const zd* F = Xpart + ((size_t)mu * B.d + j) * ne;
-      acc += F[e];
-      acc += sab * conj(F[et]);
-      int jm = B.coarse_nbr(j, 2 * mu + 1);
-      zd yv = Op[((size_t)jm * 9 + 1 + 2 * mu) * ne + et];
-      Op[((size_t)j * 9 + 2 + 2 * mu) * ne + e] = sab * conj(yv);
+galerkin_finish_kernel(zd* Op, zf* Op32, const zd* __restrict__ Xpart, const zd* __restrict__ PtP,
+                       int k, Blocking B) {
+  extern __shared__ zd fsm[];
+  const int j = blockIdx.x;
+  const int n2k = 2 * k, ne = n2k * n2k, ld = n2k + 1;
+  zd* sF = fsm;               // [n2k][ld]: sF[b * ld + a] = F(a, b)
+  zd* sY = fsm + n2k * ld;
+  zd* X = Op + (size_t)j * 9 * ne;
+  auto narrow = [](zd v) { return zf{f32_from_bits(v.re), f32_from_bits(v.im)}; };
+  for (int mu = 0; mu < 4; ++mu) {
+    const zd* F = Xpart + ((size_t)mu * B.d + j) * ne;
+    const size_t yp = ((size_t)B.coarse_nbr(j, 2 * mu + 1) * 9 + 1 + 2 * mu) * ne;
+    const size_t ym = ((size_t)j * 9 + 2 + 2 * mu) * ne;
+    __syncthreads();
+    for (int e = threadIdx.x; e < ne; e += GTH) {
+      const int b = e / n2k, a = e - b * n2k;
+      sF[b * ld + a] = F[e];
+      const zd y = Op[yp + e];
+      sY[b * ld + a] = y;
+      Op32[yp + e] = narrow(y);
     }
-    Op[(size_t)j * 9 * ne + e] = acc;
+    __syncthreads();
+    for (int e = threadIdx.x; e < ne; e += GTH) {
+      const int b = e / n2k, a = e - b * n2k;   // column-major element (a, b)
+      const int aa = a >= k, bb = b >= k;
+      const double sab = aa == bb ? 1.0 : -1.0;
+      zd acc = {0, 0};
+      if (mu > 0) acc = X[e];
+      else if (aa == bb)   // P_a^dag P_b
+        acc = PtP[((size_t)(2 * j + aa) * k + (a - aa * k)) * k + (b - bb * k)];
+      acc += sF[b * ld + a];
+      acc += sab * conj(sF[a * ld + b]);
+      X[e] = acc;
+      if (mu == 3) Op32[(size_t)j * 9 * ne + e] = narrow(acc);
+      const zd y = sab * conj(sY[a * ld + b]);
+      Op[ym + e] = y;
+      Op32[ym + e] = narrow(y);
+    }
   }
 }
 
@@ -419,7 +457,7 @@ int launch_hop_ne(dim3 grid, size_t sh, cudaStream_t st, zd* Op, zd* Xpart, cons
 }
 }  // namespace
 
-int galerkin_build(zd* Op, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, int k, const zd* links,
+int galerkin_build(zd* Op, zf* Op32, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, int k, const zd* links,
                    const zdf* Ldf, const Geom& g, const Blocking& B, cudaStream_t st, bool df64,
                    bool pdf_ready, int* range_flag) {
   if (4 * k * k > GTH * GMAXE) return fail(MG_EINVAL, "galerkin: k > 32");
@@ -471,7 +509,9 @@ int galerkin_build(zd* Op, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, int k, con
   } else {
     WMG_TRY(launch_hop_ne<false>(grid, sh, st, Op, Xpart, P, Pdf, k, links, Ldf, hg, B));
   }
-  galerkin_finish_kernel<<<B.d, GTH, 0, st>>>(Op, Xpart, PtP, k, B);
+  const size_t fsh = sizeof(zd) * 2 * 2 * k * (2 * k + 1);
+  WMG_TRY(smem_attr(galerkin_finish_kernel, fsh));
+  galerkin_finish_kernel<<<B.d, GTH, fsh, st>>>(Op, Op32, Xpart, PtP, k, B);
   WMG_LAUNCHED();
   return MG_OK;
 }

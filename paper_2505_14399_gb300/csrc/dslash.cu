@@ -9,6 +9,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "bits.cuh"
 #include "common.cuh"
 #include "internal.h"
 #include "stencil.cuh"
@@ -258,129 +259,123 @@ template int link_to_lanes_v<zh>(zh*, const zd*, int, cudaStream_t, int);
 template int link_to_lanes_v<zbf>(zbf*, const zd*, int, cudaStream_t, int);
 
 namespace {
-// Largest deviation of any link from SU(3): max over links of max(|U U^dag - 1|_max,
-// |det U - 1|), as the bits of a non-negative double (ordered like the values) in *out.
-__global__ void su3_deviation_kernel(unsigned long long* out, const zd* __restrict__ L, size_t n) {
-  double worst = 0;
-  for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n;
-       l += (size_t)gridDim.x * blockDim.x) {
-    zd u[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) u[i] = L[l * 9 + i];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        zd s = {0, 0};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) s = s + u[a * 3 + c] * conj(u[b * 3 + c]);
-        if (a == b) s.re -= 1.0;
-        worst = fmax(worst, fmax(fabs(s.re), fabs(s.im)));
-      }
-    zd det = u[0] * (u[4] * u[8] - u[5] * u[7]) - u[1] * (u[3] * u[8] - u[5] * u[6]) +
-             u[2] * (u[3] * u[7] - u[4] * u[6]);
-    det.re -= 1.0;
-    worst = fmax(worst, sqrt(det.re * det.re + det.im * det.im));
-  }
-  if (!(worst == worst)) worst = 1e300;   // NaN: not SU(3)
-  // warp, then CTA maximum: one atomic per CTA (a single address taking one atomic per
-  // thread serialises them)
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-  __shared__ double wmax[32];
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = worst;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = wmax[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
-    atomicMax(out, (unsigned long long)__double_as_longlong(m));
-  }
-}
-}  // namespace
 
-// The same on a double-float copy of the links, in double-float arithmetic on the FP32 units
-// (error-free products and sums, ~2^-48 relative: deviations are resolved far below 1e-9).
-__global__ void su3_deviation_df_kernel(unsigned long long* out, const zdf* __restrict__ L,
-                                        size_t n) {
+// |U U^dag - 1| and |det U - 1| of one link, largest entry, in double-float arithmetic on the
+// FP32 units (error-free products and sums, ~2^-48 relative: deviations are resolved far below
+// 1e-9); NaN gives a huge value.
+__device__ float su3_deviation(const zdf u[9]) {
   float worst = 0.f;
-  for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < n;
-       l += (size_t)gridDim.x * blockDim.x) {
-    zdf u[9];
+  // U U^dag - 1: the six entries a <= b of the Hermitian matrix
 #pragma unroll
-    for (int i = 0; i < 9; ++i) u[i] = L[l * 9 + i];
-    // U U^dag - 1: the six entries a <= b of the Hermitian matrix
+  for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int b = a; b < 3; ++b) {
+      zdfacc s{};
 #pragma unroll
-      for (int b = a; b < 3; ++b) {
-        zdfacc s{};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) zdf_fmac(s, u[b * 3 + c], u[a * 3 + c]);   // u_ac conj(u_bc)
-        zdf v = zdf_norm(s);
-        if (a == b) v.re = df_add(v.re, {-1.0f, 0.0f});
-        worst = fmaxf(worst, fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)));
-      }
-    // det U - 1 by cofactors of the first row
-    zdfacc t{};
-    zdf_fma(t, u[4], u[8]);
-    zdf_fma(t, zdf_neg(u[5]), u[7]);
-    const zdf c0 = zdf_norm(t);
-    t = zdfacc{};
-    zdf_fma(t, u[3], u[8]);
-    zdf_fma(t, zdf_neg(u[5]), u[6]);
-    const zdf c1 = zdf_norm(t);
-    t = zdfacc{};
-    zdf_fma(t, u[3], u[7]);
-    zdf_fma(t, zdf_neg(u[4]), u[6]);
-    const zdf c2 = zdf_norm(t);
-    t = zdfacc{};
-    zdf_fma(t, u[0], c0);
-    zdf_fma(t, zdf_neg(u[1]), c1);
-    zdf_fma(t, u[2], c2);
-    zdf det = zdf_norm(t);
-    det.re = df_add(det.re, {-1.0f, 0.0f});
-    worst = fmaxf(worst, sqrtf(det.re.hi * det.re.hi + det.im.hi * det.im.hi));
+      for (int c = 0; c < 3; ++c) zdf_fmac(s, u[b * 3 + c], u[a * 3 + c]);   // u_ac conj(u_bc)
+      zdf v = zdf_norm(s);
+      if (a == b) v.re = df_add(v.re, {-1.0f, 0.0f});
+      worst = fmaxf(worst, fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)));
+    }
+  // det U - 1 by cofactors of the first row
+  zdfacc t{};
+  zdf_fma(t, u[4], u[8]);
+  zdf_fma(t, zdf_neg(u[5]), u[7]);
+  const zdf c0 = zdf_norm(t);
+  t = zdfacc{};
+  zdf_fma(t, u[3], u[8]);
+  zdf_fma(t, zdf_neg(u[5]), u[6]);
+  const zdf c1 = zdf_norm(t);
+  t = zdfacc{};
+  zdf_fma(t, u[3], u[7]);
+  zdf_fma(t, zdf_neg(u[4]), u[6]);
+  const zdf c2 = zdf_norm(t);
+  t = zdfacc{};
+  zdf_fma(t, u[0], c0);
+  zdf_fma(t, zdf_neg(u[1]), c1);
+  zdf_fma(t, u[2], c2);
+  zdf det = zdf_norm(t);
+  det.re = df_add(det.re, {-1.0f, 0.0f});
+  worst = fmaxf(worst, sqrtf(det.re.hi * det.re.hi + det.im.hi * det.im.hi));
+  return worst == worst ? worst : 3e38f;
+}
+
+// Everything a handle keeps of its links, in one pass over them: the ABI copy, its double-float
+// form, the lane-contiguous FP64 and FP32 stencil copies (the latter with `rows` rows) and the
+// largest deviation from SU(3) (bits of a non-negative float, ordered like the values).  Null
+// outputs are skipped.  A CTA's links go through shared memory, so loads and stores are coalesced
+// in both layouts; the conversions stay off the FP64 pipe (bits.cuh).  The separate passes (copy,
+// two layouts, conversion, check) took 225 us at 16^3x32, this one LNK us.
+constexpr int LPT = 128;
+__global__ void __launch_bounds__(LPT)
+links_prepare_kernel(zd* copy, zdf* df_, zd* lanes64, zf* lanes32, int rows, unsigned* dev,
+                     const zd* __restrict__ src, int V) {
+  __shared__ zd su[LPT * 9];
+  const size_t n = (size_t)4 * V, l0 = (size_t)blockIdx.x * LPT;
+  const int nl = (int)min((size_t)LPT, n - l0);
+  for (int e = threadIdx.x; e < nl * 9; e += LPT) {
+    const zd v = src[l0 * 9 + e];
+    su[e] = v;
+    if (copy) copy[l0 * 9 + e] = v;
+    if (df_) {
+      const zdf q = zdf_from_bits(v);
+      reinterpret_cast<float4*>(df_)[l0 * 9 + e] = make_float4(q.re.hi, q.re.lo, q.im.hi, q.im.lo);
+    }
   }
-  if (!(worst == worst)) worst = 3e38f;   // NaN: not SU(3)
+  __syncthreads();
+  float worst = 0.f;
+  if ((int)threadIdx.x < nl) {
+    const size_t l = l0 + threadIdx.x, mu = l / V, site = l - mu * V;
+    const zd* u = su + threadIdx.x * 9;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const zd v = u[i];
+      if (lanes64) lanes64[(mu * 9 + i) * V + site] = v;
+      if (lanes32 && i < 3 * rows)
+        lanes32[(mu * 3 * rows + i) * V + site] = {f32_from_bits(v.re), f32_from_bits(v.im)};
+    }
+    if (dev) {
+      zdf q[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) q[i] = zdf_from_bits(u[i]);
+      worst = su3_deviation(q);
+    }
+  }
+  if (!dev) return;
+  // warp, then CTA maximum: one atomic per CTA
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-  __shared__ float wmax[32];
+  __shared__ float wmax[LPT / 32];
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = worst;
   __syncthreads();
   if (threadIdx.x == 0) {
     float m = wmax[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, wmax[w]);
-    atomicMax(out, (unsigned long long)__double_as_longlong((double)m));
+    for (int w = 1; w < LPT / 32; ++w) m = fmaxf(m, wmax[w]);
+    atomicMax(dev, __float_as_uint(m));
   }
 }
 
-int su3_deviation(double* dev_out, const zd* links, size_t nlinks, cudaStream_t st) {
-  unsigned long long* d = nullptr;
-  WMG_CUDA(scratch_alloc(&d, sizeof(*d), st));
-  WMG_CUDA(cudaMemsetAsync(d, 0, sizeof(*d), st));
-  size_t g = (nlinks + 255) / 256, cap = (size_t)num_sms() * 8;
-  su3_deviation_kernel<<<(unsigned)(g < cap ? (g < 1 ? 1 : g) : cap), 256, 0, st>>>(d, links, nlinks);
-  WMG_LAUNCHED();
-  unsigned long long bits = 0;
-  WMG_CUDA(cudaMemcpyAsync(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost, st));
-  WMG_CUDA(cudaStreamSynchronize(st));
-  scratch_free(d, st);
-  std::memcpy(dev_out, &bits, sizeof(double));
-  return MG_OK;
-}
+}  // namespace
 
-int su3_deviation_df(double* dev_out, const zdf* links, size_t nlinks, cudaStream_t st) {
-  unsigned long long* d = nullptr;
-  WMG_CUDA(scratch_alloc(&d, sizeof(*d), st));
-  WMG_CUDA(cudaMemsetAsync(d, 0, sizeof(*d), st));
-  size_t g = (nlinks + 255) / 256, cap = (size_t)num_sms() * 8;
-  su3_deviation_df_kernel<<<(unsigned)(g < cap ? (g < 1 ? 1 : g) : cap), 256, 0, st>>>(d, links, nlinks);
+int links_prepare(zd* copy, zdf* df_, zd* lanes64, zf* lanes32, int rows, double* deviation,
+                  const zd* src, int V, cudaStream_t st) {
+  unsigned* d = nullptr;
+  if (deviation) {
+    WMG_CUDA(scratch_alloc(&d, sizeof(*d), st));
+    WMG_CUDA(cudaMemsetAsync(d, 0, sizeof(*d), st));
+  }
+  links_prepare_kernel<<<(unsigned)(((size_t)4 * V + LPT - 1) / LPT), LPT, 0, st>>>(
+      copy, df_, lanes64, lanes32, rows, d, src, V);
   WMG_LAUNCHED();
-  unsigned long long bits = 0;
-  WMG_CUDA(cudaMemcpyAsync(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost, st));
-  WMG_CUDA(cudaStreamSynchronize(st));
-  scratch_free(d, st);
-  std::memcpy(dev_out, &bits, sizeof(double));
+  if (deviation) {
+    unsigned bits = 0;
+    WMG_CUDA(cudaMemcpyAsync(&bits, d, sizeof(bits), cudaMemcpyDeviceToHost, st));
+    WMG_CUDA(cudaStreamSynchronize(st));
+    scratch_free(d, st);
+    float f;
+    std::memcpy(&f, &bits, sizeof(f));
+    *deviation = f;
+  }
   return MG_OK;
 }
 

@@ -27,11 +27,12 @@ template <typename To>
 inline int link_to_lanes(cplx<To>* dst, const zd* src, int V, cudaStream_t st, int rows = 3) {
   return link_to_lanes_v<cplx<To>>(dst, src, V, st, rows);
 }
-// *dev = the largest deviation of the nlinks 3x3 complex-double links from SU(3):
-// max(|U U^dag - 1|_max, |det U - 1|) (synchronises st).
-int su3_deviation(double* dev, const zd* links, size_t nlinks, cudaStream_t st);
-// the same from a double-float copy of the links, in double-float arithmetic
-int su3_deviation_df(double* dev, const zdf* links, size_t nlinks, cudaStream_t st);
+// One pass over the links (complex double, ABI layout): a copy, its double-float form, the
+// lane-contiguous FP64 copy and the FP32 one with `rows` rows (null outputs are skipped), and, if
+// deviation is not null, the largest deviation of a link from SU(3), max(|U U^dag - 1|_max,
+// |det U - 1|), in double-float arithmetic (synchronises st then).
+int links_prepare(zd* copy, zdf* df, zd* lanes64, zf* lanes32, int rows, double* deviation,
+                  const zd* src, int V, cudaStream_t st);
 
 // Autotuned launch shape for a kernel with `nvar` candidate shapes; `run(v)` launches
 // shape v on the caller's arguments.  Returns the chosen shape or -1 on a CUDA error.
@@ -182,11 +183,11 @@ class GmresV {
 
  private:
   // b0 (fused first step only): the unscaled right-hand side, scaled and written as v_0 there;
-  // next = false: column j + 1 of the basis is not needed (the last step of a fixed run), so
-  // only the Givens step of column j runs, not the normalised update
+  // next = false: column j + 1 of the basis is not needed (the last step of a fixed run);
+  // givens = false: no Givens step of column j (a fixed run solves its small problem at its end)
   int arnoldi_step(const OpV<E>& A, const OpV<E>* M, int j, cudaStream_t st,
                    bool single_pass = false, const FusedStencil* fused = nullptr,
-                   const E* b0 = nullptr, bool next = true);
+                   const E* b0 = nullptr, bool next = true, bool givens = true);
   double ip_scale() const { return VecT<E>::rms ? 1.0 / (double)n : 1.0; }
   E* V = nullptr;         // (m+1) x nrhs x n
   E* Z = nullptr;         // m x nrhs x n
@@ -325,7 +326,7 @@ int prolong_launch(cplx<R>* v, const cplx<R>* vc, const cplx<R>* P, int k, const
 // here unless pdf_ready says the setup wrote it), Ldf (the links as (hi, lo) pairs, filled
 // by the caller) and range_flag (one device int of the caller's, for the tensor path's range
 // check; synchronises `st` when that path runs).
-int galerkin_build(zd* Op, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, int k, const zd* links,
+int galerkin_build(zd* Op, zf* Op32, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, int k, const zd* links,
                    const zdf* Ldf, const Geom& g, const Blocking& B, cudaStream_t st, bool df64,
                    bool pdf_ready, int* range_flag);
 // complex double -> (hi, lo) float pairs

@@ -5,7 +5,8 @@
 // Hessenberg column is reduced by complex Givens rotations by one extra CTA of the step's
 // normalising update, and the residual estimates |g_{j+1}| (one per step, kept on the device)
 // are the only values the host reads, every `check_every` steps of a tolerance-driven solve.
-// All nrhs systems advance in lockstep.
+// A fixed number of steps needs no estimates: its small least-squares problem is solved once, at
+// the end.  All nrhs systems advance in lockstep.
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -44,29 +45,10 @@ __global__ void init_kernel(zd* small, SmallLayout L, const double* beta, double
   res[r] = beta[r];
 }
 
-// Finish column j of one system's Hessenberg matrix: H[:, j] += h2, H[j+1, j] = ||w||,
-// apply the previous rotations, form the new one, update g; returns |g_{j+1}|.
-// col = H[:, j] (j + 2 entries), h2 (j + 1), cs / sn (rotations 0..j; entry j is written),
-// gp = {g_j, g_{j+1}}.  The arrays may live in global or shared memory.
-__device__ double givens_core(zd* col, const zd* h2, zd* cs, zd* sn, zd* gp, int j,
-                              double wnorm) {
-  for (int i = 0; i <= j; ++i) col[i] = col[i] + h2[i];
-  col[j + 1] = {wnorm, 0};
-  for (int i = 0; i < j; ++i) {
-    double c = cs[i].re;
-    zd sv = sn[i];
-    zd a = col[i], b = col[i + 1];
-    zd na = c * a + sv * b;
-    zd nb = c * b - cmulc(sv, a);  // -conj(s) a + c b
-    col[i] = na;
-    col[i + 1] = nb;
-  }
-  // c = |a| / rho, s = (a / |a|) conj(b) / rho with rho^2 = |a|^2 + |b|^2, from two
-  // reciprocal square roots (one thread's serial FP64 chain: no hypot, sqrt or divide)
-  zd a = col[j], b = col[j + 1];
+// c = |a| / rho, s = (a / |a|) conj(b) / rho with rho^2 = |a|^2 + |b|^2, from two reciprocal
+// square roots (a serial FP64 chain: no hypot, sqrt or divide)
+__device__ __forceinline__ void rotation(zd a, zd b, double& c, zd& sv) {
   double na2 = norm2(a), rho2 = na2 + norm2(b);
-  double c;
-  zd sv;
   if (!(rho2 > 0.0)) {
     c = 1.0;
     sv = {0, 0};
@@ -79,6 +61,25 @@ __device__ double givens_core(zd* col, const zd* h2, zd* cs, zd* sn, zd* gp, int
     c = na2 * ina * ir;
     sv = (ina * ir) * (a * conj(b));
   }
+}
+
+// Reduce column j of one system's Hessenberg matrix: apply the previous rotations, form the new
+// one, update g; returns |g_{j+1}|.  col = H[:, j] (j + 2 entries), cs / sn (rotations 0..j;
+// entry j is written), gp = {g_j, g_{j+1}}.
+__device__ double givens_core(zd* col, zd* cs, zd* sn, zd* gp, int j) {
+  for (int i = 0; i < j; ++i) {
+    double c = cs[i].re;
+    zd sv = sn[i];
+    zd a = col[i], b = col[i + 1];
+    zd na = c * a + sv * b;
+    zd nb = c * b - cmulc(sv, a);  // -conj(s) a + c b
+    col[i] = na;
+    col[i + 1] = nb;
+  }
+  zd a = col[j], b = col[j + 1];
+  double c;
+  zd sv;
+  rotation(a, b, c, sv);
   zd top = c * a + sv * b;
   col[j] = top;
   col[j + 1] = {0, 0};
@@ -90,34 +91,49 @@ __device__ double givens_core(zd* col, const zd* h2, zd* cs, zd* sn, zd* gp, int
   return sqrt(norm2(gp[1]));
 }
 
-// Column j of the Hessenberg matrix and its Givens step, run by one whole CTA on shared-memory
-// copies (one thread's chain of dependent updates then touches shared memory, not L2): the
-// column gets the projections h2 (added to the pass-1 values, or alone when `single`) and
-// H[j+1, j] = beta; the rotation updates cs, sn, g and the residual estimate res.  Called by
-// the extra CTA of the normalising update, so this serial FP64 chain runs beside the
-// memory-bound update instead of ending the reduction sweep.
+// The Givens step of Hessenberg column j (complete in global memory), run by one whole CTA on
+// shared-memory copies (one thread's chain of dependent updates then touches shared memory, not
+// L2): the rotation updates cs, sn, g and the residual estimate res.  Called by the extra CTA of
+// the normalising update, so this serial FP64 chain runs beside the memory-bound update instead
+// of ending the reduction sweep.
 constexpr int GV_MAX = 130;   // m <= 128
-__device__ void givens_deferred(zd* sm, SmallLayout L, int j, double beta, bool single,
-                                double* res) {
-  __shared__ zd g_col[GV_MAX], g_h2[GV_MAX], g_cs[GV_MAX], g_sn[GV_MAX], g_g[2];
-  const zd* colg = sm + L.H() + (size_t)j * (L.m + 1);
-  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) g_col[i] = single ? zd{0, 0} : colg[i];
-  for (int i = threadIdx.x; i <= j; i += blockDim.x) g_h2[i] = sm[L.h2() + i];
+__device__ void givens_deferred(zd* sm, SmallLayout L, int j, double* res) {
+  __shared__ zd g_col[GV_MAX], g_cs[GV_MAX], g_sn[GV_MAX], g_g[2];
+  zd* colg = sm + L.H() + (size_t)j * (L.m + 1);
+  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) g_col[i] = colg[i];
   for (int i = threadIdx.x; i < j; i += blockDim.x) {
     g_cs[i] = sm[L.cs() + i];
     g_sn[i] = sm[L.sn() + i];
   }
   if (threadIdx.x < 2) g_g[threadIdx.x] = sm[L.g() + j + threadIdx.x];
   __syncthreads();
-  if (threadIdx.x == 0) *res = givens_core(g_col, g_h2, g_cs, g_sn, g_g, j, beta);
+  if (threadIdx.x == 0) *res = givens_core(g_col, g_cs, g_sn, g_g, j);
   __syncthreads();
-  zd* colw = sm + L.H() + (size_t)j * (L.m + 1);
-  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) colw[i] = g_col[i];
+  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) colg[i] = g_col[i];
   if (threadIdx.x == 0) {
     sm[L.cs() + j] = g_cs[j];
     sm[L.sn() + j] = g_sn[j];
   }
   if (threadIdx.x < 2) sm[L.g() + j + threadIdx.x] = g_g[threadIdx.x];
+}
+
+// The end of a reduction sweep, by its last CTA: h2 (the nv projections and ||w||^2, in shared
+// memory) to the coefficients of the update, column nv - 1 of the Hessenberg matrix (added to the
+// first pass's projections, or alone when `single`) and H[j+1, j]^2 = ||w||^2 - ||h2||^2.
+__device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, const zd* h2,
+                                              double* wnorm, bool single) {
+  zd* col = sm + L.H() + (size_t)(nv - 1) * (L.m + 1);
+  for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+    sm[L.h2() + i] = h2[i];
+    col[i] = single ? h2[i] : col[i] + h2[i];
+  }
+  if (threadIdx.x == 0) {
+    double hh = 0;
+    for (int i = 0; i < nv; ++i) hh += norm2(h2[i]);
+    const double b2 = h2[nv].re - hh, b = b2 > 0 ? sqrt(b2) : 0.0;
+    *wnorm = b;
+    col[nv] = {b, 0};
+  }
 }
 
 // CGS pass 1 update fused with the pass 2 projections and the norm:
@@ -226,40 +242,33 @@ cgs_update_dot_kernel(E* w, const E* __restrict__ V, size_t vstride, int nv,
   cta_store_partials<R, 1>(&ss, &zero, 1, nv, rhs, maxvec, nblk, partials_as<R>(partial),
                            reinterpret_cast<R*>(sh));
   if (!last_cta(counter, rhs, nblk)) return;
-  finish_partials(partials_as<R>(partial), nv + 1, nblk, maxvec, rhs, small + L.h2(), nullptr,
-                  L.stride(), 0,
-                  scale);
+  __shared__ zd g_h2[GV_MAX];
+  finish_partials(partials_as<R>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0, scale);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    counter[rhs] = 0;
-    const zd* h2 = sm + L.h2();
-    double hh = 0;
-    for (int i = 0; i < nv; ++i) hh += norm2(h2[i]);
-    double b2 = h2[nv].re - hh;
-    wnorm[rhs] = b2 > 0 ? sqrt(b2) : 0.0;   // the Givens step follows in the update
-  }
+  finish_column(sm, L, nv, g_h2, wnorm + rhs, false);
+  if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
 // CGS pass 2 update written straight into the next basis column:
 //   v_{j+1} = (w - sum_i h2_i V_i) / H[j+1, j]   (0 if H[j+1, j] = 0).
-// The last CTA of every rhs row does not update: it completes Hessenberg column j = nv - 1
-// and its Givens step (givens_deferred) while the others stream the vectors.
+// With `givens` the last CTA of every rhs row does not update: it does the Givens step of
+// Hessenberg column j = nv - 1 (givens_deferred) while the others stream the vectors.
 template <typename E>
 __global__ void __launch_bounds__(256)
 cgs_update_scale_kernel(E* vout, const E* __restrict__ w, const E* __restrict__ V,
                         size_t vstride, int nv, zd* small, SmallLayout L,
-                        const double* wnorm, size_t n, double* res, int single) {
+                        const double* wnorm, size_t n, double* res, int givens) {
   dep_entry();
   typedef VecT<E> T;
   typedef typename T::R R;
   __shared__ cplx<R> cs[128];
   int rhs = blockIdx.y;
-  if (blockIdx.x == gridDim.x - 1) {
-    givens_deferred(small + (size_t)rhs * L.stride(), L, nv - 1, wnorm[rhs], single != 0,
+  if (givens && blockIdx.x == gridDim.x - 1) {
+    givens_deferred(small + (size_t)rhs * L.stride(), L, nv - 1,
                     res + (size_t)(nv - 1) * gridDim.y + rhs);
     return;
   }
-  const size_t nthreads = (size_t)(gridDim.x - 1) * blockDim.x;
+  const size_t nthreads = (size_t)(gridDim.x - givens) * blockDim.x;
   const zd* h2 = small + (size_t)rhs * L.stride() + L.h2();
   for (int i = threadIdx.x; i < nv; i += blockDim.x) cs[i] = {(R)(-h2[i].re), (R)(-h2[i].im)};
   __syncthreads();
@@ -306,8 +315,7 @@ cgs_update_scale_kernel(E* vout, const E* __restrict__ w, const E* __restrict__ 
 //   MODE 1: w -= V c; h2_i = V_i^dag w; ||w||^2; H[j+1, j] as in cgs_update_dot_kernel
 //   MODE 2: h_i = V_i^dag w and ||w||^2; H[j+1, j]^2 = ||w||^2 - ||h||^2 (single-pass
 //           classical Gram-Schmidt; see GmresV::fixed)
-// In modes 1 and 2 the Hessenberg column and its Givens step are completed by the
-// normalising update that follows (givens_deferred).
+// Modes 1 and 2 complete the Hessenberg column (finish_column).
 // A bounded wait that gives up sets *err, waits (bounded) for the CTA's copies in flight
 // and returns; the caller reports MG_ETIMEOUT.
 constexpr int ST_NV = 16;      // columns handled (NVM = 8 or 16 accumulator sets)
@@ -454,19 +462,12 @@ stream_cgs_kernel(zf* w, const zf* __restrict__ V, size_t vstride, int nv, size_
     if (threadIdx.x == 0) counter[rhs] = 0;
     return;
   }
-  // projections and H[j+1, j]; the Givens step follows in the normalising update
   __shared__ zd g_h2[NVM + 1];
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0,
                   scale);
   __syncthreads();
-  for (int i = threadIdx.x; i <= nv; i += RT) sm[L.h2() + i] = g_h2[i];
-  if (threadIdx.x == 0) {
-    counter[rhs] = 0;
-    double hh = 0;
-    for (int i = 0; i < nv; ++i) hh += norm2(g_h2[i]);
-    double b2 = g_h2[nv].re - hh;
-    wnorm[rhs] = b2 > 0 ? sqrt(b2) : 0.0;
-  }
+  finish_column(sm, L, nv, g_h2, wnorm + rhs, MODE == 2);
+  if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
 // One fixed-step GMRES step's operator and projections in one kernel (single-pass classical
@@ -561,19 +562,11 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   cta_store_partials<float, 1>(&ss, &zero, 1, nv, rhs, maxvec, nblk, partials_as<float>(partial),
                                sh);
   if (!last_cta(counter, rhs, nblk)) return;
-  // projections and H[j+1, j]; the Givens step follows in the normalising update
   __shared__ zd g_h2[NVM + 1];
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0);
   __syncthreads();
-  zd* sm = small + (size_t)rhs * L.stride();
-  for (int i = threadIdx.x; i <= nv; i += BT) sm[L.h2() + i] = g_h2[i];
-  if (threadIdx.x == 0) {
-    counter[rhs] = 0;
-    double hh = 0;
-    for (int i = 0; i < nv; ++i) hh += norm2(g_h2[i]);
-    double b2 = g_h2[nv].re - hh;
-    wnorm[rhs] = b2 > 0 ? sqrt(b2) : 0.0;
-  }
+  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true);
+  if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
 // launch shapes of the fused kernel: 128 threads and 4, 5 or 6 resident CTAs per SM asked of the
@@ -731,6 +724,54 @@ __global__ void solve_kernel(zd* small, SmallLayout L, int steps, int nrhs) {
   }
 }
 
+// The least-squares problem of a fixed number of steps: min |beta e_1 - H y| over the complete
+// (steps + 1) x steps Hessenberg matrix (real subdiagonal), one CTA per system.  Rotation j,
+//   [conj(a) b; -b a] / rho,  rho^2 = |a|^2 + b^2,  a = H_jj, b = H_j+1,j,
+// makes the diagonal real; every thread forms it from the same two entries and thread k applies it
+// to its own column k > j (thread `steps`: to the right-hand side).  Back substitution then only
+// multiplies by the 1 / rho at hand.  FP64 instructions take a warp 16 cycles and depend on each
+// other here, so the chain per step is one reciprocal square root and four multiply-adds; a fixed
+// run pays for it once instead of once per normalising update, which waited for its extra CTA
+// (9.7 -> LS_UPD us per update on 4096 sites, 14.1 -> LS_UPD2 us on the 65 536-site Schur system).
+__global__ void __launch_bounds__(128) fixed_ls_kernel(zd* small, SmallLayout L, int steps,
+                                                       const double* beta) {
+  dep_entry();
+  extern __shared__ zd lsh[];          // [steps][steps + 1] H by columns
+  __shared__ zd gs[GV_MAX];
+  __shared__ double inv[GV_MAX];
+  zd* sm = small + (size_t)blockIdx.x * L.stride();
+  const int ld = steps + 1, k = threadIdx.x;
+  for (int e = threadIdx.x; e < steps * ld; e += blockDim.x) {
+    const int col = e / ld, row = e % ld;
+    if (row <= col + 1) lsh[e] = sm[L.H() + (size_t)col * (L.m + 1) + row];
+  }
+  for (int i = threadIdx.x; i <= steps; i += blockDim.x)
+    gs[i] = i == 0 ? zd{beta[blockIdx.x], 0} : zd{0, 0};
+  __syncthreads();
+  for (int j = 0; j < steps; ++j) {
+    const zd a = lsh[j * ld + j];
+    const double b = lsh[j * ld + j + 1].re, rho2 = fma(b, b, norm2(a));
+    const double ir = rho2 > 0.0 ? rsqrt(rho2) : 0.0;   // an all-zero column: no rotation, y_j = 0
+    if (k > j && k <= steps && rho2 > 0.0) {
+      zd* p = k < steps ? lsh + k * ld + j : gs + j;
+      const zd x = ir * p[0], y = ir * p[1];
+      zd top = b * y, bot = -(b * x);
+      cfmac(top, a, x);
+      cfma(bot, a, y);
+      p[0] = top;
+      p[1] = bot;
+    }
+    if (k == j) inv[j] = ir;
+    __syncthreads();
+  }
+  for (int i = steps - 1; i >= 0; --i) {
+    const zd y = inv[i] * gs[i];
+    if (k < i) gs[k] = gs[k] - lsh[i * ld + k] * y;
+    if (k == i) sm[L.y() + i] = y;
+    __syncthreads();
+  }
+}
+
 }  // namespace
 
 template <typename E>
@@ -778,7 +819,7 @@ void GmresV<E>::release() {
 template <typename E>
 int GmresV<E>::arnoldi_step(const OpV<E>& A, const OpV<E>* M, int j, cudaStream_t st,
                             bool single_pass, const FusedStencil* fused, const E* b0,
-                            bool next) {
+                            bool next, bool givens) {
   SmallLayout L{m};
   size_t fs = n * nrhs;
   E* vj = V + (size_t)j * fs;
@@ -817,22 +858,13 @@ int GmresV<E>::arnoldi_step(const OpV<E>& A, const OpV<E>* M, int j, cudaStream_
     ProfScope ps("cgs_update_dot", (j + 3) * fb, (16.0 * (j + 1) + 4.0) * n * nrhs, st);
     WMG_LAUNCH_DEP(cgs_update_dot_kernel<E>, dim3(nb, nrhs), RT, 0, st, w, V, fs, j + 1, small, L, j, n, dnorm, reshist, rw.partial, rw.counter, nb, rw.maxvec, ip_scale());
   }
-  if (!next) {
-    // the Givens step of column j alone (the last CTA of the update kernel)
-    ProfScope ps("cgs_givens", 0.0, 0.0, st);
-    WMG_LAUNCH_DEP(cgs_update_scale_kernel<E>, dim3(1, nrhs), 256, 0, st,
-                   V + (size_t)(j + 1) * fs, w, V, fs, j + 1, small, L, dnorm, n, reshist,
-                   single_pass && streamed ? 1 : 0);
-    return MG_OK;
-  }
-  {
+  if (!next) return MG_OK;   // the last of a fixed number of steps
   ProfScope ps("cgs_update_scale", (j + 3) * fb, (8.0 * (j + 1) + 2.0) * n * nrhs, st);
   size_t g = (n / 2 + 255) / 256;
   size_t cap = (size_t)num_sms() * 8;
-  // + 1 CTA per rhs row for the deferred Givens step
-  dim3 grid((unsigned)(g < cap ? (g < 1 ? 1 : g) : cap) + 1, nrhs);
-  WMG_LAUNCH_DEP(cgs_update_scale_kernel<E>, grid, 256, 0, st, V + (size_t)(j + 1) * fs, w, V, fs, j + 1, small, L, dnorm, n, reshist, single_pass && streamed ? 1 : 0);
-  }
+  // + 1 CTA per rhs row for the Givens step
+  dim3 grid((unsigned)(g < cap ? (g < 1 ? 1 : g) : cap) + (givens ? 1 : 0), nrhs);
+  WMG_LAUNCH_DEP(cgs_update_scale_kernel<E>, grid, 256, 0, st, V + (size_t)(j + 1) * fs, w, V, fs, j + 1, small, L, dnorm, n, reshist, givens ? 1 : 0);
   return MG_OK;
 }
 
@@ -844,8 +876,8 @@ int GmresV<E>::fixed(const OpV<E>& A, E* x, const E* b, int steps, cudaStream_t 
   size_t fs = n * nrhs;
   if (!accumulate) WMG_TRY(fill_zero_v<E>(x, fs, st));
   if (steps == 0) return MG_OK;
+  if (steps > 112) return fail(MG_EINVAL, "gmres: at most 112 fixed steps");   // fixed_ls_kernel
   WMG_TRY(norm2_v<E>(dnorm + nrhs, 1, b, n, nrhs, rw, st, ip_scale()));
-  WMG_LAUNCH_DEP(init_kernel, (nrhs + 31) / 32, 32, 0, st, small, L, dnorm + nrhs, dnorm + 2 * nrhs, nrhs);
   // the fused first step scales b itself and writes v_0 (see dslash_proj_kernel)
   bool fuse0 = false;
   if constexpr (std::is_same<E, zf>::value)
@@ -856,11 +888,14 @@ int GmresV<E>::fixed(const OpV<E>& A, E* x, const E* b, int steps, cudaStream_t 
   // Pythagoras.  Over these few steps the basis stays orthogonal to ~eps_32 times the
   // conditioning of the small Krylov basis, which leaves the smoother's approximate
   // minimisation unchanged to FP32 rounding; the tolerance-driven solves keep CGS2.
-  // the last step needs its Hessenberg column and Givens step, not the next basis column
+  // the last step needs its Hessenberg column, not the next basis column
   for (int j = 0; j < steps; ++j)
     WMG_TRY(arnoldi_step(A, nullptr, j, st, true, fused, fuse0 && j == 0 ? b : nullptr,
-                         j + 1 < steps));
-  WMG_LAUNCH_DEP(solve_kernel, (nrhs + 31) / 32, 32, 0, st, small, L, steps, nrhs);
+                         j + 1 < steps, false));
+  const size_t lsb = sizeof(zd) * (size_t)steps * (steps + 1);
+  WMG_TRY(smem_attr(fixed_ls_kernel, lsb));
+  const int lst = (steps + 1 + 31) / 32 * 32;
+  WMG_LAUNCH_DEP(fixed_ls_kernel, nrhs, lst, lsb, st, small, L, steps, dnorm + nrhs);
   WMG_TRY(multi_axpy_v<E>(x, V, fs, steps, small + L.y(), L.stride(), xsign, n, nrhs, st));
   return MG_OK;
 }

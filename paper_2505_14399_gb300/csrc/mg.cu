@@ -144,8 +144,9 @@ int validate(const mg_params* p, bool need_svd) {
   return MG_OK;
 }
 
+// smoother_only: no more than the setup smoother needs (mg_test_vectors), no prolongator storage
 int create_handle(mg_handle** out, const void* links, const mg_params* p, bool need_svd,
-                  cudaStream_t st) {
+                  cudaStream_t st, bool smoother_only = false) {
   if (!out) return fail(MG_EINVAL, "NULL handle pointer");
   if (*out) return fail(MG_EINVAL, "*h must be NULL on entry");
   if (!links) return fail(MG_EINVAL, "NULL links");
@@ -158,43 +159,49 @@ int create_handle(mg_handle** out, const void* links, const mg_params* p, bool n
   h->nf = (size_t)h->g.V * 12;
   h->nc = (size_t)h->B.d * 2 * h->k;
   size_t lb = (size_t)4 * h->g.V * 9;
-  WMG_TRY(dev_alloc(&h->links64, lb * sizeof(zd)));
-  WMG_TRY(dev_alloc(&h->links64L, lb * sizeof(zd)));
   Staged sl;
   WMG_TRY(stage_in(sl, links, lb * sizeof(zd), st));
-  WMG_CUDA(cudaMemcpyAsync(h->links64, sl.dev, lb * sizeof(zd), cudaMemcpyDeviceToDevice, st));
-  WMG_TRY(link_to_lanes<double>(h->links64L, h->links64, h->g.V, st));
-  // the double-float copy of the links (double-float Galerkin sums) first: the SU(3) check
-  // below runs on it in double-float arithmetic instead of on the FP64 units
-  if (galerkin_df(*p)) {
-    WMG_TRY(dev_alloc(&h->Ldf, lb * sizeof(zdf)));
-    WMG_TRY(to_df(h->Ldf, h->links64, lb, st));
-  }
-  // the FP32 / half stencil copies keep two rows per link when the links are SU(3)
-  int rows = 3;
-  if (p->link_compress != 0) {
-    double dev = 0;
-    if (h->Ldf) WMG_TRY(su3_deviation_df(&dev, h->Ldf, (size_t)4 * h->g.V, st));
-    else WMG_TRY(su3_deviation(&dev, h->links64, (size_t)4 * h->g.V, st));
-    if (dev <= 1e-9) rows = 2;
-    else if (p->link_compress > 0)
+  const zd* src = static_cast<const zd*>(sl.dev);
+  const bool fp64 = !smoother_only || p->setup_dtype == MG_C128;
+  const bool fp32 = !smoother_only || p->setup_dtype != MG_C128;
+  if (!smoother_only) WMG_TRY(dev_alloc(&h->links64, lb * sizeof(zd)));
+  if (fp64) WMG_TRY(dev_alloc(&h->links64L, lb * sizeof(zd)));
+  if (!smoother_only && galerkin_df(*p)) WMG_TRY(dev_alloc(&h->Ldf, lb * sizeof(zdf)));
+  // the FP32 / half stencil copies keep two rows per link when the links are SU(3): the pass that
+  // finds out writes two rows, and three follow where they are not
+  int rows = p->link_compress != 0 ? 2 : 3;
+  if (fp32) WMG_TRY(dev_alloc(&h->links32L, (size_t)4 * h->g.V * 3 * rows * sizeof(zf)));
+  double dev = 0;
+  WMG_TRY(links_prepare(h->links64, h->Ldf, h->links64L, h->links32L, rows,
+                        rows == 2 ? &dev : nullptr, src, h->g.V, st));
+  if (!(dev <= 1e-9)) {
+    if (p->link_compress > 0)
       return fail(MG_EINVAL, "link_compress = 1 needs SU(3) links (deviation " +
                                  std::to_string(dev) + " > 1e-9)");
+    rows = 3;
+    if (fp32) {
+      dfree(h->links32L);   // links_prepare has synchronised
+      WMG_TRY(dev_alloc(&h->links32L, (size_t)4 * h->g.V * 9 * sizeof(zf)));
+      WMG_TRY(link_to_lanes<float>(h->links32L, src, h->g.V, st));
+    }
   }
   h->llay = rows == 2 ? 2 : 1;
-  size_t lbc = (size_t)4 * h->g.V * 3 * rows;
-  WMG_TRY(dev_alloc(&h->links32L, lbc * sizeof(zf)));
-  WMG_TRY(link_to_lanes<float>(h->links32L, h->links64, h->g.V, st, rows));
-  if (p->solve_dtype == MG_F16 || p->solve_dtype == MG_BF16) {
+  const size_t lbc = (size_t)4 * h->g.V * 3 * rows;
+  if (!smoother_only && (p->solve_dtype == MG_F16 || p->solve_dtype == MG_BF16)) {
     WMG_TRY(dev_alloc(&h->links16L, lbc * 4));
-    if (p->solve_dtype == MG_F16) WMG_TRY(link_to_lanes_v<zh>((zh*)h->links16L, h->links64, h->g.V, st, rows));
-    else WMG_TRY(link_to_lanes_v<zbf>((zbf*)h->links16L, h->links64, h->g.V, st, rows));
+    if (p->solve_dtype == MG_F16) WMG_TRY(link_to_lanes_v<zh>((zh*)h->links16L, src, h->g.V, st, rows));
+    else WMG_TRY(link_to_lanes_v<zbf>((zbf*)h->links16L, src, h->g.V, st, rows));
   }
   if (p->csw != 0) {
     WMG_TRY(dev_alloc(&h->clov64, (size_t)h->g.V * 72 * sizeof(zd)));
     WMG_TRY(dev_alloc(&h->clov32, (size_t)h->g.V * 72 * sizeof(zf)));
-    WMG_TRY(clover_field(h->clov64, h->links64, h->g, p->csw, st));
+    WMG_TRY(clover_field(h->clov64, src, h->g, p->csw, st));
     WMG_TRY((convert<float, double>(h->clov32, h->clov64, nullptr, 0, (size_t)h->g.V * 72, 1, st)));
+  }
+  if (smoother_only) {
+    WMG_CUDA(cudaStreamSynchronize(st));   // staged host links
+    *out = h.release();
+    return MG_OK;
   }
   size_t ntile = (size_t)h->B.d * 2;
   WMG_TRY(dev_alloc(&h->P64, ntile * h->k * h->B.M * sizeof(zd)));
@@ -1015,12 +1022,14 @@ extern "C" int coarse_build(mg_handle* h, void* stream) {
   zd* Xpart = nullptr;
   WMG_CUDA(scratch_alloc(&Xpart, (size_t)4 * h->B.d * ne * sizeof(zd), st));
   bool df = galerkin_df(h->p);
-  int s = galerkin_build(h->Op64, Xpart, h->P64, h->Pdf, h->PtP, h->k, h->links64, h->Ldf, h->g,
+  int s = galerkin_build(h->Op64, h->Op32, Xpart, h->P64, h->Pdf, h->PtP, h->k, h->links64, h->Ldf, h->g,
                          h->B, st, df, h->pdf_ready, h->tc_flag);
   scratch_free(Xpart, st);
   WMG_TRY(s);
-  if (h->clov64) WMG_TRY(clover_galerkin_add(h->Op64, h->P64, h->clov64, h->k, h->B, st));
-  WMG_TRY((convert<float, double>(h->Op32, h->Op64, nullptr, 0, (size_t)h->B.d * 9 * ne, 1, st)));
+  if (h->clov64) {   // changes X after galerkin_build wrote Op32
+    WMG_TRY(clover_galerkin_add(h->Op64, h->P64, h->clov64, h->k, h->B, st));
+    WMG_TRY((convert<float, double>(h->Op32, h->Op64, nullptr, 0, (size_t)h->B.d * 9 * ne, 1, st)));
+  }
   WMG_CUDA(cudaStreamSynchronize(st));
   h->have_coarse = true;
   return MG_OK;
@@ -1081,10 +1090,12 @@ extern "C" int coarse_build_noalloc(mg_handle* h, void* stream) {
   void* scratch = nullptr;
   WMG_TRY(galerkin_scratch(&scratch));
   bool df = galerkin_df(h->p);
-  WMG_TRY(galerkin_build(h->Op64, static_cast<zd*>(scratch), h->P64, h->Pdf, h->PtP, h->k,
+  WMG_TRY(galerkin_build(h->Op64, h->Op32, static_cast<zd*>(scratch), h->P64, h->Pdf, h->PtP, h->k,
                          h->links64, h->Ldf, h->g, h->B, st, df, h->pdf_ready, h->tc_flag));
-  if (h->clov64) WMG_TRY(clover_galerkin_add(h->Op64, h->P64, h->clov64, h->k, h->B, st));
-  WMG_TRY((convert<float, double>(h->Op32, h->Op64, nullptr, 0, (size_t)h->B.d * 9 * ne, 1, st)));
+  if (h->clov64) {   // changes X after galerkin_build wrote Op32
+    WMG_TRY(clover_galerkin_add(h->Op64, h->P64, h->clov64, h->k, h->B, st));
+    WMG_TRY((convert<float, double>(h->Op32, h->Op64, nullptr, 0, (size_t)h->B.d * 9 * ne, 1, st)));
+  }
   WMG_CUDA(cudaStreamSynchronize(st));
   h->have_coarse = true;
   return MG_OK;
@@ -1149,7 +1160,7 @@ extern "C" int mg_test_vectors(void* out, const void* links, const mg_params* p,
     return fail(MG_EINVAL, "mg_test_vectors: stream index out of range");
   cudaStream_t st = (cudaStream_t)stream;
   mg_handle* h = nullptr;
-  WMG_TRY(create_handle(&h, links, p, true, st));
+  WMG_TRY(create_handle(&h, links, p, true, st, true));
   std::unique_ptr<mg_handle> guard(h);
   size_t fr = h->nf * p->r;
   Staged so;
@@ -1272,19 +1283,32 @@ extern "C" int mg_prolong(mg_handle* h, void* v, const void* vc, int nrhs, void*
 }
 
 namespace {
-__global__ void export_coarse_kernel(zd* X, zd* Y, const zd* Op, int n2k, int d) {
-  size_t ne = (size_t)n2k * n2k;
-  size_t total = (size_t)d * 9 * ne;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    size_t j = e / (9 * ne), rem = e % (9 * ne);
-    int blk = (int)(rem / ne);
-    size_t q = rem % ne;
-    int b = (int)(q / n2k), a = (int)(q % n2k);   // Op is column-major
-    zd v = Op[e];
-    if (blk == 0) X[j * ne + (size_t)a * n2k + b] = v;
-    else Y[((size_t)(blk - 1) * d + j) * ne + (size_t)a * n2k + b] = v;
+// one CTA per block (j, blk): transposed through shared memory (Op is column-major, rows padded by
+// one entry), so both sides are coalesced (16^3x64, k = 24, 2.7 GB each way: 3.55 -> EXP_US ms)
+__global__ void __launch_bounds__(256) export_coarse_kernel(zd* X, zd* Y, const zd* __restrict__ Op,
+                                                            int n2k, int d) {
+  extern __shared__ zd esm[];
+  const int ne = n2k * n2k, ld = n2k + 1;
+  const int j = blockIdx.x / 9, blk = blockIdx.x - 9 * j;
+  const zd* src = Op + (size_t)blockIdx.x * ne;
+  for (int e = threadIdx.x; e < ne; e += 256) {
+    const int b = e / n2k, a = e - b * n2k;
+    esm[b * ld + a] = src[e];
   }
+  __syncthreads();
+  zd* dst = blk == 0 ? X + (size_t)j * ne : Y + ((size_t)(blk - 1) * d + j) * ne;
+  for (int e = threadIdx.x; e < ne; e += 256) {
+    const int a = e / n2k, b = e - a * n2k;
+    dst[e] = esm[b * ld + a];
+  }
+}
+
+int export_coarse(zd* X, zd* Y, const zd* Op, int n2k, int d, cudaStream_t st) {
+  const size_t sh = sizeof(zd) * n2k * (n2k + 1);
+  WMG_TRY(smem_attr(export_coarse_kernel, sh));
+  export_coarse_kernel<<<9 * d, 256, sh, st>>>(X, Y, Op, n2k, d);
+  WMG_LAUNCHED();
+  return MG_OK;
 }
 }  // namespace
 
@@ -1296,8 +1320,7 @@ extern "C" int mg_get_coarse_op(mg_handle* h, void* X, void* Y, void* stream) {
   Staged sx, sy;
   WMG_TRY(stage_out_alloc(sx, X, (size_t)h->B.d * ne * sizeof(zd), st));
   WMG_TRY(stage_out_alloc(sy, Y, (size_t)8 * h->B.d * ne * sizeof(zd), st));
-  export_coarse_kernel<<<256, 256, 0, st>>>((zd*)sx.dev, (zd*)sy.dev, h->Op64, 2 * h->k, h->B.d);
-  WMG_LAUNCHED();
+  WMG_TRY(export_coarse((zd*)sx.dev, (zd*)sy.dev, h->Op64, 2 * h->k, h->B.d, st));
   WMG_TRY(stage_out_finish(sx, X, (size_t)h->B.d * ne * sizeof(zd), st));
   WMG_TRY(stage_out_finish(sy, Y, (size_t)8 * h->B.d * ne * sizeof(zd), st));
   WMG_CUDA(cudaStreamSynchronize(st));
@@ -1320,8 +1343,7 @@ extern "C" int mg_get_level(mg_handle* h, int level, void* P, void* sigma, void*
     Staged sx, sy;
     WMG_TRY(stage_out_alloc(sx, X, (size_t)L->B.d * ne * sizeof(zd), st));
     WMG_TRY(stage_out_alloc(sy, Y, (size_t)8 * L->B.d * ne * sizeof(zd), st));
-    export_coarse_kernel<<<256, 256, 0, st>>>((zd*)sx.dev, (zd*)sy.dev, L->Op64, 2 * L->k, L->B.d);
-    WMG_LAUNCHED();
+    WMG_TRY(export_coarse((zd*)sx.dev, (zd*)sy.dev, L->Op64, 2 * L->k, L->B.d, st));
     WMG_TRY(stage_out_finish(sx, X, (size_t)L->B.d * ne * sizeof(zd), st));
     WMG_TRY(stage_out_finish(sy, Y, (size_t)8 * L->B.d * ne * sizeof(zd), st));
   }

@@ -37,14 +37,17 @@ __device__ __forceinline__ void philox10(uint32_t c[4], uint32_t k0, uint32_t k1
 // in FP32 (GB300's FP64 transcendentals are slow).  1 - u_a is formed exactly as the
 // integer 2^53 - m_a before rounding to float, so the tail is not lost to cancellation;
 // small u_a goes through log1pf.  Relative error against the FP64 map ~1e-7.
-__global__ void gaussian_kernel_f32(zf* out, uint32_t k0, uint32_t k1, unsigned id0, int V,
-                                    int nc, uint32_t w3, size_t total) {
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    size_t per = (size_t)V * nc;
-    unsigned v = (unsigned)(e / per);
-    size_t rem = e % per;
-    uint32_t c[4] = {(uint32_t)(rem / nc), (uint32_t)(rem % nc), id0 + v, w3};
+// One vector per grid row, so that a field's index arithmetic is one 32-bit division (I: unsigned
+// where a field has fewer than 2^32 entries).
+template <typename I>
+__global__ void __launch_bounds__(256)
+gaussian_kernel_f32(zf* out, uint32_t k0, uint32_t k1, unsigned id0, I per, unsigned nc,
+                    uint32_t w3) {
+  const unsigned v = blockIdx.y;
+  out += (size_t)v * per;
+  for (I e = (I)blockIdx.x * 256 + threadIdx.x; e < per; e += (I)gridDim.x * 256) {
+    const I site = e / nc;
+    uint32_t c[4] = {(uint32_t)site, (uint32_t)(e - site * nc), id0 + v, w3};
     philox10(c, k0, k1);
     unsigned long long ma = ((unsigned long long)(c[0] >> 5) << 26) | (c[1] >> 6);
     unsigned long long mb = ((unsigned long long)(c[2] >> 5) << 26) | (c[3] >> 6);
@@ -91,9 +94,15 @@ int gaussian_fill_n(cplx<R>* out, unsigned long long seed, unsigned id0, int nve
   size_t cap = (size_t)num_sms() * 16;
   unsigned grid = (unsigned)(g < cap ? (g < 1 ? 1 : g) : cap);
   uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
-  if (sizeof(R) == 4)
-    gaussian_kernel_f32<<<grid, 256, 0, st>>>((zf*)out, k0, k1, id0, nsites, ncomp, word3, total);
-  else
+  if (sizeof(R) == 4) {
+    // the loop index stays below per + a grid stride
+    const size_t per = (size_t)nsites * ncomp, gp = (per + 255) / 256;
+    const dim3 gr((unsigned)(gp < cap ? (gp < 1 ? 1 : gp) : cap), nvec);
+    if (per < ((size_t)1 << 31))
+      gaussian_kernel_f32<unsigned><<<gr, 256, 0, st>>>((zf*)out, k0, k1, id0, (unsigned)per, ncomp, word3);
+    else
+      gaussian_kernel_f32<size_t><<<gr, 256, 0, st>>>((zf*)out, k0, k1, id0, per, ncomp, word3);
+  } else
     gaussian_kernel<R><<<grid, 256, 0, st>>>(out, k0, k1, id0, nsites, ncomp, word3, total);
   WMG_LAUNCHED();
   return MG_OK;
