@@ -306,8 +306,10 @@ int ReduceWork::alloc(size_t n, int nrhs, int mv) {
   size_t nb = (n + 4 * RT - 1) / (4 * RT);
   size_t cap = (size_t)num_sms() * 6;
   nblk = (int)(nb < 1 ? 1 : (nb > cap ? cap : nb));
-  size_t per96 = (n / 12 + 95) / 96;
-  this->cap = (int)(per96 > (size_t)nblk ? per96 : (size_t)nblk);
+  const size_t sites = n / 12, per96 = (sites + 95) / 96, per32 = (sites + 31) / 32;
+  size_t slots = per96 > (size_t)nblk ? per96 : (size_t)nblk;
+  if (per32 <= 4096 && per32 > slots) slots = per32;
+  this->cap = (int)slots;
   maxvec = mv;
   nrhs_cap = nrhs;
   WMG_TRY(dev_alloc(&partial, sizeof(double) * 2 * (size_t)this->cap * maxvec * nrhs));

@@ -60,70 +60,41 @@ dslash_kernel(typename S::elem* __restrict__ out, const typename S::elem* __rest
   }
 }
 
-// Two threads per site, warp-uniform: the first 64 threads of a CTA take the forward hops
-// of 64 sites, the other 64 the backward hops of the same sites; the halves meet in shared
-// memory.  Twice the threads with half the dependent work each, for lattices too small to
-// fill the GPU with one thread per site.
+// One thread per site and hop (hop_lanes), consecutive sites; lane pairs write one spin each.
 template <typename S, int DAG, int LL>
 __global__ void __launch_bounds__(128)
-dslash_split_kernel(typename S::elem* __restrict__ out, const typename S::elem* __restrict__ in,
-                    const typename S::elem* __restrict__ links, KGeom g, int parity, int nsites,
-                    size_t in_stride, size_t out_stride) {
+dslash_hop_kernel(typename S::elem* __restrict__ out, const typename S::elem* __restrict__ in,
+                  const typename S::elem* __restrict__ links, KGeom g, int parity, int nsites,
+                  size_t in_stride, size_t out_stride) {
   dep_entry();
   typedef typename S::real R;
-  __shared__ cplx<R> sacc[12][64];
-  const int half = threadIdx.x >> 6, ls = threadIdx.x & 63;
-  int i = 0, site = 0, c[4] = {0, 0, 0, 0};
-  const bool active = stencil_work(g, parity, nsites, ls, 64, i, site, c);
+  const int i = blockIdx.x * (blockDim.x >> 3) + (threadIdx.x >> 3), hop = threadIdx.x & 7;
+  const bool active = i < nsites;
+  int c[4] = {0, 0, 0, 0}, site = 0;
+  if (active) site = stencil_site(g, parity, i, c);
   const size_t rhs = blockIdx.y;
-  const bool half_in = parity >= 0;
-  const size_t in_off = rhs * in_stride;
-  cplx<R> acc[12];
+  const typename S::elem* inr = in + rhs * in_stride;
+  cplx<R> acc[3];
+  hop_lanes<DAG, S, LL>(g, active, site, c, hop, inr, parity >= 0, links, acc);
+  if (!active || (hop & 1)) return;
+  const R mk = (R)(-g.kappa);
+  const size_t e0 = (size_t)i * 12 + 3 * (hop >> 1);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
-  if (active) {
-    if (half == 0) {
-      hop_fwd<0, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_fwd<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_fwd<2, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_fwd<3, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-    } else {
-      hop_bwd<0, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_bwd<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_bwd<2, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_bwd<3, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
+  for (int k = 0; k < 3; ++k) {
+    cplx<R> r = mk * acc[k];
+    if (parity < 0) {
+      const cplx<R> x = S::ld(inr, e0 + k);
+      r = {fma(mk, acc[k].re, x.re), fma(mk, acc[k].im, x.im)};
+    } else if (g.sub) {
+      r = S::ld(static_cast<const typename S::elem*>(g.sub) + rhs * out_stride, e0 + k) - r;
     }
-  }
-  if (half == 1) {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) sacc[k][ls] = acc[k];
-  }
-  __syncthreads();
-  if (half != 0 || !active) return;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] += sacc[k][ls];
-  R mk = (R)(-g.kappa);
-  cplx<R> res[12];
-  if (parity < 0) {
-    cplx<R> p[12];
-    SiteIO<S>::load(in + in_off, (size_t)site, p);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      res[k].re = fma(mk, acc[k].re, p[k].re);
-      res[k].im = fma(mk, acc[k].im, p[k].im);
-    }
-    SiteIO<S>::store(out + rhs * out_stride, (size_t)site, res);
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) res[k] = mk * acc[k];
-    apply_sub<S>(g, rhs * out_stride, i, res);
-    SiteIO<S>::store(out + rhs * out_stride, (size_t)i, res);
+    S::st(out + rhs * out_stride, e0 + k, r);
   }
 }
 
 // Launch variants of an aligned call, searched by the autotuner per (dtype, layout, parity,
 // dagger, volume, nrhs): 0 and 1 one site per thread, 128 threads, registers uncapped and capped
-// at 128; 2 two threads per site (dslash_split_kernel); 3 one site per thread at 80 registers; 4
+// at 128; 2 one thread per site and hop (dslash_hop_kernel); 3 one site per thread at 80 registers; 4
 // and 5 take 2 and 4 right-hand sides per thread (dslash_mrhs_kernel), candidates only when nrhs
 // > 1.  Complex double stops at 2: its later forms spill kilobytes per thread.
 constexpr int kNumVariants = 6, kNumSingle = 4, kNumF64 = 3;
@@ -142,11 +113,11 @@ void launch_variant(int v, void* out, const void* in, const void* links, const K
                     int parity, int nsites, int nrhs, cudaStream_t st, size_t is, size_t os) {
   if (v == 2) {
     typedef typename S::elem E;
-    KGeom k64 = k;
-    k64.tile = pick_tile(k.L, parity, 64);
-    dim3 grid(stencil_ctas(k64.tile, nsites, 64), nrhs);
-    launch_dep(dslash_split_kernel<S, DAG, LL>, grid, 128, 0, st, (E*)out, (const E*)in,
-               (const E*)links, k64, parity, nsites, is, os);
+    // one warp per CTA until every SM has a few of them
+    const int t = (long long)nsites * nrhs < 4LL * 16 * num_sms() ? 32 : 128;
+    dim3 grid((nsites + t / 8 - 1) / (t / 8), nrhs);
+    launch_dep(dslash_hop_kernel<S, DAG, LL>, grid, t, 0, st, (E*)out, (const E*)in,
+               (const E*)links, k, parity, nsites, is, os);
     return;
   }
   if constexpr (!std::is_same<S, StC128>::value) {

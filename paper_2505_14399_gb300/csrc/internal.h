@@ -49,6 +49,7 @@ struct ReduceWork {
   int nblk = 0;
   int cap = 0;        // partial slots per vector: >= nblk, and one per 96 sites of a fine
                       // field, so the fused stencil kernel may launch a CTA per 96-site tile
+                      // (per 32 sites on lattices of up to 2^17 of them)
   int maxvec = 0;
   int nrhs_cap = 0;
   int alloc(size_t n, int nrhs, int maxvec);

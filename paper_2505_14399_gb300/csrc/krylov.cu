@@ -569,9 +569,120 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
+// The same step with one thread per site and hop (hop_lanes): for small lattices, whose launches
+// last as long as one thread's chain of eight hops.  A lane pair holds one spin of its site; the
+// two lanes take the basis columns of either parity.
+constexpr int HPT = 256;    // 32 sites
+template <int NVM, bool FIRST, int LL>
+__global__ void __launch_bounds__(HPT)
+dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
+                       const float2* __restrict__ links, stencil::KGeom g, zd* small, SmallLayout L,
+                       double* wnorm, double* partial, unsigned* counter, int maxvec,
+                       const zf* __restrict__ b0, const double* beta0, const zf* __restrict__ sin,
+                       int par) {
+  using namespace stencil;
+  dep_entry();
+  constexpr int NH = (NVM + 1) / 2, NWP = HPT / 32;
+  __shared__ float sh[NWP][2 * NVM + 1];
+  const int rhs = blockIdx.y;
+  const int nsites = par ? g.V / 2 : g.V;
+  zf* vb = V + (size_t)rhs * n;
+  const zf* vin = FIRST ? b0 + (size_t)rhs * n : vb + (size_t)(nv - 1) * vstride;
+  float sc = 1.0f;
+  if (FIRST) {
+    double bb = beta0[rhs];
+    sc = bb > 0 ? (float)(1.0 / bb) : 0.0f;
+  }
+  zf* wr = w + (size_t)rhs * n;
+  const float2* vst = reinterpret_cast<const float2*>(par ? sin + (size_t)rhs * n : vin);
+  const int site = blockIdx.x * (HPT / 8) + (threadIdx.x >> 3), hop = threadIdx.x & 7;
+  const bool active = site < nsites;
+  int c[4] = {0, 0, 0, 0}, ls = 0;
+  if (active) ls = stencil_site(g, par ? 0 : -1, site, c);
+  zf acc[3];
+  hop_lanes<0, StC64, LL>(g, active, ls, c, hop, vst, par != 0, links, acc);
+  float ar[NH], ai[NH], ss = 0.f;
+#pragma unroll
+  for (int q = 0; q < NH; ++q) { ar[q] = 0.f; ai[q] = 0.f; }
+  if (active) {
+    const size_t e0 = (size_t)site * 12 + 3 * (hop >> 1);
+    const int odd = hop & 1;
+    const float mk = par ? (float)g.kappa : (float)(-g.kappa);
+    zf p[3], x0[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      x0[k] = vin[e0 + k];
+      p[k] = {sc * fmaf(mk, acc[k].re, x0[k].re), sc * fmaf(mk, acc[k].im, x0[k].im)};
+      ss = fmaf(p[k].re, p[k].re, ss);
+      ss = fmaf(p[k].im, p[k].im, ss);
+      x0[k] = sc * x0[k];
+    }
+    if (odd) ss = 0.f;   // the pair holds the same values
+    if (!odd) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        wr[e0 + k] = p[k];
+        if (FIRST) vb[e0 + k] = x0[k];   // v_0
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NH; ++q) {
+      const int col = 2 * q + odd;
+      if (col < nv) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const zf v = FIRST ? x0[k] : vb[(size_t)col * vstride + e0 + k];
+          ar[q] = fmaf(v.re, p[k].re, ar[q]);
+          ar[q] = fmaf(v.im, p[k].im, ar[q]);
+          ai[q] = fmaf(v.re, p[k].im, ai[q]);
+          ai[q] = fmaf(-v.im, p[k].re, ai[q]);
+        }
+      }
+    }
+  }
+  // sums over the lanes of either parity, then over the warps
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NH; ++q) {
+    if (2 * q < nv) {
+#pragma unroll
+      for (int o = 2; o < 32; o <<= 1) {
+        ar[q] += __shfl_xor_sync(0xffffffffu, ar[q], o);
+        ai[q] += __shfl_xor_sync(0xffffffffu, ai[q], o);
+      }
+      if (lane < 2 && 2 * q + lane < nv) {
+        sh[wid][2 * (2 * q + lane)] = ar[q];
+        sh[wid][2 * (2 * q + lane) + 1] = ai[q];
+      }
+    }
+  }
+  ss = warp_sum_r(ss);
+  if (lane == 0) sh[wid][2 * NVM] = ss;
+  __syncthreads();
+  const int nblk = gridDim.x;
+  if ((int)threadIdx.x < 2 * nv + 2) {
+    const int t = threadIdx.x;
+    float v = 0.f;
+    if (t < 2 * nv) {
+      for (int i = 0; i < NWP; ++i) v += sh[i][t];
+    } else if (t == 2 * nv) {
+      for (int i = 0; i < NWP; ++i) v += sh[i][2 * NVM];
+    }
+    partials_as<float>(partial)[(((size_t)rhs * maxvec + (t >> 1)) * nblk + blockIdx.x) * 2 + (t & 1)] = v;
+    __threadfence();
+  }
+  if (!last_cta(counter, rhs, nblk)) return;
+  __shared__ zd g_h2[NVM + 1];
+  finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0);
+  __syncthreads();
+  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true);
+  if (threadIdx.x == 0) counter[rhs] = 0;
+}
+
 // launch shapes of the fused kernel: 128 threads and 4, 5 or 6 resident CTAs per SM asked of the
-// register allocator (128, 96 or 80 registers).
-constexpr int kProjShapes = 3;
+// register allocator (128, 96 or 80 registers); 3 is dslash_proj_hop_kernel, a candidate where
+// the partial slots hold its CTAs of 32 sites.
+constexpr int kProjShapes = 4;
 
 template <int NVM, bool FIRST, int LL>
 void launch_proj_v(int v, int nv, int nrhs, cudaStream_t st, zf* w, zf* V, size_t fs, size_t n,
@@ -584,7 +695,12 @@ void launch_proj_v(int v, int nv, int nrhs, cudaStream_t st, zf* w, zf* V, size_
     *err = launch_dep(kernel, grid, 128, 0, st, w, V, fs, nv, n, L32, kg, small, L, dnorm,
                       rw.partial, rw.counter, rw.maxvec, b0, beta0, sin, par);
   };
-  if (v == 1) go(dslash_proj_kernel<NVM, FIRST, LL, 128, 5>);
+  if (v == 3) {
+    const int ns = par ? kg.V / 2 : kg.V;
+    *err = launch_dep(dslash_proj_hop_kernel<NVM, FIRST, LL>, dim3((ns + HPT / 8 - 1) / (HPT / 8), nrhs),
+                      HPT, 0, st, w, V, fs, nv, n, L32, kg, small, L, dnorm, rw.partial, rw.counter,
+                      rw.maxvec, b0, beta0, sin, par);
+  } else if (v == 1) go(dslash_proj_kernel<NVM, FIRST, LL, 128, 5>);
   else if (v == 2) go(dslash_proj_kernel<NVM, FIRST, LL, 128, 6>);
   else go(dslash_proj_kernel<NVM, FIRST, LL, 128, 4>);
 }
@@ -612,7 +728,8 @@ int launch_proj(int nv, bool first, int nrhs, cudaStream_t st, zf* w, zf* V, siz
   // tuning key: a dtype code of its own per (columns class, link layout), parity -2; the
   // kernel is idempotent (it rewrites w, its partials and its Hessenberg column from inputs
   // it does not modify), so the tuner may run it several times
-  int v = tuned_variant(1000 + 100 * par + 10 * nvm + LL, -2, 0, kg.V, nrhs, st, kProjShapes, run);
+  const int nshape = (ns + HPT / 8 - 1) / (HPT / 8) <= rw.cap ? kProjShapes : kProjShapes - 1;
+  int v = tuned_variant(1000 + 100 * par + 10 * nvm + LL, -2, 0, kg.V, nrhs, st, nshape, run);
   if (v < 0) return fail(MG_ECUDA, "fused stencil autotune failed");
   run(v);
   count_launch();

@@ -354,6 +354,118 @@ __device__ __forceinline__ void hop_pair(const KGeom& g, int site, const int c[4
   hop_bwd<MU, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
 }
 
+// ---- one thread per site and hop
+// For lattices that leave the chip idle with a thread per site (4^4: two CTAs; 8^4: 32) the chain
+// of eight dependent hops is the launch: FP64 on 4^4 17.8 us, of which the launch itself is a
+// few.  Here eight lanes share a site, lane `hop` takes direction hop / 2 (forward when even) with
+// the spin projector's phases as operands, and the 12 sums are reduced and scattered over the
+// lanes: every pair of lanes ends with the three colours of one spin.
+
+// i sigma_mu d for mu < 3, d for mu = 3, as (f0 d[w], f1 d[1 - w]) with units f and w = 1 for mu < 2
+template <typename R>
+struct HopPhase {
+  bool swap;
+  R re0, im0, re1, im1;
+};
+template <typename R>
+__device__ __forceinline__ HopPhase<R> hop_phase(int mu) {
+  HopPhase<R> p;
+  p.swap = mu < 2;
+  p.re0 = (mu & 1) ? R(1) : R(0);          // mu 1, 3: 1; mu 0, 2: i
+  p.im0 = (mu & 1) ? R(0) : R(1);
+  p.re1 = mu == 1 ? R(-1) : p.re0;         // mu 1: -1, mu 2: -i
+  p.im1 = mu == 2 ? R(-1) : p.im0;
+  return p;
+}
+
+// The hop's term of H psi at `site`, reduced over the site's eight lanes: out = components 3 sp ..
+// 3 sp + 2 of sum_mu w_mu [...], sp = hop >> 1.  All 32 lanes call it; inactive sites pass active =
+// false and get zeros.
+template <int DAG, typename S, int LL>
+__device__ __forceinline__ void hop_lanes(const KGeom& g, bool active, int site, const int c[4],
+                                          int hop, const typename S::elem* in, bool half_in,
+                                          const typename S::elem* links,
+                                          cplx<typename S::real> out[3]) {
+  typedef typename S::real R;
+  const int mu = hop >> 1;
+  const bool fwd = (hop & 1) == 0;
+  cplx<R> gg[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) gg[i] = {0, 0};
+  const HopPhase<R> f = hop_phase<R>(mu);
+  R s = (fwd != (DAG != 0)) ? R(-1) : R(1);   // projector sign
+  R cf = 0;
+  if (active) {
+    const int L = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
+    const int st = mu == 0 ? g.stride[0] : mu == 1 ? g.stride[1] : mu == 2 ? g.stride[2] : g.stride[3];
+    const int cm = mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3];
+    const int bc = mu == 0 ? g.bc[0] : mu == 1 ? g.bc[1] : mu == 2 ? g.bc[2] : g.bc[3];
+    const R w = mu == 0 ? wgt<R>(g, 0) : mu == 1 ? wgt<R>(g, 1) : mu == 2 ? wgt<R>(g, 2) : wgt<R>(g, 3);
+    const bool wrap = fwd ? cm == L - 1 : cm == 0;
+    const int step = wrap ? -(L - 1) * st : st;
+    const int nb = fwd ? site + step : site - step;
+    cf = (wrap && bc < 0) ? -w : w;
+    cplx<R> p[12], u[9], h[6];
+    SiteIO<S>::load(in, half_in ? (size_t)(nb >> 1) : (size_t)nb, p);
+    load_link<S, LL>(links, g.V, mu, fwd ? site : nb, u);
+    // h = psi_up - s i sigma psi_dn (mu < 3), psi_up + s psi_dn (mu = 3)
+    const R sp = mu < 3 ? -s : s;
+    const R r0 = sp * f.re0, i0 = sp * f.im0, r1 = sp * f.re1, i1 = sp * f.im1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const cplx<R> d0 = f.swap ? p[9 + k] : p[6 + k], d1 = f.swap ? p[6 + k] : p[9 + k];
+      h[k] = {fma(r0, d0.re, fma(-i0, d0.im, p[k].re)), fma(r0, d0.im, fma(i0, d0.re, p[k].im))};
+      h[3 + k] = {fma(r1, d1.re, fma(-i1, d1.im, p[3 + k].re)),
+                  fma(r1, d1.im, fma(i1, d1.re, p[3 + k].im))};
+    }
+    // U h or U^dag h
+    const R cj = fwd ? R(1) : R(-1);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      cplx<R> t0 = {0, 0}, t1 = {0, 0};
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const cplx<R> q = fwd ? u[a * 3 + b] : u[b * 3 + a];
+        const cplx<R> m = {q.re, cj * q.im};
+        cfma(t0, m, h[b]);
+        cfma(t1, m, h[3 + b]);
+      }
+      gg[a] = t0;
+      gg[3 + a] = t1;
+    }
+  }
+  // upper pair cf g, lower pair cf s i sigma g (cf s g): lanes 0-3 keep the upper, 4-7 the lower
+  const R cs = cf * s;
+  const R r0 = cs * f.re0, i0 = cs * f.im0, r1 = cs * f.re1, i1 = cs * f.im1;
+  const bool low = (hop & 4) != 0;
+  cplx<R> keep[6];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const cplx<R> g0 = f.swap ? gg[3 + k] : gg[k], g1 = f.swap ? gg[k] : gg[3 + k];
+    const cplx<R> up0 = cf * gg[k], up1 = cf * gg[3 + k];
+    const cplx<R> lo0 = {fma(r0, g0.re, -i0 * g0.im), fma(r0, g0.im, i0 * g0.re)};
+    const cplx<R> lo1 = {fma(r1, g1.re, -i1 * g1.im), fma(r1, g1.im, i1 * g1.re)};
+    const cplx<R> s0 = low ? up0 : lo0, s1 = low ? up1 : lo1;
+    keep[k] = low ? lo0 : up0;
+    keep[3 + k] = low ? lo1 : up1;
+    keep[k].re += __shfl_xor_sync(0xffffffffu, s0.re, 4);
+    keep[k].im += __shfl_xor_sync(0xffffffffu, s0.im, 4);
+    keep[3 + k].re += __shfl_xor_sync(0xffffffffu, s1.re, 4);
+    keep[3 + k].im += __shfl_xor_sync(0xffffffffu, s1.im, 4);
+  }
+  const bool odd = (hop & 2) != 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const cplx<R> send = odd ? keep[k] : keep[3 + k];
+    cplx<R> t = odd ? keep[3 + k] : keep[k];
+    t.re += __shfl_xor_sync(0xffffffffu, send.re, 2);
+    t.im += __shfl_xor_sync(0xffffffffu, send.im, 2);
+    t.re += __shfl_xor_sync(0xffffffffu, t.re, 1);
+    t.im += __shfl_xor_sync(0xffffffffu, t.im, 1);
+    out[k] = t;
+  }
+}
+
 // Site index of thread i (parity < 0: lexicographic; else the i-th site of that parity)
 // and its coordinates.
 __device__ __forceinline__ int stencil_site(const KGeom& g, int parity, int i, int c[4]) {
