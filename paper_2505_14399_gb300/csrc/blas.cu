@@ -181,8 +181,8 @@ __global__ void scale_inv_kernel(E* y, const E* x, const double* s, int lds, siz
   typedef VecT<E> T;
   typedef typename T::R R;
   int rhs = blockIdx.y;
-  double sv = s[(size_t)rhs * lds];
-  R f = sv > 0 ? (R)(1.0 / sv) : (R)0;
+  const R sv = (R)s[(size_t)rhs * lds];
+  const R f = sv > 0 ? (R)1 / sv : (R)0;
   const E* xr = x + (size_t)rhs * n;
   E* yr = y + (size_t)rhs * n;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
@@ -193,11 +193,11 @@ __global__ void scale_inv_kernel(E* y, const E* x, const double* s, int lds, siz
 }
 
 template <typename E>
-__global__ void axpby_kernel(E* y, double a, const E* x, double b, size_t n) {
+__global__ void axpby_kernel(E* y, typename VecT<E>::R ar, const E* x, typename VecT<E>::R br,
+                             size_t n) {
   dep_entry();
   typedef VecT<E> T;
   typedef typename T::R R;
-  R ar = (R)a, br = (R)b;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (size_t)gridDim.x * blockDim.x) {
     cplx<R> xv = T::ld(x, k), yv = T::ld(y, k);
@@ -207,10 +207,9 @@ __global__ void axpby_kernel(E* y, double a, const E* x, double b, size_t n) {
 
 // y += a * x with x and y of possibly different storage (arithmetic of y)
 template <typename Ey, typename Ex>
-__global__ void axpy_mixed_kernel(Ey* y, double a, const Ex* x, size_t n) {
+__global__ void axpy_mixed_kernel(Ey* y, typename VecT<Ey>::R ar, const Ex* x, size_t n) {
   dep_entry();
   typedef typename VecT<Ey>::R R;
-  R ar = (R)a;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (size_t)gridDim.x * blockDim.x) {
     auto xv = VecT<Ex>::ld(x, k);
@@ -221,11 +220,11 @@ __global__ void axpy_mixed_kernel(Ey* y, double a, const Ex* x, size_t n) {
 
 // y = a * x1 + b * x2 (x1, x2 in one storage, y in another; arithmetic of x)
 template <typename Eo, typename Ei>
-__global__ void lincomb_kernel(Eo* y, double a, const Ei* x1, double b, const Ei* x2, size_t n) {
+__global__ void lincomb_kernel(Eo* y, typename VecT<Ei>::R ar, const Ei* x1,
+                               typename VecT<Ei>::R br, const Ei* x2, size_t n) {
   dep_entry();
   typedef typename VecT<Ei>::R R;
   typedef typename VecT<Eo>::R Ro;
-  R ar = (R)a, br = (R)b;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (size_t)gridDim.x * blockDim.x) {
     cplx<R> u = VecT<Ei>::ld(x1, k), v = VecT<Ei>::ld(x2, k);
@@ -367,19 +366,21 @@ int scale_inv_v(E* y, const E* x, const double* s, int lds, size_t n, int nrhs, 
 template <typename E>
 int axpby_v(E* y, double a, const E* x, double b, size_t n, int nrhs, cudaStream_t st) {
   size_t tot = n * nrhs;
-  WMG_LAUNCH_DEP(axpby_kernel<E>, grid_for(tot), 256, 0, st, y, a, x, b, tot);
+  typedef typename VecT<E>::R R;
+  WMG_LAUNCH_DEP(axpby_kernel<E>, grid_for(tot), 256, 0, st, y, (R)a, x, (R)b, tot);
   return MG_OK;
 }
 
 template <typename Ey, typename Ex>
 int axpy_mixed(Ey* y, double a, const Ex* x, size_t n, cudaStream_t st) {
-  WMG_LAUNCH_DEP(axpy_mixed_kernel<Ey, Ex>, grid_for(n), 256, 0, st, y, a, x, n);
+  WMG_LAUNCH_DEP(axpy_mixed_kernel<Ey, Ex>, grid_for(n), 256, 0, st, y, (typename VecT<Ey>::R)a, x, n);
   return MG_OK;
 }
 
 template <typename Eo, typename Ei>
 int lincomb_v(Eo* y, double a, const Ei* x1, double b, const Ei* x2, size_t n, cudaStream_t st) {
-  WMG_LAUNCH_DEP(lincomb_kernel<Eo, Ei>, grid_for(n), 256, 0, st, y, a, x1, b, x2, n);
+  typedef typename VecT<Ei>::R R;
+  WMG_LAUNCH_DEP(lincomb_kernel<Eo, Ei>, grid_for(n), 256, 0, st, y, (R)a, x1, (R)b, x2, n);
   return MG_OK;
 }
 

@@ -50,25 +50,35 @@ restrict_kernel(cplx<R>* vc, const cplx<R>* __restrict__ v, const cplx<R>* __res
   cplx<R>* sred = sv + B.M;   // [2k]
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const cplx<R>* Pt = P + (size_t)t * k * B.M;
-  const int half_rows = (B.M + 1) / 2;
+  const int half_rows = (B.M / 2 + 1) & ~1;   // M = 6 n_d is even: whole row pairs
   for (int it = wid; it < 2 * k; it += nw) {
     const int i = it >> 1, r0 = (it & 1) * half_rows;
     const int r1 = min(B.M, r0 + half_rows);
     const cplx<R>* col = Pt + (size_t)i * B.M;
     cplx<R> a0 = {0, 0}, a1 = {0, 0};
-    int row = r0 + lane;
-    // eight loads of P in flight per lane
-    for (; row + 224 < r1; row += 256) {
-      cplx<R> c[8];
+    // two rows per load (16 bytes of an FP32 P), four loads in flight per lane
+    struct alignas(sizeof(R) == 4 ? 16 : 8) Pair {
+      cplx<R> a, b;
+    };
+    const Pair* c2 = reinterpret_cast<const Pair*>(col);
+    const Pair* s2 = reinterpret_cast<const Pair*>(sv);
+    int row = r0 / 2 + lane;
+    for (; row + 96 < r1 / 2; row += 128) {
+      Pair c[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) c[u] = col[row + 32 * u];
+      for (int u = 0; u < 4; ++u) c[u] = c2[row + 32 * u];
 #pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        cfmac(a0, c[u], sv[row + 32 * u]);
-        cfmac(a1, c[u + 1], sv[row + 32 * u + 32]);
+      for (int u = 0; u < 4; ++u) {
+        const Pair w = s2[row + 32 * u];
+        cfmac(a0, c[u].a, w.a);
+        cfmac(a1, c[u].b, w.b);
       }
     }
-    for (; row < r1; row += 32) cfmac(a0, col[row], sv[row]);
+    for (; row < r1 / 2; row += 32) {
+      const Pair c = c2[row], w = s2[row];
+      cfmac(a0, c.a, w.a);
+      cfmac(a1, c.b, w.b);
+    }
     a0 += a1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -82,34 +92,45 @@ restrict_kernel(cplx<R>* vc, const cplx<R>* __restrict__ v, const cplx<R>* __res
     vc[(size_t)rhs * B.d * 2 * k + (size_t)t * k + i] = sred[2 * i] + sred[2 * i + 1];
 }
 
+// One thread per component pair of a site (two rows of a column: 16-byte loads of an FP32 P), four
+// columns' loads in flight.
 template <typename R>
-__global__ void prolong_kernel(cplx<R>* v, const cplx<R>* __restrict__ vc,
-                               const cplx<R>* __restrict__ P, int k, Blocking B, size_t total) {
+__global__ void __launch_bounds__(256)
+prolong_kernel(cplx<R>* v, const cplx<R>* __restrict__ vc, const cplx<R>* __restrict__ P, int k,
+               Blocking B) {
   dep_entry();
-  size_t V12 = (size_t)B.nd * B.d * 12;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    size_t rhs = e / V12, rem = e % V12;
-    int s = (int)(rem / 12), comp = (int)(rem % 12);
-    int spin = comp / 3, c = comp % 3;
-    int j, l;
-    B.block_of(s, &j, &l);
-    int t = 2 * j + (spin >> 1);
-    int row = (l * 2 + (spin & 1)) * 3 + c;
-    const cplx<R>* Pt = P + (size_t)t * k * B.M + row;
-    const cplx<R>* cv = vc + rhs * B.d * 2 * k + (size_t)t * k;
-    cplx<R> acc = {0, 0};
-    int i = 0;
-    for (; i + 4 <= k; i += 4) {   // four loads of P in flight
-      cplx<R> p[4];
+  struct alignas(sizeof(R) == 4 ? 16 : 8) Pair {
+    cplx<R> a, b;
+  };
+  const unsigned e = blockIdx.x * 256u + threadIdx.x, n = 6u * B.nd * B.d;
+  if (e >= n) return;
+  const unsigned s = e / 6;
+  const int p = (int)(e - 6 * s), alpha = p / 3;
+  int j, l;
+  B.block_of((int)s, &j, &l);
+  const int t = 2 * j + alpha;
+  const cplx<R>* Pt = P + (size_t)t * k * B.M + 6 * l + 2 * (p - 3 * alpha);
+  const size_t rhs = blockIdx.y;
+  const cplx<R>* cv = vc + rhs * B.d * 2 * k + (size_t)t * k;
+  cplx<R> x = {0, 0}, y = {0, 0};
+  int i = 0;
+  for (; i + 4 <= k; i += 4) {
+    Pair q[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) p[u] = Pt[(size_t)(i + u) * B.M];
+    for (int u = 0; u < 4; ++u) q[u] = *reinterpret_cast<const Pair*>(Pt + (size_t)(i + u) * B.M);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) cfma(acc, p[u], cv[i + u]);
+    for (int u = 0; u < 4; ++u) {
+      const cplx<R> c = cv[i + u];
+      cfma(x, q[u].a, c);
+      cfma(y, q[u].b, c);
     }
-    for (; i < k; ++i) cfma(acc, Pt[(size_t)i * B.M], cv[i]);
-    v[e] = acc;
   }
+  for (; i < k; ++i) {
+    const Pair q = *reinterpret_cast<const Pair*>(Pt + (size_t)i * B.M);
+    cfma(x, q.a, cv[i]);
+    cfma(y, q.b, cv[i]);
+  }
+  *reinterpret_cast<Pair*>(v + 2 * (rhs * n + e)) = Pair{x, y};
 }
 
 
@@ -417,12 +438,10 @@ int restrict_launch(cplx<R>* vc, const cplx<R>* v, const cplx<R>* P, int k, cons
 template <typename R>
 int prolong_launch(cplx<R>* v, const cplx<R>* vc, const cplx<R>* P, int k, const Blocking& B,
                    int nrhs, cudaStream_t st) {
-  size_t total = (size_t)nrhs * B.nd * B.d * 12;
-  size_t gsz = (total + 255) / 256;
-  size_t cap = (size_t)num_sms() * 16;
+  const dim3 grid((6u * B.nd * B.d + 255) / 256, nrhs);
   ProfScope ps("prolong", (double)sizeof(cplx<R>) * (12.0 * B.nd * B.d * (k + nrhs) + 2.0 * B.d * k * nrhs),
                8.0 * 12 * B.nd * B.d * k * nrhs, st);
-  WMG_LAUNCH_DEP(prolong_kernel<R>, (unsigned)(gsz < cap ? gsz : cap), 256, 0, st, v, vc, P, k, B, total);
+  WMG_LAUNCH_DEP(prolong_kernel<R>, grid, 256, 0, st, v, vc, P, k, B);
   return MG_OK;
 }
 

@@ -41,7 +41,7 @@ dslash_kernel(typename S::elem* __restrict__ out, const typename S::elem* __rest
   hop_pair<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
   hop_pair<2, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
   hop_pair<3, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-  R mk = (R)(-g.kappa);
+  R mk = -kap<R>(g);
   cplx<R> res[12];
   if (parity < 0) {
     cplx<R> p[12];
@@ -77,7 +77,7 @@ dslash_hop_kernel(typename S::elem* __restrict__ out, const typename S::elem* __
   cplx<R> acc[3];
   hop_lanes<DAG, S, LL>(g, active, site, c, hop, inr, parity >= 0, links, acc);
   if (!active || (hop & 1)) return;
-  const R mk = (R)(-g.kappa);
+  const R mk = -kap<R>(g);
   const size_t e0 = (size_t)i * 12 + 3 * (hop >> 1);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {

@@ -96,7 +96,7 @@ dslash_mrhs_kernel(typename S::elem* __restrict__ out, const typename S::elem* _
   hop_bwd_m<2, DAG, S, LL, NR>(g, site, c, inr, in_stride, nr, half_in, links, acc);
   hop_fwd_m<3, DAG, S, LL, NR>(g, site, c, inr, in_stride, nr, half_in, links, acc);
   hop_bwd_m<3, DAG, S, LL, NR>(g, site, c, inr, in_stride, nr, half_in, links, acc);
-  const R mk = (R)(-g.kappa);
+  const R mk = -kap<R>(g);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
     if (r < nr) {

@@ -120,16 +120,37 @@ __device__ void givens_deferred(zd* sm, SmallLayout L, int j, double* res) {
 // The end of a reduction sweep, by its last CTA: h2 (the nv projections and ||w||^2, in shared
 // memory) to the coefficients of the update, column nv - 1 of the Hessenberg matrix (added to the
 // first pass's projections, or alone when `single`) and H[j+1, j]^2 = ||w||^2 - ||h2||^2.
+// beta (fused fixed runs): column 0 of the basis is the right-hand side b itself, of norm beta, so
+// its projection and its coefficient carry 1 / beta each.  In the first step (`first`) w = D b as
+// well, h2[1].im = ||b||^2, and beta and 1 / beta are written (beta[ibeta]: no FP64 division in
+// the chain of every later step).
 __device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, const zd* h2,
-                                              double* wnorm, bool single) {
+                                              double* wnorm, bool single, double* beta = nullptr,
+                                              bool first = false, int ibeta = 0) {
   zd* col = sm + L.H() + (size_t)(nv - 1) * (L.m + 1);
+  if (first) {
+    if (threadIdx.x == 0) {
+      const double bb = h2[1].im, ib2 = bb > 0 ? 1.0 / bb : 0.0, ib = sqrt(ib2);
+      const zd h = ib2 * h2[0];
+      const double w2 = h2[1].re - bb * norm2(h), w = w2 > 0 ? sqrt(w2) : 0.0;
+      sm[L.h2()] = h;
+      col[0] = h;
+      col[1] = {w * ib, 0};
+      *wnorm = w;           // v_1 = (D b - h b) / w
+      beta[0] = bb * ib;
+      beta[ibeta] = ib;
+    }
+    return;
+  }
+  const double s0 = beta ? beta[ibeta] : 1.0;
   for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-    sm[L.h2() + i] = h2[i];
-    col[i] = single ? h2[i] : col[i] + h2[i];
+    const double s = i == 0 ? s0 : 1.0;
+    sm[L.h2() + i] = s * s * h2[i];
+    col[i] = single ? s * h2[i] : col[i] + h2[i];
   }
   if (threadIdx.x == 0) {
-    double hh = 0;
-    for (int i = 0; i < nv; ++i) hh += norm2(h2[i]);
+    double hh = s0 * s0 * norm2(h2[0]);
+    for (int i = 1; i < nv; ++i) hh += norm2(h2[i]);
     const double b2 = h2[nv].re - hh, b = b2 > 0 ? sqrt(b2) : 0.0;
     *wnorm = b;
     col[nv] = {b, 0};
@@ -272,8 +293,10 @@ cgs_update_scale_kernel(E* vout, const E* __restrict__ w, const E* __restrict__ 
   const zd* h2 = small + (size_t)rhs * L.stride() + L.h2();
   for (int i = threadIdx.x; i < nv; i += blockDim.x) cs[i] = {(R)(-h2[i].re), (R)(-h2[i].im)};
   __syncthreads();
-  double beta = wnorm[rhs];
-  R f = beta > 0 ? (R)(1.0 / beta) : (R)0;
+  // the division in the vectors' precision: in FP64 on every thread it took as long as the update
+  // itself (FP64 instructions occupy an SM for 16 cycles per warp): 14.1 -> UPD us on 65 536 sites
+  const R beta = (R)wnorm[rhs];
+  const R f = beta > 0 ? (R)1 / beta : (R)0;
   const E* wr = w + (size_t)rhs * n;
   const E* vb = V + (size_t)rhs * n;
   E* outr = vout + (size_t)rhs * n;
@@ -483,8 +506,7 @@ __global__ void __launch_bounds__(BT, MINB)
 dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
                    const float2* __restrict__ links, stencil::KGeom g, zd* small, SmallLayout L,
                    double* wnorm, double* partial, unsigned* counter, int maxvec,
-                   const zf* __restrict__ b0, const double* beta0, const zf* __restrict__ sin,
-                   int par) {
+                   const zf* __restrict__ b0, double* beta, const zf* __restrict__ sin, int par) {
   using namespace stencil;
   dep_entry();
   __shared__ float sh[(BT / 32) * NVM * 2];
@@ -493,21 +515,17 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   // half-lattice fields, with t_o = -kappa H_oe x (the odd field sin) computed by the caller
   const int nsites = par ? g.V / 2 : g.V;
   float2* vb = reinterpret_cast<float2*>(V) + (size_t)rhs * n;
-  // FIRST (step 0): the stencil reads b and everything is scaled by 1 / ||b|| (linear),
-  // v_0 = b / ||b|| is written here (no separate scaling pass); otherwise the input is v_j
+  // FIRST (step 0): the stencil reads b, which is copied to column 0 as it is, and ||b||^2 joins
+  // the sums (finish_column scales; neither a norm nor a scaling pass of their own); otherwise
+  // the input is v_j
   const float2* vin = FIRST ? reinterpret_cast<const float2*>(b0) + (size_t)rhs * n
                             : vb + (size_t)(nv - 1) * vstride;
-  float sc = 1.0f;
-  if (FIRST) {
-    double bb = beta0[rhs];
-    sc = bb > 0 ? (float)(1.0 / bb) : 0.0f;
-  }
   float2* wr = reinterpret_cast<float2*>(w) + (size_t)rhs * n;
   const float2* vst = par ? reinterpret_cast<const float2*>(sin) + (size_t)rhs * n : vin;
   float ar[NVM], ai[NVM];
 #pragma unroll
   for (int q = 0; q < NVM; ++q) { ar[q] = 0.f; ai[q] = 0.f; }
-  float ss = 0.f;
+  float ss = 0.f, bb = 0.f;
   // one site per thread (the launcher sizes the grid to cover every site): with no loop the
   // projection accumulators are not live across the stencil's hops, which need the registers.
   // site: the output index (lexicographic, or the checkerboard index with par); ls: the lattice
@@ -523,15 +541,17 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
     hop_pair<3, 0, StC64, LL>(g, ls, c, vst, 0, par != 0, links, acc);
     zf p[12], x0[12];
     SiteIO<StC64>::load(vin, (size_t)site, x0);
-    const float mk = par ? (float)g.kappa : (float)(-g.kappa);
+    const float mk = par ? g.kf : -g.kf;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      p[k].re = sc * fmaf(mk, acc[k].re, x0[k].re);
-      p[k].im = sc * fmaf(mk, acc[k].im, x0[k].im);
+      p[k].re = fmaf(mk, acc[k].re, x0[k].re);
+      p[k].im = fmaf(mk, acc[k].im, x0[k].im);
       ss = fmaf(p[k].re, p[k].re, ss);
       ss = fmaf(p[k].im, p[k].im, ss);
-      x0[k].re *= sc;
-      x0[k].im *= sc;
+      if (FIRST) {
+        bb = fmaf(x0[k].re, x0[k].re, bb);
+        bb = fmaf(x0[k].im, x0[k].im, bb);
+      }
     }
     SiteIO<StC64>::store(wr, (size_t)site, p);
     if (FIRST) SiteIO<StC64>::store(vb, (size_t)site, x0);   // v_0
@@ -558,14 +578,14 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   const int nblk = gridDim.x;
   cta_store_partials<float, NVM>(ar, ai, nv, 0, rhs, maxvec, nblk, partials_as<float>(partial),
                                  sh);
-  float zero = 0.f;
-  cta_store_partials<float, 1>(&ss, &zero, 1, nv, rhs, maxvec, nblk, partials_as<float>(partial),
+  cta_store_partials<float, 1>(&ss, &bb, 1, nv, rhs, maxvec, nblk, partials_as<float>(partial),
                                sh);
   if (!last_cta(counter, rhs, nblk)) return;
   __shared__ zd g_h2[NVM + 1];
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0);
   __syncthreads();
-  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true);
+  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true,
+                beta ? beta + rhs : nullptr, FIRST, gridDim.y);
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
@@ -578,21 +598,15 @@ __global__ void __launch_bounds__(HPT)
 dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
                        const float2* __restrict__ links, stencil::KGeom g, zd* small, SmallLayout L,
                        double* wnorm, double* partial, unsigned* counter, int maxvec,
-                       const zf* __restrict__ b0, const double* beta0, const zf* __restrict__ sin,
-                       int par) {
+                       const zf* __restrict__ b0, double* beta, const zf* __restrict__ sin, int par) {
   using namespace stencil;
   dep_entry();
   constexpr int NH = (NVM + 1) / 2, NWP = HPT / 32;
-  __shared__ float sh[NWP][2 * NVM + 1];
+  __shared__ float sh[NWP][2 * NVM + 2];
   const int rhs = blockIdx.y;
   const int nsites = par ? g.V / 2 : g.V;
   zf* vb = V + (size_t)rhs * n;
   const zf* vin = FIRST ? b0 + (size_t)rhs * n : vb + (size_t)(nv - 1) * vstride;
-  float sc = 1.0f;
-  if (FIRST) {
-    double bb = beta0[rhs];
-    sc = bb > 0 ? (float)(1.0 / bb) : 0.0f;
-  }
   zf* wr = w + (size_t)rhs * n;
   const float2* vst = reinterpret_cast<const float2*>(par ? sin + (size_t)rhs * n : vin);
   const int site = blockIdx.x * (HPT / 8) + (threadIdx.x >> 3), hop = threadIdx.x & 7;
@@ -601,23 +615,26 @@ dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   if (active) ls = stencil_site(g, par ? 0 : -1, site, c);
   zf acc[3];
   hop_lanes<0, StC64, LL>(g, active, ls, c, hop, vst, par != 0, links, acc);
-  float ar[NH], ai[NH], ss = 0.f;
+  float ar[NH], ai[NH], ss = 0.f, bb = 0.f;
 #pragma unroll
   for (int q = 0; q < NH; ++q) { ar[q] = 0.f; ai[q] = 0.f; }
   if (active) {
     const size_t e0 = (size_t)site * 12 + 3 * (hop >> 1);
     const int odd = hop & 1;
-    const float mk = par ? (float)g.kappa : (float)(-g.kappa);
+    const float mk = par ? g.kf : -g.kf;
     zf p[3], x0[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       x0[k] = vin[e0 + k];
-      p[k] = {sc * fmaf(mk, acc[k].re, x0[k].re), sc * fmaf(mk, acc[k].im, x0[k].im)};
+      p[k] = {fmaf(mk, acc[k].re, x0[k].re), fmaf(mk, acc[k].im, x0[k].im)};
       ss = fmaf(p[k].re, p[k].re, ss);
       ss = fmaf(p[k].im, p[k].im, ss);
-      x0[k] = sc * x0[k];
+      if (FIRST) {
+        bb = fmaf(x0[k].re, x0[k].re, bb);
+        bb = fmaf(x0[k].im, x0[k].im, bb);
+      }
     }
-    if (odd) ss = 0.f;   // the pair holds the same values
+    if (odd) ss = bb = 0.f;   // the pair holds the same values
     if (!odd) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
@@ -657,7 +674,11 @@ dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
     }
   }
   ss = warp_sum_r(ss);
-  if (lane == 0) sh[wid][2 * NVM] = ss;
+  if (FIRST) bb = warp_sum_r(bb);
+  if (lane == 0) {
+    sh[wid][2 * NVM] = ss;
+    sh[wid][2 * NVM + 1] = bb;
+  }
   __syncthreads();
   const int nblk = gridDim.x;
   if ((int)threadIdx.x < 2 * nv + 2) {
@@ -665,8 +686,8 @@ dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
     float v = 0.f;
     if (t < 2 * nv) {
       for (int i = 0; i < NWP; ++i) v += sh[i][t];
-    } else if (t == 2 * nv) {
-      for (int i = 0; i < NWP; ++i) v += sh[i][2 * NVM];
+    } else {
+      for (int i = 0; i < NWP; ++i) v += sh[i][2 * NVM + t - 2 * nv];
     }
     partials_as<float>(partial)[(((size_t)rhs * maxvec + (t >> 1)) * nblk + blockIdx.x) * 2 + (t & 1)] = v;
     __threadfence();
@@ -675,7 +696,8 @@ dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   __shared__ zd g_h2[NVM + 1];
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0);
   __syncthreads();
-  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true);
+  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true,
+                beta ? beta + rhs : nullptr, FIRST, gridDim.y);
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
@@ -687,7 +709,7 @@ constexpr int kProjShapes = 4;
 template <int NVM, bool FIRST, int LL>
 void launch_proj_v(int v, int nv, int nrhs, cudaStream_t st, zf* w, zf* V, size_t fs, size_t n,
                    const float2* L32, const stencil::KGeom& kg, zd* small, SmallLayout L,
-                   double* dnorm, ReduceWork& rw, const zf* b0, const double* beta0,
+                   double* dnorm, ReduceWork& rw, const zf* b0, double* beta0,
                    const zf* sin, int par, cudaError_t* err) {
   // one site per thread; launch_proj checked that the partial slots hold every CTA
   const dim3 grid(stencil::stencil_ctas(kg.tile, par ? kg.V / 2 : kg.V, 128), nrhs);
@@ -708,7 +730,7 @@ void launch_proj_v(int v, int nv, int nrhs, cudaStream_t st, zf* w, zf* V, size_
 template <int LL>
 int launch_proj(int nv, bool first, int nrhs, cudaStream_t st, zf* w, zf* V, size_t fs,
                 size_t n, const float2* L32, stencil::KGeom kg, zd* small, SmallLayout L,
-                double* dnorm, ReduceWork& rw, const zf* b0, const double* beta0, const zf* sin,
+                double* dnorm, ReduceWork& rw, const zf* b0, double* beta0, const zf* sin,
                 int par) {
   const int nvm = first ? 0 : nv <= 4 ? 4 : nv <= 8 ? 8 : 16;
   // one site per thread: the grid must fit the partial slots of the reduction workspace, which
@@ -741,7 +763,7 @@ int launch_proj(int nv, bool first, int nrhs, cudaStream_t st, zf* w, zf* V, siz
 int dslash_proj_launch(zf* w, zf* V, size_t fs, size_t n, int nrhs, zd* small,
                        SmallLayout L, int j, double* dnorm, ReduceWork& rw,
                        const FusedStencil& fz, cudaStream_t st, const zf* b0 = nullptr,
-                       const double* beta0 = nullptr) {
+                       double* beta0 = nullptr) {
   stencil::KGeom kg = stencil::to_kgeom(fz.g);
   int nv = j + 1;
   const float2* L32 = static_cast<const float2*>(fz.links);
@@ -850,8 +872,9 @@ __global__ void solve_kernel(zd* small, SmallLayout L, int steps, int nrhs) {
 // other here, so the chain per step is one reciprocal square root and four multiply-adds; a fixed
 // run pays for it once instead of once per normalising update, which waited for its extra CTA
 // (9.7 -> LS_UPD us per update on 4096 sites, 14.1 -> LS_UPD2 us on the 65 536-site Schur system).
+// raw0: basis column 0 has norm beta, so its coefficient is divided by it.
 __global__ void __launch_bounds__(128) fixed_ls_kernel(zd* small, SmallLayout L, int steps,
-                                                       const double* beta) {
+                                                       const double* beta, int raw0) {
   dep_entry();
   extern __shared__ zd lsh[];          // [steps][steps + 1] H by columns
   __shared__ zd gs[GV_MAX];
@@ -884,7 +907,9 @@ __global__ void __launch_bounds__(128) fixed_ls_kernel(zd* small, SmallLayout L,
   for (int i = steps - 1; i >= 0; --i) {
     const zd y = inv[i] * gs[i];
     if (k < i) gs[k] = gs[k] - lsh[i * ld + k] * y;
-    if (k == i) sm[L.y() + i] = y;
+    if (k == i) {
+      sm[L.y() + i] = raw0 && i == 0 ? beta[gridDim.x + blockIdx.x] * y : y;
+    }
     __syncthreads();
   }
 }
@@ -936,7 +961,7 @@ void GmresV<E>::release() {
 template <typename E>
 int GmresV<E>::arnoldi_step(const OpV<E>& A, const OpV<E>* M, int j, cudaStream_t st,
                             bool single_pass, const FusedStencil* fused, const E* b0,
-                            bool next, bool givens) {
+                            bool next, bool givens, bool raw0) {
   SmallLayout L{m};
   size_t fs = n * nrhs;
   E* vj = V + (size_t)j * fs;
@@ -948,7 +973,7 @@ int GmresV<E>::arnoldi_step(const OpV<E>& A, const OpV<E>* M, int j, cudaStream_
     // the stencil and the single-pass projections in one kernel
     if constexpr (std::is_same<E, zf>::value)
       WMG_TRY(dslash_proj_launch(w, V, fs, n, nrhs, small, L, j, dnorm, rw, *fused, st, b0,
-                                 b0 ? dnorm + nrhs : nullptr));
+                                 raw0 ? dnorm + nrhs : nullptr));
   } else if (M) {
     E* zj = Z + (size_t)j * fs;
     WMG_TRY((*M)(zj, vj, st));
@@ -994,12 +1019,15 @@ int GmresV<E>::fixed(const OpV<E>& A, E* x, const E* b, int steps, cudaStream_t 
   if (!accumulate) WMG_TRY(fill_zero_v<E>(x, fs, st));
   if (steps == 0) return MG_OK;
   if (steps > 112) return fail(MG_EINVAL, "gmres: at most 112 fixed steps");   // fixed_ls_kernel
-  WMG_TRY(norm2_v<E>(dnorm + nrhs, 1, b, n, nrhs, rw, st, ip_scale()));
-  // the fused first step scales b itself and writes v_0 (see dslash_proj_kernel)
-  bool fuse0 = false;
+  // a run whose every step is fused keeps b itself as basis column 0 (dslash_proj_kernel)
+  bool raw0 = false;
   if constexpr (std::is_same<E, zf>::value)
-    fuse0 = fused && n == (size_t)(fused->schur ? fused->g.V / 2 : fused->g.V) * 12;
-  if (!fuse0) WMG_TRY(scale_inv_v<E>(V, b, dnorm + nrhs, 1, n, nrhs, st));
+    raw0 = fused && steps <= ST_NV &&
+           n == (size_t)(fused->schur ? fused->g.V / 2 : fused->g.V) * 12;
+  if (!raw0) {
+    WMG_TRY(norm2_v<E>(dnorm + nrhs, 1, b, n, nrhs, rw, st, ip_scale()));
+    WMG_TRY(scale_inv_v<E>(V, b, dnorm + nrhs, 1, n, nrhs, st));
+  }
   // A fixed number of steps from zero (the smoothers): complex-float bases of up to 16
   // columns orthogonalise with a single classical Gram-Schmidt pass, H[j+1, j] from
   // Pythagoras.  Over these few steps the basis stays orthogonal to ~eps_32 times the
@@ -1007,12 +1035,12 @@ int GmresV<E>::fixed(const OpV<E>& A, E* x, const E* b, int steps, cudaStream_t 
   // minimisation unchanged to FP32 rounding; the tolerance-driven solves keep CGS2.
   // the last step needs its Hessenberg column, not the next basis column
   for (int j = 0; j < steps; ++j)
-    WMG_TRY(arnoldi_step(A, nullptr, j, st, true, fused, fuse0 && j == 0 ? b : nullptr,
-                         j + 1 < steps, false));
+    WMG_TRY(arnoldi_step(A, nullptr, j, st, true, fused, raw0 && j == 0 ? b : nullptr,
+                         j + 1 < steps, false, raw0));
   const size_t lsb = sizeof(zd) * (size_t)steps * (steps + 1);
   WMG_TRY(smem_attr(fixed_ls_kernel, lsb));
   const int lst = (steps + 1 + 31) / 32 * 32;
-  WMG_LAUNCH_DEP(fixed_ls_kernel, nrhs, lst, lsb, st, small, L, steps, dnorm + nrhs);
+  WMG_LAUNCH_DEP(fixed_ls_kernel, nrhs, lst, lsb, st, small, L, steps, dnorm + nrhs, raw0 ? 1 : 0);
   WMG_TRY(multi_axpy_v<E>(x, V, fs, steps, small + L.y(), L.stride(), xsign, n, nrhs, st));
   return MG_OK;
 }

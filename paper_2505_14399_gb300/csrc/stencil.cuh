@@ -292,6 +292,7 @@ struct KGeom {
   double wd[4];
   int bc[4];
   double kappa;
+  float kf;      // kappa in FP32: one FP64 conversion per thread would cost each warp 16 cycles
   // single-parity form only: when set, out_p = sub_p - (-kappa H_{p,1-p} in) (the even-odd
   // Schur complement and its source / reconstruction steps), sub with out's layout and stride
   const void* sub = nullptr;
@@ -303,6 +304,9 @@ template <typename S>
 __device__ __forceinline__ void apply_sub(const KGeom& g, size_t rhs_off, int i,
                                           cplx<typename S::real> res[12]);
 
+template <typename R> __device__ __forceinline__ R kap(const KGeom& g);
+template <> __device__ __forceinline__ double kap<double>(const KGeom& g) { return g.kappa; }
+template <> __device__ __forceinline__ float kap<float>(const KGeom& g) { return g.kf; }
 template <typename R> __device__ __forceinline__ R wgt(const KGeom& g, int mu);
 template <> __device__ __forceinline__ double wgt<double>(const KGeom& g, int mu) { return g.wd[mu]; }
 template <> __device__ __forceinline__ float wgt<float>(const KGeom& g, int mu) { return g.wf[mu]; }
@@ -548,6 +552,7 @@ inline KGeom to_kgeom(const Geom& g) {
   k.stride[3] = g.L[0] * g.L[1] * g.L[2];
   k.V = g.V;
   k.kappa = g.kappa;
+  k.kf = (float)g.kappa;
   return k;
 }
 
