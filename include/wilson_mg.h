@@ -101,7 +101,7 @@ typedef struct mg_params {
                                 only in the mixed forms (SVD: setup_dtype MG_C64;
                                 Galerkin: solve_dtype other than MG_C128).  A double-float
                                 Galerkin with k <= 24 runs its contraction on the tensor
-                                pipe as exact bf16 digit products (same accuracy) when
+                                pipe as exact fp16 digit products (same accuracy) when
                                 every entry is in range (orthonormal P, unitary links),
                                 else on the FP32 units                                   */
   int link_compress;         /* link copies of the FP32 / half stencils: 1 keep the first
@@ -144,7 +144,7 @@ const char* mg_last_error(void);
 long long mg_kernel_launches(void);
 
 /* JSON list of the launch shapes the autotuner has chosen so far, one object per problem key
- * ("kernel": "dslash" | "dslash_proj" | "galerkin_tc", the key fields, "variant", "ms");
+ * ("kernel": "dslash" | "dslash_proj", the key fields, "variant", "ms");
  * library-owned string, valid until the next call. */
 const char* mg_autotune_report(void);
 

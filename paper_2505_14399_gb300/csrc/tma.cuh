@@ -1,4 +1,5 @@
-// Bulk asynchronous copies (the TMA engine's untiled form) and mbarrier waits, as inline PTX.
+// Asynchronous copies (the TMA engine's untiled bulk form, per-thread 16-byte ones) and mbarrier
+// waits, as inline PTX.
 //
 // A bulk copy moves `bytes` (a multiple of 16) from a 16-byte aligned global address into
 // a 16-byte aligned shared-memory buffer and reports completion as transaction bytes on an
@@ -42,6 +43,17 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
           "r"(smem_addr(dst)),
       "l"(src), "r"(bytes), "r"(smem_addr(bar))
       : "memory");
+}
+
+// 16-byte asynchronous copies by this thread, in groups
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {

@@ -95,26 +95,35 @@ def test_tile_reciprocals_of_the_stencil_are_exact():
 
 
 def test_digit_split_by_magic_sums():
-    """The kernel's digit split: v plus 1.5 2^k (and 128 units) in units of 2^-14, 2^-30, 2^-46 and
-    2^-54, the remainders renormalised by fast two-sums, digits from the bytes of the sums' words.
-    Every remainder is exact as rationals, every digit has |d| <= 128, and the value minus its
-    expansion sum_i d_i 2^(-6-8i) is at most 2^-55 (half of the last unit)."""
+    """The kernel's digit split: v plus 1.546875 2^k (and 128 units) in units of 2^-14, 2^-30, 2^-46
+    and 2^-54, the remainders renormalised by fast two-sums, digits as fp16 numbers s 2^-8 from the
+    bytes of the sums' words.  Every remainder is exact as rationals, every digit has |s| <= 128,
+    and the value minus its expansion sum_i s_i 2^(-6-8i) is at most 2^-55 (half of the last
+    unit)."""
     def word(x):
         return int(np.array(x, dtype=F).view(np.uint32))
 
-    magic = [F(float.fromhex("0x1.8p9") + float.fromhex("0x1p-7")),
-             F(float.fromhex("0x1.8p-7") + float.fromhex("0x1p-23")),
-             F(float.fromhex("0x1.8p-23") + float.fromhex("0x1p-39")),
-             F(float.fromhex("0x1.8p-31") + float.fromhex("0x1p-40"))]
+    def half(bits, scale, off):
+        """scale * (fp16 of these bits) + off, exact in fp16; returns 2^8 times it."""
+        y = Fraction(float(np.array(bits, dtype=np.uint16).view(np.float16))) * scale + off
+        assert Fraction(float(np.float16(float(y)))) == y
+        assert (y * 256).denominator == 1
+        return int(y * 256)
+
+    magic = [F(float.fromhex("0x1.8cp9") + float.fromhex("0x1p-7")),
+             F(float.fromhex("0x1.8cp-7") + float.fromhex("0x1p-23")),
+             F(float.fromhex("0x1.8cp-23") + float.fromhex("0x1p-39")),
+             F(float.fromhex("0x1.8p-31") + float.fromhex("0x1.18p-40"))]
     units = [Fraction(1, 2 ** e) for e in (14, 30, 46, 54)]
-    for m, u, off in zip(magic, units, (128, 128, 128, 2 ** 14)):
-        # exact constants: 1.5 2^23 units and the offset, in a word whose bit 23 is clear
-        assert Fraction(float(m)) == u * (3 * 2 ** 22 + off) and not word(m) >> 23 & 1
+    for m, u, man in zip(magic, units, (0xc60080, 0xc60080, 0xc60080, 0xc04600)):
+        # exact constants, in a word whose bit 23 is clear
+        assert Fraction(float(m)) == u * man and not word(m) >> 23 & 1
     rng = np.random.default_rng(3)
     xs = _values() + [s * (2 - 2.0 ** -23) for s in (1, -1)]
     # remainders at their largest: halves of the first two units, on both sides
     xs += [float(n) * 2.0 ** -14 + s * 2.0 ** -15 + t * 2.0 ** -31
            for n in rng.integers(-20000, 20000, 200) for s in (1, -1) for t in (1, 0, -1)]
+    half_off = Fraction(-9, 2)
     for x in xs:
         hi = F(x)
         lo = F(x - float(hi))
@@ -127,14 +136,15 @@ def test_digit_split_by_magic_sums():
             n = Fraction(float(F(a - m)))
             w = word(a)
             if i < 3:
-                ds += [((w >> 8) & 0xFFFF) - 2 ** 14, (w & 0xFF) - 128]
+                ds += [half((w >> 8) & 0xFFFF, 1, -6),
+                       half((w >> 16) & 0xFF00 | w & 0xFF, 4 ** i, half_off)]
                 assert 256 * ds[-2] + ds[-1] == n / u
                 r = F(h - F(a - m))
                 h = F(r + l)
                 l = F(l - F(h - r))
                 assert Fraction(float(h)) + Fraction(float(l)) == before - n, (x, i)
             else:
-                ds.append((w & 0xFFFF) - 2 ** 14)
+                ds.append(half(w & 0xFFFF, 1, -6))
                 assert ds[-1] == n / u
         assert all(abs(d) <= 128 for d in ds), (x, ds)
         v = Fraction(float(hi)) + Fraction(float(lo))
@@ -142,3 +152,46 @@ def test_digit_split_by_magic_sums():
         assert abs(v - expansion) <= Fraction(1, 2 ** 55), x
     # three batches of 48 stacked rows, 7 digit pairs each, stay exact in FP32
     assert 3 * 7 * 48 * 128 ** 2 < 2 ** 24
+
+
+def test_integer_conversions_between_float_formats():
+    """The conversions that stay off the FP64 pipe, as integer operations on the words: double to
+    FP32 (nearest even), double to a double-float pair, a normalised pair to double (nearest), FP32
+    to double -- bit for bit what the conversions give, within the exponents they claim."""
+    rng = np.random.default_rng(0)
+    f2u = lambda x: int(np.array(x, dtype=F).view(np.uint32))
+    u2f = lambda u: float(np.array(u, dtype=np.uint32).view(F))
+    d2u = lambda x: int(np.array(x, dtype=np.float64).view(np.uint64))
+    u2d = lambda u: float(np.array(u, dtype=np.uint64).view(np.float64))
+    n = 4000
+    x = ((rng.integers(0, 2, n).astype(np.uint64) << np.uint64(63)) |
+         (rng.integers(1023 - 125, 1023 + 126, n).astype(np.uint64) << np.uint64(52)) |
+         rng.integers(0, 1 << 52, n, dtype=np.uint64)).view(np.float64)
+    for x in list(x) + [1.5 + 2.0 ** -24, 1.5 + 3 * 2.0 ** -24, 2 - 2.0 ** -25, 2 - 2.0 ** -53]:
+        x = float(x)
+        q = d2u(x)
+        h, l = q >> 32, q & 0xFFFFFFFF
+        ex, sign = (h >> 20) & 0x7FF, h & 0x80000000
+        f0, t = ((ex - 896) << 23) | ((h & 0xFFFFF) << 3) | (l >> 29), l & 0x1FFFFFFF
+        f = f0 + (1 if t > 1 << 28 or (t == 1 << 28 and f0 & 1) else 0)
+        assert u2f(sign | f) == float(F(x)), x
+        if 949 <= ex < 949 + 201:
+            up = t >> 28
+            hi = u2f(sign | (f0 + up))
+            lo = float(F(t - (up << 29)) * F(u2f(sign | ((ex - 948) << 23))))
+            H = float(F(x))
+            assert (hi, lo) == (H, float(F(x - H))) or (t == 1 << 28 and hi + lo == x), x
+        hi = float(F(x))
+        ulp = float(np.spacing(F(abs(hi)))) / 2
+        for lo in (float(F(x - hi)), 0.0, float(F(0.3 * (x - hi))), ulp, -ulp):
+            u = f2u(hi)
+            a = u & 0x7FFFFFFF
+            e = a >> 23
+            if 80 <= e < 230:
+                p = float(F(lo) * F(u2f(((306 - e) << 23) | (u & 0x80000000))))
+                s = (((a & 0x7FFFFF) | 0x800000) << 29) + int(np.rint(p))
+                if 1 << 52 <= s < 1 << 53:
+                    w = (((u & 0x80000000) | ((e + 896) << 20) | ((s >> 32) & 0xFFFFF)) << 32)
+                    assert u2d(w | (s & 0xFFFFFFFF)) == hi + lo, (hi, lo)
+            w = (((u & 0x80000000) | ((a >> 3) + 0x38000000)) << 32) | ((u << 29) & 0xFFFFFFFF)
+            assert u2d(w) == hi
