@@ -126,8 +126,7 @@ def load_peaks():
 # over the launches of one warm-up and one timed step) from one ncu capture of this bench
 # command on its workload, reported as roofline.traffic for that kernel; an entry is removed
 # whenever its kernel changes, until it is captured again.
-NCU_TRAFFIC = {("galerkin_tc", "c2_16^3x32_near_critical"): 1.9608e9,
-               ("dslash_proj", "c2_16^3x32_near_critical"): 516.9e6}
+NCU_TRAFFIC = {}
 
 
 def kernel_bound(name, alu, peaks, peak_kind):
@@ -141,7 +140,7 @@ def kernel_bound(name, alu, peaks, peak_kind):
         # instructions (1 mul, 3 fma, 8 add/sub), so the peak is the FP32 FMA rate / 12
         return "alu", alu["fp32"] / 12.0, "TFLOP/s", "measured FP32 FMA rate / 12"
     if name.endswith("_tc"):
-        # the method's FP64-equivalent flops; the exact bf16 digit-plane products it issues on
+        # the method's FP64-equivalent flops; the exact fp16 digit-plane products it issues on
         # the tensor pipe are reported beside them.  Its time is set by the double-float staging
         # (colour transport, digit split) on the FP32 units, so that is the peak it is set against
         return "alu", alu["fp32"] / 12.0, "TFLOP/s", "measured FP32 FMA rate / 12 (staging)"

@@ -237,27 +237,30 @@ gram_df_kernel(zd* G, float* cn, int cld, const zdf* __restrict__ tiles, int cma
       Gt[i * c + j] = i == j ? zd{l, 0.0} : zd{0.0, 0.0};
       if (i == j && cn) cn[(size_t)t * cld + i] = (float)l;
     }
+  // sums over the eight lanes of a block, scattered: lane g ends with value g (entry g >> 1, real
+  // part or, g odd, imaginary part) after 4 + 2 + 1 additions
+  df x[8];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    df v[2];
+  for (int v = 0; v < 8; ++v) {
+    const f32x2 h = th[v >> 2][v & 1], l = tl[v >> 2][v & 1];
+    x[v] = (v & 2) ? df_two_sum(f2_hi(h), f2_hi(l)) : df_two_sum(f2_lo(h), f2_lo(l));
+  }
 #pragma unroll
-    for (int z = 0; z < 2; ++z) {
-      const f32x2 h = th[q >> 1][z], l = tl[q >> 1][z];
-      df x = (q & 1) ? df_two_sum(f2_hi(h), f2_hi(l)) : df_two_sum(f2_lo(h), f2_lo(l));
+  for (int o = GDF_G / 2; o > 0; o >>= 1) {
+    const bool up = (g & o) != 0;
 #pragma unroll
-      for (int o = 1; o < GDF_G; o <<= 1) {
-        const df y = {__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
-        x = (g & o) ? df_add(y, x) : df_add(x, y);   // one order in every lane
-      }
-      v[z] = x;
+    for (int v = 0; v < o; ++v) {
+      const df send = up ? x[v] : x[v + o], keep = up ? x[v + o] : x[v];
+      const df y = {__shfl_xor_sync(0xffffffffu, send.hi, o), __shfl_xor_sync(0xffffffffu, send.lo, o)};
+      x[v] = df_add(keep, y);
     }
-    const int i = 2 * I + (q >> 1), j = 2 * J + (q & 1);
-    if (work && g == 0 && i <= j && j < c && j >= kd) {
-      const zd w = {df_val(v[0]), i == j ? 0.0 : df_val(v[1])};
-      Gt[i * c + j] = w;
-      if (i != j) Gt[j * c + i] = conj(w);
-      else if (cn) cn[(size_t)t * cld + i] = df_to_float(v[0]);
-    }
+  }
+  const int i = 2 * I + (g >> 2), j = 2 * J + ((g >> 1) & 1), im = g & 1;
+  if (work && i <= j && j < c && j >= kd) {
+    const double w = im && i == j ? 0.0 : df_val_bits(x[0]);
+    reinterpret_cast<double*>(Gt + i * c + j)[im] = w;
+    if (i != j) reinterpret_cast<double*>(Gt + j * c + i)[im] = im ? -w : w;
+    else if (cn && !im) cn[(size_t)t * cld + i] = df_to_float(x[0]);
   }
 }
 
