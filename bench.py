@@ -137,12 +137,14 @@ def kernel_bound(name, alu, peaks, peak_kind):
         return "latency", None, "TFLOP/s", "none"
     if name.endswith("_df64"):
         # double-float: one real multiply-add (2 FP64-equivalent flops) costs 12 FP32
-        # instructions (1 mul, 3 fma, 8 add/sub), so the peak is the FP32 FMA rate / 12
+        # instructions in its plain form (1 mul, 3 fma, 8 add/sub), so the peak is the FP32 FMA
+        # rate / 12; the biased sums of the SVD take 6, so they may exceed it
         return "alu", alu["fp32"] / 12.0, "TFLOP/s", "measured FP32 FMA rate / 12"
     if name.endswith("_tc"):
         # the method's FP64-equivalent flops; the exact fp16 digit-plane products it issues on
         # the tensor pipe are reported beside them.  Its time is set by the double-float staging
-        # (colour transport, digit split) on the FP32 units, so that is the peak it is set against
+        # (colour transport, digit split) on the FP32 units, so that is the peak it is set against;
+        # the products themselves are on the tensor cores, so it may exceed it
         return "alu", alu["fp32"] / 12.0, "TFLOP/s", "measured FP32 FMA rate / 12 (staging)"
     if name.endswith("_fp64") or name.startswith("galerkin") or name == "dslash_c128":
         # the FP64 stencil runs at the FP64 FMA rate (1/74 of FP32 on this part), not at HBM

@@ -9,8 +9,8 @@
 // fixed-point digits in base 256,
 //     v = sum_{i < NS} s_i 2^{-6-8i},  s_i integers, |s_i| <= 128,  NS = 7
 // (error at most 2^-55),
-// each digit exact in fp16 (kept as s_i 2^-8).  A product of digit planes is an integer matrix product:
-// fp16 x fp16 tensor-core MMAs with FP32 accumulation are exact while the partial sums stay
+// each digit exact in fp16 (kept as s_i 2^-8).  A product of digit planes is an integer matrix
+// product: fp16 x fp16 tensor-core MMAs with FP32 accumulation are exact while the partial sums stay
 // below 2^24, which holds for three staging batches (7 digit pairs x 3 x 48 stacked rows x
 // 128^2 = 0.984 2^24).  Digit pairs i + j = d of the same weight 2^{-12-8d} share FP32
 // accumulator columns; pairs with i + j >= NS (weight below 2^-68) are dropped.  After every
@@ -36,13 +36,14 @@
 // split, on two columns at once in packed FP32 instructions) and every third batch's fold are on
 // the critical path.  With warp-level mma.sync (bf16 digits) the products, their ldmatrix reads
 // and the accumulators lived in the staging warps, which met at two barriers per batch: 2.57 ms
-// at 16^3x32, k = 12 (blocks of 4^4) and 18.6 ms at 16^3x64, k = 24 (2x2x2x4); here 1.55 and
-// 10.1 ms.  Bound now by the staging warps' FP32 and issue slots (k = 12: about 5000 cycles a
-// batch, two CTAs per SM), for small blocks also by a CTA's start and its two outputs (k = 24,
-// 32 sites: 85 000 cycles, of them 10 000 before the first batch, 13 000 in four folds, 9000 in
-// the outputs).  Tried and slower: Ch and Pt staged by different warps (2.27 ms, k = 12), a
-// persistent grid whose feeder warp copies and issues everything (2.5 ms: the feeder is a serial
-// chain; 3.4 ms with 96-byte bulk copies).
+// at 16^3x32, k = 12 (blocks of 4^4) and 18.6 ms at 16^3x64, k = 24 (2x2x2x4); here 1.42 and
+// 9.25 ms.  Bound now by the staging warps' FP32 and issue slots (k = 12: about 4700 cycles a
+// batch, two CTAs per SM), for small blocks also by a CTA's start, four folds and two outputs (k =
+// 24, 32 sites: together a third of its 78 000 cycles).  P(x) is loaded between the transport and
+// the digits: before the transport its eight registers made the loop spill (1.54 against 1.48 ms,
+// 9.5 against 9.3 ms with the rest as it is).  Tried and slower: Ch and Pt staged by different
+// warps (2.27 ms, k = 12), a persistent grid whose feeder warp copies and issues everything (2.5
+// ms: the feeder is a serial chain; 3.4 ms with 96-byte bulk copies).
 
 #include "bits.cuh"
 #include "common.cuh"
@@ -115,6 +116,11 @@ __device__ __forceinline__ zdf2 zdf2_pair(const zdf& a, const zdf& b) {
   return {{f2_pack(a.re.hi, b.re.hi), f2_pack(a.re.lo, b.re.lo)},
           {f2_pack(a.im.hi, b.im.hi), f2_pack(a.im.lo, b.im.lo)}};
 }
+// a / b for 0 <= a < 2^20, b > 0: the quotient of the floats is within 2^-22 a / b of
+// (a + 1/2) / b, which is at least 1 / (2 b) away from an integer
+__device__ __forceinline__ int small_div(int a, int b) {
+  return (int)__fdividef((float)a + 0.5f, (float)b);
+}
 __device__ __forceinline__ df2 df2_xor(df2 a, f32x2 m) { return {a.hi ^ m, a.lo ^ m}; }
 __device__ __forceinline__ f32x2 sign_mask(bool neg) { return neg ? 0x8000000080000000ull : 0ull; }
 
@@ -144,22 +150,38 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
 
   // ---- per-site tables, hops inside the aggregate first (pass 0), then the crossing ones: a
   // hop crosses when its local coordinate mu is the last one
-  int lstride = 1;
-  for (int m = 0; m < mu; ++m) lstride *= B.b[m];
-  const int bm = B.b[mu];
-  const int n0 = nd / bm * (bm - 1), n1 = nd - n0;
+  const int b0 = B.b[0], b1 = B.b[1], b2 = B.b[2];
+  const int lstride = mu == 0 ? 1 : mu == 1 ? b0 : mu == 2 ? b0 * b1 : b0 * b1 * b2;
+  const int bm = mu == 0 ? b0 : mu == 1 ? b1 : mu == 2 ? b2 : B.b[3];
+  const int n1 = small_div(nd, bm), n0 = nd - n1;
+  int jc[4];
+  jc[0] = j % B.C[0];
+  int jr = j / B.C[0];
+  jc[1] = jr % B.C[1]; jr /= B.C[1];
+  jc[2] = jr % B.C[2]; jc[3] = jr / B.C[2];
   const int bstride = mu == 0 ? 1 : mu == 1 ? B.C[0] : mu == 2 ? B.C[0] * B.C[1]
                                                              : B.C[0] * B.C[1] * B.C[2];
-  const bool last = j / bstride % B.C[mu] == B.C[mu] - 1;   // crossing hops leave the lattice
-  const int jn = last ? j - (B.C[mu] - 1) * bstride : j + bstride;
+  const int Cm = mu == 0 ? B.C[0] : mu == 1 ? B.C[1] : mu == 2 ? B.C[2] : B.C[3];
+  const int jm = mu == 0 ? jc[0] : mu == 1 ? jc[1] : mu == 2 ? jc[2] : jc[3];
+  const int bcm = mu == 0 ? g.bc[0] : mu == 1 ? g.bc[1] : mu == 2 ? g.bc[2] : g.bc[3];
+  const bool last = jm == Cm - 1;   // crossing hops leave the lattice
+  const int jn = last ? j - (Cm - 1) * bstride : j + bstride;
   const int tj = 2 * j * k * M, tn = 2 * jn * k * M;
+  const int x0 = jc[0] * b0 +
+                 B.L[0] * (jc[1] * b1 + B.L[1] * (jc[2] * b2 + B.L[2] * jc[3] * B.b[3]));
   for (int l = tid; l < nd; l += NT) {
-    const int q = l / lstride, lo = l - q * lstride, hi = q / bm, cm = q - hi * bm;
+    const int r1 = small_div(l, b0), r2 = small_div(r1, b1), r3 = small_div(r2, b2);
+    const int c0 = l - r1 * b0, c1 = r1 - r2 * b1, c2 = r2 - r3 * b2;
+    const int cm = mu == 0 ? c0 : mu == 1 ? c1 : mu == 2 ? c2 : r3;
+    // hi: the coordinates above mu, lo: below (as a local index)
+    const int hi = mu == 0 ? r1 : mu == 1 ? r2 : mu == 2 ? r3 : 0;
+    const int lo = l - lstride * (cm + bm * hi);
     const bool cross = cm == bm - 1;
     const int e = cross ? n0 + lo + lstride * hi : lo + lstride * (cm + (bm - 1) * hi);
+    const int x = x0 + c0 + B.L[0] * (c1 + B.L[1] * (c2 + B.L[2] * r3));
     tx[e] = tj + l * 6;
     ty[e] = cross ? tn + (l - (bm - 1) * lstride) * 6 : tj + (l + lstride) * 6;
-    tu[e] = 2 * (B.site(j, l) * 9) + ((cross && last && g.bc[mu] < 0) ? 1 : 0);
+    tu[e] = 2 * (x * 9) + ((cross && last && bcm < 0) ? 1 : 0);
   }
   if (wid == C::WARPS - 1) tc5_alloc(&s_tmem, C::TCOLS);
   if (tid == 0) {
@@ -179,7 +201,7 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int p = tid + u * NT;
-    const int h = p / (6 * n2k), rem = p - h * 6 * n2k;
+    const int h = small_div(p, 6 * n2k), rem = p - h * 6 * n2k;
     const int col = rem / 6, part = rem - 6 * col;
     const int chi = col >= k, i = col - (chi ? k : 0);
     // pair q = chi KP / 2 + i / 2 keeps its columns in slots q and KP + q: the staging threads,
@@ -190,7 +212,11 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
     cpd[u] = (h * 6 + part) * NRP + q + ((i & 1) ? KP : 0);
   }
   // staging: a column pair sq (one chirality: padded to an even count) of one batch row
-  const int sg = wid / T4, pg = wid % T4, lrow = lane >> 2, sq = 4 * pg + (lane & 3);
+  // Warp w runs on scheduler w % 4, so both CTAs of an SM would give their ninth item to the same
+  // one (T4 = 3): the accumulator allocation tells them apart (1.48 -> 1.42 ms at k = 12).
+  const int cta = (int)((tmem & 0xffffu) / C::TCOLS);
+  const int item = T4 == 3 && wid >= 8 ? 8 + (((wid - 8) ^ cta) & 1) : wid;
+  const int sg = item / T4, pg = item % T4, lrow = lane >> 2, sq = 4 * pg + (lane & 3);
   const bool dn = sq >= KP / 2;
   const int si = 2 * (sq - (dn ? KP / 2 : 0)), scol = (dn ? k : 0) + si;
   const int scol1 = si + 1 < k ? M : 0;   // an odd k's last pair repeats its column
@@ -217,16 +243,13 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
   };
   unsigned char* const sA = tc_raw + 3 * PLANE * sg + 128 * pg + 4 * lane;
   unsigned char* const sB = tc_raw + C::A_BYTES + 2 * TC_NS * PLANE * sg + 128 * pg + 4 * lane;
-  const bool stager = wid < C::ITEMS && sq < KP;
+  const bool stager = item < C::ITEMS && sq < KP;
   const Row w = row_of(8 * sg + lrow);
   // fold: quarter of the lanes, column group
   const int fq = wid & 3, fg = wid >> 2;
   const int frow = C::M == 128 ? 32 * fq + lane : lane < 16 ? 16 * fq + lane : 2 * NR;
   const bool folder = fg < C::FG && (C::M == 128 ? 32 : 16) * fq < 2 * NR;
   const uint32_t ftm = tmem + ((uint32_t)(32 * fq) << 16) + (uint32_t)(fg * C::CPG);
-
-  // output: first element of this thread
-  const int ob = tid / n2k, oa = tid - ob * n2k;
 
   const int nb0 = (n0 + NB - 1) / NB, nbt = nb0 + (n1 + NB - 1) / NB;
   auto batch = [&](int t, int& e0, int& nb) {
@@ -305,13 +328,14 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
     __syncthreads();
     zd* out = pass == 1 ? Op + ((size_t)j * 9 + 1 + dir) * ne
                         : Xpart + ((size_t)mu * B.d + j) * ne;
-    int b = ob, a = oa;
+    const int db = small_div(NT, n2k), da = NT - db * n2k;
+    int b = small_div(tid, n2k), a = tid - b * n2k;
     for (int e = tid; e < ne; e += NT) {
       const int sb = b < k ? b : KP + b - k, sa = a < k ? a : KP + a - k;
       const df re = sOut[(size_t)sb * LO + sa], im = sOut[(size_t)(NR + sb) * LO + sa];
       out[e] = {coef * df_val_bits(re), coef * df_val_bits(im)};   // column-major
-      b += NT / n2k;
-      a += NT % n2k;
+      b += db;
+      a += da;
       if (a >= n2k) { a -= n2k; ++b; }
     }
   };
@@ -323,16 +347,6 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
     unsigned char* const A = sA + (size_t)buf * C::BUF;
     unsigned char* const Bp = sB + (size_t)buf * C::BUF;
     const bool act = stager && w.h < nb;
-    // P(x), used last: straight from global memory, swapped for odd powers of i
-    float2 pxv[4];
-    if (act) {
-      const float2* px = reinterpret_cast<const float2*>(Pdf + (size_t)tx[e0 + w.h] +
-                                                         (size_t)scol * M + w.spin + w.cc);
-      pxv[0] = __ldg(px + w.odd);
-      pxv[1] = __ldg(px + !w.odd);
-      pxv[2] = __ldg(px + 2 * scol1 + w.odd);
-      pxv[3] = __ldg(px + 2 * scol1 + !w.odd);
-    }
     if (t >= 2) wait_mma(t - 2);   // its products have read this digit buffer
     // Ch (spin-projected, transported P(x + mu)) and Pt (reconstruction-folded P(x)) in
     // double-float, written as digit planes: every digit of the two columns of a pair goes
@@ -354,6 +368,11 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
         dfacc2_fma(tim, ur, mr, v.im, c2 == 0);
         dfacc2_fma(tim, ui, mi.hi, v.re, false);
       }
+      // P(x), used last: straight from global memory, swapped for odd powers of i
+      const float2* px = reinterpret_cast<const float2*>(Pdf + (size_t)tx[e0 + w.h] +
+                                                         (size_t)scol * M + w.spin + w.cc);
+      const float2 pxv[4] = {__ldg(px + w.odd), __ldg(px + !w.odd), __ldg(px + 2 * scol1 + w.odd),
+                             __ldg(px + 2 * scol1 + !w.odd)};
       const df2 nre = df2_norm(tre), nim = df2_norm(tim);
       bad |= !(tc_in_range(nre) && tc_in_range(nim));
       unsigned dr[TC_NS], di[TC_NS];
@@ -399,7 +418,7 @@ galerkin_tc_kernel(zd* Op, zd* Xpart, const zdf* __restrict__ Pdf, int k,
       nacc = 0;
       __syncthreads();           // the accumulators (and the output's buffer) have been read
     }
-    if (tid == NT - 32) {
+    if (item == C::WARPS - 1 && lane == 0) {
       tc5_fence_after();
       constexpr uint32_t idesc = tc5_idesc_f16_mn(C::M, 0);
       const uint32_t a0 = smem_addr(tc_raw + (size_t)buf * C::BUF), b0 = a0 + C::A_BYTES;
