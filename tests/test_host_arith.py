@@ -195,3 +195,16 @@ def test_integer_conversions_between_float_formats():
                     assert u2d(w | (s & 0xFFFFFFFF)) == hi + lo, (hi, lo)
             w = (((u & 0x80000000) | ((a >> 3) + 0x38000000)) << 32) | ((u << 29) & 0xFFFFFFFF)
             assert u2d(w) == hi
+
+
+def test_small_quotients_by_float_division():
+    """The Galerkin kernel's quotients a / b (a < 2^20): the float division of a + 1/2 by b, in
+    error by up to 2 units in the last place, still truncates to floor(a / b)."""
+    rng = np.random.default_rng(4)
+    for b in list(range(1, 130)) + [144, 288, 768, 1000, 4096, 65536]:
+        a = np.concatenate([np.arange(4096), rng.integers(0, 1 << 20, 2000),
+                            b * rng.integers(0, (1 << 20) // b, 500), (1 << 20) - 1 - np.arange(64)])
+        q = ((a.astype(F) + F(0.5)) / F(b)).astype(F)
+        for step in (-2, 0, 2):
+            p = (q.view(np.int32) + step).view(F)
+            assert np.array_equal(p.astype(np.int64), a // b), (b, step)
