@@ -235,7 +235,7 @@ gram_df_kernel(zd* G, float* cn, int cld, const zdf* __restrict__ tiles, int cma
       const int i = e / kd, j = e % kd;
       const double l = lamp[(size_t)t * cprev + i];
       Gt[i * c + j] = i == j ? zd{l, 0.0} : zd{0.0, 0.0};
-      if (i == j && cn) cn[(size_t)t * cld + i] = (float)l;
+      if (i == j && cn) cn[(size_t)t * cld + i] = fmaxf((float)l, 0.0f);   // noise: either sign
     }
   // sums over the eight lanes of a block, scattered: lane g ends with value g (entry g >> 1, real
   // part or, g odd, imaginary part) after 4 + 2 + 1 additions
@@ -602,8 +602,12 @@ update_df_kernel(zdf* out, int cmax_out, const zdf* __restrict__ tiles, int cmax
     for (int q = threadIdx.x; q < c; q += 32) m = fmaxf(m, sqrtf(cn[(size_t)t * cld + q]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    // Any positive weights n_c bound the sums, but one far below its column's true norm makes R, and
+    // with it the bias of its whole group, too large.  A kept null direction's norm is eigenvalue
+    // noise, down to zero (the column itself stays below 1e-7 of the largest), so no weight is below
+    // 2^-24 of the largest; columns of that size are below what the Gram matrix resolves.
     for (int q = threadIdx.x; q < cpad; q += 32) {
-      const float n = q < c ? sqrtf(cn[(size_t)t * cld + q]) : 0.f;
+      const float n = q < c ? fmaxf(sqrtf(cn[(size_t)t * cld + q]), 0x1p-24f * m) : 0.f;
       sI[q] = n > 1e-20f ? 1.0f / n : 0.0f;   // below: n^2 has lost its digits
       sN[q] = m > 0.f ? n / m : 0.f;
     }

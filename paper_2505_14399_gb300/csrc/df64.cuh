@@ -139,10 +139,13 @@ __device__ __forceinline__ void bacc2_fma(bacc2& acc, df2 a, df2 b) {
   acc.s = s;
 }
 
-// C for partial sums within +-bound (bound >= 0): 3 times the power of two above it
+// C for partial sums within +-bound (bound >= 0): 3 times the power of two above it, at most 3 2^126
+// (the largest for which C + 2^126 is finite).  A bound that is not finite gives a sum that is not:
+// its exponent bits alone would wrap to -0, a sum without its error terms.
 __device__ __forceinline__ float bacc_bias(float bound) {
-  const unsigned u = (__float_as_uint(bound) & 0x7f800000u) + 0x00800000u;
-  return 3.0f * __uint_as_float(u);
+  const unsigned e = __float_as_uint(bound) & 0x7f800000u;
+  if (e == 0x7f800000u) return __uint_as_float(0x7fffffffu);
+  return 3.0f * __uint_as_float(min(e + 0x00800000u, 0x7e800000u));
 }
 
 // complex df64 value and accumulator
