@@ -365,21 +365,21 @@ __device__ __forceinline__ void hop_pair(const KGeom& g, int site, const int c[4
 // the spin projector's phases as operands, and the 12 sums are reduced and scattered over the
 // lanes: every pair of lanes ends with the three colours of one spin.
 
-// i sigma_mu d for mu < 3, d for mu = 3, as (f0 d[w], f1 d[1 - w]) with units f and w = 1 for mu < 2
+// The two components of i sigma_mu d for mu < 3, d for mu = 3, are d[w], d[1 - w] (w = 1 for mu <
+// 2) times one unit, i for even mu and 1 for odd, the second negated for mu = 1 and 2.  The unit is
+// applied by exchanging real and imaginary parts, not by multiplying with its zero part: half of
+// the multiply-adds, and an infinite component does not turn its neighbours into NaN.
 template <typename R>
 struct HopPhase {
-  bool swap;
-  R re0, im0, re1, im1;
+  bool swap, imag;
+  R sgn1;                       // sign of the second component
+  // the part of d that gives the real part (times -1 if imag) and the imaginary part
+  __device__ __forceinline__ R re(cplx<R> d) const { return imag ? d.im : d.re; }
+  __device__ __forceinline__ R im(cplx<R> d) const { return imag ? d.re : d.im; }
 };
 template <typename R>
 __device__ __forceinline__ HopPhase<R> hop_phase(int mu) {
-  HopPhase<R> p;
-  p.swap = mu < 2;
-  p.re0 = (mu & 1) ? R(1) : R(0);          // mu 1, 3: 1; mu 0, 2: i
-  p.im0 = (mu & 1) ? R(0) : R(1);
-  p.re1 = mu == 1 ? R(-1) : p.re0;         // mu 1: -1, mu 2: -i
-  p.im1 = mu == 2 ? R(-1) : p.im0;
-  return p;
+  return {mu < 2, (mu & 1) == 0, (mu == 1 || mu == 2) ? R(-1) : R(1)};
 }
 
 // The hop's term of H psi at `site`, reduced over the site's eight lanes: out = components 3 sp ..
@@ -414,13 +414,12 @@ __device__ __forceinline__ void hop_lanes(const KGeom& g, bool active, int site,
     load_link<S, LL>(links, g.V, mu, fwd ? site : nb, u);
     // h = psi_up - s i sigma psi_dn (mu < 3), psi_up + s psi_dn (mu = 3)
     const R sp = mu < 3 ? -s : s;
-    const R r0 = sp * f.re0, i0 = sp * f.im0, r1 = sp * f.re1, i1 = sp * f.im1;
+    const R i0 = sp, r0 = f.imag ? -sp : sp, i1 = f.sgn1 * i0, r1 = f.sgn1 * r0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const cplx<R> d0 = f.swap ? p[9 + k] : p[6 + k], d1 = f.swap ? p[6 + k] : p[9 + k];
-      h[k] = {fma(r0, d0.re, fma(-i0, d0.im, p[k].re)), fma(r0, d0.im, fma(i0, d0.re, p[k].im))};
-      h[3 + k] = {fma(r1, d1.re, fma(-i1, d1.im, p[3 + k].re)),
-                  fma(r1, d1.im, fma(i1, d1.re, p[3 + k].im))};
+      h[k] = {fma(r0, f.re(d0), p[k].re), fma(i0, f.im(d0), p[k].im)};
+      h[3 + k] = {fma(r1, f.re(d1), p[3 + k].re), fma(i1, f.im(d1), p[3 + k].im)};
     }
     // U h or U^dag h
     const R cj = fwd ? R(1) : R(-1);
@@ -440,15 +439,15 @@ __device__ __forceinline__ void hop_lanes(const KGeom& g, bool active, int site,
   }
   // upper pair cf g, lower pair cf s i sigma g (cf s g): lanes 0-3 keep the upper, 4-7 the lower
   const R cs = cf * s;
-  const R r0 = cs * f.re0, i0 = cs * f.im0, r1 = cs * f.re1, i1 = cs * f.im1;
+  const R i0 = cs, r0 = f.imag ? -cs : cs, i1 = f.sgn1 * i0, r1 = f.sgn1 * r0;
   const bool low = (hop & 4) != 0;
   cplx<R> keep[6];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const cplx<R> g0 = f.swap ? gg[3 + k] : gg[k], g1 = f.swap ? gg[k] : gg[3 + k];
     const cplx<R> up0 = cf * gg[k], up1 = cf * gg[3 + k];
-    const cplx<R> lo0 = {fma(r0, g0.re, -i0 * g0.im), fma(r0, g0.im, i0 * g0.re)};
-    const cplx<R> lo1 = {fma(r1, g1.re, -i1 * g1.im), fma(r1, g1.im, i1 * g1.re)};
+    const cplx<R> lo0 = {r0 * f.re(g0), i0 * f.im(g0)};
+    const cplx<R> lo1 = {r1 * f.re(g1), i1 * f.im(g1)};
     const cplx<R> s0 = low ? up0 : lo0, s1 = low ? up1 : lo1;
     keep[k] = low ? lo0 : up0;
     keep[3 + k] = low ? lo1 : up1;
