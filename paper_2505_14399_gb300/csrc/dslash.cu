@@ -1,11 +1,6 @@
 // Wilson-Dirac stencil (the operator D of Eq. 1), full and single-parity, any storage.
 //
-// One thread per output site and right-hand side.  Each of the 8 hops loads the
-// neighbour spinor, projects it to a 2-spin half spinor with (1 -/+ gamma_mu) in the
-// chiral basis, multiplies by U_mu(x) or U_mu(x-mu)^dag, and reconstructs the lower
-// spin pair from the upper one.  Spinor loads are 32-byte vector loads of the
-// [site][spin][colour] layout (16-byte where the fields are only so aligned); links are read
-// through the read-only path.
+// The kernels are in dslash_forms.cuh; here are the choice of launch shape, link layouts and tiles.
 #include <cstring>
 #include <type_traits>
 
@@ -20,124 +15,23 @@ namespace {
 
 using namespace stencil;
 
-// parity < 0: out = in - kappa H in (full lattice).  parity p >= 0: out_p = -kappa H in_{1-p}
-// on half-lattice (checkerboard-indexed) fields.
-template <typename S, int DAG, int TPB, int MINB, int LL>
-__global__ void __launch_bounds__(TPB, MINB)
-dslash_kernel(typename S::elem* __restrict__ out, const typename S::elem* __restrict__ in,
-              const typename S::elem* __restrict__ links, KGeom g, int parity, int nsites,
-              size_t in_stride, size_t out_stride) {
-  dep_entry();
-  typedef typename S::real R;
-  const size_t rhs = blockIdx.y;
-  int i, site, c[4];
-  if (!stencil_work(g, parity, nsites, threadIdx.x, TPB, i, site, c)) return;
-  cplx<R> acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
-  bool half_in = parity >= 0;
-  size_t in_off = rhs * in_stride;
-  hop_pair<0, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-  hop_pair<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-  hop_pair<2, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-  hop_pair<3, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-  R mk = -kap<R>(g);
-  cplx<R> res[12];
-  if (parity < 0) {
-    cplx<R> p[12];
-    SiteIO<S>::load(in + in_off, (size_t)site, p);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      res[k].re = fma(mk, acc[k].re, p[k].re);
-      res[k].im = fma(mk, acc[k].im, p[k].im);
-    }
-    SiteIO<S>::store(out + rhs * out_stride, (size_t)site, res);
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) res[k] = mk * acc[k];
-    apply_sub<S>(g, rhs * out_stride, i, res);
-    SiteIO<S>::store(out + rhs * out_stride, (size_t)i, res);
-  }
-}
+// Launch shapes (dslash_forms.cuh), searched by the autotuner per (dtype, link form, alignment,
+// parity, dagger, volume, nrhs): 0 and 1 one site per thread, 128 threads, registers uncapped and
+// capped at 128; 2 one thread per site and hop.  FP32 arithmetic: 3 one site per thread at 80
+// registers, 4 and 5 take 2 and 4 right-hand sides per thread, candidates when nrhs > 1; 6, 7 and 8
+// (4-byte types) are 3, 4 and 5 on consecutive sites, ABI links read element by element: with the
+// links shared by several right-hand sides, the windows' selects and the tiles can cost more than
+// they save (bf16, 12 right-hand sides at 16^3x32: 103 -> 98 us).  FP64: 3 two threads per site, 4
+// as 0 with consecutive sites (12x10x14x18: 72 us instead of 77, the tile's part-filled warps cost
+// FP64 issue); 2 and 4 right-hand sides per thread spill kilobytes (78 and 139 us against 22 at 8^4,
+// 2 right-hand sides).
+constexpr int kNumForms = 6, kNumSingle = 4, kNumF64 = 5, kNumHalf = 9;
 
-// One thread per site and hop (hop_lanes), consecutive sites; lane pairs write one spin each.
-template <typename S, int DAG, int LL>
-__global__ void __launch_bounds__(128)
-dslash_hop_kernel(typename S::elem* __restrict__ out, const typename S::elem* __restrict__ in,
-                  const typename S::elem* __restrict__ links, KGeom g, int parity, int nsites,
-                  size_t in_stride, size_t out_stride) {
-  dep_entry();
-  typedef typename S::real R;
-  const int i = blockIdx.x * (blockDim.x >> 3) + (threadIdx.x >> 3), hop = threadIdx.x & 7;
-  const bool active = i < nsites;
-  int c[4] = {0, 0, 0, 0}, site = 0;
-  if (active) site = stencil_site(g, parity, i, c);
-  const size_t rhs = blockIdx.y;
-  const typename S::elem* inr = in + rhs * in_stride;
-  cplx<R> acc[3];
-  hop_lanes<DAG, S, LL>(g, active, site, c, hop, inr, parity >= 0, links, acc);
-  if (!active || (hop & 1)) return;
-  const R mk = -kap<R>(g);
-  const size_t e0 = (size_t)i * 12 + 3 * (hop >> 1);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    cplx<R> r = mk * acc[k];
-    if (parity < 0) {
-      const cplx<R> x = S::ld(inr, e0 + k);
-      r = {fma(mk, acc[k].re, x.re), fma(mk, acc[k].im, x.im)};
-    } else if (g.sub) {
-      r = S::ld(static_cast<const typename S::elem*>(g.sub) + rhs * out_stride, e0 + k) - r;
-    }
-    S::st(out + rhs * out_stride, e0 + k, r);
-  }
-}
-
-// Launch variants of an aligned call, searched by the autotuner per (dtype, layout, parity,
-// dagger, volume, nrhs): 0 and 1 one site per thread, 128 threads, registers uncapped and capped
-// at 128; 2 one thread per site and hop (dslash_hop_kernel); 3 one site per thread at 80 registers; 4
-// and 5 take 2 and 4 right-hand sides per thread (dslash_mrhs_kernel), candidates only when nrhs
-// > 1.  Complex double stops at 2: its later forms spill kilobytes per thread.
-constexpr int kNumVariants = 6, kNumSingle = 4, kNumF64 = 3;
-
-template <typename S, int DAG, int MINB, int LL>
-void launch_shape(void* out, const void* in, const void* links, const KGeom& k, int parity,
-                  int nsites, int nrhs, cudaStream_t st, size_t in_stride, size_t out_stride) {
-  typedef typename S::elem E;
-  dim3 grid(stencil_ctas(k.tile, nsites, 128), nrhs);
-  launch_dep(dslash_kernel<S, DAG, 128, MINB, LL>, grid, 128, 0, st, (E*)out, (const E*)in,
-             (const E*)links, k, parity, nsites, in_stride, out_stride);
-}
-
-template <typename S, int DAG, int LL>
-void launch_variant(int v, void* out, const void* in, const void* links, const KGeom& k,
-                    int parity, int nsites, int nrhs, cudaStream_t st, size_t is, size_t os) {
-  if (v == 2) {
-    typedef typename S::elem E;
-    // one warp per CTA until every SM has a few of them
-    const int t = (long long)nsites * nrhs < 4LL * 16 * num_sms() ? 32 : 128;
-    dim3 grid((nsites + t / 8 - 1) / (t / 8), nrhs);
-    launch_dep(dslash_hop_kernel<S, DAG, LL>, grid, t, 0, st, (E*)out, (const E*)in,
-               (const E*)links, k, parity, nsites, is, os);
-    return;
-  }
-  if constexpr (!std::is_same<S, StC128>::value) {
-    if (v == 3) return launch_shape<S, DAG, 6, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os);
-    if (v >= 4)
-      return launch_dslash_mrhs<S>(v == 4 ? 2 : 4, DAG, LL, out, in, links, k, parity, nsites, nrhs, st, is, os);
-  }
-  if (v == 1) launch_shape<S, DAG, 4, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os);
-  else launch_shape<S, DAG, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, is, os);
-}
-
-template <typename S, int LL>
-void launch_dag(int v, int dagger, void* out, const void* in, const void* links, const KGeom& k,
-                int parity, int nsites, int nrhs, cudaStream_t st, size_t is, size_t os) {
-  if (dagger) launch_variant<S, 1, LL>(v, out, in, links, k, parity, nsites, nrhs, st, is, os);
-  else launch_variant<S, 0, LL>(v, out, in, links, k, parity, nsites, nrhs, st, is, os);
-}
-
-// S: the storage type; SN: its form for fields that are only 16-byte aligned (or, where the ABI
-// links are not 16-byte aligned, for links read element by element): one launch shape.
+// S: the storage type; SN: its form for fields that are only 16-byte aligned.  Fields or ABI links
+// less aligned than S's accesses and the windowed links want run the same shapes on 16-byte accesses
+// and element loads, under tuning keys of their own; in FP32 arithmetic on consecutive sites, which
+// suit those accesses better than tiles (complex float at 16^3x32, 1 / 4 / 12 right-hand sides: 20.4
+// / 63 / 165 us, with tiles 21.6 / 71 / 186).
 template <typename S, typename SN>
 int launch_typed(void* out, const void* in, const void* links, const Geom& g, int parity,
                  int dagger, int nrhs, cudaStream_t st, size_t in_stride, size_t out_stride,
@@ -156,45 +50,32 @@ int launch_typed(void* out, const void* in, const void* links, const Geom& g, in
   bool wide = !site32 || (al & 31) == 0;
   // the windowed link loads (load_link, LL = 3) start at a 16-byte boundary
   if (layout == 0 && !f64) wide = wide && ((uintptr_t)links & 15) == 0;
+  if (!wide && !f64) k.tile.on = 0;
+  auto run = [&](int v) {
+    if (!wide) {
+      launch_stencil<SN>(v, dagger, layout, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+      return;
+    }
+    int ll = layout == 0 && !f64 ? 3 : layout;
+    KGeom kv = k;
+    if (v >= kNumForms) {   // half storage only
+      if (layout == 0) ll = 0;
+      v -= 3;
+      kv.tile.on = 0;
+    }
+    launch_stencil<S>(v, dagger, ll, out, in, links, kv, parity, nsites, nrhs, st, in_stride, out_stride);
+  };
+  const int forms = f64 ? kNumF64 : nrhs == 1 ? kNumSingle
+                    : wide && es == 4 ? kNumHalf : kNumForms;
+  int v = tuned_variant(dtype + 16 * layout + (wide ? 0 : 64), parity, dagger, g.V, nrhs, st, forms, run);
+  if (v < 0) return fail(MG_ECUDA, "dslash autotune failed");
   // algorithmic bytes: in + out spinors per rhs and each link once (parity: all 4V links),
   // 18 reals per link whatever the stored form
   double real_bytes = (double)sizeof(typename S::real) * (sizeof(typename S::elem) == 4 ? 0.5 : 1.0);
   double per_site = parity < 0 ? 48.0 * nrhs + 72.0 : 48.0 * nrhs + 144.0;
   const char* name = dtype == MG_C128 ? "dslash_c128" : dtype == MG_C64 ? "dslash_c64"
                      : dtype == MG_F16 ? "dslash_f16" : "dslash_bf16";
-  const double pbytes = per_site * real_bytes * nsites, pflops = 1320.0 * nsites * nrhs;
-  if (!wide) {
-    ProfScope ps(name, pbytes, pflops, st);
-    const bool d = dagger != 0;
-    auto one = [&](auto ll) {
-      constexpr int LL = decltype(ll)::value;
-      if (d) launch_shape<SN, 1, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else launch_shape<SN, 0, 1, LL>(out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-    };
-    if (layout == 0) one(std::integral_constant<int, 0>{});
-    if constexpr (site32) {
-      if (layout == 1) one(std::integral_constant<int, 1>{});
-      if constexpr (!f64) if (layout == 2) one(std::integral_constant<int, 2>{});
-    }
-    WMG_LAUNCHED();
-    return MG_OK;
-  }
-  auto run = [&](int v) {
-    if constexpr (f64) {
-      if (layout == 0) launch_dag<S, 0>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else launch_dag<S, 1>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-    } else {
-      // two stored rows (FP32 and half storage only: the FP64 stencil is bound by its FMA
-      // rate, where rebuilding the third row would cost more than the bytes it saves)
-      if (layout == 0) launch_dag<S, 3>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else if (layout == 1) launch_dag<S, 1>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-      else launch_dag<S, 2>(v, dagger, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
-    }
-  };
-  int v = tuned_variant(dtype + 16 * layout, parity, dagger, g.V, nrhs, st,
-                        f64 ? kNumF64 : nrhs > 1 ? kNumVariants : kNumSingle, run);
-  if (v < 0) return fail(MG_ECUDA, "dslash autotune failed");
-  ProfScope ps(name, pbytes, pflops, st);
+  ProfScope ps(name, per_site * real_bytes * nsites, 1320.0 * nsites * nrhs, st);
   run(v);
   WMG_LAUNCHED();
   return MG_OK;

@@ -4,6 +4,8 @@
 // colour transport by U or U^dag, reconstruction, and one hop in each direction.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 #include "vec.cuh"
@@ -563,12 +565,23 @@ inline int stencil_ctas(const TileMap& m, int nsites, int per) {
   return m.on ? nsites / m.sites : (nsites + per - 1) / per;
 }
 
-// Stencil with 2 or 4 right-hand sides per thread (nr), defined in dslash_mrhs.cu for the
-// FP32-arithmetic storage types; layouts as load_link's LL.
+// Whether storage S is compiled for links of form LL (load_link).  The windowed form is for fields
+// with S's widest accesses; element-wise ABI links are for what is less aligned, and a choice for
+// half storage.
 template <typename S>
-void launch_dslash_mrhs(int nr, int dagger, int layout, void* out, const void* in,
-                        const void* links, const KGeom& k, int parity, int nsites, int nrhs,
-                        cudaStream_t st, size_t in_stride, size_t out_stride);
+constexpr bool link_form(int ll) {
+  if (std::is_same<typename S::real, double>::value) return ll < 2;
+  if (std::is_same<S, StC64>::value) return ll > 0;
+  if (std::is_same<S, StC64N>::value) return ll < 3;
+  return true;
+}
+
+// The stencil in launch shape v with links of form ll (dslash_forms.cuh, one instantiation per
+// storage type in dslash_<storage>.cu).
+template <typename S>
+void launch_stencil(int v, int dagger, int ll, void* out, const void* in, const void* links,
+                    const KGeom& k, int parity, int nsites, int nrhs, cudaStream_t st,
+                    size_t in_stride, size_t out_stride);
 
 }  // namespace stencil
 }  // namespace wmg

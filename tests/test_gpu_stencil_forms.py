@@ -9,6 +9,8 @@ import sys
 
 import pytest
 
+from paper_2505_14399_gb300 import api, synthetic
+
 pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -46,6 +48,20 @@ for dims in ((6, 10, 2, 6), (3, 5, 7, 2)):
                 for r in range(5):
                     e = rel(y[r], wilson.dslash_parity(hh[r], Uh, dims, 0.13, 1, W, BC))
                     assert e < TOL[dtype], ("parity", dtype, sf, sl, r, e)
+# the lane-contiguous copies of the half types, three and two rows per link
+dims = (6, 10, 2, 6)
+U, psi = synthetic.haar_links(dims, 9), synthetic.gaussian_rhs(dims, 6, 5)
+for dtype in ("f16", "bf16"):
+    for lc in (0, 1):
+        p = api.params(dims, (2, 2, 2, 2), 0.13, 4, 4, 1, hop_weight=W, bc=BC, solve_dtype=dtype,
+                       link_compress=lc)
+        h = api.Hierarchy(torch.from_numpy(U).cuda(), p, setup=False)
+        x = _dev(psi, dtype, 0)
+        xh, y = _host(x, dtype), _host(h.apply_fine(x), dtype)
+        h.close()
+        for r in range(5):
+            e = rel(y[r], wilson.dslash(xh[r], U, dims, 0.13, W, BC))
+            assert e < TOL[dtype], ("lanes", dtype, lc, r, e)
 # one infinite component at a time (every spin, both parts): which outputs are NaN, which infinite
 dims = (6, 4, 6, 4)
 U = synthetic.haar_links(dims, 7)
@@ -79,6 +95,23 @@ def first():
     return _run(0)
 
 
-@pytest.mark.parametrize("variant", range(1, 6))
+@pytest.mark.parametrize("variant", range(1, 9))
 def test_forced_shape_every_storage_and_alignment(first, variant):
     assert _run(variant) == first
+
+
+@pytest.mark.parametrize("shift_f,shift_l", [(16, 0), (0, 8), (16, 8)])
+def test_less_aligned_calls_are_tuned_too(shift_f, shift_l):
+    """Their shapes are candidates of the tuner as for aligned calls, under a key of their own."""
+    from paper_2505_14399_gb300 import _lib
+    from test_gpu_dslash_alignment import _dev
+    dims = (10, 6, 4, 2 + shift_f // 8 + shift_l)           # keys of this test only
+    U, psi = synthetic.haar_links(dims, 5), synthetic.gaussian_rhs(dims, 6, 3)
+    count = _lib.lib().mg_kernel_launches
+    for sf, sl in ((0, 0), (shift_f, shift_l)):
+        Ud, x, y = _dev(U, "c64", sl), _dev(psi, "c64", sf), _dev(psi, "c64", sf)
+        n = [count()]
+        for _ in range(2):
+            api.dslash(x, Ud, dims, 0.12, out=y)
+            n.append(count())
+        assert n[1] - n[0] > 1 and n[2] - n[1] == 1, (sf, sl, n)
