@@ -6,6 +6,7 @@ CPU fallback for any entry point.
 """
 import ctypes as C
 import functools
+import math
 import os
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -136,19 +137,32 @@ def check(status, where):
 
 @functools.lru_cache(maxsize=256)
 def _ivec(v):
-    return (C.c_int * 4)(*[int(x) for x in v])
+    return (C.c_int * 4)(*v)
 
 
 @functools.lru_cache(maxsize=256)
-def _dvec(v):
-    return (C.c_double * 4)(*[float(x) for x in v])
+def _dvec(v, signs):
+    return (C.c_double * 4)(*v)
+
+
+# Only tuples of Python's own numbers are keys as they are: other numbers may change in place, hash
+# by identity or not at all, and are converted at every call.
+_INT = {int}
+_NUM = {int, float}
 
 
 def ivec(v):
     """Four C ints; arrays of equal values are shared (the library only reads them)."""
-    return _ivec(tuple(v))
+    v = tuple(v)
+    if not _INT.issuperset(map(type, v)):
+        v = tuple([int(x) for x in v])
+    return _ivec(v)
 
 
 def dvec(v):
     """Four C doubles; arrays of equal values are shared (the library only reads them)."""
-    return _dvec(tuple(v))
+    v = tuple(v)
+    if not _NUM.issuperset(map(type, v)):
+        v = tuple([float(x) for x in v])
+    # zeros of either sign compare equal
+    return _dvec(v, tuple([math.copysign(1.0, x) for x in v]) if 0 in v else None)
