@@ -7,10 +7,11 @@
 // the default shape).  WMG_DSLASH_VARIANT=<i> in the environment forces a shape.
 //
 // Persistence: with WMG_AUTOTUNE_CACHE=<file> the choices are also kept in that file, one JSON
-// object per line ({"device": ..., "dtype": ..., "parity": ..., "dagger": ..., "volume": ...,
-// "nrhs": ..., "variant": ..., "ms": ..., "all_ms": [every candidate's time]}); the file is
-// read once per process and every new choice is appended, so later processes on the same
-// kind of GPU skip the timing.  Entries of other device names are ignored.
+// object per line ({"device": ..., "shapes": ..., "dtype": ..., "parity": ..., "dagger": ...,
+// "volume": ..., "nrhs": ..., "variant": ..., "ms": ..., "all_ms": [every candidate's time]}); the
+// file is read once per process and every new choice is appended, so later processes on the same
+// kind of GPU skip the timing.  Entries of other device names are ignored, and so are those of
+// another shape table, whose variant numbers mean other kernels.
 #include <cstdio>
 #include <cstdlib>
 #include <map>
@@ -26,6 +27,10 @@
 namespace wmg {
 
 namespace {
+// Version of the shape numbering (csrc/dslash.cu, csrc/krylov.cu): goes up with every change of what
+// a variant number launches.  Tables 1 and 2 wrote no version.
+constexpr int kShapeTable = 3;
+
 typedef std::tuple<int, int, int, int, int> Key;
 std::map<Key, std::pair<int, float>> g_cache;
 std::mutex g_mu;
@@ -53,7 +58,8 @@ void load_cache_file() {
   if (!path) return;
   FILE* f = std::fopen(path, "r");
   if (!f) return;
-  const std::string want = "{\"device\":\"" + device_name() + "\",";
+  const std::string want = "{\"device\":\"" + device_name() +
+                           "\",\"shapes\":" + std::to_string(kShapeTable) + ",";
   char line[512];
   while (std::fgets(line, sizeof(line), f)) {
     std::string s(line);
@@ -76,9 +82,9 @@ void append_cache_file(const Key& k, int var, float ms, const std::vector<float>
   FILE* f = std::fopen(path, "a");
   if (!f) return;
   std::fprintf(f,
-               "{\"device\":\"%s\",\"dtype\":%d,\"parity\":%d,\"dagger\":%d,\"volume\":%d,"
-               "\"nrhs\":%d,\"variant\":%d,\"ms\":%.6g,\"all_ms\":[",
-               device_name().c_str(), std::get<0>(k), std::get<1>(k), std::get<2>(k),
+               "{\"device\":\"%s\",\"shapes\":%d,\"dtype\":%d,\"parity\":%d,\"dagger\":%d,"
+               "\"volume\":%d,\"nrhs\":%d,\"variant\":%d,\"ms\":%.6g,\"all_ms\":[",
+               device_name().c_str(), kShapeTable, std::get<0>(k), std::get<1>(k), std::get<2>(k),
                std::get<3>(k), std::get<4>(k), var, ms);
   for (size_t i = 0; i < all.size(); ++i) std::fprintf(f, i ? ",%.6g" : "%.6g", all[i]);
   std::fprintf(f, "]}\n");
@@ -149,10 +155,9 @@ const char* tune_report() {
   for (auto& kv : g_cache) {
     if (!first) os << ",";
     first = false;
-    // key ranges: stencil dtype codes below 1000, the fused stencil + projections 1000-1999,
-    // from 2000 entries of older cache files (the tensor-pipe Galerkin has no shapes to tune now)
+    // key ranges: stencil dtype codes below 1000, the fused stencil + projections from 1000
     const int dt = std::get<0>(kv.first);
-    const char* kern = dt >= 2000 ? "galerkin_tc" : dt >= 1000 ? "dslash_proj" : "dslash";
+    const char* kern = dt >= 1000 ? "dslash_proj" : "dslash";
     os << "{\"kernel\":\"" << kern << "\",\"dtype\":" << dt
        << ",\"parity\":" << std::get<1>(kv.first) << ",\"dagger\":" << std::get<2>(kv.first)
        << ",\"volume\":" << std::get<3>(kv.first) << ",\"nrhs\":" << std::get<4>(kv.first)
