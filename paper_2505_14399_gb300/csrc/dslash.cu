@@ -114,9 +114,11 @@ namespace {
 
 // |U U^dag - 1| and |det U - 1| of one link, largest entry, in double-float arithmetic on the
 // FP32 units (error-free products and sums, ~2^-48 relative: deviations are resolved far below
-// 1e-9); NaN gives a huge value.
+// 1e-9).  Entries that are not finite, or whose products leave the FP32 range, give a huge value: a
+// deviation that is not a number (inf - inf in the error-free sums) is one.
 __device__ float su3_deviation(const zdf u[9]) {
   float worst = 0.f;
+  auto take = [&](float d) { worst = d <= 3e38f ? fmaxf(worst, d) : 3e38f; };
   // U U^dag - 1: the six entries a <= b of the Hermitian matrix
 #pragma unroll
   for (int a = 0; a < 3; ++a)
@@ -127,7 +129,8 @@ __device__ float su3_deviation(const zdf u[9]) {
       for (int c = 0; c < 3; ++c) zdf_fmac(s, u[b * 3 + c], u[a * 3 + c]);   // u_ac conj(u_bc)
       zdf v = zdf_norm(s);
       if (a == b) v.re = df_add(v.re, {-1.0f, 0.0f});
-      worst = fmaxf(worst, fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)));
+      take(fabsf(v.re.hi));
+      take(fabsf(v.im.hi));
     }
   // det U - 1 by cofactors of the first row
   zdfacc t{};
@@ -148,8 +151,8 @@ __device__ float su3_deviation(const zdf u[9]) {
   zdf_fma(t, u[2], c2);
   zdf det = zdf_norm(t);
   det.re = df_add(det.re, {-1.0f, 0.0f});
-  worst = fmaxf(worst, sqrtf(det.re.hi * det.re.hi + det.im.hi * det.im.hi));
-  return worst == worst ? worst : 3e38f;
+  take(sqrtf(det.re.hi * det.re.hi + det.im.hi * det.im.hi));
+  return worst;
 }
 
 // Everything a handle keeps of its links, in one pass over them: the ABI copy, its double-float
