@@ -15,6 +15,7 @@
 // contribution sigma_3 C^dag sigma_3 of a forward one C (exactly, up to rounding), which
 // halves the FP64 work.  A second kernel adds the diagonal term P_j^dag P_j and the
 // mirrored blocks in a fixed order.
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -93,16 +94,19 @@ restrict_kernel(cplx<R>* vc, const cplx<R>* __restrict__ v, const cplx<R>* __res
 }
 
 // One thread per component pair of a site (two rows of a column: 16-byte loads of an FP32 P), four
-// columns' loads in flight.
+// columns' loads in flight.  In FP64 the multiply-adds are the bound and small CTAs leave a shorter
+// last wave.
 template <typename R>
-__global__ void __launch_bounds__(256)
+constexpr int prolong_threads() { return sizeof(R) == 8 ? 64 : 256; }
+template <typename R>
+__global__ void __launch_bounds__(prolong_threads<R>())
 prolong_kernel(cplx<R>* v, const cplx<R>* __restrict__ vc, const cplx<R>* __restrict__ P, int k,
                Blocking B) {
   dep_entry();
   struct alignas(sizeof(R) == 4 ? 16 : 8) Pair {
     cplx<R> a, b;
   };
-  const unsigned e = blockIdx.x * 256u + threadIdx.x, n = 6u * B.nd * B.d;
+  const unsigned e = blockIdx.x * (unsigned)prolong_threads<R>() + threadIdx.x, n = 6u * B.nd * B.d;
   if (e >= n) return;
   const unsigned s = e / 6;
   const int p = (int)(e - 6 * s), alpha = p / 3;
@@ -438,10 +442,14 @@ int restrict_launch(cplx<R>* vc, const cplx<R>* v, const cplx<R>* P, int k, cons
 template <typename R>
 int prolong_launch(cplx<R>* v, const cplx<R>* vc, const cplx<R>* P, int k, const Blocking& B,
                    int nrhs, cudaStream_t st) {
-  const dim3 grid((6u * B.nd * B.d + 255) / 256, nrhs);
+  constexpr int T = prolong_threads<R>();
   ProfScope ps("prolong", (double)sizeof(cplx<R>) * (12.0 * B.nd * B.d * (k + nrhs) + 2.0 * B.d * k * nrhs),
                8.0 * 12 * B.nd * B.d * k * nrhs, st);
-  WMG_LAUNCH_DEP(prolong_kernel<R>, grid, 256, 0, st, v, vc, P, k, B);
+  for (int r0 = 0; r0 < nrhs; r0 += 65535) {   // grid rows
+    const dim3 grid((6u * B.nd * B.d + T - 1) / T, std::min(nrhs - r0, 65535));
+    WMG_LAUNCH_DEP(prolong_kernel<R>, grid, T, 0, st, v + (size_t)r0 * 12 * B.nd * B.d,
+                   vc + (size_t)r0 * 2 * B.d * k, P, k, B);
+  }
   return MG_OK;
 }
 
