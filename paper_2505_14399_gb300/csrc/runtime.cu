@@ -92,7 +92,12 @@ cudaMemPool_t scratch_pool(int dev) {
     pr.location.type = cudaMemLocationTypeDevice;
     pr.location.id = dev;
     cudaMemPool_t pool = nullptr;
-    if (cudaMemPoolCreate(&pool, &pr) != cudaSuccess) {
+    // a stream of this or another thread may be under capture: creating a pool is no part of it
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMemPoolCreate(&pool, &pr);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
@@ -191,6 +196,10 @@ cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
+  // under capture the allocation is the graph's, not a pool's
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+  if (cs != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, st);
   cudaMemPool_t pool = scratch_pool(dev);
   if (!pool) return cudaMallocAsync(p, bytes, st);
   return cudaMallocFromPoolAsync(p, bytes, pool, st);
