@@ -143,6 +143,11 @@ const char* mg_last_error(void);
 /* Number of kernels this library has launched since load (diagnostic counter). */
 long long mg_kernel_launches(void);
 
+/* Gives the device and pinned host memory that the library keeps between calls (blocks of destroyed
+ * handles, idle scratch) back to the driver; synchronises the current device.  Not needed for the
+ * library's own allocations, which do the same before they fail. */
+int mg_release_memory(void);
+
 /* JSON list of the launch shapes the autotuner has chosen so far, one object per problem key
  * ("kernel": "dslash" | "dslash_proj", the key fields, "variant", "ms");
  * library-owned string, valid until the next call. */

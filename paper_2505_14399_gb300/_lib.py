@@ -66,6 +66,7 @@ SIGNATURES = {
     "mg_last_error": (C.c_char_p, []),
     "mg_kernel_launches": (C.c_longlong, []),
     "mg_autotune_report": (C.c_char_p, []),
+    "mg_release_memory": (I, []),
     "mg_selftest_barrier_timeout": (I, [P]),
     "mg_probe_fma_peak": (I, [I, P, P]),
     "mg_profile_enable": (I, [I, I]),

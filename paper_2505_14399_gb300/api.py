@@ -127,6 +127,11 @@ def clover_dslash(inp, links, clover, dims, kappa, hop_weight=(1, 1, 1, 1), bc=(
     return out
 
 
+def release_memory():
+    """Give the memory that the library keeps between calls back to the device (for torch, say)."""
+    L.check(L.lib().mg_release_memory(), "mg_release_memory")
+
+
 def test_vectors(links, p, stream_index, device=None):
     """The r smoothed test vectors of one stream (Eq. 2), complex128 (r, V, 4, 3)."""
     V = p.dims[0] * p.dims[1] * p.dims[2] * p.dims[3]

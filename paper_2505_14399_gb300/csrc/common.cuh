@@ -30,6 +30,8 @@ void host_free(void* p);
 // Stream-ordered scratch of one call, from the library's own pool; see runtime.cu.
 cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st);
 void scratch_free(void* p, cudaStream_t st);
+// Free blocks and unused scratch back to the driver.
+int release_memory();
 template <typename T>
 inline cudaError_t scratch_alloc(T** p, size_t bytes, cudaStream_t st) {
   return scratch_alloc_bytes(reinterpret_cast<void**>(p), bytes, st);

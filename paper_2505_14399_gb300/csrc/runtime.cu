@@ -76,8 +76,8 @@ size_t round_block(size_t b) {
 // time (0.3 ms for the 16 MB of a 16^3x32 Galerkin build, 2.5 ms for the 1.2 GB of a 16^3x64 one
 // with k = 24, 0.6 ms for the two temporaries of a test-vector stream).  This pool keeps up to
 // kScratchKeep bytes that no call uses; the rest goes back at the next synchronisation, and all
-// of it when a device allocation of the library fails.  Order and reuse across streams and
-// threads are the pool's, as for cudaMallocAsync.
+// of it when an allocation of the library fails or mg_release_memory asks for it.  Order and reuse
+// across streams and threads are the pool's, as for cudaMallocAsync.
 constexpr unsigned long long kScratchKeep = 2ull << 30;
 constexpr int kScratchDevices = 64;
 std::mutex g_scratch_pool_mu;
@@ -108,9 +108,23 @@ cudaMemPool_t scratch_pool(int dev) {
   return g_scratch_pool[dev];
 }
 
-void trim_scratch(int dev) {
-  cudaMemPool_t pool = scratch_pool(dev);
-  if (pool) cudaMemPoolTrimTo(pool, 0);
+void trim_scratch() {
+  std::lock_guard<std::mutex> lock(g_scratch_pool_mu);
+  for (cudaMemPool_t pool : g_scratch_pool)
+    if (pool) cudaMemPoolTrimTo(pool, 0);
+}
+
+// Gives back what no call uses: the free blocks (of both kinds if `host`) and the scratch pools.
+// The caller holds c.mu.
+void release_unused(MemCache& c, bool host) {
+  cudaDeviceSynchronize();
+  for (auto& kv : c.free_dev) cudaFree(kv.second);
+  c.free_dev.clear();
+  if (host) {
+    for (auto& kv : c.free_host) cudaFreeHost(kv.second);
+    c.free_host.clear();
+  }
+  trim_scratch();
 }
 
 int cached_alloc(void** p, size_t bytes, bool host) {
@@ -131,13 +145,7 @@ int cached_alloc(void** p, size_t bytes, bool host) {
   cudaError_t e = host ? cudaMallocHost(p, key.second) : cudaMalloc(p, key.second);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    cudaDeviceSynchronize();
-    for (auto& kv : fl) {
-      if (host) cudaFreeHost(kv.second);
-      else cudaFree(kv.second);
-    }
-    fl.clear();
-    if (!host) trim_scratch(dev);
+    release_unused(c, host);
     e = host ? cudaMallocHost(p, key.second) : cudaMalloc(p, key.second);
   }
   if (e != cudaSuccess) {
@@ -202,10 +210,28 @@ cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
   if (cs != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, st);
   cudaMemPool_t pool = scratch_pool(dev);
   if (!pool) return cudaMallocAsync(p, bytes, st);
-  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+  e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    {
+      MemCache& c = mem_cache();
+      std::lock_guard<std::mutex> lock(c.mu);
+      release_unused(c, false);
+    }
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  }
+  return e;
 }
 
 void scratch_free(void* p, cudaStream_t st) { cudaFreeAsync(p, st); }
+
+int release_memory() {
+  MemCache& c = mem_cache();
+  std::lock_guard<std::mutex> lock(c.mu);
+  release_unused(c, true);
+  WMG_CUDA(cudaGetLastError());
+  return MG_OK;
+}
 
 int smem_attr_raw(const void* fn, size_t bytes) {
   static std::mutex mu;
@@ -381,6 +407,8 @@ extern "C" const char* mg_profile_report(void) {
 }
 
 extern "C" const char* mg_last_error(void) { return wmg::g_last_error.c_str(); }
+
+extern "C" int mg_release_memory(void) { return wmg::release_memory(); }
 
 extern "C" long long mg_kernel_launches(void) { return wmg::g_launches.load(); }
 
