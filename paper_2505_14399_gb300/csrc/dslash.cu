@@ -47,6 +47,8 @@ int launch_typed(void* out, const void* in, const void* links, const Geom& g, in
   const size_t es = sizeof(typename S::elem);
   uintptr_t al = (uintptr_t)out | (uintptr_t)in | (uintptr_t)k.sub;
   if (nrhs > 1) al |= (in_stride * es) | (out_stride * es);
+  if (al & 15) return fail(MG_EINVAL, "dslash: spinor fields must be 16-byte aligned");
+  if ((uintptr_t)links & (es - 1)) return fail(MG_EINVAL, "dslash: links misaligned for their dtype");
   bool wide = !site32 || (al & 31) == 0;
   // the windowed link loads (load_link, LL = 3) start at a 16-byte boundary
   if (layout == 0 && !f64) wide = wide && ((uintptr_t)links & 15) == 0;
@@ -353,10 +355,6 @@ extern "C" int wilson_dslash(void* out, const void* in, const void* links, const
   WMG_TRY(stage_in(sin, in, fbytes, st));
   WMG_TRY(stage_in(sl, links, lbytes, st));
   WMG_TRY(stage_out_alloc(sout, out, fbytes, st));
-  if (((uintptr_t)sin.dev | (uintptr_t)sout.dev) & 15)
-    return fail(MG_EINVAL, "wilson_dslash: spinor fields must be 16-byte aligned");
-  if ((uintptr_t)sl.dev & (eb >= 8 ? 7 : 3))
-    return fail(MG_EINVAL, "wilson_dslash: links misaligned for their dtype");
   WMG_TRY(dslash_launch(dtype, sout.dev, sin.dev, sl.dev, g, parity, dagger, nrhs, st, 0, 0));
   WMG_TRY(stage_out_finish(sout, out, fbytes, st));
   return MG_OK;

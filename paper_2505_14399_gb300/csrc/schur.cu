@@ -194,8 +194,6 @@ extern "C" int wilson_schur(void* out, const void* in, const void* links, const 
   WMG_TRY(stage_in(sin, in, fbytes, st));
   WMG_TRY(stage_in(sl, links, (size_t)4 * g.V * 9 * eb, st));
   WMG_TRY(stage_out_alloc(sout, out, fbytes, st));
-  if (((uintptr_t)sin.dev | (uintptr_t)sout.dev) & 15)
-    return fail(MG_EINVAL, "wilson_schur: spinor fields must be 16-byte aligned");
   void* tmp = nullptr;
   WMG_CUDA(scratch_alloc(&tmp, fbytes, st));
   int s = MG_OK;
