@@ -181,8 +181,13 @@ __global__ void scale_inv_kernel(E* y, const E* x, const double* s, int lds, siz
   typedef VecT<E> T;
   typedef typename T::R R;
   int rhs = blockIdx.y;
-  const R sv = (R)s[(size_t)rhs * lds];
-  const R f = sv > 0 ? (R)1 / sv : (R)0;
+  __shared__ R fs;   // one FP64 division per CTA, rounded once
+  if (threadIdx.x == 0) {
+    const double sv = s[(size_t)rhs * lds];
+    fs = sv > 0 ? (R)(1.0 / sv) : (R)0;
+  }
+  __syncthreads();
+  const R f = fs;
   const E* xr = x + (size_t)rhs * n;
   E* yr = y + (size_t)rhs * n;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;

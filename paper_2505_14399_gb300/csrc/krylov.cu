@@ -119,14 +119,16 @@ __device__ void givens_deferred(zd* sm, SmallLayout L, int j, double* res) {
 
 // The end of a reduction sweep, by its last CTA: h2 (the nv projections and ||w||^2, in shared
 // memory) to the coefficients of the update, column nv - 1 of the Hessenberg matrix (added to the
-// first pass's projections, or alone when `single`) and H[j+1, j]^2 = ||w||^2 - ||h2||^2.
+// first pass's projections, or alone when `single`) and H[j+1, j]^2 = ||w||^2 - ||h2||^2, with its
+// reciprocal for the update (wnorm[iw]: a FP32 update rounds it once and divides nothing).
 // beta (fused fixed runs): column 0 of the basis is the right-hand side b itself, of norm beta, so
 // its projection and its coefficient carry 1 / beta each.  In the first step (`first`) w = D b as
 // well, h2[1].im = ||b||^2, and beta and 1 / beta are written (beta[ibeta]: no FP64 division in
 // the chain of every later step).
 __device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, const zd* h2,
-                                              double* wnorm, bool single, double* beta = nullptr,
-                                              bool first = false, int ibeta = 0) {
+                                              double* wnorm, int iw, bool single,
+                                              double* beta = nullptr, bool first = false,
+                                              int ibeta = 0) {
   zd* col = sm + L.H() + (size_t)(nv - 1) * (L.m + 1);
   if (first) {
     if (threadIdx.x == 0) {
@@ -136,7 +138,8 @@ __device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, con
       sm[L.h2()] = h;
       col[0] = h;
       col[1] = {w * ib, 0};
-      *wnorm = w;           // v_1 = (D b - h b) / w
+      wnorm[0] = w;           // v_1 = (D b - h b) / w
+      wnorm[iw] = w2 > 0 ? rsqrt(w2) : 0.0;
       beta[0] = bb * ib;
       beta[ibeta] = ib;
     }
@@ -152,7 +155,8 @@ __device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, con
     double hh = s0 * s0 * norm2(h2[0]);
     for (int i = 1; i < nv; ++i) hh += norm2(h2[i]);
     const double b2 = h2[nv].re - hh, b = b2 > 0 ? sqrt(b2) : 0.0;
-    *wnorm = b;
+    wnorm[0] = b;
+    wnorm[iw] = b2 > 0 ? rsqrt(b2) : 0.0;
     col[nv] = {b, 0};
   }
 }
@@ -266,7 +270,7 @@ cgs_update_dot_kernel(E* w, const E* __restrict__ V, size_t vstride, int nv,
   __shared__ zd g_h2[GV_MAX];
   finish_partials(partials_as<R>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0, scale);
   __syncthreads();
-  finish_column(sm, L, nv, g_h2, wnorm + rhs, false);
+  finish_column(sm, L, nv, g_h2, wnorm + rhs, 4 * gridDim.y, false);
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
@@ -293,10 +297,16 @@ cgs_update_scale_kernel(E* vout, const E* __restrict__ w, const E* __restrict__ 
   const zd* h2 = small + (size_t)rhs * L.stride() + L.h2();
   for (int i = threadIdx.x; i < nv; i += blockDim.x) cs[i] = {(R)(-h2[i].re), (R)(-h2[i].im)};
   __syncthreads();
-  // the division in the vectors' precision: in FP64 on every thread it took as long as the update
-  // itself (FP64 instructions occupy an SM for 16 cycles per warp): 14.1 -> 10.1 us on 65 536 sites
-  const R beta = (R)wnorm[rhs];
-  const R f = beta > 0 ? (R)1 / beta : (R)0;
+  // FP32: the FP64 reciprocal of the reduction's end, rounded once.  A FP64 division on every thread
+  // took as long as the update itself (FP64 instructions occupy an SM for 16 cycles per warp): 14.1
+  // -> 10.1 us on 65 536 sites
+  R f;
+  if constexpr (sizeof(R) == 8) {
+    const double beta = wnorm[rhs];
+    f = beta > 0 ? 1.0 / beta : 0.0;
+  } else {
+    f = (R)wnorm[4 * gridDim.y + rhs];
+  }
   const E* wr = w + (size_t)rhs * n;
   const E* vb = V + (size_t)rhs * n;
   E* outr = vout + (size_t)rhs * n;
@@ -489,7 +499,7 @@ stream_cgs_kernel(zf* w, const zf* __restrict__ V, size_t vstride, int nv, size_
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0,
                   scale);
   __syncthreads();
-  finish_column(sm, L, nv, g_h2, wnorm + rhs, MODE == 2);
+  finish_column(sm, L, nv, g_h2, wnorm + rhs, 4 * gridDim.y, MODE == 2);
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
 
@@ -584,7 +594,7 @@ dslash_proj_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   __shared__ zd g_h2[NVM + 1];
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0);
   __syncthreads();
-  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true,
+  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, 4 * gridDim.y, true,
                 beta ? beta + rhs : nullptr, FIRST, gridDim.y);
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
@@ -696,7 +706,7 @@ dslash_proj_hop_kernel(zf* w, zf* V, size_t vstride, int nv, size_t n,
   __shared__ zd g_h2[NVM + 1];
   finish_partials(partials_as<float>(partial), nv + 1, nblk, maxvec, rhs, g_h2, nullptr, 0, 0);
   __syncthreads();
-  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, true,
+  finish_column(small + (size_t)rhs * L.stride(), L, nv, g_h2, wnorm + rhs, 4 * gridDim.y, true,
                 beta ? beta + rhs : nullptr, FIRST, gridDim.y);
   if (threadIdx.x == 0) counter[rhs] = 0;
 }
@@ -930,7 +940,7 @@ int GmresV<E>::alloc(size_t n_, int nrhs_, int m_, bool flexible_) {
   WMG_TRY(dev_alloc(&w, fb));
   SmallLayout L{m};
   WMG_TRY(dev_alloc(&small, sizeof(zd) * L.stride() * nrhs));
-  WMG_TRY(dev_alloc(&dnorm, sizeof(double) * nrhs * 4));
+  WMG_TRY(dev_alloc(&dnorm, sizeof(double) * nrhs * 5));
   WMG_TRY(dev_alloc(&reshist, sizeof(double) * nrhs * m));
   WMG_TRY(host_alloc(&host_res, sizeof(double) * nrhs * (m + 2)));
   WMG_TRY(rw.alloc(n, nrhs, m + 1));
@@ -957,7 +967,8 @@ void GmresV<E>::release() {
   m = 0;
 }
 
-// dnorm layout: [0..nrhs) current ||w||, [nrhs..2nrhs) beta, [2nrhs..3nrhs) residual estimate
+// dnorm layout: [0..nrhs) current ||w||, [nrhs..2nrhs) beta, [2nrhs..3nrhs) residual estimate (fused
+// fixed runs: 1 / beta), [3nrhs..4nrhs) norms of the next cycle's residual, [4nrhs..5nrhs) 1 / ||w||
 template <typename E>
 int GmresV<E>::arnoldi_step(const OpV<E>& A, const OpV<E>* M, int j, cudaStream_t st,
                             bool single_pass, const FusedStencil* fused, const E* b0,
