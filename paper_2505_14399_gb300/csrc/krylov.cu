@@ -124,7 +124,8 @@ __device__ void givens_deferred(zd* sm, SmallLayout L, int j, double* res) {
 // beta (fused fixed runs): column 0 of the basis is the right-hand side b itself, of norm beta, so
 // its projection and its coefficient carry 1 / beta each.  In the first step (`first`) w = D b as
 // well, h2[1].im = ||b||^2, and beta and 1 / beta are written (beta[ibeta]: no FP64 division in
-// the chain of every later step).
+// the chain of every later step).  Where a norm of b or D b leaves the FP32 range the run ends with
+// x = 0, as for b = 0.
 __device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, const zd* h2,
                                               double* wnorm, int iw, bool single,
                                               double* beta = nullptr, bool first = false,
@@ -132,15 +133,17 @@ __device__ __forceinline__ void finish_column(zd* sm, SmallLayout L, int nv, con
   zd* col = sm + L.H() + (size_t)(nv - 1) * (L.m + 1);
   if (first) {
     if (threadIdx.x == 0) {
-      const double bb = h2[1].im, ib2 = bb > 0 ? 1.0 / bb : 0.0, ib = sqrt(ib2);
-      const zd h = ib2 * h2[0];
-      const double w2 = h2[1].re - bb * norm2(h), w = w2 > 0 ? sqrt(w2) : 0.0;
+      const double bb = h2[1].im, ww = h2[1].re;
+      const bool ok = bb > 0 && bb <= 3.4028234663852886e38 && ww <= 3.4028234663852886e38;
+      const double ib2 = ok ? 1.0 / bb : 0.0, ib = sqrt(ib2);
+      const zd h = ok ? ib2 * h2[0] : zd{0, 0};
+      const double w2 = ok ? ww - bb * norm2(h) : 0.0, w = w2 > 0 ? sqrt(w2) : 0.0;
       sm[L.h2()] = h;
       col[0] = h;
       col[1] = {w * ib, 0};
       wnorm[0] = w;           // v_1 = (D b - h b) / w
       wnorm[iw] = w2 > 0 ? rsqrt(w2) : 0.0;
-      beta[0] = bb * ib;
+      beta[0] = ok ? bb * ib : 0.0;
       beta[ibeta] = ib;
     }
     return;

@@ -40,3 +40,18 @@ def test_norm_reciprocal_is_rounded_once():
     twice = np.sort([_psi(x, F(1) / F(m)) for x, m in zip(a, n)])[::-1]
     assert np.abs(once - twice).max() > 1e-9       # the inputs tell the two apart
     assert np.abs(S - once).max() < 1e-12 + 1e-6 * once.max()
+
+
+def test_norm_beyond_fp32_leaves_the_vectors_as_they_are():
+    """Initial guesses phi whose squared norm overflows FP32 are not smoothed (as phi = 0 is not):
+    the setup's results are those of phi itself, finite."""
+    dims, block = (4, 4, 4, 4), (2, 2, 2, 2)
+    v = (4e17 * synthetic.gaussian_rhs(dims, 6, 8)).astype(np.complex64)
+    p = api.params(dims, block, 0.12, 4, 4, 2, setup_dtype="c64", solve_dtype="c64")
+    out = []
+    for smooth in (True, False):
+        h = api.Hierarchy(to_dev(synthetic.smooth_links(dims, 5)), p, vectors=to_dev(v), smooth=smooth)
+        out.append((h.prolongator()[0].cpu().numpy(), h.sigma_history().cpu().numpy()))
+        h.close()
+    assert np.all(np.isfinite(out[0][0])) and np.all(out[0][1] > 0)
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
