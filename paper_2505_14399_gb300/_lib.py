@@ -6,7 +6,6 @@ CPU fallback for any entry point.
 """
 import ctypes as C
 import functools
-import math
 import os
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -136,34 +135,40 @@ def check(status, where):
     return status
 
 
-@functools.lru_cache(maxsize=256)
-def _ivec(v):
-    return (C.c_int * 4)(*v)
-
-
-@functools.lru_cache(maxsize=256)
-def _dvec(v, signs):
-    return (C.c_double * 4)(*v)
-
-
-# Only tuples of Python's own numbers are keys as they are: other numbers may change in place, hash
-# by identity or not at all, and are converted at every call.
-_INT = {int}
+_I4 = C.c_int * 4
+_D4 = C.c_double * 4
 _NUM = {int, float}
 
 
+@functools.lru_cache(maxsize=256)
+def _ivec(v):
+    return _I4(*v)
+
+
+@functools.lru_cache(maxsize=256)
+def _dvec(v):
+    return _D4(*v)
+
+
+# Arrays of equal values are shared (the library only reads them), with tuples of Python's own
+# numbers as keys: other numbers may change in place, hash by identity or not at all, and zeros of
+# either sign compare equal, so those are converted at every call.
 def ivec(v):
-    """Four C ints; arrays of equal values are shared (the library only reads them)."""
+    """Four C ints."""
     v = tuple(v)
-    if not _INT.issuperset(map(type, v)):
-        v = tuple([int(x) for x in v])
-    return _ivec(v)
+    if len(v) == 4:
+        a, b, c, d = v
+        if type(a) is type(b) is type(c) is type(d) is int:
+            return _ivec(v)
+    return _I4(*[int(x) for x in v])
 
 
 def dvec(v):
-    """Four C doubles; arrays of equal values are shared (the library only reads them)."""
+    """Four C doubles."""
     v = tuple(v)
-    if not _NUM.issuperset(map(type, v)):
-        v = tuple([float(x) for x in v])
-    # zeros of either sign compare equal
-    return _dvec(v, tuple([math.copysign(1.0, x) for x in v]) if 0 in v else None)
+    if len(v) == 4:
+        a, b, c, d = v
+        if (type(a) in _NUM and type(b) in _NUM and type(c) in _NUM and type(d) in _NUM
+                and a and b and c and d):
+            return _dvec(v)
+    return _D4(*[float(x) for x in v])
