@@ -29,7 +29,7 @@ namespace wmg {
 namespace {
 // Version of the shape numbering (csrc/dslash.cu, csrc/krylov.cu): goes up with every change of what
 // a variant number launches.  Tables 1 and 2 wrote no version.
-constexpr int kShapeTable = 3;
+constexpr int kShapeTable = 4;
 
 typedef std::tuple<int, int, int, int, int> Key;
 std::map<Key, std::pair<int, float>> g_cache;

@@ -21,11 +21,13 @@ using namespace stencil;
 // registers, 4 and 5 take 2 and 4 right-hand sides per thread, candidates when nrhs > 1; 6, 7 and 8
 // (4-byte types) are 3, 4 and 5 on consecutive sites, ABI links read element by element: with the
 // links shared by several right-hand sides, the windows' selects and the tiles can cost more than
-// they save (bf16, 12 right-hand sides at 16^3x32: 103 -> 98 us).  FP64: 3 two threads per site, 4
-// as 0 with consecutive sites (12x10x14x18: 72 us instead of 77, the tile's part-filled warps cost
-// FP64 issue); 2 and 4 right-hand sides per thread spill kilobytes (78 and 139 us against 22 at 8^4,
-// 2 right-hand sides).
-constexpr int kNumForms = 6, kNumSingle = 4, kNumF64 = 5, kNumHalf = 9;
+// they save (bf16, 12 right-hand sides at 16^3x32: 103 -> 98 us).  FP64: 3 as 0 with consecutive
+// sites (12x10x14x18: 62 us instead of 77, the tile's part-filled warps cost FP64 issue); 2 and 4
+// right-hand sides per thread spill kilobytes (78 and 139 us against 19 at 8^4, 2 right-hand sides).
+// Two threads per site in FP64 (20 us there, alone) are slower in a chain of dependent launches: their
+// 128 CTAs are placed while the SMs still drain, several to one SM (a solve at 8^3x16: 11.2 ms
+// against 8.8 with one thread per site and hop).
+constexpr int kNumForms = 6, kNumSingle = 4, kNumF64 = 4, kNumHalf = 9;
 
 // S: the storage type; SN: its form for fields that are only 16-byte aligned.  Fields or ABI links
 // less aligned than S's accesses and the windowed links want run the same shapes on 16-byte accesses
@@ -58,14 +60,14 @@ int launch_typed(void* out, const void* in, const void* links, const Geom& g, in
       launch_stencil<SN>(v, dagger, layout, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
       return;
     }
-    int ll = layout == 0 && !f64 ? 3 : layout;
-    KGeom kv = k;
     if (v >= kNumForms) {   // half storage only
-      if (layout == 0) ll = 0;
-      v -= 3;
-      kv.tile.on = 0;
+      KGeom kc = k;
+      kc.tile.on = 0;
+      launch_stencil<S>(v - 3, dagger, layout, out, in, links, kc, parity, nsites, nrhs, st, in_stride, out_stride);
+      return;
     }
-    launch_stencil<S>(v, dagger, ll, out, in, links, kv, parity, nsites, nrhs, st, in_stride, out_stride);
+    launch_stencil<S>(v, dagger, layout == 0 && !f64 ? 3 : layout, out, in, links, k, parity, nsites,
+                      nrhs, st, in_stride, out_stride);
   };
   const int forms = f64 ? kNumF64 : nrhs == 1 ? kNumSingle
                     : wide && es == 4 ? kNumHalf : kNumForms;

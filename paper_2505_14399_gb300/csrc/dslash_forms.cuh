@@ -7,7 +7,7 @@
 // U_mu(x) or U_mu(x-mu)^dag, and reconstructs the lower spin pair from the upper one.  Spinor loads
 // are 32-byte vector loads of the [site][spin][colour] layout (16-byte where the fields are only so
 // aligned); links are read through the read-only path.  Further shapes take one thread per site and
-// hop, two threads per site, or 2 and 4 right-hand sides per thread: there each link is loaded once
+// hop, or 2 and 4 right-hand sides per thread: there each link is loaded once
 // and applied to NR spinors (the test-vector streams of the setup smoothing, Eq. 2, and batched
 // solves), and every thread keeps NR independent neighbour loads in flight per hop.
 #pragma once
@@ -94,67 +94,6 @@ dslash_hop_kernel(typename S::elem* __restrict__ out, const typename S::elem* __
     }
     S::st(out + rhs * out_stride, e0 + k, r);
   }
-}
-
-// Two threads per site, warp-uniform: the first 64 threads of a CTA take the forward hops of 64
-// consecutive sites, the other 64 the backward hops of the same sites; the halves meet in shared
-// memory.  FP64 only: between one thread per site and hop (whose shuffles and selects cost more than
-// they hide there) and one per site, 8192 sites x right-hand sides take 22 us instead of 24 and 32.
-template <typename S, int DAG, int LL>
-__global__ void __launch_bounds__(128)
-dslash_split_kernel(typename S::elem* __restrict__ out, const typename S::elem* __restrict__ in,
-                    const typename S::elem* __restrict__ links, KGeom g, int parity, int nsites,
-                    size_t in_stride, size_t out_stride) {
-  dep_entry();
-  typedef typename S::real R;
-  __shared__ cplx<R> sacc[12][64];
-  const int half = threadIdx.x >> 6, ls = threadIdx.x & 63;
-  const int i = blockIdx.x * 64 + ls;
-  const bool active = i < nsites;
-  const size_t rhs = blockIdx.y;
-  const bool half_in = parity >= 0;
-  const size_t in_off = rhs * in_stride;
-  cplx<R> acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
-  int site = 0, c[4] = {0, 0, 0, 0};
-  if (active) {
-    site = stencil_site(g, parity, i, c);
-    if (half == 0) {
-      hop_fwd<0, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_fwd<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_fwd<2, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_fwd<3, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-    } else {
-      hop_bwd<0, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_bwd<1, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_bwd<2, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-      hop_bwd<3, DAG, S, LL>(g, site, c, in, in_off, half_in, links, acc);
-    }
-  }
-  if (half == 1) {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) sacc[k][ls] = acc[k];
-  }
-  __syncthreads();
-  if (half != 0 || !active) return;
-  const R mk = -kap<R>(g);
-  cplx<R> res[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] += sacc[k][ls];
-  if (parity < 0) {
-    SiteIO<S>::load(in + in_off, (size_t)site, res);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      res[k].re = fma(mk, acc[k].re, res[k].re);
-      res[k].im = fma(mk, acc[k].im, res[k].im);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) res[k] = mk * acc[k];
-    apply_sub<S>(g, rhs * out_stride, i, res);
-  }
-  SiteIO<S>::store(out + rhs * out_stride, (size_t)i, res);
 }
 
 template <int MU, int DAG, typename S, int LL, int NR>
@@ -299,11 +238,6 @@ void launch_form(int v, void* out, const void* in, const void* links, const KGeo
   }
   if constexpr (f64) {
     if (v == 3) {
-      launch_dep(dslash_split_kernel<S, DAG, LL>, dim3((nsites + 63) / 64, nrhs), 128, 0, st, (E*)out,
-                 (const E*)in, (const E*)links, k, parity, nsites, is, os);
-      return;
-    }
-    if (v == 4) {
       KGeom kc = k;
       kc.tile.on = 0;
       return launch_site<S, DAG, LL, 1>(out, in, links, kc, parity, nsites, nrhs, st, is, os);
@@ -340,9 +274,9 @@ void launch_stencil(int v, int dagger, int ll, void* out, const void* in, const 
 
 }  // namespace stencil
 
-#define WMG_STENCIL(S)                                                                           \
-  template void stencil::launch_stencil<S>(int, int, int, void*, const void*,           \
-                                                    const void*, const stencil::KGeom&, int, int, \
-                                                    int, cudaStream_t, size_t, size_t);
+#define WMG_STENCIL(S)                                                                        \
+  template void stencil::launch_stencil<S>(int, int, int, void*, const void*, const void*,    \
+                                           const stencil::KGeom&, int, int, int, cudaStream_t, \
+                                           size_t, size_t);
 
 }  // namespace wmg

@@ -295,6 +295,7 @@ struct KGeom {
   int bc[4];
   double kappa;
   float kf;      // kappa in FP32: one FP64 conversion per thread would cost each warp 16 cycles
+  bool unit;     // all four hop weights are 1
   // single-parity form only: when set, out_p = sub_p - (-kappa H_{p,1-p} in) (the even-odd
   // Schur complement and its source / reconstruction steps), sub with out's layout and stride
   const void* sub = nullptr;
@@ -363,25 +364,35 @@ __device__ __forceinline__ void hop_pair(const KGeom& g, int site, const int c[4
 // ---- one thread per site and hop
 // For lattices that leave the chip idle with a thread per site (4^4: two CTAs; 8^4: 32) the chain
 // of eight dependent hops is the launch: FP64 on 4^4 17.8 us, of which the launch itself is a
-// few.  Here eight lanes share a site, lane `hop` takes direction hop / 2 (forward when even) with
+// few (7.7 us in this form).  Here eight lanes share a site, lane `hop` takes direction hop / 2 (forward when even) with
 // the spin projector's phases as operands, and the 12 sums are reduced and scattered over the
 // lanes: every pair of lanes ends with the three colours of one spin.
 
+// -x where `neg`, off the FP64 pipe
+__device__ __forceinline__ float flip(float x, bool neg) {
+  return __uint_as_float(__float_as_uint(x) ^ (neg ? 0x80000000u : 0u));
+}
+__device__ __forceinline__ double flip(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000u : 0), __double2loint(x));
+}
+
 // The two components of i sigma_mu d for mu < 3, d for mu = 3, are d[w], d[1 - w] (w = 1 for mu <
 // 2) times one unit, i for even mu and 1 for odd, the second negated for mu = 1 and 2.  The unit is
-// applied by exchanging real and imaginary parts, not by multiplying with its zero part: half of
-// the multiply-adds, and an infinite component does not turn its neighbours into NaN.
+// applied by exchanging real and imaginary parts and flipping signs, not by multiplying with it: an
+// infinite component does not turn its neighbours into NaN, and FP64 multiply-adds, the bound of a
+// filled chip, are left to the products and sums (8192 sites: 24.1 -> 18.6 us).
 template <typename R>
 struct HopPhase {
-  bool swap, imag;
-  R sgn1;                       // sign of the second component
-  // the part of d that gives the real part (times -1 if imag) and the imaginary part
-  __device__ __forceinline__ R re(cplx<R> d) const { return imag ? d.im : d.re; }
-  __device__ __forceinline__ R im(cplx<R> d) const { return imag ? d.re : d.im; }
+  bool swap, imag, neg1;        // neg1: the second component's sign
+  // component c of the result, from d = its d[w] or d[1 - w], negated where `neg`
+  __device__ __forceinline__ cplx<R> turn(cplx<R> d, int c, bool neg) const {
+    const bool n = neg != (c && neg1);
+    return {flip(imag ? d.im : d.re, n != imag), flip(imag ? d.re : d.im, n)};
+  }
 };
 template <typename R>
 __device__ __forceinline__ HopPhase<R> hop_phase(int mu) {
-  return {mu < 2, (mu & 1) == 0, (mu == 1 || mu == 2) ? R(-1) : R(1)};
+  return {mu < 2, (mu & 1) == 0, mu == 1 || mu == 2};
 }
 
 // The hop's term of H psi at `site`, reduced over the site's eight lanes: out = components 3 sp ..
@@ -399,39 +410,38 @@ __device__ __forceinline__ void hop_lanes(const KGeom& g, bool active, int site,
 #pragma unroll
   for (int i = 0; i < 6; ++i) gg[i] = {0, 0};
   const HopPhase<R> f = hop_phase<R>(mu);
-  R s = (fwd != (DAG != 0)) ? R(-1) : R(1);   // projector sign
-  R cf = 0;
+  const bool neg = fwd != (DAG != 0);   // projector sign
+  R w = 0;
+  bool cneg = false;                    // coefficient: w, negated at an antiperiodic boundary
   if (active) {
     const int L = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
     const int st = mu == 0 ? g.stride[0] : mu == 1 ? g.stride[1] : mu == 2 ? g.stride[2] : g.stride[3];
     const int cm = mu == 0 ? c[0] : mu == 1 ? c[1] : mu == 2 ? c[2] : c[3];
     const int bc = mu == 0 ? g.bc[0] : mu == 1 ? g.bc[1] : mu == 2 ? g.bc[2] : g.bc[3];
-    const R w = mu == 0 ? wgt<R>(g, 0) : mu == 1 ? wgt<R>(g, 1) : mu == 2 ? wgt<R>(g, 2) : wgt<R>(g, 3);
+    w = mu == 0 ? wgt<R>(g, 0) : mu == 1 ? wgt<R>(g, 1) : mu == 2 ? wgt<R>(g, 2) : wgt<R>(g, 3);
     const bool wrap = fwd ? cm == L - 1 : cm == 0;
     const int step = wrap ? -(L - 1) * st : st;
     const int nb = fwd ? site + step : site - step;
-    cf = (wrap && bc < 0) ? -w : w;
+    cneg = wrap && bc < 0;
     cplx<R> p[12], u[9], h[6];
     SiteIO<S>::load(in, half_in ? (size_t)(nb >> 1) : (size_t)nb, p);
     load_link<S, LL>(links, g.V, mu, fwd ? site : nb, u);
     // h = psi_up - s i sigma psi_dn (mu < 3), psi_up + s psi_dn (mu = 3)
-    const R sp = mu < 3 ? -s : s;
-    const R i0 = sp, r0 = f.imag ? -sp : sp, i1 = f.sgn1 * i0, r1 = f.sgn1 * r0;
+    const bool np = neg != (mu < 3);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const cplx<R> d0 = f.swap ? p[9 + k] : p[6 + k], d1 = f.swap ? p[6 + k] : p[9 + k];
-      h[k] = {fma(r0, f.re(d0), p[k].re), fma(i0, f.im(d0), p[k].im)};
-      h[3 + k] = {fma(r1, f.re(d1), p[3 + k].re), fma(i1, f.im(d1), p[3 + k].im)};
+      h[k] = p[k] + f.turn(d0, 0, np);
+      h[3 + k] = p[3 + k] + f.turn(d1, 1, np);
     }
     // U h or U^dag h
-    const R cj = fwd ? R(1) : R(-1);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       cplx<R> t0 = {0, 0}, t1 = {0, 0};
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
         const cplx<R> q = fwd ? u[a * 3 + b] : u[b * 3 + a];
-        const cplx<R> m = {q.re, cj * q.im};
+        const cplx<R> m = {q.re, flip(q.im, !fwd)};
         cfma(t0, m, h[b]);
         cfma(t1, m, h[3 + b]);
       }
@@ -439,17 +449,20 @@ __device__ __forceinline__ void hop_lanes(const KGeom& g, bool active, int site,
       gg[3 + a] = t1;
     }
   }
-  // upper pair cf g, lower pair cf s i sigma g (cf s g): lanes 0-3 keep the upper, 4-7 the lower
-  const R cs = cf * s;
-  const R i0 = cs, r0 = f.imag ? -cs : cs, i1 = f.sgn1 * i0, r1 = f.sgn1 * r0;
+  // unit weights (uniform over the launch) need no multiplications
+  if (!g.unit) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) gg[k] = w * gg[k];
+  }
+  // upper pair g, lower pair s i sigma g (s g): lanes 0-3 keep the upper, 4-7 the lower
   const bool low = (hop & 4) != 0;
   cplx<R> keep[6];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const cplx<R> g0 = f.swap ? gg[3 + k] : gg[k], g1 = f.swap ? gg[k] : gg[3 + k];
-    const cplx<R> up0 = cf * gg[k], up1 = cf * gg[3 + k];
-    const cplx<R> lo0 = {r0 * f.re(g0), i0 * f.im(g0)};
-    const cplx<R> lo1 = {r1 * f.re(g1), i1 * f.im(g1)};
+    const cplx<R> up0 = {flip(gg[k].re, cneg), flip(gg[k].im, cneg)};
+    const cplx<R> up1 = {flip(gg[3 + k].re, cneg), flip(gg[3 + k].im, cneg)};
+    const cplx<R> lo0 = f.turn(g0, 0, cneg != neg), lo1 = f.turn(g1, 1, cneg != neg);
     const cplx<R> s0 = low ? up0 : lo0, s1 = low ? up1 : lo1;
     keep[k] = low ? lo0 : up0;
     keep[3 + k] = low ? lo1 : up1;
@@ -541,7 +554,9 @@ __device__ __forceinline__ void apply_sub(const KGeom& g, size_t rhs_off, int i,
 
 inline KGeom to_kgeom(const Geom& g) {
   KGeom k;
+  k.unit = true;
   for (int m = 0; m < 4; ++m) {
+    k.unit = k.unit && g.w[m] == 1.0;
     k.L[m] = g.L[m];
     k.wf[m] = (float)g.w[m];
     k.wd[m] = g.w[m];
