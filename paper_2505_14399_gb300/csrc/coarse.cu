@@ -514,28 +514,33 @@ int galerkin_build(zd* Op, zf* Op32, zd* Xpart, const zd* P, zdf* Pdf, zd* PtP, 
   // 6 rows x (2k)^2 complex multiply-adds); the tensor path also records the fp16 digit-plane
   // products it issues for them
   if (tc && !range_flag) return fail(MG_EINVAL, "galerkin: no range flag");
-  const double tc_flops = tc ? galerkin_tc_issued_flops(k, B) : 0.0;
-  ProfScope ps(tc ? "galerkin_tc" : df64 ? "galerkin_df64" : "galerkin_fp64",
-               16.0 * (12.0 * B.nd * B.d * k * 5 + 36.0 * B.nd * B.d),
-               768.0 * k * k * B.nd * B.d, tc ? tc_flops : 0.0, st);
+  {
+    // the contraction alone; the finish pass below is profiled apart
+    ProfScope ps(tc ? "galerkin_tc" : df64 ? "galerkin_df64" : "galerkin_fp64",
+                 16.0 * (12.0 * B.nd * B.d * k * 5 + 36.0 * B.nd * B.d),
+                 768.0 * k * k * B.nd * B.d, tc ? galerkin_tc_issued_flops(k, B) : 0.0, st);
+    if (tc) {
+      WMG_CUDA(cudaMemsetAsync(range_flag, 0, sizeof(int), st));
+      WMG_TRY(galerkin_hops_tc(Op, Xpart, Pdf, k, Ldf, hg, B, range_flag, st));
+    } else if (df64) {
+      WMG_TRY(launch_hop_ne<true>(grid, sh, st, Op, Xpart, P, Pdf, k, links, Ldf, hg, B));
+    } else {
+      WMG_TRY(launch_hop_ne<false>(grid, sh, st, Op, Xpart, P, Pdf, k, links, Ldf, hg, B));
+    }
+  }
   if (tc) {
     // tensor pipe (exact digit-plane products); entries outside its fixed-point range (links
     // that are not unitary, a prolongator that is not orthonormal) fall back to the FP32 units
-    int* flag = range_flag;
-    WMG_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), st));
-    WMG_TRY(galerkin_hops_tc(Op, Xpart, Pdf, k, Ldf, hg, B, flag, st));
     int h_flag = 0;
-    WMG_CUDA(cudaMemcpyAsync(&h_flag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    WMG_CUDA(cudaMemcpyAsync(&h_flag, range_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     WMG_CUDA(cudaStreamSynchronize(st));
     if (h_flag) {
       ProfScope pf("galerkin_tc_range_fallback", 0.0, 0.0, st);
       WMG_TRY(launch_hop_ne<true>(grid, sh, st, Op, Xpart, P, Pdf, k, links, Ldf, hg, B));
     }
-  } else if (df64) {
-    WMG_TRY(launch_hop_ne<true>(grid, sh, st, Op, Xpart, P, Pdf, k, links, Ldf, hg, B));
-  } else {
-    WMG_TRY(launch_hop_ne<false>(grid, sh, st, Op, Xpart, P, Pdf, k, links, Ldf, hg, B));
   }
+  // partials and +mu blocks in; X, -mu blocks and the FP32 copy of all nine out
+  ProfScope pf("coarse_finish", 4.0 * k * k * B.d * (16.0 * (8 + 5) + 8.0 * 9), 64.0 * k * k * B.d, st);
   const size_t fsh = sizeof(zd) * 2 * 2 * k * (2 * k + 1);
   WMG_TRY(smem_attr(galerkin_finish_kernel, fsh));
   galerkin_finish_kernel<<<B.d, GTH, fsh, st>>>(Op, Op32, Xpart, PtP, k, B);
