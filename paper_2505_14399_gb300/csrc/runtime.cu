@@ -204,7 +204,7 @@ cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  // under capture the allocation is the graph's, not a pool's
+  // an allocation from a pool cannot be captured (it invalidates the capture); this one is the graph's
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
   if (cs != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, st);
