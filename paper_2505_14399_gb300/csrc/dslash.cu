@@ -32,8 +32,12 @@ constexpr int kNumForms = 6, kNumSingle = 4, kNumF64 = 4, kNumHalf = 9;
 // S: the storage type; SN: its form for fields that are only 16-byte aligned.  Fields or ABI links
 // less aligned than S's accesses and the windowed links want run the same shapes on 16-byte accesses
 // and element loads, under tuning keys of their own; in FP32 arithmetic on consecutive sites, which
-// suit those accesses better than tiles (complex float at 16^3x32, 1 / 4 / 12 right-hand sides: 20.4
-// / 63 / 165 us, with tiles 21.6 / 71 / 186).
+// mostly suit those accesses better than tiles (complex float at 16^3x32, 1 / 4 / 12 right-hand
+// sides: 20.4 / 63 / 165 us, with tiles 21.6 / 71 / 186), with the uncapped single-site shape and
+// the several-right-hand-side ones on tiles as kTiled more candidates (8^4, 12 right-hand sides: 9
+// us, consecutive sites 12-14).
+constexpr int kTiled = 3, kTiledSingle = 1;
+
 template <typename S, typename SN>
 int launch_typed(void* out, const void* in, const void* links, const Geom& g, int parity,
                  int dagger, int nrhs, cudaStream_t st, size_t in_stride, size_t out_stride,
@@ -54,10 +58,13 @@ int launch_typed(void* out, const void* in, const void* links, const Geom& g, in
   bool wide = !site32 || (al & 31) == 0;
   // the windowed link loads (load_link, LL = 3) start at a 16-byte boundary
   if (layout == 0 && !f64) wide = wide && ((uintptr_t)links & 15) == 0;
-  if (!wide && !f64) k.tile.on = 0;
+  const int forms = f64 ? kNumF64 : nrhs == 1 ? kNumSingle : kNumForms;
   auto run = [&](int v) {
     if (!wide) {
-      launch_stencil<SN>(v, dagger, layout, out, in, links, k, parity, nsites, nrhs, st, in_stride, out_stride);
+      KGeom kn = k;
+      if (!f64) kn.tile.on = k.tile.on && v >= forms;
+      if (v >= forms) v = v == forms ? 0 : v - forms + 3;   // 0, 4, 5 on tiles
+      launch_stencil<SN>(v, dagger, layout, out, in, links, kn, parity, nsites, nrhs, st, in_stride, out_stride);
       return;
     }
     if (v >= kNumForms) {   // half storage only
@@ -69,9 +76,9 @@ int launch_typed(void* out, const void* in, const void* links, const Geom& g, in
     launch_stencil<S>(v, dagger, layout == 0 && !f64 ? 3 : layout, out, in, links, k, parity, nsites,
                       nrhs, st, in_stride, out_stride);
   };
-  const int forms = f64 ? kNumF64 : nrhs == 1 ? kNumSingle
-                    : wide && es == 4 ? kNumHalf : kNumForms;
-  int v = tuned_variant(dtype + 16 * layout + (wide ? 0 : 64), parity, dagger, g.V, nrhs, st, forms, run);
+  const int more = f64 ? 0 : !wide ? (nrhs == 1 ? kTiledSingle : kTiled)
+                   : nrhs > 1 && es == 4 ? kNumHalf - kNumForms : 0;
+  int v = tuned_variant(dtype + 16 * layout + (wide ? 0 : 64), parity, dagger, g.V, nrhs, st, forms + more, run);
   if (v < 0) return fail(MG_ECUDA, "dslash autotune failed");
   // algorithmic bytes: in + out spinors per rhs and each link once (parity: all 4V links),
   // 18 reals per link whatever the stored form
