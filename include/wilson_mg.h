@@ -180,7 +180,9 @@ int mg_probe_fma_peak(int dtype, double* tflops, void* stream);
  *     sites, ordered by checkerboard index site/2 (requires every dims[mu] even).
  *   dtype: storage of out, in and links (all the same); MG_F16 / MG_BF16 accumulate
  *   in FP32.  nrhs fields are processed in one launch sharing the links.
- * Returns MG_EINVAL for bad dims / dtype / nrhs < 1 / NULL pointers.
+ *   Device fields are 16-byte aligned, links to one complex number of their dtype (here
+ *   and wherever fields and links are given below).
+ * Returns MG_EINVAL for bad dims / dtype / nrhs < 1 / NULL or misaligned pointers.
  * ------------------------------------------------------------------------------- */
 int wilson_dslash(void* out, const void* in, const void* links, const int dims[4],
                   double kappa, const double hop_weight[4], const int bc_phase[4],

@@ -206,7 +206,10 @@ cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   // an allocation from a pool cannot be captured (it invalidates the capture); this one is the graph's
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    cs = cudaStreamCaptureStatusNone;
+  }
   if (cs != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, st);
   cudaMemPool_t pool = scratch_pool(dev);
   if (!pool) return cudaMallocAsync(p, bytes, st);
