@@ -126,7 +126,8 @@ def load_peaks():
 # over the launches of one warm-up and one timed step) from one ncu capture of this bench
 # command on its workload, reported as roofline.traffic for that kernel; an entry is removed
 # whenever its kernel changes, until it is captured again.
-NCU_TRAFFIC = {}
+# profiles/dslash_proj_16x16x16x32_traffic.md
+NCU_TRAFFIC = {("dslash_proj", "c2_16^3x32_near_critical"): 520.1e6}
 
 
 def kernel_bound(name, alu, peaks, peak_kind):

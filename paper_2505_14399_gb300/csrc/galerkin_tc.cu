@@ -37,7 +37,8 @@
 // the critical path.  With warp-level mma.sync (bf16 digits) the products, their ldmatrix reads
 // and the accumulators lived in the staging warps, which met at two barriers per batch: 2.57 ms
 // at 16^3x32, k = 12 (blocks of 4^4) and 18.6 ms at 16^3x64, k = 24 (2x2x2x4); here 1.42 and
-// 9.25 ms.  Bound now by the staging warps' FP32 and issue slots (k = 12: about 4700 cycles a
+// 9.25 ms.  (These and the times below hold the finish pass and the range flag's round trip, 0.05
+// and 1.5 ms; the contraction alone takes 1.37 and 7.74 ms.)  Bound now by the staging warps' FP32 and issue slots (k = 12: about 4700 cycles a
 // batch, two CTAs per SM), for small blocks also by a CTA's start, four folds and two outputs (k =
 // 24, 32 sites: together a third of its 78 000 cycles).  P(x) is loaded between the transport and
 // the digits: before the transport its eight registers made the loop spill (1.54 against 1.48 ms,
